@@ -407,16 +407,29 @@ static size_t simt_workspace(const okq_cache* c, int layer_count, int num_splits
   return (size_t)layer_count * c->batch * c->n_kv_heads * S * sizeof(Partial);
 }
 
-// one PartialF per (CTA, (sequence, head)) overlap, then one PairPartial per (warp pair, (sequence, head))
-// overlap: slot = unit index + CTA (or global pair) index, both non-decreasing along the window axis
+// one PartialF per (CTA, (sequence, head)) overlap, then one WarpPiece per (warp, (sequence, head))
+// overlap: slot = unit index + CTA (or global warp) index, both non-decreasing along the window axis
 static size_t mma_partials_bytes(const okq_cache* c, int layer_count, int num_splits) {
   return ((size_t)layer_count * c->batch * c->n_kv_heads + mma_ctas(c, layer_count, num_splits)) * sizeof(PartialF);
 }
 static size_t mma_workspace(const okq_cache* c, int layer_count, int num_splits) {
   return mma_partials_bytes(c, layer_count, num_splits) +
-         ((size_t)layer_count * c->batch * c->n_kv_heads + (size_t)MMA_PAIRS * mma_ctas(c, layer_count, num_splits)) *
-             sizeof(PairPartial);
+         ((size_t)layer_count * c->batch * c->n_kv_heads + (size_t)DECODE_WARPS * mma_ctas(c, layer_count, num_splits)) *
+             sizeof(WarpPiece);
 }
+
+// Grid of the no-allocation form: what is accepted is fixed (the documented limit: one 12736-byte and one 12832-byte record
+// per unit and CTA resp. eighth of a CTA must fit the scratch); of the asked number of CTAs as many run as have room for
+// their warps' pieces.  0: too large.
+static int noalloc_ctas(const okq_cache* c, int layer_count, int num_splits) {
+  const size_t units = (size_t)layer_count * c->batch * c->n_kv_heads;
+  const int want = mma_ctas(c, layer_count, num_splits);
+  if ((units + want) * 12736 + (units + 8 * (size_t)want) * 12832 > (size_t)OKQ_NOALLOC_SCRATCH_BYTES) return 0;
+  const size_t fit = ((size_t)OKQ_NOALLOC_SCRATCH_BYTES - units * (sizeof(PartialF) + sizeof(WarpPiece))) /
+                     (sizeof(PartialF) + DECODE_WARPS * sizeof(WarpPiece));
+  return fit < (size_t)want ? (int)fit : want;
+}
+static_assert(sizeof(PartialF) + sizeof(WarpPiece) <= 12736 + 12832, "a request at the documented limit has room for its units");
 
 static okq_status check_decode(const okq_cache* cache, int32_t layer, int32_t layer_count, const void* q,
                                const float* signs, const float* R, int32_t n_R, void* workspace,
@@ -433,13 +446,14 @@ static okq_status check_decode(const okq_cache* cache, int32_t layer, int32_t la
 }
 
 static DecodeParams make_params(const okq_cache* cache, int32_t layer, int32_t layer_count, const void* q,
-                                float sm_scale, const float* signs, const float* R, int32_t n_R, float* out) {
+                                float sm_scale, const float* signs, const float* R, int32_t n_R, float* out,
+                                int num_splits) {
   DecodeParams P;
   P.cv = make_view(cache);
-  P.layer0 = layer; P.layer_count = layer_count; P.n_splits = 1;
+  P.layer0 = layer; P.layer_count = layer_count; P.n_splits = num_splits;
   P.group = cache->n_q_heads / cache->n_kv_heads;
   P.q = static_cast<const __half*>(q); P.signs = signs; P.R = R; P.n_R = n_R; P.sm_scale = sm_scale;
-  P.partials = nullptr; P.partials_f = nullptr; P.pair_parts = nullptr; P.out = out;
+  P.partials = nullptr; P.partials_f = nullptr; P.pieces = nullptr; P.out = out;
   return P;
 }
 
@@ -479,10 +493,9 @@ okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t l
   for (int l0 = 0; l0 < layer_count; l0 += layers_per_launch) {
     const int lc = layer_count - l0 < layers_per_launch ? layer_count - l0 : layers_per_launch;
     DecodeParams P = make_params(cache, layer + l0, lc, static_cast<const __half*>(q) + l0 * q_stride, sm_scale,
-                                 signs + (size_t)l0 * D, R + (size_t)l0 * n_R * 3 * D * D, n_R, out + l0 * q_stride);
+                                 signs + (size_t)l0 * D, R + (size_t)l0 * n_R * 3 * D * D, n_R, out + l0 * q_stride, num_splits);
     P.partials_f = static_cast<PartialF*>(workspace);
-    P.pair_parts = reinterpret_cast<PairPartial*>(static_cast<unsigned char*>(workspace) +
-                                                  mma_partials_bytes(cache, lc, num_splits));
+    P.pieces = reinterpret_cast<WarpPiece*>(static_cast<unsigned char*>(workspace) + mma_partials_bytes(cache, lc, num_splits));
     const int n_cta = mma_ctas(cache, lc, num_splits);
     st = launch_decode_mma(P, n_cta, s, g_ev_before, g_ev_after);
     if (st != OKQ_OK) return st;
@@ -499,7 +512,7 @@ okq_status okq_decode_attention_noalloc(const okq_cache* cache, int32_t layer, i
   // the largest launch of the call decides how much of the fixed scratch is needed
   const int layers_per_launch = cache->batch >= MAX_ENTRIES ? 1 : MAX_ENTRIES / cache->batch;
   const int lc_max = layer_count < layers_per_launch ? layer_count : layers_per_launch;
-  if (mma_workspace(cache, lc_max, num_splits) > (size_t)OKQ_NOALLOC_SCRATCH_BYTES) return OKQ_ERR_WORKSPACE;
+  if (noalloc_ctas(cache, lc_max, num_splits) <= 0) return OKQ_ERR_WORKSPACE;
   void* scratch = nullptr;
   st = noalloc_scratch(&scratch);
   if (st != OKQ_OK) return st;
@@ -511,11 +524,11 @@ okq_status okq_decode_attention_noalloc(const okq_cache* cache, int32_t layer, i
   for (int l0 = 0; l0 < layer_count; l0 += layers_per_launch) {
     const int lc = layer_count - l0 < layers_per_launch ? layer_count - l0 : layers_per_launch;
     DecodeParams P = make_params(cache, layer + l0, lc, static_cast<const __half*>(q) + l0 * q_stride, sm_scale,
-                                 signs + (size_t)l0 * D, R + (size_t)l0 * n_R * 3 * D * D, n_R, out + l0 * q_stride);
+                                 signs + (size_t)l0 * D, R + (size_t)l0 * n_R * 3 * D * D, n_R, out + l0 * q_stride, num_splits);
     P.partials_f = static_cast<PartialF*>(scratch);
-    P.pair_parts = reinterpret_cast<PairPartial*>(static_cast<unsigned char*>(scratch) +
-                                                  mma_partials_bytes(cache, lc, num_splits));
-    st = launch_decode_mma(P, mma_ctas(cache, lc, num_splits), s, nullptr, nullptr);
+    const int n_cta = noalloc_ctas(cache, lc, num_splits);
+    P.pieces = reinterpret_cast<WarpPiece*>(P.partials_f + (size_t)lc * cache->batch * cache->n_kv_heads + n_cta);
+    st = launch_decode_mma(P, n_cta, s, nullptr, nullptr);
     if (st != OKQ_OK) return st;
   }
   return launch_status();
@@ -528,7 +541,7 @@ okq_status okq_decode_attention_simt(const okq_cache* cache, int32_t layer, int3
   okq_status st = check_decode(cache, layer, layer_count, q, signs, R, n_R, workspace, workspace_bytes, num_splits, out);
   if (st != OKQ_OK) return st;
   if (cache->schedule != OKQ_SCHEDULE_WINDOW) return OKQ_ERR_UNSUPPORTED;   // the cross-check kernels know one schedule
-  DecodeParams P = make_params(cache, layer, layer_count, q, sm_scale, signs, R, n_R, out);
+  DecodeParams P = make_params(cache, layer, layer_count, q, sm_scale, signs, R, n_R, out, num_splits);
   P.n_splits = num_splits > 0 ? num_splits : auto_splits(cache, layer_count);
   P.partials = static_cast<Partial*>(workspace);
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -4,509 +4,71 @@
 //     S^T[head][token]   = W[head][channel] * C_k[channel][token]        (per 32-token window)
 //     O^T[channel][head] = C_v[channel][token] * P[token][head]
 // and run on mma.sync.m16n8k16 with the 2-bit codes unpacked in registers:
-//   * a code field masked out of its 32-bit word *is* an fp16 subnormal (code * 4^j * 2^-24,
+//   * a key-code field masked out of its 32-bit word *is* an fp16 subnormal (code * 4^j * 2^-24,
 //     j the field's position), so unpacking is one AND per two codes; the factor 4^j is folded
-//     into the other operand (the query weights, or the softmax numerators);
+//     into the query weights;
 //   * W = q'_c * s_gc is split into an fp16 high and low part, which fill the 16 rows of the
-//     m16 tile (8 heads x {hi, lo}), so the split costs no extra tensor work; the per-window
-//     bias sum_c q'_c m_gc goes through the same pipe against a constant operand;
-//   * the value codebook {-b,-a,a,b} is affine in the two code bits:
-//     cb[c] = (b-a)*c + (3a-b)*bit1(c) - b, so two bit-plane products plus the running sum
-//     of the weights reproduce it exactly.
-// A CTA runs 8 warp pairs.  The "score" warp of a pair computes the scores and the online
-// softmax (FlashAttention order) and hands the fp16 numerators to its "value" warp through
-// shared memory; the value warp accumulates the codebook sums of the previous window meanwhile
-// and streams the window records through a cp.async ring, two windows ahead of the score warp
-// (with MXFP4 metadata it also expands them into the fp16 planes).  One named barrier per pair
-// and iteration keeps the two in step (no spin-waits anywhere).  Windows whose tokens all belong
-// to the modality the registers hold take a straight-line path.  Values accumulate in the rotated
-// basis of the current modality, in registers for at most 32 windows at a time; each modality's
-// running sums live in shared memory.
+//     m16 tile (8 heads x {hi, lo}), so the split costs no extra tensor work;
+//   * the bias sum_c q'_c m_gc of eight consecutive windows comes out of one set of eight products,
+//     the windows' m planes being the eight columns of the B operand (one window at a time the same
+//     products would have eight equal columns);
+//   * value codes become fp16 codebook levels by byte permutes: four codes are four nibbles of a
+//     selector, one look-up gives the high bytes of their levels, and two permutes put the common low
+//     byte under them.  One product per 16 x 16 codes then replaces two bit-plane products.
+// A warp does all of a window by itself: scores, online softmax (FlashAttention order), value sums.
+// The score tile's accumulator layout is the value product's operand layout, so the numerators
+// never leave their lane.  Records arrive through a cp.async ring, PREFETCH windows ahead (bulk copies were measured too:
+// each costs the warp about 15 instructions to hand over, against 5 copies of 512 bytes with immediate offsets).
+// A warp's registers hold the value sums of one modality in its rotated basis; tokens of another
+// modality inside its range are "visitors", whose products are added straight to the warp's piece
+// in global memory (vector reductions), as are the registers every FLUSH windows.
+// What bounds it: dispatch slots.  Per window a warp issues about 600 instructions (53 of them products); LOP3, PRMT,
+// IMAD and HFMA2 take two dispatch cycles of an SM sub-partition each, a product 8.6 by itself and about 10 with the
+// masks that feed it, so more warps do not help: 12 per CTA with 168 registers each is where the accumulators, both
+// operand sets and the next window's scores fit without spills.  step7b (28 layers x 8 x 16384 tokens, 1.233 GB of
+// records), whole call: 570 us with a score and a value warp per window pair and two bit-plane products per 16 x 16
+// codes, 515 us in this form.  Two windows per turn (8 warps, 233 registers) measured 541 us, an unrolled pair of turns
+// 594 us (the loop outgrows the instruction cache).
 // The grid is persistent: CTA i owns an equal slice of the flattened (layer, sequence, head,
-// window) axis, each of its pairs an eighth of that slice, which the pair walks without any
-// block-wide step; at the end the block merges its pairs' pieces into one partial per
+// window) axis, each of its warps an equal part of that slice, which the warp walks without any
+// block-wide step; at the end the block merges its warps' pieces into one partial per
 // (sequence, head) it touched.  The combine kernel merges the partials, adds the raw fp16 tail
 // tokens, applies R_m^T once per head and normalises.
-#include <type_traits>
-#include "okq_common.cuh"
-#include "okq_device.cuh"
-#include "okq_decode_shared.cuh"
-#include "okq_decode_frag.cuh"
+#include "okq_decode_walk.cuh"
 
 namespace okq {
 
 namespace {
 
-constexpr int NPAIR = MMA_PAIRS;                // warp pairs per CTA
-constexpr int NTHREADS = NPAIR * 64;
-constexpr int NSTAGE = 4;                       // record ring per pair
-constexpr int PREFETCH = 2;                     // windows in flight ahead of the score warp
-// staged window image: the fp16-metadata record, the window's 32 modality bytes and, with MXFP4
-// metadata, the 136 stored metadata bytes (decoded into the first 512 bytes by the score warp)
-constexpr int STAGE_MOD = RECORD_BYTES, STAGE_MX = RECORD_BYTES + 32;
-template <int FMT> constexpr int stage_bytes() { return FMT == FMT_MXFP4 ? STAGE_MX + 144 : STAGE_MX; }
-constexpr float RESCALE_LOG2 = 3.0f;            // numerators stay below 2^3 * 2^6 * vnorm in fp16
-constexpr int FLUSH = 32;                       // windows a value warp accumulates in registers at most
-constexpr int SPILL_STRIDE = 36;                // floats per lane in the deposited sums: 33 used, 144-byte rows
-
-struct Handoff {
-  uint4 pb[32];         // per lane: numerators p * vnorm * 2^6 / 4^nu of its 8 tokens, fp16 pairs (nu = x,y,z,w)
-  float m[GP];          // running maximum per head after this window (log2 domain)
-  float alpha[GP];      // factor the value accumulators must be multiplied by before this window
-  int rescale;          // non-zero if any alpha != 1
-  int pad[15];
-};
-
-template <int FMT>
-struct MmaSmem {
-  __align__(16) unsigned char stage[NPAIR][NSTAGE][stage_bytes<FMT>()];
-  __align__(16) Handoff hand[NPAIR][2];
-  __align__(16) float spill[NPAIR][3][32][SPILL_STRIDE];   // [pair][modality][lane]: the lane's 33 sums, 128-bit rows
-  float spill_m[NPAIR][3][GP];
-  float fin_w[NPAIR][2][GP];   // running maximum and weight sum a pair's score warp ended its last range with
+template <int FMT> struct MmaSmem {
+  WarpSmem<FMT> w[NWARP];
+  __align__(16) uint4 qlo[NWARP][4][32];   // low parts of a warp's query fragments
   int prefix[MAX_ENTRIES + 1];
 };
 
 constexpr int MB_SEG = 32;                      // (sequence, head) units merged per batch at the end of the launch
 struct MergeSmem {
-  int pa[MB_SEG], pb[MB_SEG];                   // first and last warp pair that worked on the unit (pb < pa: none)
-  int last_kept[MB_SEG];                        // whether pair pb's piece is in shared memory (all before it are)
-  float meta[MB_SEG + NPAIR][5 * GP];           // per piece: sm[3][GP], wm[GP], wl[GP]; index = unit + pair - pa[0]
-  float M[MB_SEG][GP];                          // merged running maximum
-  float fac[MB_SEG + NPAIR][3][GP];             // per piece, modality and head: exp2(sm - M), 0 where the piece holds nothing
+  int pa[MB_SEG], pb[MB_SEG];                   // first and last warp that worked on the unit (pb < pa: none)
+  float meta[MB_SEG + NWARP][2 * GP];           // per piece: wm[GP], wl[GP]; index = unit + warp - pa[0]
+  int mask[MB_SEG + NWARP];                     // per piece: modalities it holds
+  float fac[MB_SEG + NWARP][GP];                // per piece and head: exp2(wm - merged maximum)
 };
-
-struct Segment {
-  const unsigned char* rec0;   // first record of the (layer, sequence, head)
-  const unsigned char* mod0;   // modality row of the sequence
-  int w0, n_my;                // this pair's windows of that (layer, sequence, head): first window, count
-  const __half* q;             // query rows of the KV head's group: [group][128]
-  const float* signs;          // Hadamard signs of the layer
-  PairPartial* piece;          // where the pair leaves what it accumulated ...
-  bool keep;                   // ... unless this is the last unit of the pair's range: then it stays in shared memory
-};
-
-// Scores of one packed window against the group's queries, by one warp, from a staged image of the window's key
-// part ((m, s) planes, key norms, key codes at their record offsets): the split-K kernel's score step.
-// sc[nu][e] = log2-domain score of head g = lane >> 2 against token 8 nu + 2 (lane & 3) + e.
-__device__ __forceinline__ void window_scores_mma(const unsigned char* st, const uint2 (&qreg)[16], float fsc, int lane,
-                                                  float (&sc)[4][2]) {
-  const int t = lane & 3;
-  const uint4* mp = reinterpret_cast<const uint4*>(st + OFF_KM + 64 * t);
-  const uint4* sp = reinterpret_cast<const uint4*>(st + OFF_KS + 64 * t);
-  float dbA[4] = {0.f, 0.f, 0.f, 0.f}, dbB[4] = {0.f, 0.f, 0.f, 0.f};
-  float d[4][4];
-#pragma unroll
-  for (int nu = 0; nu < 4; nu++)
-#pragma unroll
-    for (int i = 0; i < 4; i++) d[nu][i] = 0.f;
-  const uint4 kc0 = *reinterpret_cast<const uint4*>(st + OFF_KCODE + 16 * kpiece_slot(lane));
-  const uint4 kc1 = *reinterpret_cast<const uint4*>(st + OFF_KCODE + 16 * kpiece_slot(32 + lane));
-  const uint32_t kw[4][2] = {{kc0.x, kc0.y}, {kc0.z, kc0.w}, {kc1.x, kc1.y}, {kc1.z, kc1.w}};
-#pragma unroll
-  for (int kq = 0; kq < 4; kq++) {
-    const uint4 m4 = mp[kq], s4 = sp[kq];
-#pragma unroll
-    for (int half = 0; half < 2; half++) {
-      const int kappa = 2 * kq + half;
-      const uint2 q0 = qreg[2 * kappa], q1 = qreg[2 * kappa + 1];
-      uint32_t a0, a1, a2, a3;
-      if (half) mma16816(dbB, q0.x, q0.y, q1.x, q1.y, m4.z, m4.w);
-      else mma16816(dbA, q0.x, q0.y, q1.x, q1.y, m4.x, m4.y);
-      split_product(u2h(q0.x), u2h(q0.y), u2h(half ? s4.z : s4.x), a0, a1);
-      split_product(u2h(q1.x), u2h(q1.y), u2h(half ? s4.w : s4.y), a2, a3);
-      const int ww = kappa >> 2, sh = (kappa >> 1) & 1;
-      const uint32_t mk0 = half ? 0x00300030u : 0x00030003u;
-      const uint32_t mk1 = half ? 0x00c000c0u : 0x000c000cu;
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++) {
-        uint32_t src = sh ? (kw[nu][ww] >> 8) : kw[nu][ww];
-        mma16816(d[nu], a0, a1, a2, a3, src & mk0, src & mk1);
-      }
-    }
-  }
-  const uint4 kn4 = *reinterpret_cast<const uint4*>(st + OFF_KNORM + 16 * t);
-  const uint32_t knu[4] = {kn4.x, kn4.y, kn4.z, kn4.w};
-  const float bias0 = ((dbA[0] + dbB[0]) + (dbA[2] + dbB[2])) * 0x1p-24f;   // the code sums carry 2^-24, the bias does not
-#pragma unroll
-  for (int nu = 0; nu < 4; nu++) {
-    const float2 kn = __half22float2(u2h(knu[nu]));
-    sc[nu][0] = ((d[nu][0] + d[nu][2]) + bias0) * (kn.x * fsc);
-    sc[nu][1] = ((d[nu][1] + d[nu][3]) + bias0) * (kn.y * fsc);
-  }
-}
-
-// ---------------------------------------------------------------- score warp
-template <int FMT>
-__device__ __forceinline__ void score_warp(MmaSmem<FMT>& sm, const Segment& sg, int G, float sm_scale, int pair,
-                                           int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  float run_m = -INFINITY, run_l = 0.f;
-
-  uint2 qreg[16];
-  float fsc;
-  query_fragments(sg.q, sg.signs, G, sm_scale, lane, qreg, fsc);   // while the first windows are on their way
-  pair_barrier(pair);   // the value warp has the first window in place
-
-  for (int k = 0; k <= sg.n_my; k++) {
-    if (k < sg.n_my) {
-      // copied (and, with MXFP4 metadata, expanded into the fp16 planes) by the value warp, complete before the last barrier
-      unsigned char* st = sm.stage[pair][k % NSTAGE];
-      const uint4* mp = reinterpret_cast<const uint4*>(st + OFF_KM + 64 * t);
-      const uint4* sp = reinterpret_cast<const uint4*>(st + OFF_KS + 64 * t);
-      // bias sum_c q'_c m_c (two independent chains)
-      // and scores sum_c q'_c s_c code_c, one k-step (16 channels) at a time
-      float dbA[4] = {0.f, 0.f, 0.f, 0.f}, dbB[4] = {0.f, 0.f, 0.f, 0.f};
-      float d[4][4];
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++)
-#pragma unroll
-        for (int i = 0; i < 4; i++) d[nu][i] = 0.f;
-      const uint4 kc0 = *reinterpret_cast<const uint4*>(st + OFF_KCODE + 16 * kpiece_slot(lane));
-      const uint4 kc1 = *reinterpret_cast<const uint4*>(st + OFF_KCODE + 16 * kpiece_slot(32 + lane));
-      const uint32_t kw[4][2] = {{kc0.x, kc0.y}, {kc0.z, kc0.w}, {kc1.x, kc1.y}, {kc1.z, kc1.w}};
-#pragma unroll
-      for (int kq = 0; kq < 4; kq++) {
-        const uint4 m4 = mp[kq], s4 = sp[kq];
-#pragma unroll
-        for (int half = 0; half < 2; half++) {
-          const int kappa = 2 * kq + half;
-          const uint2 q0 = qreg[2 * kappa], q1 = qreg[2 * kappa + 1];
-          uint32_t a0, a1, a2, a3;
-          // bias: the stored m * 4^j is the B operand as it is (every column the same), the query fragments
-          // (hi rows, lo rows) the A operand
-          if (half) mma16816(dbB, q0.x, q0.y, q1.x, q1.y, m4.z, m4.w);
-          else mma16816(dbA, q0.x, q0.y, q1.x, q1.y, m4.x, m4.y);
-          split_product(u2h(q0.x), u2h(q0.y), u2h(half ? s4.z : s4.x), a0, a1);
-          split_product(u2h(q1.x), u2h(q1.y), u2h(half ? s4.w : s4.y), a2, a3);
-          const int ww = kappa >> 2, sh = (kappa >> 1) & 1;
-          const uint32_t mk0 = half ? 0x00300030u : 0x00030003u;
-          const uint32_t mk1 = half ? 0x00c000c0u : 0x000c000cu;
-#pragma unroll
-          for (int nu = 0; nu < 4; nu++) {
-            uint32_t src = sh ? (kw[nu][ww] >> 8) : kw[nu][ww];
-            mma16816(d[nu], a0, a1, a2, a3, src & mk0, src & mk1);
-          }
-        }
-      }
-      // online softmax (log2 domain); this lane: head g, tokens 8*nu + 2*t + e
-      const uint4 kn4 = *reinterpret_cast<const uint4*>(st + OFF_KNORM + 16 * t);
-      const uint4 vn4 = *reinterpret_cast<const uint4*>(st + OFF_VNORM + 16 * t);
-      const uint32_t knu[4] = {kn4.x, kn4.y, kn4.z, kn4.w}, vnu[4] = {vn4.x, vn4.y, vn4.z, vn4.w};
-      // the code sums carry 2^-24 (subnormal code operands), the bias sum does not
-      const float bias0 = ((dbA[0] + dbB[0]) + (dbA[2] + dbB[2])) * 0x1p-24f, bias1 = bias0;
-      // sc = score / fsc: the head's scale fsc > 0 (query scaling, 1/sqrt(d), log2 e) enters the exponent below in
-      // one multiply-add and the maximum once
-      float sc[4][2];
-      float mx = -INFINITY;
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++) {
-        float2 kn = __half22float2(u2h(knu[nu]));
-        sc[nu][0] = ((d[nu][0] + d[nu][2]) + bias0) * kn.x;
-        sc[nu][1] = ((d[nu][1] + d[nu][3]) + bias1) * kn.y;
-        mx = fmaxf(mx, fmaxf(sc[nu][0], sc[nu][1]));
-      }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      mx *= fsc;
-      // the reference maximum only moves when it is exceeded by more than 2^RESCALE_LOG2, so the
-      // value accumulators are rescaled a few times per range instead of at every new maximum
-      const float m_new = mx > run_m + RESCALE_LOG2 ? mx : run_m;
-      const float alpha = ex2(run_m - m_new);  // 0 on the first window
-      const int changed = __any_sync(0xffffffffu, m_new > run_m);
-      run_l *= alpha;
-      run_m = m_new;
-      Handoff& ho = sm.hand[pair][k & 1];
-      uint32_t pb[4];
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++) {
-        float2 vn = __half22float2(u2h(vnu[nu]));
-        const float off = (float)(6 - 2 * nu) - run_m;
-        const float cinv = (float)(1 << (2 * nu)) * (1.0f / 64.0f);
-        float p0 = ex2(fmaf(sc[nu][0], fsc, off)), p1 = ex2(fmaf(sc[nu][1], fsc, off));
-        run_l = fmaf(p0 + p1, cinv, run_l);
-        pb[nu] = pack_sat(p0 * vn.x, p1 * vn.y);
-      }
-      ho.pb[lane] = make_uint4(pb[0], pb[1], pb[2], pb[3]);
-      if (t == 0) { ho.m[g] = run_m; ho.alpha[g] = alpha; }
-      if (lane == 0) ho.rescale = changed;
-    }
-    pair_barrier(pair);
-  }
-  run_l += __shfl_xor_sync(0xffffffffu, run_l, 1);
-  run_l += __shfl_xor_sync(0xffffffffu, run_l, 2);
-  if (t == 0) {
-    if (sg.keep) { sm.fin_w[pair][0][g] = run_m; sm.fin_w[pair][1][g] = run_l; }
-    else { sg.piece->wm[g] = run_m; sg.piece->wl[g] = run_l; }
-  }
-}
-
-// ---------------------------------------------------------------- value warp
-template <int FMT>
-__device__ __forceinline__ void value_warp(MmaSmem<FMT>& sm, const Segment& sg, int pair, int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  float acc[8][4];
-#pragma unroll
-  for (int mu = 0; mu < 8; mu++)
-#pragma unroll
-    for (int i = 0; i < 4; i++) acc[mu][i] = 0.f;
-  float run_S = 0.f;
-  int cur_mod = -1;
-  int since = 0;             // windows accumulated in registers since the last deposit
-  // nothing deposited yet (the deposited registers themselves are only read where a maximum says so)
-  if (lane < 3 * GP) (&sm.spill_m[pair][0][0])[lane] = -INFINITY;
-  __syncwarp();
-  // The value warp also streams the records: it has registers to spare and the copies of window k + 2 are issued
-  // while it works on window k - 1; a window is complete (cp.async.wait_group) before the barrier after which the
-  // score warp reads it.
-  auto issue = [&](int k) {
-    if (k < sg.n_my) {
-      const int win = sg.w0 + k;
-      unsigned char* dst = sm.stage[pair][k % NSTAGE];
-      if (FMT == FMT_FP16) {
-        const unsigned char* src = sg.rec0 + (size_t)win * RECORD_BYTES;
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-          int c16 = lane + 32 * i;
-          if (c16 < RECORD_BYTES / 16) cp_async16(dst + 16 * c16, src + 16 * c16);
-        }
-      } else {
-        // body (16-byte aligned) behind the 512 bytes the decoded (m, s) will occupy; the 136
-        // metadata bytes are only 8-byte aligned
-        // two windows share one block [meta 0 | meta 1 | body 0 | body 1]: offsets in 32 bits
-        const uint32_t odd = (uint32_t)win & 1u, blk = ((uint32_t)win >> 1) * (uint32_t)MX_PAIR_BYTES;
-        const unsigned char* body = sg.rec0 + (blk + 2u * MX_META_BYTES + odd * (uint32_t)BODY_BYTES);
-        const unsigned char* meta = sg.rec0 + (blk + odd * (uint32_t)MX_META_BYTES);
-#pragma unroll
-        for (int i = 0; i < 5; i++) {
-          int c16 = lane + 32 * i;
-          if (c16 < BODY_BYTES / 16) cp_async16(dst + META_BYTES_FP16 + 16 * c16, body + 16 * c16);
-        }
-        if (lane < MX_META_BYTES / 8) cp_async8(dst + STAGE_MX + 8 * lane, meta + 8 * lane);
-      }
-      if (lane < 2) cp_async16(dst + STAGE_MOD + 16 * lane, sg.mod0 + (size_t)win * W + 16 * lane);
-    }
-    cp_async_commit();
-  };
-#pragma unroll
-  for (int k = 0; k < PREFETCH; k++) issue(k);
-  // with MXFP4 metadata: the stored (m, s) of a window that has landed, expanded into the fp16 planes of its staged image
-  auto expand_meta = [&](int k) {
-    if (FMT == FMT_MXFP4 && k < sg.n_my) {
-      __syncwarp();   // the other lanes' copies have landed too
-      unsigned char* st = sm.stage[pair][k % NSTAGE];
-      uint2 m4, s4;
-      mx_decode_lane(st + STAGE_MX, lane, m4, s4);
-      *reinterpret_cast<uint2*>(st + OFF_KM + 8 * lane) = m4;
-      *reinterpret_cast<uint2*>(st + OFF_KS + 8 * lane) = s4;
-    }
-  };
-  cp_async_wait<PREFETCH - 1>();
-  expand_meta(0);
-  pair_barrier(pair);   // window 0 is in place
-
-  // Adds the live accumulators (which refer to the running maxima ho.m) to the current modality's sums in
-  // shared memory and clears them.  Apart from modality changes this happens every FLUSH windows: the
-  // tensor cores' fp32 accumulation does not round to nearest, so a long chain of MMAs into one register
-  // drifts, and the difference against the exactly rounded weight sum run_S is amplified by the codebook's
-  // cancellation (code plane minus b times the weight sum); short chains summed with FFMA do not drift.
-  auto deposit = [&](const Handoff& ho) {
-    float4* dst = reinterpret_cast<float4*>(&sm.spill[pair][cur_mod][lane][0]);
-    float* dm = &sm.spill_m[pair][cur_mod][0];
-    const float s_lo = dm[2 * t], s_hi = dm[2 * t + 1], s_g = dm[g];
-    if (s_g == -INFINITY) {   // first deposit of this modality (the same for every head)
-#pragma unroll
-      for (int mu = 0; mu < 8; mu++) dst[mu] = make_float4(acc[mu][0], acc[mu][1], acc[mu][2], acc[mu][3]);
-      reinterpret_cast<float*>(dst)[32] = run_S;
-    } else {
-      const float f_lo = ex2(s_lo - ho.m[2 * t]), f_hi = ex2(s_hi - ho.m[2 * t + 1]), f_g = ex2(s_g - ho.m[g]);
-#pragma unroll
-      for (int mu = 0; mu < 8; mu++) {
-        float4 v = dst[mu];
-        v.x = fmaf(v.x, f_lo, acc[mu][0]); v.y = fmaf(v.y, f_hi, acc[mu][1]);
-        v.z = fmaf(v.z, f_lo, acc[mu][2]); v.w = fmaf(v.w, f_hi, acc[mu][3]);
-        dst[mu] = v;
-      }
-      float* dS = reinterpret_cast<float*>(dst) + 32;
-      *dS = fmaf(*dS, f_g, run_S);
-    }
-    __syncwarp();
-    if (t == 0) dm[g] = ho.m[g];
-    __syncwarp();
-#pragma unroll
-    for (int mu = 0; mu < 8; mu++)
-#pragma unroll
-      for (int i = 0; i < 4; i++) acc[mu][i] = 0.f;
-    run_S = 0.f;
-    since = 0;
-  };
-
-  for (int k = 0; k <= sg.n_my; k++) {
-    issue(k + PREFETCH);
-    if (k >= 1) {
-      const unsigned char* st = sm.stage[pair][(k - 1) % NSTAGE];
-      const Handoff& ho = sm.hand[pair][(k - 1) & 1];
-      if (ho.rescale) {
-        const float a_lo = ho.alpha[2 * t], a_hi = ho.alpha[2 * t + 1];
-#pragma unroll
-        for (int mu = 0; mu < 8; mu++) {
-          acc[mu][0] *= a_lo; acc[mu][1] *= a_hi; acc[mu][2] *= a_lo; acc[mu][3] *= a_hi;
-        }
-        run_S *= ho.alpha[g];
-      }
-      const unsigned char* wmod = st + STAGE_MOD;
-      const int mymod = wmod[lane];
-      const int first = __shfl_sync(0xffffffffu, mymod, 0);
-      const bool uniform = __all_sync(0xffffffffu, mymod == first);
-      const uint4 vc0 = *reinterpret_cast<const uint4*>(st + OFF_VCODE + 16 * vpiece_slot(lane));
-      const uint4 vc1 = *reinterpret_cast<const uint4*>(st + OFF_VCODE + 16 * vpiece_slot(32 + lane));
-      const uint32_t vw[8] = {vc0.x, vc0.y, vc0.z, vc0.w, vc1.x, vc1.y, vc1.z, vc1.w};
-      const uint4 pb4 = ho.pb[lane];
-      const uint32_t pb[4] = {pb4.x, pb4.y, pb4.z, pb4.w};
-      // (3a - b) / (2 (b - a)): weight of the bit-1 plane relative to the code plane
-      constexpr float DELTA_REL = (3.0f * CB_INNER - CB_OUTER) / (2.0f * (CB_OUTER - CB_INNER));
-      const __half2 drel = __float2half2_rn(DELTA_REL);
-      // the two bit-plane products of the numerators b0 (zero where a token is not of the current modality) over
-      // the 16-token halves named by halfmask, and the weight sum
-      auto half_products = [&](const uint32_t (&b0)[4], const uint32_t (&b1)[4], auto kv_c) {
-        constexpr int kv = decltype(kv_c)::value;
-        constexpr uint32_t mA = 0x00030003u << (4 * kv), mB = 0x000c000cu << (4 * kv);
-        constexpr uint32_t nA = 0x00020002u << (4 * kv), nB = 0x00080008u << (4 * kv);
-        const uint32_t p0 = b0[2 * kv], p1 = b0[2 * kv + 1], q0 = b1[2 * kv], q1 = b1[2 * kv + 1];
-        // the two bit-plane products of one m-tile hit the same accumulator: keep them four
-        // MMAs apart so the second never waits for the first
-#pragma unroll
-        for (int mq = 0; mq < 8; mq += 4) {
-          uint32_t w8[4];
-#pragma unroll
-          for (int i = 0; i < 4; i++) {
-            const uint32_t w = vw[mq + i];
-            w8[i] = w >> 8;
-            mma16816(acc[mq + i], w & mA, w8[i] & mA, w & mB, w8[i] & mB, p0, p1);
-          }
-#pragma unroll
-          for (int i = 0; i < 4; i++) {
-            const uint32_t w = vw[mq + i];
-            mma16816(acc[mq + i], w & nA, w8[i] & nA, w & nB, w8[i] & nB, q0, q1);
-          }
-        }
-      };
-      auto products = [&](const uint32_t (&b0)[4], unsigned halfmask, auto whole) {
-        uint32_t b1[4];
-#pragma unroll
-        for (int nu = 0; nu < 4; nu++) {
-          b1[nu] = h2u(__hmul2(u2h(b0[nu]), drel));
-          float2 pf = __half22float2(u2h(b0[nu]));   // weight sum from the rounded numerators
-          run_S = fmaf(pf.x + pf.y, (float)(1 << (2 * nu)) * (1.0f / 64.0f), run_S);
-        }
-        if constexpr (decltype(whole)::value) {   // both halves, straight-line, compile-time masks
-          half_products(b0, b1, std::integral_constant<int, 0>{});
-          half_products(b0, b1, std::integral_constant<int, 1>{});
-        } else {
-#pragma unroll 1   // rolled on purpose: unrolling both halves makes ptxas spill the accumulators
-          for (int kv = 0; kv < 2; kv++) {
-            if (!((halfmask >> kv) & 1)) continue;
-            const uint32_t mA = 0x00030003u << (4 * kv), mB = 0x000c000cu << (4 * kv);
-            const uint32_t nA = 0x00020002u << (4 * kv), nB = 0x00080008u << (4 * kv);
-            const uint32_t p0 = kv ? b0[2] : b0[0], p1 = kv ? b0[3] : b0[1];
-            const uint32_t q0 = kv ? b1[2] : b1[0], q1 = kv ? b1[3] : b1[1];
-#pragma unroll
-            for (int mq = 0; mq < 8; mq += 4) {
-              uint32_t w8[4];
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const uint32_t w = vw[mq + i];
-                w8[i] = w >> 8;
-                mma16816(acc[mq + i], w & mA, w8[i] & mA, w & mB, w8[i] & mB, p0, p1);
-              }
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const uint32_t w = vw[mq + i];
-                mma16816(acc[mq + i], w & nA, w8[i] & nA, w & nB, w8[i] & nB, q0, q1);
-              }
-            }
-          }
-        }
-      };
-      if (uniform && first == cur_mod) {
-        // the common case: every token of the window belongs to the modality the registers hold
-        products(pb, 3u, std::true_type{});
-      } else {
-        unsigned present = uniform ? (1u << first)
-                                   : ((__any_sync(0xffffffffu, mymod == 0) ? 1u : 0u) |
-                                      (__any_sync(0xffffffffu, mymod == 1) ? 2u : 0u) |
-                                      (__any_sync(0xffffffffu, mymod == 2) ? 4u : 0u));
-        for (int pass = 0; pass < 3 && present; pass++) {
-          int m = (cur_mod >= 0 && (present >> cur_mod) & 1) ? cur_mod : (__ffs(present) - 1);
-          present &= ~(1u << m);
-          if (m != cur_mod) {
-            if (cur_mod >= 0) deposit(ho);
-            cur_mod = m;
-          }
-          uint32_t b0[4];
-          unsigned halfmask = 3u;  // which 16-token halves hold a token of modality m
-          if (uniform) {
-#pragma unroll
-            for (int nu = 0; nu < 4; nu++) b0[nu] = pb[nu];
-          } else {
-            bool any_lo = false, any_hi = false;
-#pragma unroll
-            for (int nu = 0; nu < 4; nu++) {
-              const bool k0 = wmod[8 * nu + 2 * t] == m, k1 = wmod[8 * nu + 2 * t + 1] == m;
-              b0[nu] = pb[nu] & ((k0 ? 0x0000ffffu : 0u) | (k1 ? 0xffff0000u : 0u));
-              if (nu < 2) any_lo |= (k0 | k1); else any_hi |= (k0 | k1);
-            }
-            halfmask = (__any_sync(0xffffffffu, any_lo) ? 1u : 0u) | (__any_sync(0xffffffffu, any_hi) ? 2u : 0u);
-          }
-          products(b0, halfmask, std::false_type{});
-        }
-      }
-      // before the barrier: the score warp may overwrite this hand-off record right after it
-      if (k == sg.n_my || ++since >= FLUSH) deposit(ho);
-    }
-    cp_async_wait<1>();   // all but the copies just issued: window k + 1 is complete
-    expand_meta(k + 1);
-    pair_barrier(pair);
-  }
-  cp_async_wait<0>();
-  // leave the three modalities' accumulators (each lane its own column) and their maxima in the pair's piece
-  if (sg.keep) return;   // the block's merge reads this pair's sums where they are
-#pragma unroll 1
-  for (int m = 0; m < 3; m++) {
-    const float mm = sm.spill_m[pair][m][g];
-    if (t == 0) sg.piece->sm[m][g] = mm;
-    if (mm != -INFINITY) {
-      const float4* src = reinterpret_cast<const float4*>(&sm.spill[pair][m][lane][0]);
-      float* dst = &sg.piece->frag[m][0][lane];
-#pragma unroll
-      for (int mu = 0; mu < 8; mu++) {
-        const float4 v = src[mu];
-        dst[(4 * mu) * 32] = v.x; dst[(4 * mu + 1) * 32] = v.y; dst[(4 * mu + 2) * 32] = v.z; dst[(4 * mu + 3) * 32] = v.w;
-      }
-      dst[32 * 32] = reinterpret_cast<const float*>(src)[32];
-    }
-  }
-  __syncwarp();
-}
 
 }  // namespace
 
-// grid = n_cta (persistent), 512 threads
+// grid = n_cta (persistent), NTHREADS threads
 //
 // CTA i owns the windows [i * per, (i + 1) * per) of the flattened (layer, sequence, head, window) axis and
-// cuts them into eight contiguous ranges, one per warp pair.  A pair walks its range on its own, with no
-// block-wide step in between: where the range crosses into another (sequence, head) the score warp sets up
-// that head group's query fragments, the value warp leaves what it accumulated in a PairPartial piece and
+// cuts them into NWARP contiguous ranges.  A warp walks its range on its own, with no block-wide step in
+// between: where the range crosses into another (sequence, head) it leaves what it accumulated in a piece and
 // starts afresh.  At the end of the launch the block merges, per (sequence, head) it touched, the pieces of
-// the pairs that worked on it into one PartialF.
+// the warps that worked on it into one PartialF.
 template <int FMT>
 __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MmaSmem<FMT>& sm = *reinterpret_cast<MmaSmem<FMT>*>(smem_raw);
   const CacheView& cv = P.cv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pair = warp & (NPAIR - 1);
-  const bool is_score = warp < NPAIR;
   const int G = P.group, Hkv = cv.n_kv_heads;
   const int n_entries = P.layer_count * cv.batch;
 
@@ -514,7 +76,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
   const int total = block_prefix(cv, P.layer0, n_entries, sm.prefix);
   const int per = (total + gridDim.x - 1) / gridDim.x;
   const int pos0 = min(total, (int)blockIdx.x * per), pos1 = min(total, pos0 + per);
-  const int cnt = (pos1 - pos0 + NPAIR - 1) / NPAIR;
+  const int cnt = (pos1 - pos0 + NWARP - 1) / NWARP;
 
   struct Where { int e, h, w0, nwin; };
   auto locate = [&](int pos) {   // (entry, head, window) of a flattened position; largest e with prefix[e] <= pos
@@ -533,7 +95,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
   };
 
   {
-    int pos = min(pos1, pos0 + pair * cnt);
+    int pos = min(pos1, pos0 + warp * cnt);
     const int pos_end = min(pos1, pos + cnt);
     while (pos < pos_end) {
       const Where wh = locate(pos);
@@ -543,116 +105,93 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
       sg.mod0 = cv.modality + (size_t)b * cv.capacity;
       sg.w0 = wh.w0;
       sg.n_my = min(pos_end - pos, wh.nwin - wh.w0);
-      sg.q = P.q + (((size_t)li * cv.batch + b) * cv.n_q_heads + (size_t)wh.h * G) * D;
-      sg.signs = P.signs + (size_t)li * D;
-      sg.piece = P.pair_parts + (size_t)(wh.e * Hkv + wh.h) + ((size_t)blockIdx.x * NPAIR + pair);
-      sg.keep = pos + sg.n_my == pos_end;
-      if (is_score) score_warp<FMT>(sm, sg, G, P.sm_scale, pair, lane);
-      else value_warp<FMT>(sm, sg, pair, lane);
+      sg.piece = P.pieces + (size_t)(wh.e * Hkv + wh.h) + ((size_t)blockIdx.x * NWARP + warp);
+      const WalkEnd we = walk_segment<FMT>(sm.w[warp], sm.qlo[warp], sg, lane, [&](uint32_t (&qh)[16], float& fsc) {
+        uint2 qreg[16];
+        query_fragments(P.q + (((size_t)li * cv.batch + b) * cv.n_q_heads + (size_t)wh.h * G) * D, P.signs + (size_t)li * D, G,
+                        P.sm_scale, lane, qreg, fsc);
+#pragma unroll
+        for (int r = 0; r < 16; r++) qh[r] = qreg[r].x;
+#pragma unroll
+        for (int kq = 0; kq < 4; kq++)   // (a lane reads back only what it wrote)
+          sm.qlo[warp][kq][lane] = make_uint4(qreg[4 * kq].y, qreg[4 * kq + 1].y, qreg[4 * kq + 2].y, qreg[4 * kq + 3].y);
+      });
+      if ((lane & 3) == 0) { sg.piece->wm[lane >> 2] = we.m; sg.piece->wl[lane >> 2] = we.l; }
+      if (lane == 0) sg.piece->mask = (int)we.held;
       pos += sg.n_my;
     }
   }
   __syncthreads();   // the pieces were written by this block's own warps: visible to the block from here on
 
-  // ---- merge the pairs' pieces into one partial per (sequence, head) of the block's range, MB_SEG
+  // ---- merge the warps' pieces into one partial per (sequence, head) of the block's range, MB_SEG
   // (sequence, head) units at a time so that the loads of many units are in flight together.  The tables
   // take the place of the record ring, which is idle by now.
   if (pos0 >= pos1) return;
   MergeSmem& mg = *reinterpret_cast<MergeSmem*>(smem_raw);
+  static_assert(sizeof(MergeSmem) <= sizeof(WarpSmem<FMT>) * NWARP, "the merge tables fit the record ring");
   const Where wf = locate(pos0), wl = locate(pos1 - 1);
   const int u_first = wf.e * Hkv + wf.h, u_last = wl.e * Hkv + wl.h;
   for (int ub = u_first; ub <= u_last; ub += MB_SEG) {
     const int n_u = min(MB_SEG, u_last - ub + 1);
-    // (a) the units' window ranges inside the block's slice and the pairs that worked on them
+    // (a) the units' window ranges inside the block's slice and the warps that worked on them
     if (tid < n_u) {
       const int u = ub + tid, e = u / Hkv, h = u % Hkv;
       const int nwin = (sm.prefix[e + 1] - sm.prefix[e]) / Hkv;
       const int a0 = max(pos0, sm.prefix[e] + h * nwin), a1 = min(pos1, sm.prefix[e] + (h + 1) * nwin);
       mg.pa[tid] = a1 > a0 ? (a0 - pos0) / cnt : 0;
-      const int pb = a1 > a0 ? (a1 - 1 - pos0) / cnt : -1;   // empty: a (sequence, head) with no packed window
-      mg.pb[tid] = pb;
-      // pairs before the last end their range inside this unit, so their sums are still in shared memory; the
-      // last one's are too unless its range goes on into the next unit
-      mg.last_kept[tid] = pb >= 0 && min(pos1, pos0 + (pb + 1) * cnt) <= a1;
+      mg.pb[tid] = a1 > a0 ? (a1 - 1 - pos0) / cnt : -1;   // empty: a (sequence, head) with no packed window
     }
     __syncthreads();
-    // (b) the pieces' maxima and weight sums: one warp per (unit, pair)
-    for (int j = warp; j < n_u * NPAIR; j += NTHREADS / 32) {
-      const int su = j / NPAIR, p = j % NPAIR;
+    // (b) the pieces' maxima and weight sums: a half-warp per (unit, warp)
+    for (int j = tid >> 4; j < n_u * NWARP; j += NTHREADS / 16) {
+      const int su = j / NWARP, p = j % NWARP, c = tid & 15;
       if (p < mg.pa[su] || p > mg.pb[su]) continue;
-      float* dst = mg.meta[su + p - mg.pa[0]];
-      if (p < mg.pb[su] || mg.last_kept[su]) {
-        dst[lane] = lane < 3 * GP ? (&sm.spill_m[p][0][0])[lane] : sm.fin_w[p][0][lane - 3 * GP];
-        if (lane < GP) dst[32 + lane] = sm.fin_w[p][1][lane];
-      } else {
-        const PairPartial& pp = P.pair_parts[(size_t)(ub + su) + (size_t)blockIdx.x * NPAIR + p];
-        dst[lane] = (&pp.sm[0][0])[lane];                         // sm[3][GP], then wm[GP]
-        if (lane < GP) dst[32 + lane] = pp.wl[lane];
-      }
+      const WarpPiece& pp = P.pieces[(size_t)(ub + su) + (size_t)blockIdx.x * NWARP + p];
+      mg.meta[su + p - mg.pa[0]][c] = pp.wm[c];             // wm[GP], then wl[GP]
+      if (c == 0) mg.mask[su + p - mg.pa[0]] = pp.mask;
     }
     __syncthreads();
-    // (c) merged maximum and weight sum per (unit, head)
+    // (c) merged maximum, weight sum and the pieces' factors per (unit, head)
     if (tid < n_u * GP) {
       const int su = tid / GP, j = tid % GP;
       if (mg.pb[su] >= mg.pa[su]) {
         float mj = -INFINITY, L = 0.f;
-        for (int p = mg.pa[su]; p <= mg.pb[su]; p++) mj = fmaxf(mj, mg.meta[su + p - mg.pa[0]][3 * GP + j]);
+        for (int p = mg.pa[su]; p <= mg.pb[su]; p++) mj = fmaxf(mj, mg.meta[su + p - mg.pa[0]][j]);
         for (int p = mg.pa[su]; p <= mg.pb[su]; p++) {
-          const float* me = mg.meta[su + p - mg.pa[0]];
-          L += me[4 * GP + j] * exp2f(me[3 * GP + j] - mj);
+          const float f = exp2f(mg.meta[su + p - mg.pa[0]][j] - mj);
+          L += mg.meta[su + p - mg.pa[0]][GP + j] * f;
+          mg.fac[su + p - mg.pa[0]][j] = f;
         }
-        mg.M[su][j] = mj;
         PartialF* out = P.partials_f + (size_t)(ub + su) + blockIdx.x;
         out->m[j] = mj;
         out->l[j] = L;
       }
     }
     __syncthreads();
-    // (d) the accumulators: one item = four lanes' worth of one (unit, modality, register) row
-    // rescale factors, once per (piece, modality, head)
-    for (int j = tid; j < n_u * NPAIR * 3 * GP; j += NTHREADS) {
-      const int su = j / (NPAIR * 3 * GP), p = (j / (3 * GP)) % NPAIR, k = j % (3 * GP);
-      if (p < mg.pa[su] || p > mg.pb[su]) continue;
-      const float smv = mg.meta[su + p - mg.pa[0]][k];
-      (&mg.fac[su + p - mg.pa[0]][0][0])[k] = smv == -INFINITY ? 0.f : exp2f(smv - mg.M[su][k % GP]);
-    }
-    __syncthreads();
-    // (d) the accumulators: one item = four consecutive registers of one lane of one (unit, modality), or that
-    // lane's weight sum.  A lane's registers are one 128-bit row read where the piece is still in shared memory;
-    // registers r and r + 2 belong to head 2 (lane & 3), r + 1 and r + 3 to the next head.
-    constexpr int RG = 9, UNIT_ITEMS = 3 * RG * 32;
+    // (d) the accumulators: one item = four consecutive registers of one lane of one (unit, modality); registers r and
+    // r + 2 belong to head 2 (lane & 3), r + 1 and r + 3 to the next head
+    constexpr int RG = 8, UNIT_ITEMS = 3 * RG * 32;
     for (int it = tid; it < n_u * UNIT_ITEMS; it += NTHREADS) {
       const int su = it / UNIT_ITEMS, idx = it % UNIT_ITEMS;
       const int L = idx & 31, rg = (idx >> 5) % RG, m = idx / (RG * 32);
       const int pa = mg.pa[su], np = mg.pb[su] - pa + 1;
       if (np <= 0) continue;
-      const int inc0 = su + pa - mg.pa[0];
-      const bool last_kept = mg.last_kept[su] != 0;
-      const int hsel = rg < 8 ? 2 * (L & 3) : (L >> 2);
+      const int inc0 = su + pa - mg.pa[0], hsel = 2 * (L & 3);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int q = 0; q < NPAIR; q++) {
-        if (q >= np || mg.meta[inc0 + q][m * GP] == -INFINITY) continue;   // no such pair / no token of this modality
-        const float* fc = mg.fac[inc0 + q][m];
-        const float fe = fc[hsel], fo = rg < 8 ? fc[hsel + 1] : fe;
-        float4 x;
-        if (q < np - 1 || last_kept) {
-          const float* sp = &sm.spill[pa + q][m][L][0];
-          x = rg < 8 ? *reinterpret_cast<const float4*>(sp + 4 * rg) : make_float4(sp[32], 0.f, 0.f, 0.f);
-        } else {
-          const float* gp = &P.pair_parts[(size_t)(ub + su) + (size_t)blockIdx.x * NPAIR + pa + q].frag[m][0][L];
-          x = rg < 8 ? make_float4(gp[(4 * rg) * 32], gp[(4 * rg + 1) * 32], gp[(4 * rg + 2) * 32], gp[(4 * rg + 3) * 32])
-                     : make_float4(gp[32 * 32], 0.f, 0.f, 0.f);
-        }
+      for (int q = 0; q < NWARP; q++) {
+        if (q >= np || !((mg.mask[inc0 + q] >> m) & 1)) continue;   // no such warp / no token of this modality
+        const float fe = mg.fac[inc0 + q][hsel], fo = mg.fac[inc0 + q][hsel + 1];
+        const float4 x = __ldcg(&P.pieces[(size_t)(ub + su) + (size_t)blockIdx.x * NWARP + pa + q].frag[m][rg][L]);
         v.x = fmaf(x.x, fe, v.x); v.y = fmaf(x.y, fo, v.y); v.z = fmaf(x.z, fe, v.z); v.w = fmaf(x.w, fo, v.w);
       }
+      // in units of the bit-plane form, whose weight sums are zero here
+      constexpr float F = LEVEL_UNIT * 16.0f / PARTIAL_ACC_SCALE;
+      static_assert(P_LOG2 == -4.0f, "the factor 16 above is 2^-P_LOG2");
       PartialF* out = P.partials_f + (size_t)(ub + su) + blockIdx.x;
-      if (rg < 8) {
-        out->frag[m][4 * rg][L] = v.x; out->frag[m][4 * rg + 1][L] = v.y;
-        out->frag[m][4 * rg + 2][L] = v.z; out->frag[m][4 * rg + 3][L] = v.w;
-      } else {
-        out->Sp[m][L] = v.x;
-      }
+      out->frag[m][4 * rg][L] = v.x * F; out->frag[m][4 * rg + 1][L] = v.y * F;
+      out->frag[m][4 * rg + 2][L] = v.z * F; out->frag[m][4 * rg + 3][L] = v.w * F;
+      if (rg == 0) out->Sp[m][L] = 0.f;
     }
     __syncthreads();
   }
@@ -777,7 +316,7 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   if (n_tail > 0) stage_tail(0);   // on its way while the prefix is computed
   const int total = block_prefix(cv, P.layer0, n_entries, sm.prefix);
   const int per = total > 0 ? (total + n_cta - 1) / n_cta : 1;
-  constexpr float ACC_SCALE = (CB_OUTER - CB_INNER) * 262144.0f;  // (b - a) * 2^18
+  constexpr float ACC_SCALE = PARTIAL_ACC_SCALE;
   constexpr float LOG2E = 1.4426950408889634f;
   // Coefficient of the weight sum S: -b from the codebook identity, plus the mean of what the bit-1
   // plane loses because its relative weight (3a-b)/(2(b-a)) enters the MMA rounded to fp16 (bit 1 is
@@ -803,12 +342,9 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
     __syncthreads();
     const int wv = c >> 5, lane = c & 31;
     if (wv < npc) {
-      Segment sq;
-      sq.q = qbase;
-      sq.signs = P.signs + (size_t)li * D;
       uint2 qreg[16];
       float fsc;
-      query_fragments(sq.q, sq.signs, G, P.sm_scale, lane, qreg, fsc);
+      query_fragments(qbase, P.signs + (size_t)li * D, G, P.sm_scale, lane, qreg, fsc);
       unsigned char* st = kimg + wv * KIMG;
       if (cv.fmt == FMT_MXFP4) {   // decode the stored (m, s) into the fp16 planes of the staged image
         uint2 m4, s4;

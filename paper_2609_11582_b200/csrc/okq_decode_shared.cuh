@@ -24,14 +24,17 @@ struct PartialF {
   float frag[3][32][32];
 };
 
-// tensor-core kernel: what one warp pair accumulated over its part of one (sequence, head); the CTA
-// merges its pairs' pieces into the PartialF records at the end of the launch
-constexpr int MMA_PAIRS = 8;        // warp pairs per CTA
-constexpr int PAIR_REGS = 33;       // 32 accumulator registers + the running weight sum, per lane
-struct PairPartial {
-  float frag[3][PAIR_REGS][32];   // [modality][register][lane]
-  float sm[3][GP];                // running maximum the modality's accumulators refer to (-inf: none)
-  float wm[GP], wl[GP];           // running maximum and sum of exp2(score - maximum) per head
+// unit of PartialF's accumulators: a value sum is PARTIAL_ACC_SCALE * frag + (codebook offset) * (sum of Sp)
+constexpr float PARTIAL_ACC_SCALE = (CB_OUTER - CB_INNER) * 262144.0f;  // (b - a) * 2^18
+
+// mma.sync kernel: what one warp accumulated over its part of one (sequence, head); the CTA merges its warps'
+// pieces into the PartialF records at the end of the launch
+constexpr int DECODE_WARPS = 12;    // warps per CTA
+struct WarpPiece {
+  float4 frag[3][8][32];   // [modality][m-tile][lane]: the tile's four accumulator registers
+  float wm[GP], wl[GP];    // reference maximum (log2 domain) of everything in the piece, sum of exp2(score - maximum)
+  int mask;                // modalities the piece holds (bit m); the other modalities' sums are not written
+  int pad[3];
 };
 
 struct DecodeParams {
@@ -44,7 +47,7 @@ struct DecodeParams {
   float sm_scale;
   Partial* partials;   // CUDA-core path: [layer_count*batch*n_kv_heads][n_splits]
   PartialF* partials_f;  // tensor-core path: [n_units + n_cta]
-  PairPartial* pair_parts;  // tensor-core path: [n_units + 8 * n_cta]
+  WarpPiece* pieces;     // tensor-core path: [n_units + DECODE_WARPS * n_cta]
   float* out;          // [layer_count][batch][n_q_heads][128]
 };
 
