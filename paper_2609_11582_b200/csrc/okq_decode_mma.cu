@@ -721,6 +721,15 @@ static void combine_dispatch(const DecodeParams& P, int n_cta, cudaStream_t s) {
 int g_decode_impl = 1;
 
 okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, cudaEvent_t before, cudaEvent_t after) {
+  if (P.n_splits == 0 && g_decode_impl == 1) {   // the library's own choice of the grid
+    const int cs = decode_small_cluster(P.cv, P.layer_count, n_cta);
+    if (cs > 0) {
+      if (before) cudaEventRecord(before, s);
+      const okq_status st = launch_decode_small(P, cs, s);
+      if (after) cudaEventRecord(after, s);
+      return st;
+    }
+  }
   static thread_local unsigned long long attr_mask = 0;
   int attr_dev = 0;
   if (attr_needed(attr_mask, attr_dev)) {

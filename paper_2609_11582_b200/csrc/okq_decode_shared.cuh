@@ -82,6 +82,11 @@ okq_status launch_decode_tc(const DecodeParams& P, int n_cta, cudaStream_t s);
 // which split-K kernel launch_decode_mma uses: 0 = the tcgen05 kernel (fp16 metadata), 1 = the mma.sync warp-pair kernel
 extern int g_decode_impl;
 
+// one-launch form for few (sequence, head) units: cluster size it would use for a call (0: not applicable), launch
+constexpr int SMALL_WINDOWS_PER_WARP = 16;
+int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta);
+okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s);
+
 // launches the tensor-core split kernel (bracketed by the optional events) and its combine kernel
 okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, cudaEvent_t before, cudaEvent_t after);
 

@@ -1,0 +1,428 @@
+// Fused decode attention in one launch, for calls with few (layer, sequence, KV head) units: a model's per-layer call.
+//
+// The split-K kernel and its combine kernel are a chain of launch, prefix, partials through memory, launch, prefix,
+// merge; with a handful of windows per warp that chain is the whole time (35 + 20 us for one layer of 4 sequences at
+// 4096 tokens).  Here a thread-block cluster owns one unit: its CS x 12 warps walk the unit's windows (the same code as
+// the split-K kernel), leave their sums as pieces in global memory (L2), and after one cluster barrier every CTA merges
+// 1 / CS of the rotated channels over all pieces.  The merged sums are pushed into every CTA's shared memory, and after
+// the second barrier each CTA applies R_m^T for 1 / CS of the output columns.  The raw tail is scored by every CTA (its
+// rows are staged at the start) while the first barrier is on its way.
+// What bounds it: latency (launch, query rotation, 4 to 10 windows per warp, two cluster barriers, L2 round trips of the
+// merge).  One sequence, one head group of seven, 2048 tokens: 59 -> 14 us per call; one layer of 4 sequences x 4 heads at
+// 4111 tokens 32 -> 18.5 us against the split-K pair.
+#include <cooperative_groups.h>
+#include "okq_decode_walk.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace okq {
+
+namespace {
+
+constexpr int KROW = D + 8;                     // halfs per staged raw key row: 16-byte reads of 32 rows over all banks
+constexpr int KIMG = OFF_VCODE + 144;           // key part of a window record (+ its MXFP4 metadata bytes)
+constexpr int PC_MAX = 4;                       // packed windows among the raw-value tokens (captioning schedule)
+
+struct PieceMeta { float m[GP], l[GP]; int held; };
+
+template <int FMT, int CS> struct SmallSmem {
+  static constexpr int C = D / CS;              // output columns (and merged channels) of a CTA
+  static constexpr int NP = CS * NWARP;         // pieces of a unit
+  static constexpr int KS = 2 * NTHREADS / C;   // row slices of the product (a thread takes two columns)
+  static constexpr int TAIL = CAPTION_V_SLOTS;
+  // what takes the record ring's place once every warp of the CTA has walked its range
+  struct After {
+    __align__(16) float R[3 * D][C];            // this CTA's columns of the three matrices
+    __align__(16) __half v[TAIL][C];            // and of the raw value rows
+    __align__(16) __half k[CAPTION_K_GROUP - W][KROW];   // raw key rows behind the first 32
+    __align__(16) unsigned char img[PC_MAX][KIMG];
+    __align__(16) float tsc[TAIL][GP];          // tail scores (log2 domain), then numerators
+    __align__(16) float fac[NP][GP];            // per piece and head: exp2(piece maximum - maximum)
+    __align__(16) float4 part[NTHREADS];        // merge: sums over a share of the pieces
+    __align__(16) float vec[3 * D][GP];         // merged rotated-basis sums [modality * 128 + channel][head], each CTA's
+                                                // share written by that CTA (behind the first cluster barrier)
+    __align__(16) float prod[KS][GP][C];
+    float red[NWARP][GP];
+    float M[GP], L[GP];
+  };
+  union { WarpSmem<FMT> w[NWARP]; After a; };
+  // written by the other CTAs of the cluster at any time
+  PieceMeta meta[NP];
+  __align__(16) __half k0[W][KROW], q[GP][KROW];   // staged at the start: the first 32 raw key rows, the queries
+  // query fragments of the unit in mma A order, high and low parts: [kq][lane][r & 3], and the heads' scales
+  __align__(16) uint32_t qhi[4][32][4], qlo[4][32][4];
+  float fsc[GP];
+};
+
+// Rotated query of head g as fragments in shared memory, by one warp with four channels per lane: the transform of
+// query_fragments with its butterflies over the lanes (every warp of the CTA needs the same fragments).
+__device__ __forceinline__ void head_fragments(const __half* qrow, const float* signs, float sm_scale, int g, bool have, int lane,
+                                               uint32_t (*qhi)[32][4], uint32_t (*qlo)[32][4], float* fsc) {
+  float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (have) {
+    x = load_row4(qrow, lane);
+    const float4 sv = *reinterpret_cast<const float4*>(signs + 4 * lane);
+    x.x *= sv.x; x.y *= sv.y; x.z *= sv.z; x.w *= sv.w;
+  }
+  x = warp_fwht(x, lane);
+  x.x *= RSQRT_D; x.y *= RSQRT_D; x.z *= RSQRT_D; x.w *= RSQRT_D;
+  float mx = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w)));
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+  int ex = 0;
+  if (mx > 0.f) frexpf(mx, &ex);           // mx < 2^ex
+  const int kh = 14 - ex, r = lane >> 1;   // |q'| * 2^kh < 2^14; channels 4 lane .. 4 lane + 3 = fragment r, t = 2 (lane & 1) + {0, 1}
+  const float sc = exp2f((float)kh) / (float)(1 << (2 * (r & 3)));
+  if (lane == 0) fsc[g] = exp2f((float)(24 - kh)) * sm_scale * 1.4426950408889634f;
+  const float v[4] = {x.x * sc, x.y * sc, x.z * sc, x.w * sc};
+#pragma unroll
+  for (int i = 0; i < 2; i++) {
+    const __half2 hi = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
+    const float2 hf = __half22float2(hi);
+    const int l = 4 * g + 2 * (lane & 1) + i;
+    qhi[r >> 2][l][r & 3] = h2u(hi);
+    qlo[r >> 2][l][r & 3] = h2u(__floats2half2_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y));
+  }
+}
+
+}  // namespace
+
+// grid CS * units, clusters of CS; unit = (layer, sequence, KV head)
+template <int FMT, int CS>
+__global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
+  using SM = SmallSmem<FMT, CS>;
+  constexpr int C = SM::C;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SM& sm = *reinterpret_cast<SM*>(smem_raw);
+  typename SM::After& af = sm.a;
+  const CacheView& cv = P.cv;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int unit = blockIdx.x / CS, rank = blockIdx.x % CS;
+  const int h = unit % cv.n_kv_heads, e = unit / cv.n_kv_heads, b = e % cv.batch, li = e / cv.batch, layer = P.layer0 + li;
+  const int G = P.group;
+  const int seq = cv.seq_len[layer * cv.batch + b];
+  // tokens [0, v_pk) have packed values (and keys); of the rest, [v_pk, k_pk) have packed keys (captioning schedule only)
+  const int v_pk = cv.v_packed(seq), k_pk = cv.k_packed(seq), nwin = v_pk / W, n_tail = seq - v_pk;
+  const int npc = (k_pk - v_pk) / W, n_rawk = seq - k_pk;
+  const __half* qbase = P.q + (((size_t)li * cv.batch + b) * cv.n_q_heads + (size_t)h * G) * D;
+  const float* signs = P.signs + (size_t)li * D;
+  const __half* kt = cv.k_tail + cv.k_tail_off(layer, b, h);
+  const __half* vt = cv.v_tail + cv.v_tail_off(layer, b, h);
+
+  // ---- on their way from the start: queries and the first raw keys
+  for (int i = tid; i < G * (D / 8); i += NTHREADS) cp_async16(&sm.q[i / (D / 8)][8 * (i % (D / 8))], qbase + 8 * i);
+  for (int i = tid; i < min(W, n_rawk) * (D / 8); i += NTHREADS)
+    cp_async16(&sm.k0[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(k_pk + i / (D / 8)) * D + 8 * (i % (D / 8)));
+  cp_async_commit();
+
+  cluster.barrier_arrive();   // every CTA of the cluster runs before its shared memory is written from outside
+  // ---- this warp's windows
+  const int cnt = (nwin + CS * NWARP - 1) / (CS * NWARP);
+  const int gw = rank * NWARP + warp, w0 = min(nwin, gw * cnt), w1 = min(nwin, w0 + cnt);
+  WarpPiece* const pieces = P.pieces + (size_t)unit * (CS * NWARP);
+  WalkEnd we{-INFINITY, 0.f, 0u};
+  auto queries = [&]() {   // the CTA's first eight warps, then everyone waits
+    if (warp < GP) head_fragments(qbase + warp * D, signs, P.sm_scale, warp, warp < G, lane, sm.qhi, sm.qlo, sm.fsc);
+    asm volatile("bar.sync 1, %0;\n" ::"n"(NTHREADS) : "memory");
+  };
+  if (w1 > w0) {
+    Segment sg;
+    sg.rec0 = cv.unit(layer, b, h);
+    sg.mod0 = cv.modality + (size_t)b * cv.capacity;
+    sg.w0 = w0;
+    sg.n_my = w1 - w0;
+    sg.piece = pieces + gw;
+    we = walk_segment<FMT>(sm.w[warp], reinterpret_cast<const uint4(*)[32]>(sm.qlo), sg, lane, [&](uint32_t (&qh)[16], float& fsc) {
+      queries();
+      fsc = sm.fsc[lane >> 2];
+#pragma unroll
+      for (int kq = 0; kq < 4; kq++) {
+        const uint4 x = *reinterpret_cast<const uint4*>(sm.qhi[kq][lane]);
+        qh[4 * kq] = x.x; qh[4 * kq + 1] = x.y; qh[4 * kq + 2] = x.z; qh[4 * kq + 3] = x.w;
+      }
+    });
+  } else {
+    queries();
+  }
+  cluster.barrier_wait();
+  // ---- the piece's header goes to every CTA of the cluster
+  for (int r = 0; r < CS; r++) {
+    PieceMeta* pm = cluster.map_shared_rank(&sm.meta[gw], r);
+    if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
+    if (lane == 0) pm->held = (int)we.held;
+  }
+  cluster.barrier_arrive();   // (release: the pieces and their headers)
+  cp_async_wait<0>();
+  __syncthreads();            // the record rings are idle: their space holds the rest from here on
+
+  // ---- rest of the tail, value rows and matrices
+  for (int i = tid; i < (n_rawk - W) * (D / 8); i += NTHREADS)
+    cp_async16(&af.k[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(k_pk + W + i / (D / 8)) * D + 8 * (i % (D / 8)));
+  for (int w = 0; w < npc; w++) {
+    const int win = nwin + w;
+    unsigned char* img = af.img[w];
+    if (FMT == FMT_FP16) {
+      const unsigned char* rec = cv.meta(layer, b, h, win);   // the record starts with its (m, s) planes
+      if (tid < OFF_VCODE / 16) cp_async16(img + 16 * tid, rec + 16 * tid);
+    } else {
+      const unsigned char* body = cv.body(layer, b, h, win);
+      const unsigned char* meta = cv.meta(layer, b, h, win);
+      if (tid < 4) cp_async16(img + OFF_KNORM + 16 * tid, body + B_KNORM + 16 * tid);
+      else if (tid < 4 + 64) cp_async16(img + OFF_KCODE + 16 * (tid - 4), body + B_KCODE + 16 * (tid - 4));
+      else if (tid < 4 + 64 + MX_META_BYTES / 8) cp_async8(img + OFF_VCODE + 8 * (tid - 68), meta + 8 * (tid - 68));
+    }
+  }
+  cp_async_commit();
+  for (int i = tid; i < n_tail * (C / 8); i += NTHREADS)
+    cp_async16(&af.v[i / (C / 8)][8 * (i % (C / 8))], vt + cv.v_slot(v_pk + i / (C / 8)) * D + rank * C + 8 * (i % (C / 8)));
+  {
+    const float* R = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D + rank * C;
+    for (int i = tid; i < 3 * D * (C / 4); i += NTHREADS)
+      cp_async16(&af.R[i / (C / 4)][4 * (i % (C / 4))], R + (size_t)(i / (C / 4)) * D + 4 * (i % (C / 4)));
+  }
+  cp_async_commit();
+
+  // ---- tail scores (log2 domain)
+  constexpr float LOG2E = 1.4426950408889634f;
+  if (n_tail > 0) {
+    if (npc > 0 || n_rawk > W) { cp_async_wait<1>(); __syncthreads(); }
+    if (warp < npc) {   // packed keys: one warp per window, on the tensor cores
+      uint2 qreg[16];
+#pragma unroll
+      for (int r = 0; r < 16; r++) qreg[r] = make_uint2(sm.qhi[r >> 2][lane][r & 3], sm.qlo[r >> 2][lane][r & 3]);
+      const float fsc = sm.fsc[lane >> 2];
+      unsigned char* st = af.img[warp];
+      if (FMT == FMT_MXFP4) {
+        uint2 m4, s4;
+        mx_decode_lane(st + OFF_VCODE, lane, m4, s4);
+        *reinterpret_cast<uint2*>(st + OFF_KM + 8 * lane) = m4;
+        *reinterpret_cast<uint2*>(st + OFF_KS + 8 * lane) = s4;
+        __syncwarp();
+      }
+      float sc[4][2];
+      window_scores_mma(st, qreg, fsc, lane, sc);
+      const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+      for (int nu = 0; nu < 4; nu++)
+#pragma unroll
+        for (int e2 = 0; e2 < 2; e2++) af.tsc[warp * W + 8 * nu + 2 * t + e2][g] = g < G ? sc[nu][e2] : -INFINITY;
+    }
+    for (int i = tid; i < n_rawk * GP; i += NTHREADS) {   // raw keys: a token and a head per thread, four sums
+      const int tok = i / GP, j = i % GP;
+      float s = -INFINITY;
+      if (j < G) {
+        const __half* krow = tok < W ? sm.k0[tok] : af.k[tok - W];
+        float a4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int k = 0; k < D; k += 8) {
+          const uint4 kv = *reinterpret_cast<const uint4*>(krow + k), qv = *reinterpret_cast<const uint4*>(&sm.q[j][k]);
+          const uint32_t kx[4] = {kv.x, kv.y, kv.z, kv.w}, qx[4] = {qv.x, qv.y, qv.z, qv.w};
+#pragma unroll
+          for (int u = 0; u < 4; u++) {
+            const float2 kf = __half22float2(u2h(kx[u])), qf = __half22float2(u2h(qx[u]));
+            a4[u] = fmaf(qf.x, kf.x, a4[u]);
+            a4[u] = fmaf(qf.y, kf.y, a4[u]);
+          }
+        }
+        s = ((a4[0] + a4[1]) + (a4[2] + a4[3])) * P.sm_scale * LOG2E;
+      }
+      af.tsc[npc * W + tok][j] = s;
+    }
+  }
+  cluster.barrier_wait();     // (acquire) all pieces of the unit and their headers are there
+  __syncthreads();            // (and the tail scores)
+
+  // ---- softmax bookkeeping: thread = (head j, stripe of 48)
+  {
+    const int j = tid & (GP - 1), stripe = tid / GP;
+    float M = -INFINITY;
+    for (int p = stripe; p < SM::NP; p += NTHREADS / GP) M = fmaxf(M, sm.meta[p].m[j]);
+    for (int i = stripe; i < n_tail; i += NTHREADS / GP) M = fmaxf(M, af.tsc[i][j]);
+    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
+    M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
+    if (lane < GP) af.red[warp][j] = M;
+    __syncthreads();
+    M = af.red[0][j];
+#pragma unroll
+    for (int w = 1; w < NWARP; w++) M = fmaxf(M, af.red[w][j]);
+    __syncthreads();
+    float L = 0.f;
+    for (int p = stripe; p < SM::NP; p += NTHREADS / GP) {
+      const float pm = sm.meta[p].m[j];
+      const float f = pm == -INFINITY ? 0.f : exp2f(pm - M);
+      af.fac[p][j] = f;
+      L += sm.meta[p].l[j] * f;
+    }
+    for (int i = stripe; i < n_tail; i += NTHREADS / GP) {
+      const float x = exp2f(af.tsc[i][j] - M);   // 0 for the heads beyond the group (-inf scores)
+      af.tsc[i][j] = x;
+      L += x;
+    }
+    L += __shfl_xor_sync(0xffffffffu, L, 8);
+    L += __shfl_xor_sync(0xffffffffu, L, 16);
+    if (lane < GP) af.red[warp][j] = L;
+    __syncthreads();
+    if (tid < GP) {
+      float s = 0.f;
+      for (int w = 0; w < NWARP; w++) s += af.red[w][tid];
+      af.L[tid] = s;
+    }
+  }
+  // ---- merge of the pieces for channels [rank * C, rank * C + C): item = (modality, m-tile, lane), a float4 of the piece
+  // = channels g and g + 8 of the tile for heads 2 t and 2 t + 1 (clusters of 16: half a tile, one of the two channels)
+  {
+    constexpr int MT = C >= 16 ? C / 16 : 1, ITEMS = 3 * MT * 32, SHARES = NTHREADS / ITEMS;
+    static_assert(NTHREADS % ITEMS == 0, "whole shares");
+    const int share = tid / ITEMS, it = tid % ITEMS;
+    const int L32 = it & 31, mt = (it >> 5) % MT, m = it / (32 * MT);
+    const int mu = C >= 16 ? rank * MT + mt : rank / 2;
+    const int j0 = 2 * (L32 & 3);
+    const int used = cnt > 0 ? (nwin + cnt - 1) / cnt : 0;   // pieces beyond have no windows
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    constexpr int IN_FLIGHT = 12;   // loads of a thread fetched together: the pieces come from L2
+    for (int p0 = share; p0 < used; p0 += IN_FLIGHT * SHARES) {
+      float4 x[IN_FLIGHT];
+#pragma unroll
+      for (int i = 0; i < IN_FLIGHT; i++) {
+        const int p = p0 + i * SHARES;
+        const bool have = p < used && ((sm.meta[p < used ? p : 0].held >> m) & 1);
+        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (have) x[i] = __ldcg(&pieces[p].frag[m][mu][L32]);
+      }
+#pragma unroll
+      for (int i = 0; i < IN_FLIGHT; i++) {
+        const int p = min(p0 + i * SHARES, used - 1);
+        const float2 f = *reinterpret_cast<const float2*>(&af.fac[p][j0]);
+        v.x = fmaf(x[i].x, f.x, v.x); v.y = fmaf(x[i].y, f.y, v.y); v.z = fmaf(x[i].z, f.x, v.z); v.w = fmaf(x[i].w, f.y, v.w);
+      }
+    }
+    af.part[tid] = v;
+    __syncthreads();
+    if (tid < ITEMS) {
+      for (int s = 1; s < SHARES; s++) {
+        const float4 x = af.part[s * ITEMS + tid];
+        v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+      }
+      constexpr float F = LEVEL_UNIT * 16.0f;   // numerators carry 2^P_LOG2 = 1/16
+      static_assert(P_LOG2 == -4.0f, "");
+      const int ch = 16 * mu + (L32 >> 2);
+      for (int r = 0; r < CS; r++) {   // to every CTA of the cluster
+        float* dst = cluster.map_shared_rank(&af.vec[0][0], r);
+        if (C >= 16 || (rank & 1) == 0) *reinterpret_cast<float2*>(dst + (m * D + ch) * GP + j0) = make_float2(v.x * F, v.y * F);
+        if (C >= 16 || (rank & 1) == 1) *reinterpret_cast<float2*>(dst + (m * D + ch + 8) * GP + j0) = make_float2(v.z * F, v.w * F);
+      }
+    }
+  }
+  cluster.sync();
+  cp_async_wait<0>();
+  __syncthreads();   // matrices and value rows have landed
+
+  // ---- out[j][c] = (raw[j][c] + sum_r R[r][c] vec[r][j]) / L: thread = (two columns, slice of rows), all heads
+  {
+    constexpr int KS = SM::KS, ROWS = 3 * D / KS;
+    static_assert(KS * ROWS == 3 * D, "whole slices");
+    const int c = 2 * (tid % (C / 2)), ks = tid / (C / 2);
+    float2 o[GP];
+#pragma unroll
+    for (int j = 0; j < GP; j++) o[j] = make_float2(0.f, 0.f);
+    auto add_row = [&](float2 x, const float* w) {
+      const float4 a = *reinterpret_cast<const float4*>(w), bq = *reinterpret_cast<const float4*>(w + 4);
+      const float wj[GP] = {a.x, a.y, a.z, a.w, bq.x, bq.y, bq.z, bq.w};
+#pragma unroll
+      for (int j = 0; j < GP; j++) { o[j].x = fmaf(x.x, wj[j], o[j].x); o[j].y = fmaf(x.y, wj[j], o[j].y); }
+    };
+#pragma unroll 8
+    for (int r = ks * ROWS; r < (ks + 1) * ROWS; r++) add_row(*reinterpret_cast<const float2*>(&af.R[r][c]), af.vec[r]);
+    for (int i = ks; i < n_tail; i += KS)   // raw value rows
+      add_row(__half22float2(*reinterpret_cast<const __half2*>(&af.v[i][c])), af.tsc[i]);
+#pragma unroll
+    for (int j = 0; j < GP; j++) *reinterpret_cast<float2*>(&af.prod[ks][j][c]) = o[j];
+    __syncthreads();
+    for (int i = tid; i < G * C; i += NTHREADS) {
+      const int j = i / C, cc = i % C;
+      float s = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < KS; k++) s += af.prod[k][j][cc];
+      const float L = af.L[j];
+      P.out[(((size_t)li * cv.batch + b) * cv.n_q_heads + h * G + j) * D + rank * C + cc] = L > 0.f ? s / L : 0.f;
+    }
+  }
+}
+
+template <int FMT, int CS>
+static void small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int units) {
+  cfg = {};
+  cfg.gridDim = dim3(units * CS);
+  cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = sizeof(SmallSmem<FMT, CS>);
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CS; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+}
+
+// clusters of this size the current device runs at once (0 if it cannot run them); looked up once per device and thread
+template <int FMT, int CS>
+static int small_clusters() {
+  static_assert(sizeof(SmallSmem<FMT, CS>) <= 227 * 1024, "shared memory of one CTA");
+  static thread_local int cached_dev = -1, cached = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev == cached_dev) return cached;
+  cudaError_t e = cudaFuncSetAttribute(k_decode_small<FMT, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<FMT, CS>));
+  if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(k_decode_small<FMT, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  int n = 0;
+  if (e == cudaSuccess) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    small_config<FMT, CS>(cfg, at, 1);
+    e = cudaOccupancyMaxActiveClusters(&n, k_decode_small<FMT, CS>, &cfg);
+  }
+  if (e != cudaSuccess) { (void)cudaGetLastError(); n = 0; }   // the split-K kernel takes the call
+  cached = n;
+  cached_dev = dev;
+  return n;
+}
+
+template <int FMT, int CS>
+static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  small_config<FMT, CS>(cfg, at, units);
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, k_decode_small<FMT, CS>, P);
+}
+
+template <int FMT>
+static int small_cluster(long long units, int n_cta) {
+  if (units * 16 <= n_cta && units <= small_clusters<FMT, 16>()) return 16;
+  if (units * 8 <= n_cta && units <= small_clusters<FMT, 8>()) return 8;
+  if (units * 4 <= n_cta && units <= small_clusters<FMT, 4>()) return 4;
+  return 0;
+}
+
+// Cluster size for a call, 0 if the split-K kernel should take it.  The clusters of all units have to be resident at once
+// (7 clusters of 16, 15 of 8, 33 of 4 on this GPU: a cluster stays inside one of its eight groups of SMs), and a warp's
+// share of the longest possible sequence has to be short: the units are not balanced against one another, and with fewer
+// CTAs than SMs a long walk costs more than the second launch saves.
+int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta) {
+  const long long units = (long long)layer_count * cv.batch * cv.n_kv_heads;
+  if (units * 4 > n_cta || cv.capacity / W > 16 * NWARP * SMALL_WINDOWS_PER_WARP) return 0;
+  const int cs = cv.fmt == FMT_MXFP4 ? small_cluster<FMT_MXFP4>(units, n_cta) : small_cluster<FMT_FP16>(units, n_cta);
+  return cv.capacity / W <= cs * NWARP * SMALL_WINDOWS_PER_WARP ? cs : 0;
+}
+
+template <int CS>
+static cudaError_t small_format(const DecodeParams& P, int units, cudaStream_t s) {
+  return P.cv.fmt == FMT_MXFP4 ? small_launch<FMT_MXFP4, CS>(P, units, s) : small_launch<FMT_FP16, CS>(P, units, s);
+}
+
+okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s) {
+  const int units = P.layer_count * P.cv.batch * P.cv.n_kv_heads;
+  const cudaError_t e = cs == 16 ? small_format<16>(P, units, s) : cs == 8 ? small_format<8>(P, units, s) : small_format<4>(P, units, s);
+  if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
+  return OKQ_OK;
+}
+
+}  // namespace okq

@@ -1,4 +1,5 @@
-// One warp's pass over packed windows, used by the split-K kernel (okq_decode_mma.cu): scores, online softmax and value sums of a contiguous range of windows.
+// One warp's pass over packed windows, shared by the split-K kernel (okq_decode_mma.cu) and the one-launch kernel for few
+// (sequence, head) units (okq_decode_small.cu): scores, online softmax and value sums of a contiguous range of windows.
 #pragma once
 #include "okq_common.cuh"
 #include "okq_device.cuh"
