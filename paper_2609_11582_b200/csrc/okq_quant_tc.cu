@@ -34,6 +34,7 @@
 
 #include "okq_common.cuh"
 #include "okq_device.cuh"
+#include "okq_quant_tail.cuh"
 
 namespace okq {
 
@@ -388,6 +389,10 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     // norm role: token rows 32*eq + lane, channels [32 q, 32 q + 32); epilogue role: channels 32*eq + lane (the
     // warp's tensor-memory lane quarter), window ewq
     const int eq = warp & 3, ewq = warp >> 2;
+    // while the first tile is on its way: this CTA's share of the modality bytes and of the raw tail rows
+    for (int bb = 0; bb < cv.batch; bb++) bulk_modality(cv, bb, modality, n_tokens, blockIdx.x * NT + tid, gridDim.x * NT);
+    for (int u = blockIdx.x; u < cv.batch * cv.n_kv_heads; u += gridDim.x)
+      bulk_tail_rows(cv, layer, u / cv.n_kv_heads, u % cv.n_kv_heads, vrows, vs_b, vs_h, vs_t, n_tokens, true, tid, NT);
     Slots slots;
     uint32_t jobidx = 0;
     bool dead = false;
