@@ -1,20 +1,26 @@
 // Offline calibration of the per-modality value rotations (Eq. 5, R_m = H U_m^T).
 //
-//   k_calib_rows / k_calib_cols   alpha = softmax(q k^T * scale) in 64 x 64 tiles on the tensor cores
+//   k_calib_pass<0>, <1>          alpha = softmax(q k^T * scale) in 128 x 64 tiles on the tensor cores
 //                                 (mma.sync, fp16 products, fp32 sums): first the row maximum and
 //                                 normaliser, then the column sums of alpha^2
 //   k_calib_wsum                  w_j: fixed-order sum of the per-(query tile, head) column sums
 //   k_calib_wmax, k_calib_moments C_m = sum w_j v_j^T v_j, tensor cores, values staged transposed
 //   k_calib_csum                  fixed-order sum of the per-chunk partial moments
-//   k_calib_eigen                 cyclic Jacobi (fp64, one block), ordering, signs, R = H U^T
+//   k_calib_eigen                 cyclic Jacobi (fp64, one cluster), ordering, signs, R = H U^T
+#include <cooperative_groups.h>
+
 #include "../../include/okq_calib.h"
 #include "okq_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace okq {
 namespace {
 
-constexpr int TQ = 64;          // queries per block (4 warps x 16 rows) and keys per tile
-constexpr int KS_STRIDE = D + 8;  // halves per staged key row: 272 bytes, conflict-free fragment reads
+constexpr int TQ = 128;         // queries per block: 4 warps x 32 rows
+constexpr int TK = 64;          // keys per staged tile
+constexpr int TQ_WS = 64;       // query tile the documented workspace size is counted in
+constexpr int KS_STRIDE = D + 8;  // halfs per staged key row: 272 bytes, conflict-free fragment reads
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1) {
@@ -23,122 +29,203 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// One pass over the key tiles of a 64-query block of one head.
-//   PASS 0: row maximum m and normaliser l of the softmax -> rowstat[(g * n + i) * 2 + {0, 1}]
-//   PASS 1: column sums of alpha^2 over the block's queries -> partial[(itile * G + g) * n + j]
-// grid (n_itiles, G), 128 threads.
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ float ex2f(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// One pass over the key tiles of a 128-query block of one head; scores in the log2 domain, s = (q . k) * scale2.
+//   PASS 0: rowstat[g * n + i] = -2 (m_i + log2 l_i), m_i = max_j s_ij, l_i = sum_j 2^(s_ij - m_i)
+//   PASS 1: column sums of alpha^2 = 2^(2 s + rowstat) over the block's queries -> partial[(itile * G + g) * n + j]
+// A warp owns 32 query rows (its fragments stay in registers, so each key fragment serves two products) and keeps the
+// running maximum and sum of its own columns per lane; the four lanes of a row meet once at the end.  Keys pass through
+// two cp.async buffers.  What bounds it: the products' dispatch (8.6 cycles of a sub-partition each) and one exponential
+// per score.  8192 tokens x 7 heads, both passes: 1.29 ms with 16 rows per warp, unbuffered tiles, scalar fragment loads and
+// expf of every score with a shuffle reduction per tile; see below for this form.
+// Block order: longest first, every other wave of blocks reversed, so that an SM's blocks add up to about the same.
 template <int PASS>
-__global__ void __launch_bounds__(128) k_calib_pass(const __half* __restrict__ q, const __half* __restrict__ k, int G, int n,
-                                                   float scale, int causal, float* __restrict__ rowstat,
-                                                   float* __restrict__ partial) {
-  __shared__ __align__(16) __half ks[TQ * KS_STRIDE];
-  __shared__ float colsum[4][TQ];
+__global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict__ q, const __half* __restrict__ k, int G, int n,
+                                                      float scale2, int causal, int n_sm, float* __restrict__ rowstat,
+                                                      float* __restrict__ partial) {
+  __shared__ __align__(16) __half ks[2][TK * KS_STRIDE];
+  __shared__ float colsum[4][TK];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int itile = blockIdx.x, head = blockIdx.y;
-  const int i0 = itile * TQ + warp * 16 + g, i1 = i0 + 8;   // this lane's two query rows
-  // A fragments of the queries: rows i0 / i1, 8 k-steps of 16 channels
-  uint32_t qa[8][4];
+  const int n_it = (n + TQ - 1) / TQ, n_blk = gridDim.x;
+  int id = blockIdx.x;
+  {
+    const int wave = id / n_sm, first = wave * n_sm, last = min(n_blk, first + n_sm) - 1;
+    if (wave & 1) id = first + last - id;
+  }
+  const int itile = n_it - 1 - id / G, head = id % G;
   const __half* qh = q + (size_t)head * n * D;
+  // the maximum below assumes a positive scale: a negative one goes into the queries' signs, zero into zero queries
+  const uint32_t flip = scale2 < 0.f ? 0x80008000u : 0u;
+  const bool no_q = scale2 == 0.f;
+  scale2 = no_q ? 1.0f : fabsf(scale2);
+  int row[2][2];   // this lane's query rows: [m-tile][upper / lower half]
+  uint32_t qa[2][8][4];
 #pragma unroll
-  for (int s = 0; s < 8; s++) {
-    const int c = 16 * s + 2 * t;
-    qa[s][0] = i0 < n ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i0 * D + c) : 0u;
-    qa[s][1] = i1 < n ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i1 * D + c) : 0u;
-    qa[s][2] = i0 < n ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i0 * D + c + 8) : 0u;
-    qa[s][3] = i1 < n ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i1 * D + c + 8) : 0u;
-  }
-  float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
-  if (PASS == 1) {
-    if (i0 < n) { m0 = rowstat[((size_t)head * n + i0) * 2]; l0 = 1.0f / rowstat[((size_t)head * n + i0) * 2 + 1]; }
-    if (i1 < n) { m1 = rowstat[((size_t)head * n + i1) * 2]; l1 = 1.0f / rowstat[((size_t)head * n + i1) * 2 + 1]; }
-  }
-  const int n_jt = causal ? itile + 1 : (n + TQ - 1) / TQ;
-  for (int jt = 0; jt < n_jt; jt++) {
-    __syncthreads();   // the previous tile's fragments and column sums have been consumed
-    for (int idx = tid; idx < TQ * (D / 8); idx += 128) {
-      const int r = idx >> 4, c8 = idx & 15, j = jt * TQ + r;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (j < n) v = *reinterpret_cast<const uint4*>(k + (size_t)j * D + c8 * 8);
-      *reinterpret_cast<uint4*>(&ks[r * KS_STRIDE + c8 * 8]) = v;
-    }
-    __syncthreads();
-    float s[8][4];
+  for (int mt = 0; mt < 2; mt++) {
+    row[mt][0] = itile * TQ + warp * 32 + mt * 16 + g;
+    row[mt][1] = row[mt][0] + 8;
 #pragma unroll
-    for (int nt = 0; nt < 8; nt++) {
-      float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int st = 0; st < 8; st++) {
-        const __half* kr = &ks[(nt * 8 + g) * KS_STRIDE + 16 * st + 2 * t];
-        mma16816(d, qa[st][0], qa[st][1], qa[st][2], qa[st][3], *reinterpret_cast<const uint32_t*>(kr),
-                 *reinterpret_cast<const uint32_t*>(kr + 8));
-      }
-      // d[0], d[1]: row i0, keys j, j+1;  d[2], d[3]: row i1
-      const int j = jt * TQ + nt * 8 + 2 * t;
+    for (int s = 0; s < 8; s++)
 #pragma unroll
       for (int e = 0; e < 4; e++) {
-        const int jj = j + (e & 1), ii = (e & 2) ? i1 : i0;
-        const bool live = jj < n && ii < n && (!causal || jj <= ii);
-        s[nt][e] = live ? d[e] * scale : -INFINITY;
+        const int i = row[mt][e & 1], c = 16 * s + 2 * t + 8 * (e >> 1);
+        qa[mt][s][e] = i < n && !no_q ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i * D + c) ^ flip : 0u;
+      }
+  }
+  float m[2][2], l[2][2];   // PASS 0: running maximum and sum; PASS 1: l = rowstat
+#pragma unroll
+  for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+    for (int hf = 0; hf < 2; hf++) {
+      m[mt][hf] = -INFINITY;
+      l[mt][hf] = PASS == 0 ? 0.f : (row[mt][hf] < n ? rowstat[(size_t)head * n + row[mt][hf]] : -INFINITY);
+    }
+  const int n_jt = causal ? min((n + TK - 1) / TK, (itile * TQ + TQ - 1) / TK + 1) : (n + TK - 1) / TK;
+  auto fetch = [&](int jt) {
+    if (jt < n_jt)
+#pragma unroll
+      for (int u = 0; u < TK * (D / 8) / 128; u++) {
+        const int idx = tid + 128 * u, r = idx >> 4, c8 = idx & 15, j = min(n - 1, jt * TK + r);   // (rows past the end: masked)
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&ks[jt & 1][r * KS_STRIDE + c8 * 8]);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(k + (size_t)j * D + c8 * 8));
+      }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  fetch(0);
+  for (int jt = 0; jt < n_jt; jt++) {
+    fetch(jt + 1);
+    asm volatile("cp.async.wait_group 1;\n" ::);
+    __syncthreads();
+    const __half* kt = ks[jt & 1];
+    // masks matter on the last tiles only
+    const bool edge = (jt + 1) * TK > n || (causal && (jt + 1) * TK - 1 > itile * TQ + warp * 32);
+#pragma unroll
+    for (int half = 0; half < 2; half++) {   // 32 keys at a time
+      float d[2][4][4];
+#pragma unroll
+      for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+        for (int nt = 0; nt < 4; nt++)
+#pragma unroll
+          for (int e = 0; e < 4; e++) d[mt][nt][e] = 0.f;
+#pragma unroll
+      for (int s2 = 0; s2 < 4; s2++)         // two k-steps per fragment load
+#pragma unroll
+        for (int nt = 0; nt < 4; nt++) {
+          uint32_t kb[4];
+          ldsm_x4(kb, kt + (half * 32 + nt * 8 + (lane & 7)) * KS_STRIDE + 32 * s2 + 8 * (lane >> 3));
+#pragma unroll
+          for (int mt = 0; mt < 2; mt++) {
+            mma16816(d[mt][nt], qa[mt][2 * s2][0], qa[mt][2 * s2][1], qa[mt][2 * s2][2], qa[mt][2 * s2][3], kb[0], kb[1]);
+            mma16816(d[mt][nt], qa[mt][2 * s2 + 1][0], qa[mt][2 * s2 + 1][1], qa[mt][2 * s2 + 1][2], qa[mt][2 * s2 + 1][3], kb[2], kb[3]);
+          }
+        }
+      if (edge) {
+#pragma unroll
+        for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+          for (int nt = 0; nt < 4; nt++)
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+              const int j = jt * TK + half * 32 + nt * 8 + 2 * t + (e & 1), i = row[mt][e >> 1];
+              if (j >= n || i >= n || (causal && j > i)) d[mt][nt][e] = -INFINITY;
+            }
+      }
+      if (PASS == 0) {
+#pragma unroll
+        for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+          for (int hf = 0; hf < 2; hf++) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int nt = 0; nt < 4; nt++) mx = fmaxf(mx, fmaxf(d[mt][nt][2 * hf], d[mt][nt][2 * hf + 1]));
+            const float mn = fmaxf(m[mt][hf], mx * scale2);
+            if (mn != -INFINITY) {
+              float a = l[mt][hf] * ex2f(m[mt][hf] - mn);   // 0 for the first finite maximum
+#pragma unroll
+              for (int nt = 0; nt < 4; nt++)
+                a += ex2f(fmaf(d[mt][nt][2 * hf], scale2, -mn)) + ex2f(fmaf(d[mt][nt][2 * hf + 1], scale2, -mn));
+              l[mt][hf] = a;
+              m[mt][hf] = mn;
+            }
+          }
+      } else {
+        const float two = 2.0f * scale2;
+        float c[8];   // column 8 (i >> 1) + 2 t + (i & 1): sums over this lane's four rows
+#pragma unroll
+        for (int nt = 0; nt < 4; nt++)
+#pragma unroll
+          for (int e = 0; e < 2; e++)
+            c[2 * nt + e] = (ex2f(fmaf(d[0][nt][e], two, l[0][0])) + ex2f(fmaf(d[0][nt][2 + e], two, l[0][1]))) +
+                            (ex2f(fmaf(d[1][nt][e], two, l[1][0])) + ex2f(fmaf(d[1][nt][2 + e], two, l[1][1])));
+        // over the eight row groups, each lane ending with one column: n-tile bits 1, 0 and e by lane bits 4, 3, 2
+#pragma unroll
+        for (int w = 4, bit = 16; w >= 1; w >>= 1, bit >>= 1) {
+          const bool up = (lane & bit) != 0;
+#pragma unroll
+          for (int i = 0; i < w; i++) {
+            const float give = up ? c[i] : c[i + w], keep = up ? c[i + w] : c[i];
+            c[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+          }
+        }
+        colsum[warp][half * 32 + 8 * (g >> 1) + 2 * t + (g & 1)] = c[0];
       }
     }
-    if (PASS == 0) {
-      float t0 = -INFINITY, t1 = -INFINITY;
-#pragma unroll
-      for (int nt = 0; nt < 8; nt++) {
-        t0 = fmaxf(t0, fmaxf(s[nt][0], s[nt][1]));
-        t1 = fmaxf(t1, fmaxf(s[nt][2], s[nt][3]));
-      }
-      t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2));
-      t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
-      const float n0 = fmaxf(m0, t0), n1 = fmaxf(m1, t1);
-      float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-      for (int nt = 0; nt < 8; nt++) {
-        if (n0 != -INFINITY) a0 += expf(s[nt][0] - n0) + expf(s[nt][1] - n0);
-        if (n1 != -INFINITY) a1 += expf(s[nt][2] - n1) + expf(s[nt][3] - n1);
-      }
-      a0 += __shfl_xor_sync(0xffffffffu, a0, 1); a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-      a1 += __shfl_xor_sync(0xffffffffu, a1, 1); a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
-      l0 = (m0 == -INFINITY ? 0.f : l0 * expf(m0 - n0)) + a0; m0 = n0;
-      l1 = (m1 == -INFINITY ? 0.f : l1 * expf(m1 - n1)) + a1; m1 = n1;
-    } else {
-#pragma unroll
-      for (int nt = 0; nt < 8; nt++) {
-        float c0 = 0.f, c1 = 0.f;   // keys j, j+1: squares of this lane's two rows
-        if (s[nt][0] != -INFINITY) { const float a = expf(s[nt][0] - m0) * l0; c0 += a * a; }
-        if (s[nt][2] != -INFINITY) { const float a = expf(s[nt][2] - m1) * l1; c0 += a * a; }
-        if (s[nt][1] != -INFINITY) { const float a = expf(s[nt][1] - m0) * l0; c1 += a * a; }
-        if (s[nt][3] != -INFINITY) { const float a = expf(s[nt][3] - m1) * l1; c1 += a * a; }
-#pragma unroll
-        for (int dl = 4; dl < 32; dl <<= 1) {   // over the eight row groups g
-          c0 += __shfl_xor_sync(0xffffffffu, c0, dl);
-          c1 += __shfl_xor_sync(0xffffffffu, c1, dl);
-        }
-        if (g == 0) { colsum[warp][nt * 8 + 2 * t] = c0; colsum[warp][nt * 8 + 2 * t + 1] = c1; }
-      }
-      __syncthreads();
-      if (tid < TQ) {
-        const int j = jt * TQ + tid;
+    __syncthreads();   // the tile has been read (and the column sums are in place)
+    if (PASS == 1) {
+      if (tid < TK) {
+        const int j = jt * TK + tid;
         if (j < n)
           partial[((size_t)itile * G + head) * n + j] = (colsum[0][tid] + colsum[1][tid]) + (colsum[2][tid] + colsum[3][tid]);
       }
+      __syncthreads();
     }
   }
-  if (PASS == 0 && t == 0) {
-    if (i0 < n) { rowstat[((size_t)head * n + i0) * 2] = m0; rowstat[((size_t)head * n + i0) * 2 + 1] = l0; }
-    if (i1 < n) { rowstat[((size_t)head * n + i1) * 2] = m1; rowstat[((size_t)head * n + i1) * 2 + 1] = l1; }
+  asm volatile("cp.async.wait_group 0;\n" ::);
+  if (PASS == 0) {
+#pragma unroll
+    for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+      for (int hf = 0; hf < 2; hf++) {
+        float mm = m[mt][hf], ll = l[mt][hf];
+#pragma unroll
+        for (int dl = 1; dl < 4; dl <<= 1) {
+          const float mo = __shfl_xor_sync(0xffffffffu, mm, dl), lo = __shfl_xor_sync(0xffffffffu, ll, dl);
+          const float mn = fmaxf(mm, mo);
+          ll = (mm == -INFINITY ? 0.f : ll * ex2f(mm - mn)) + (mo == -INFINITY ? 0.f : lo * ex2f(mo - mn));
+          mm = mn;
+        }
+        if (t == 0 && row[mt][hf] < n) rowstat[(size_t)head * n + row[mt][hf]] = -2.0f * (mm + log2f(ll));
+      }
   }
 }
 
-// w_j = sum over (query tile, head) of the column sums, in index order.  One thread per key.
-__global__ void k_calib_wsum(const float* __restrict__ partial, int G, int n, int causal, float* __restrict__ w) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const int n_it = (n + TQ - 1) / TQ;
+// w_j = sum over (query tile, head) of the column sums, in a fixed order: a warp per 32 keys' slice, its lanes one key each;
+// the block's warps take every eighth (tile, head) row and meet in shared memory
+__global__ void __launch_bounds__(256) k_calib_wsum(const float* __restrict__ partial, int G, int n, int causal, float* __restrict__ w) {
+  __shared__ float part[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, j = blockIdx.x * 32 + lane;
+  const int rows = (n + TQ - 1) / TQ * G, r0 = causal ? (blockIdx.x * 32) / TQ * G : 0;
   float acc = 0.f;
-  for (int it = causal ? j / TQ : 0; it < n_it; it++)
-    for (int g = 0; g < G; g++) acc += partial[((size_t)it * G + g) * n + j];
-  w[j] = acc;
+  if (j < n)
+#pragma unroll 4
+    for (int r = r0 + warp; r < rows; r += 8) acc += partial[(size_t)r * n + j];
+  part[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && j < n) {
+    float s = 0.f;
+    for (int i = 0; i < 8; i++) s += part[i][lane];
+    w[j] = s;
+  }
 }
 
 // ---------------------------------------------------------------- weighted moments
@@ -250,124 +337,267 @@ __global__ void k_calib_csum(const float* __restrict__ partial, int n_chunks, co
 
 constexpr int EIG_THREADS = 1024;
 constexpr int MAX_SWEEPS = 30;
+constexpr int NPOS = D / 2;                        // pairs per round
+constexpr int NBLK = NPOS * (NPOS - 1) / 2;        // 2 x 2 blocks above the diagonal
+constexpr int ROUNDS = D - 1;
+constexpr int V_CTAS = 4, V_COLS = D / V_CTAS;     // blocks that carry the eigenvectors, columns of each
 
-// Cyclic Jacobi on a symmetric 128 x 128 matrix in fp64, one block.  A lives in shared memory (128 KB), the
-// accumulated rotations as V^T (row l = eigenvector l) in global memory.  A sweep is 127 rounds of 64
-// disjoint pairs (round-robin pairing); a round computes its 64 rotations, then applies them to the rows
-// and to the columns of A and to the rows of V^T.  Stops after a sweep in which no rotation was needed.
-// Then: eigenvalues in descending order, every eigenvector with its largest-magnitude component positive,
-// R = H U^T with H = Had_128 diag(signs) / sqrt(128).
+// Cyclic Jacobi on a symmetric 128 x 128 matrix in fp64, one cluster of 1 + V_CTAS blocks.
+//
+// The round-robin pairing is kept as a ring (Brent and Luk): after every round each index moves one place, so the pair
+// k of a round is always positions (top k, bottom k) and a sweep of 127 rounds brings everybody home.  Block 0 holds the
+// matrix in position order, upper half only, as 2 x 2 blocks (pair k, pair l), one plane per block element: a thread owns
+// two blocks, reads them at fixed addresses, applies its rows' and its columns' rotation in registers and stores the
+// results where the move takes them, at fixed addresses of a second buffer.  Per round that is 128 KB of shared-memory
+// traffic and two block barriers; with the matrix in place, rows first and columns then, it was 512 KB, the
+// eigenvectors' rows through L2 and three barriers (5.2 us per round).
+// The rotations of a sweep go to the other blocks, which apply them to V^T (row = eigenvector estimate, V_COLS columns
+// each) while block 0 works on the next sweep.
+// The angle is taken in fp32 (the residual element is computed, not assumed zero, so that only costs a factor 1e-7 per
+// visit); cosine and sine are orthonormal to fp64 by two Newton steps.  Stops after a sweep whose largest tangent was
+// below 1e-8: what is left is quadratically smaller.
+// Then: eigenvalues in descending order, every eigenvector with its largest-magnitude component positive, R = H U^T with
+// H = Had_128 diag(signs) / sqrt(128), a Hadamard transform per column.
+struct EigA {
+  double buf[2][4 * NBLK + NPOS + D];   // off-diagonal planes [2 * row part + column part][block], pairs' elements, diagonal
+  double2 cs[NPOS];
+  double red[32];
+  unsigned maxt;                        // largest |tangent| of the sweep (float bits); 0: nothing rotated
+};
+struct EigV {
+  double v[D][V_COLS];                  // V^T, rows by index
+  double t[2][ROUNDS * NPOS];           // tangents of a sweep, written by block 0
+  double lam[D];
+  double best[V_CTAS][D];               // per slice and eigenvector: the slice's component of largest magnitude
+  int done[2];
+  int order[D];
+};
+constexpr int EIG_SMEM = sizeof(EigA) > sizeof(EigV) ? (int)sizeof(EigA) : (int)sizeof(EigV);
+static_assert(EIG_SMEM <= 227 * 1024, "shared memory of one block");
+
+// position 2 k: top of pair k, 2 k + 1: bottom
+__device__ __forceinline__ int eig_move(int pos) {
+  const int k = pos >> 1;
+  if ((pos & 1) == 0) return k == 0 ? 0 : (k == NPOS - 1 ? 2 * k + 1 : 2 * (k + 1));
+  return k == 0 ? 2 : 2 * (k - 1) + 1;
+}
+// index that sits at a position in round r
+__device__ __forceinline__ int eig_index(int pos, int r) {
+  const int k = pos >> 1;
+  if (pos == 0) return 0;
+  int x = ((pos & 1) ? 2 * NPOS - 2 - k : k - 1) - r;
+  return (x < 0 ? x + ROUNDS : x) + 1;
+}
+// blocks (k, l), k < l, numbered so that 32 warps own 63 each: warp w the rows w and 63 - w
+__device__ __forceinline__ int eig_block(int k, int l) {
+  return k < NPOS / 2 ? k * (NPOS - 1) + l - k - 1 : (NPOS - 1 - k) * (NPOS - 1) + k + (l - k - 1);
+}
+// where the element of positions (a, b) is kept
+__device__ __forceinline__ int eig_slot(int a, int b) {
+  if ((a >> 1) == (b >> 1)) return 4 * NBLK + (a >> 1);
+  if ((a >> 1) > (b >> 1)) { const int x = a; a = b; b = x; }
+  return (2 * (a & 1) + (b & 1)) * NBLK + eig_block(a >> 1, b >> 1);
+}
+__device__ __forceinline__ double2 eig_cos_sin(double t) {   // c = 1 / sqrt(1 + t^2) to fp64, s = t c
+  const double x = fma(t, t, 1.0), hx = 0.5 * x;
+  double y = (double)rsqrtf((float)x);
+  y = y * fma(-hx * y, y, 1.5);
+  y = y * fma(-hx * y, y, 1.5);
+  return make_double2(y, t * y);
+}
+
 __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __restrict__ C, const float* __restrict__ signs,
-                                                           double* __restrict__ vt, float* __restrict__ R,
-                                                           float* __restrict__ lambda, int* __restrict__ sweeps_out) {
+                                                           float* __restrict__ R, float* __restrict__ lambda,
+                                                           int* __restrict__ sweeps_out) {
   extern __shared__ __align__(16) unsigned char eig_raw[];
-  double* A = reinterpret_cast<double*>(eig_raw);                 // [128][128]
-  __shared__ double rc[64], rs[64];
-  __shared__ int rp[64], rq[64];
-  __shared__ int rotated;
-  __shared__ int order[D];
-  __shared__ double flip[D];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < D * D; idx += EIG_THREADS) {
-    const int a = idx / D, b = idx % D;
-    A[idx] = 0.5 * ((double)C[a * D + b] + (double)C[b * D + a]);
-    vt[idx] = a == b ? 1.0 : 0.0;
-  }
-  // the scale below which an off-diagonal element is left alone
-  __shared__ double tiny;
-  if (tid == 0) {
-    double tr = 0.0;
-    for (int i = 0; i < D; i++) tr += fabs((double)C[i * D + i]);
-    tiny = tr * 1e-18;
-  }
-  __syncthreads();
-  int sweeps = 0;
-  for (; sweeps < MAX_SWEEPS; sweeps++) {
-    if (tid == 0) rotated = 0;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x;
+  EigV& sv = *reinterpret_cast<EigV*>(eig_raw);
+  cluster.sync();   // every block runs before its shared memory is written from outside
+  if (rank == 0) {
+    EigA& sa = *reinterpret_cast<EigA*>(eig_raw);
+    // largest magnitude (the matrix is scaled by a power of two to at most 1) and trace
+    double mx = 0.0, tr = 0.0;
+    for (int i = tid; i < D * D; i += EIG_THREADS) mx = fmax(mx, fabs((double)C[i]));
+    if (tid < D) tr = fabs((double)C[tid * D + tid]);
+    for (int d = 16; d; d >>= 1) {
+      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+      tr += __shfl_xor_sync(0xffffffffu, tr, d);
+    }
+    if (lane == 0) sa.red[warp] = mx;
     __syncthreads();
-    for (int round = 0; round < D - 1; round++) {
-      if (tid < 64) {
-        int p, q;
-        if (tid == 0) { p = round; q = D - 1; }
-        else { p = (round + tid) % (D - 1); q = (round - tid + (D - 1)) % (D - 1); }
-        if (p > q) { const int x = p; p = q; q = x; }
-        const double apq = A[p * D + q], app = A[p * D + p], aqq = A[q * D + q];
-        double c = 1.0, s = 0.0;
-        if (fabs(apq) > tiny && fabs(apq) > 1e-17 * sqrt(fabs(app * aqq))) {
-          const double tau = (aqq - app) / (2.0 * apq);
-          const double tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          c = 1.0 / sqrt(1.0 + tt * tt);
-          s = tt * c;
-          rotated = 1;
+    for (int i = 0; i < 32; i++) mx = fmax(mx, sa.red[i]);
+    __syncthreads();
+    if (lane == 0 && warp < 4) sa.red[warp] = tr;
+    __syncthreads();
+    int ex = 0;
+    if (mx > 0.0) frexp(mx, &ex);   // mx < 2^ex
+    const double scale = ldexp(1.0, -ex);
+    // the size below which an off-diagonal element is left alone
+    const double tiny = fmax(((sa.red[0] + sa.red[1]) + (sa.red[2] + sa.red[3])) * scale * 1e-18, 1e-30);
+    for (int i = tid; i < D * D; i += EIG_THREADS) {
+      const int a = i / D, b = i % D;
+      if (a > b) continue;
+      const int ia = eig_index(a, 0), ib = eig_index(b, 0);
+      const double x = 0.5 * ((double)C[ia * D + ib] + (double)C[ib * D + ia]) * scale;
+      if (a == b) sa.buf[0][4 * NBLK + NPOS + a] = x;
+      else sa.buf[0][eig_slot(a, b)] = x;
+    }
+    // this thread's two blocks: where they are read, the rows' and columns' pairs, where their elements go
+    int rd[2], pk[2], pl[2], wr[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int j = lane + 32 * u;
+      const bool first = j < NPOS - 1 - warp;
+      pk[u] = first ? warp : NPOS - 1 - warp;
+      pl[u] = first ? warp + 1 + j : NPOS - warp + (j - (NPOS - 1 - warp));
+      rd[u] = warp * (NPOS - 1) + j;
+      if (j >= NPOS - 1) { rd[u] = -1; pk[u] = 0; pl[u] = 1; }
+#pragma unroll
+      for (int e = 0; e < 4; e++) wr[u][e] = eig_slot(eig_move(2 * pk[u] + (e >> 1)), eig_move(2 * pl[u] + (e & 1)));
+    }
+    const int dk = tid & (NPOS - 1);
+    const int d_off = eig_slot(eig_move(2 * dk), eig_move(2 * dk + 1));
+    const int d_top = 4 * NBLK + NPOS + eig_move(2 * dk), d_bot = 4 * NBLK + NPOS + eig_move(2 * dk + 1);
+    double* t_remote[V_CTAS];
+#pragma unroll
+    for (int r = 0; r < V_CTAS; r++) t_remote[r] = cluster.map_shared_rank(&sv.t[0][0], r + 1);
+    if (tid == 0) sa.maxt = 0;
+    __syncthreads();
+    int cur = 0, sweeps = 0, sweep = 0;
+    for (;; sweep++) {
+      const int tbase = (sweep & 1) * ROUNDS * NPOS;
+#pragma unroll 1
+      for (int round = 0; round < ROUNDS; round++) {
+        const double* in = sa.buf[cur];
+        double* out = sa.buf[cur ^ 1];
+        if (tid < NPOS) {
+          const double app = in[4 * NBLK + NPOS + 2 * dk], aqq = in[4 * NBLK + NPOS + 2 * dk + 1], apq = in[4 * NBLK + dk];
+          double t = 0.0, res = apq;
+          double2 cs = make_double2(1.0, 0.0);
+          if (fabs(apq) > tiny && apq * apq > 1e-34 * fabs(app * aqq)) {
+            const float tau = __fdividef((float)(aqq - app), 2.0f * (float)apq);
+            const float tf = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+            t = (double)tf;
+            cs = eig_cos_sin(t);
+            res = cs.x * cs.x * fma(1.0 - t * t, apq, t * (app - aqq));
+            atomicMax(&sa.maxt, __float_as_uint(fabsf(tf)));
+          }
+          sa.cs[dk] = cs;
+          out[d_top] = app - t * (apq + res);
+          out[d_bot] = aqq + t * (apq + res);
+          out[d_off] = res;
+#pragma unroll
+          for (int r = 0; r < V_CTAS; r++) t_remote[r][tbase + round * NPOS + dk] = t;
         }
-        rc[tid] = c; rs[tid] = s; rp[tid] = p; rq[tid] = q;
+        double x[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+          if (rd[u] >= 0)
+#pragma unroll
+            for (int e = 0; e < 4; e++) x[u][e] = in[e * NBLK + rd[u]];
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+          if (rd[u] >= 0) {
+            const double2 ck = sa.cs[pk[u]], cl = sa.cs[pl[u]];
+            const double r00 = ck.x * x[u][0] - ck.y * x[u][2], r01 = ck.x * x[u][1] - ck.y * x[u][3];
+            const double r10 = ck.y * x[u][0] + ck.x * x[u][2], r11 = ck.y * x[u][1] + ck.x * x[u][3];
+            out[wr[u][0]] = cl.x * r00 - cl.y * r01;
+            out[wr[u][1]] = cl.y * r00 + cl.x * r01;
+            out[wr[u][2]] = cl.x * r10 - cl.y * r11;
+            out[wr[u][3]] = cl.y * r10 + cl.x * r11;
+          }
+        __syncthreads();
+        cur ^= 1;
       }
+      const float mt = __uint_as_float(sa.maxt);
+      if (mt > 0.0f) sweeps++;
+      const bool done = mt <= 1e-8f || sweep + 1 >= MAX_SWEEPS;
+      if (tid < V_CTAS) cluster.map_shared_rank(&sv.done[0], tid + 1)[sweep & 1] = done;
       __syncthreads();
-      // rows: A <- J^T A, and V^T <- J^T V^T (the rows of V^T are the eigenvector estimates)
-      for (int idx = tid; idx < 64 * D; idx += EIG_THREADS) {
-        const int kk = idx >> 7, j = idx & (D - 1);
-        const double c = rc[kk], s = rs[kk];
-        if (s != 0.0) {
-          const int p = rp[kk], q = rq[kk];
-          const double ap = A[p * D + j], aq = A[q * D + j];
-          A[p * D + j] = c * ap - s * aq;
-          A[q * D + j] = s * ap + c * aq;
-          const double vp = vt[p * D + j], vq = vt[q * D + j];
-          vt[p * D + j] = c * vp - s * vq;
-          vt[q * D + j] = s * vp + c * vq;
-        }
-      }
-      __syncthreads();
-      // columns: A <- A J
-      for (int idx = tid; idx < 64 * D; idx += EIG_THREADS) {
-        const int kk = idx & 63, i = idx >> 6;
-        const double c = rc[kk], s = rs[kk];
-        if (s != 0.0) {
-          const int p = rp[kk], q = rq[kk];
-          const double ap = A[i * D + p], aq = A[i * D + q];
-          A[i * D + p] = c * ap - s * aq;
-          A[i * D + q] = s * ap + c * aq;
+      if (tid == 0) sa.maxt = 0;
+      cluster.sync();   // the sweep's tangents are in place; the sweep before has been applied
+      if (done) break;
+    }
+    if (tid == 0 && sweeps_out) *sweeps_out = sweeps;
+    if (tid < D) {
+      const double l = sa.buf[cur][4 * NBLK + NPOS + tid] * ldexp(1.0, ex);
+      const int idx = eig_index(tid, 0);
+      for (int r = 0; r < V_CTAS; r++) cluster.map_shared_rank(&sv.lam[0], r + 1)[idx] = l;
+    }
+    cluster.sync();   // eigenvalues are out
+    cluster.sync();   // (the other blocks exchange their slices' largest components)
+    return;
+  }
+  const int col0 = (rank - 1) * V_COLS;
+  for (int i = tid; i < D * V_COLS; i += EIG_THREADS) sv.v[i / V_COLS][i % V_COLS] = i / V_COLS == col0 + i % V_COLS ? 1.0 : 0.0;
+  for (int sweep = 0;; sweep++) {
+    cluster.sync();
+    const double* ts = sv.t[sweep & 1];
+    for (int round = 0; round < ROUNDS; round++) {
+      // a warp takes two pairs, a lane one column
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        const int k = warp + 32 * u;
+        const double t = ts[round * NPOS + k];
+        if (t != 0.0) {
+          const double2 cs = eig_cos_sin(t);
+          double* vp = &sv.v[eig_index(2 * k, round)][lane];
+          double* vq = &sv.v[eig_index(2 * k + 1, round)][lane];
+          const double a = *vp, b = *vq;
+          *vp = cs.x * a - cs.y * b;
+          *vq = cs.y * a + cs.x * b;
         }
       }
       __syncthreads();
     }
-    if (!rotated) break;
-    __syncthreads();
+    if (sv.done[sweep & 1]) break;
   }
-  if (tid == 0 && sweeps_out) *sweeps_out = sweeps;
-  // descending order (ties by index) and sign convention
-  if (tid < D) {
-    const double li = A[tid * D + tid];
-    int rank = 0;
-    for (int j = 0; j < D; j++) {
-      const double lj = A[j * D + j];
-      rank += (lj > li) || (lj == li && j < tid);
-    }
-    order[rank] = tid;
-    double best = 0.0, val = 1.0;
-    for (int j = 0; j < D; j++) {
-      const double x = vt[tid * D + j];
+  cluster.sync();   // eigenvalues are here
+  if (tid < D) {    // the slice's component of largest magnitude (the first of equals), to all slices
+    double best = 0.0, val = 0.0;
+    for (int j = 0; j < V_COLS; j++) {
+      const double x = sv.v[tid][j];
       if (fabs(x) > best) { best = fabs(x); val = x; }
     }
-    flip[tid] = val < 0.0 ? -1.0 : 1.0;
-  }
-  __syncthreads();
-  if (tid < D) lambda[tid] = (float)A[order[tid] * D + order[tid]];
-  // R[c][k] = sum_l H[c][l] * U[k][l], U[k][l] = component k of the l-th eigenvector (in sorted order)
-  for (int idx = tid; idx < D * D; idx += EIG_THREADS) {
-    const int c = idx / D, k = idx % D;
-    double acc = 0.0;
-    for (int l = 0; l < D; l++) {
-      const int src = order[l];
-      const double h = ((__popc(c & l) & 1) ? -1.0 : 1.0) * (double)signs[l];
-      acc += h * flip[src] * vt[src * D + k];
+    for (int r = 0; r < V_CTAS; r++) cluster.map_shared_rank(&sv.best[0][0], r + 1)[(rank - 1) * D + tid] = val;
+    const double li = sv.lam[tid];
+    int pos = 0;   // descending order, ties by index
+    for (int j = 0; j < D; j++) {
+      const double lj = sv.lam[j];
+      pos += (lj > li) || (lj == li && j < tid);
     }
-    R[idx] = (float)(acc * 0.08838834764831845);   // 1 / sqrt(128)
+    sv.order[pos] = tid;
+    if (rank == 1) lambda[pos] = (float)li;
+  }
+  cluster.sync();
+  {  // R[c][k] = sum_l H[c][l] U[k][l]: warp = column k, lane holds l = lane + 32 i
+    double x[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int l = lane + 32 * i, src = sv.order[l];
+      double best = 0.0, val = 1.0;
+      for (int r = 0; r < V_CTAS; r++)
+        if (fabs(sv.best[r][src]) > best) { best = fabs(sv.best[r][src]); val = sv.best[r][src]; }
+      x[i] = (val < 0.0 ? -1.0 : 1.0) * (double)signs[l] * sv.v[src][warp];
+    }
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const double o = __shfl_xor_sync(0xffffffffu, x[i], d);
+        x[i] = (lane & d) ? o - x[i] : x[i] + o;
+      }
+    const double y0 = x[0] + x[1], y1 = x[0] - x[1], y2 = x[2] + x[3], y3 = x[2] - x[3];
+    const double o[4] = {y0 + y2, y1 + y3, y0 - y2, y1 - y3};
+#pragma unroll
+    for (int i = 0; i < 4; i++) R[(size_t)(lane + 32 * i) * D + col0 + warp] = (float)(o[i] * 0.08838834764831845);   // 1 / sqrt(128)
   }
 }
 
 size_t attn_bytes(int group, int n) {
-  const size_t n_it = (size_t)(n + TQ - 1) / TQ;
+  const size_t n_it = (size_t)(n + TQ_WS - 1) / TQ_WS;
   return ((size_t)group * n * 2 + n_it * group * n) * sizeof(float);
 }
 size_t moments_bytes() { return (size_t)MAX_CHUNKS * 3 * D * D * sizeof(float) + 16; }
@@ -397,12 +627,13 @@ okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   float* rowstat = static_cast<float*>(workspace);
   float* partial = rowstat + (size_t)group * n * 2;
-  const dim3 grid((n + TQ - 1) / TQ, group);
+  const int grid = (n + TQ - 1) / TQ * group, n_sm = sm_count();
   const __half* q = static_cast<const __half*>(q_fp16);
   const __half* k = static_cast<const __half*>(k_fp16);
-  k_calib_pass<0><<<grid, 128, 0, s>>>(q, k, group, n, sm_scale, causal, rowstat, partial);
-  k_calib_pass<1><<<grid, 128, 0, s>>>(q, k, group, n, sm_scale, causal, rowstat, partial);
-  k_calib_wsum<<<(n + 127) / 128, 128, 0, s>>>(partial, group, n, causal, w_out);
+  const float scale2 = sm_scale * 1.4426950408889634f;
+  k_calib_pass<0><<<grid, 128, 0, s>>>(q, k, group, n, scale2, causal, n_sm, rowstat, partial);
+  k_calib_pass<1><<<grid, 128, 0, s>>>(q, k, group, n, scale2, causal, n_sm, rowstat, partial);
+  k_calib_wsum<<<(n + 31) / 32, 256, 0, s>>>(partial, group, n, causal, w_out);
   return launch_status();
 }
 
@@ -430,12 +661,22 @@ okq_status okq_calib_rotation(const float* C, const float* signs, void* workspac
   static thread_local unsigned long long attr_mask = 0;
   int attr_dev = 0;
   if (attr_needed(attr_mask, attr_dev)) {
-    cudaError_t e = cudaFuncSetAttribute(k_calib_eigen, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EIGEN_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(k_calib_eigen, cudaFuncAttributeMaxDynamicSharedMemorySize, EIG_SMEM);
     if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
     attr_done(attr_mask, attr_dev);
   }
-  k_calib_eigen<<<1, EIG_THREADS, EIGEN_BYTES, static_cast<cudaStream_t>(stream)>>>(C, signs, static_cast<double*>(workspace), R_out,
-                                                                                  lambda_out, sweeps_out);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1 + V_CTAS);
+  cfg.blockDim = dim3(EIG_THREADS);
+  cfg.dynamicSmemBytes = EIG_SMEM;
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 1 + V_CTAS; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, k_calib_eigen, C, signs, R_out, lambda_out, sweeps_out);
+  if (le != cudaSuccess) { set_last_cuda_error((int)le); return OKQ_ERR_CUDA; }
   return launch_status();
 }
 
