@@ -562,11 +562,17 @@ __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __rest
       if (fabs(x) > best) { best = fabs(x); val = x; }
     }
     for (int r = 0; r < V_CTAS; r++) cluster.map_shared_rank(&sv.best[0][0], r + 1)[(rank - 1) * D + tid] = val;
+    // descending order, ties by index, on the numbers' bit patterns made monotone: a permutation whatever the input (NaN too)
+    auto key = [](double x) {
+      const long long b = __double_as_longlong(x + 0.0);   // (-0 counts as 0)
+      return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+    };
     const double li = sv.lam[tid];
-    int pos = 0;   // descending order, ties by index
+    const long long ki = key(li);
+    int pos = 0;
     for (int j = 0; j < D; j++) {
-      const double lj = sv.lam[j];
-      pos += (lj > li) || (lj == li && j < tid);
+      const long long kj = key(sv.lam[j]);
+      pos += (kj > ki) || (kj == ki && j < tid);
     }
     sv.order[pos] = tid;
     if (rank == 1) lambda[pos] = (float)li;
