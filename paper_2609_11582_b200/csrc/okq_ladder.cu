@@ -2,56 +2,17 @@
 // Plain CUDA-core kernels that follow the 2-bit path's arithmetic with the number of levels changed:
 //   k_ladder_keys    Eq. 2 + Eq. 4: one block per 32-token window of one (sequence, KV head)
 //   k_ladder_values  Eq. 6 + Eq. 3: likewise, the rotation as one fused-multiply-add chain per coordinate
-//   k_ladder_decode  Eq. 1 in the rotated space: one block per (sequence, KV head) walks the windows
+// (decode attention: okq_ladder_decode.cu)
 // The value levels are the Lloyd-Max quantiser of N(0, 1/128) with 2^b levels (fixed point of: level = mean of its
 // cell, threshold = mid-point of neighbouring levels), held as constants.
 #include "../../include/okq_ladder.h"
-#include "okq_common.cuh"
-#include "okq_device.cuh"
+#include "okq_ladder.cuh"
 
 namespace okq {
 
 namespace {
 
 constexpr int GP_L = OKQ_MAX_GROUP;   // padded GQA group
-
-// ascending levels / thresholds for b = 2, 3, 4 (index b - 2); the middle threshold is 0 by symmetry
-__constant__ float c_levels[3][16] = {
-    {-0x1.116a30p-3f, -0x1.47d908p-5f, 0x1.47d908p-5f, 0x1.116a30p-3f},
-    {-0x1.858b36p-3f, -0x1.e68c10p-4f, -0x1.11b402p-4f, -0x1.62ef2ep-6f, 0x1.62ef2ep-6f, 0x1.11b402p-4f, 0x1.e68c10p-4f,
-     0x1.858b36p-3f},
-    {-0x1.eea6ccp-3f, -0x1.76883ap-3f, -0x1.24e5cep-3f, -0x1.c6cde4p-4f, -0x1.5529e8p-4f, -0x1.db8b5ep-5f, -0x1.18fa1cp-5f,
-     -0x1.73df2ap-7f, 0x1.73df2ap-7f, 0x1.18fa1cp-5f, 0x1.db8b5ep-5f, 0x1.5529e8p-4f, 0x1.c6cde4p-4f, 0x1.24e5cep-3f,
-     0x1.76883ap-3f, 0x1.eea6ccp-3f}};
-__constant__ float c_thresholds[3][16] = {
-    {-0x1.636072p-4f, 0.0f, 0x1.636072p-4f},
-    {-0x1.3c689ep-3f, -0x1.7c200ap-4f, -0x1.6a6fccp-5f, 0.0f, 0x1.6a6fccp-5f, 0x1.7c200ap-4f, 0x1.3c689ep-3f},
-    {-0x1.b29782p-3f, -0x1.4db704p-3f, -0x1.042660p-3f, -0x1.8dfbe6p-4f, -0x1.2177ccp-4f, -0x1.7a42bcp-5f, -0x1.75f1e6p-6f, 0.0f,
-     0x1.75f1e6p-6f, 0x1.7a42bcp-5f, 0x1.2177ccp-4f, 0x1.8dfbe6p-4f, 0x1.042660p-3f, 0x1.4db704p-3f, 0x1.b29782p-3f}};
-const float h_levels[3][16] = {
-    {-0x1.116a30p-3f, -0x1.47d908p-5f, 0x1.47d908p-5f, 0x1.116a30p-3f},
-    {-0x1.858b36p-3f, -0x1.e68c10p-4f, -0x1.11b402p-4f, -0x1.62ef2ep-6f, 0x1.62ef2ep-6f, 0x1.11b402p-4f, 0x1.e68c10p-4f,
-     0x1.858b36p-3f},
-    {-0x1.eea6ccp-3f, -0x1.76883ap-3f, -0x1.24e5cep-3f, -0x1.c6cde4p-4f, -0x1.5529e8p-4f, -0x1.db8b5ep-5f, -0x1.18fa1cp-5f,
-     -0x1.73df2ap-7f, 0x1.73df2ap-7f, 0x1.18fa1cp-5f, 0x1.db8b5ep-5f, 0x1.5529e8p-4f, 0x1.c6cde4p-4f, 0x1.24e5cep-3f,
-     0x1.76883ap-3f, 0x1.eea6ccp-3f}};
-const float h_thresholds[3][16] = {
-    {-0x1.636072p-4f, 0.0f, 0x1.636072p-4f},
-    {-0x1.3c689ep-3f, -0x1.7c200ap-4f, -0x1.6a6fccp-5f, 0.0f, 0x1.6a6fccp-5f, 0x1.7c200ap-4f, 0x1.3c689ep-3f},
-    {-0x1.b29782p-3f, -0x1.4db704p-3f, -0x1.042660p-3f, -0x1.8dfbe6p-4f, -0x1.2177ccp-4f, -0x1.7a42bcp-5f, -0x1.75f1e6p-6f, 0.0f,
-     0x1.75f1e6p-6f, 0x1.7a42bcp-5f, 0x1.2177ccp-4f, 0x1.8dfbe6p-4f, 0x1.042660p-3f, 0x1.4db704p-3f, 0x1.b29782p-3f}};
-
-struct LadderView {
-  int batch, n_kv_heads, n_q_heads, capacity, bits;
-  unsigned char* k_codes;
-  __half* k_norm;
-  __half* k_meta;
-  unsigned char* v_codes;
-  __half* v_norm;
-  unsigned char* modality;
-  __host__ __device__ size_t unit(int b, int h) const { return (size_t)b * n_kv_heads + h; }
-  __host__ __device__ int row_bytes() const { return 16 * bits; }
-};
 
 // packs the 32 codes cd[0..31] (channels 32 part .. 32 part + 31 of one token) into 4 * bits bytes of its bit stream
 __device__ __forceinline__ void pack_quarter(const unsigned char* cd, int bits, unsigned char* dst) {
@@ -234,168 +195,6 @@ __global__ void __launch_bounds__(128) k_ladder_values(LadderView cv, const __ha
 namespace okq {
 namespace {
 
-constexpr int LD_THREADS = 256;
-
-struct DecodeSmemL {
-  float qrot[GP_L][D];        // rotated queries H D q / sqrt(128)
-  float wgt[GP_L][D];         // q'_c s_c of the window
-  float lev[16];              // value levels
-  float m[D], s[D];
-  float bias[GP_L];
-  float sc[GP_L][W];          // scores, then numerators p * |v|
-  float alpha[GP_L];
-  float acc[3][GP_L][D];      // end: rotated-basis sums per modality
-  float linv[GP_L];
-  unsigned char mod[W];
-  __align__(16) unsigned char kc[W * 64], vc[W * 64];   // the window's code rows (W * 16 * bits bytes each), staged
-};
-
-// grid (heads, batch), 256 threads: warp j = head j for the query rotation and the softmax; thread (c, hh) = channel
-// c, heads 4 hh .. 4 hh + 3 for the value sums
-__global__ void __launch_bounds__(LD_THREADS) k_ladder_decode(LadderView cv, int n_tokens, const __half* __restrict__ q,
-                                                             float sm_scale, const float* __restrict__ signs,
-                                                             const float* __restrict__ R, int n_R, float* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  DecodeSmemL& sm = *reinterpret_cast<DecodeSmemL*>(smem_raw);
-  const int h = blockIdx.x, b = blockIdx.y;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int G = cv.n_q_heads / cv.n_kv_heads, bits = cv.bits;
-  const size_t u = cv.unit(b, h);
-  const int rb = cv.row_bytes();
-  constexpr float LOG2E = 1.4426950408889634f;
-  // rotated queries
-  {
-    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (warp < G) {
-      const float4 x = load_row4(q + ((size_t)b * cv.n_q_heads + (size_t)h * G + warp) * D, lane);
-      const float4 sg = *reinterpret_cast<const float4*>(signs + 4 * lane);
-      y = warp_fwht(make_float4(sg.x * x.x, sg.y * x.y, sg.z * x.z, sg.w * x.w), lane);
-    }
-    sm.qrot[warp][4 * lane + 0] = y.x * RSQRT_D; sm.qrot[warp][4 * lane + 1] = y.y * RSQRT_D;
-    sm.qrot[warp][4 * lane + 2] = y.z * RSQRT_D; sm.qrot[warp][4 * lane + 3] = y.w * RSQRT_D;
-  }
-  if (tid < 16) sm.lev[tid] = c_levels[bits - 2][tid];
-  const int c = tid & (D - 1), hh = tid >> 7;
-  float acc[3][4];
-#pragma unroll
-  for (int m = 0; m < 3; m++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) acc[m][j] = 0.f;
-  float run_m = -INFINITY, run_l = 0.f;   // per warp = head (every lane holds the same value)
-  __syncthreads();
-  const int n_win = n_tokens / W;
-  for (int win = 0; win < n_win; win++) {
-    const size_t tok0 = u * cv.capacity + (size_t)win * W;
-    if (tid < D) {
-      const __half* meta = cv.k_meta + ((u * (cv.capacity / W) + win) * D + tid) * 2;
-      sm.m[tid] = __half2float(meta[0]); sm.s[tid] = __half2float(meta[1]);
-    }
-    if (tid < W) sm.mod[tid] = cv.modality[(size_t)b * cv.capacity + (size_t)win * W + tid];
-    {   // the window's rows are contiguous: W * rb bytes = 2 * bits * 32 pieces of 16 bytes per side
-      const int n16 = W * rb / 16;
-      const uint4* ksrc = reinterpret_cast<const uint4*>(cv.k_codes + tok0 * rb);
-      const uint4* vsrc = reinterpret_cast<const uint4*>(cv.v_codes + tok0 * rb);
-      if (tid < n16) reinterpret_cast<uint4*>(sm.kc)[tid] = ksrc[tid];
-      else if (tid >= 128 && tid - 128 < n16) reinterpret_cast<uint4*>(sm.vc)[tid - 128] = vsrc[tid - 128];
-    }
-    __syncthreads();
-    {   // weights and bias of head `warp`
-      float bsum = 0.f;
-#pragma unroll
-      for (int k4 = 0; k4 < 4; k4++) {
-        const int cc = 4 * lane + k4;
-        const float qv = sm.qrot[warp][cc];
-        sm.wgt[warp][cc] = qv * sm.s[cc];
-        bsum = fmaf(qv, sm.m[cc], bsum);
-      }
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) bsum += __shfl_xor_sync(0xffffffffu, bsum, d);
-      if (lane == 0) sm.bias[warp] = bsum;
-    }
-    __syncthreads();
-    // scores: warp w takes tokens 4 w .. 4 w + 3, a lane four channels
-    for (int tt = 0; tt < 4; tt++) {
-      const int t = 4 * warp + tt;
-      const unsigned char* row = sm.kc + t * rb;
-      float cd[4];
-#pragma unroll
-      for (int k4 = 0; k4 < 4; k4++) cd[k4] = (float)load_code(row, bits, 4 * lane + k4);
-      const float kn = __half2float(cv.k_norm[tok0 + t]) * sm_scale * LOG2E;
-#pragma unroll
-      for (int j = 0; j < GP_L; j++) {
-        float d = 0.f;
-#pragma unroll
-        for (int k4 = 0; k4 < 4; k4++) d = fmaf(sm.wgt[j][4 * lane + k4], cd[k4], d);
-#pragma unroll
-        for (int sft = 1; sft < 32; sft <<= 1) d += __shfl_xor_sync(0xffffffffu, d, sft);
-        if (lane == 0) sm.sc[j][t] = (d + sm.bias[j]) * kn;
-      }
-    }
-    __syncthreads();
-    {   // online softmax of head `warp` over the window's 32 tokens (lane = token)
-      const float x = sm.sc[warp][lane];
-      float mx = x;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-      const float m_new = fmaxf(run_m, mx);
-      const float al = exp2f(run_m - m_new);
-      const float p = exp2f(x - m_new);
-      float ps = p;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) ps += __shfl_xor_sync(0xffffffffu, ps, d);
-      run_l = run_l * al + ps;
-      run_m = m_new;
-      sm.sc[warp][lane] = p * __half2float(cv.v_norm[tok0 + lane]);
-      if (lane == 0) sm.alpha[warp] = al;
-    }
-    __syncthreads();
-    {   // value sums in the rotated basis of each token's modality
-      float al[4];
-#pragma unroll
-      for (int j = 0; j < 4; j++) al[j] = sm.alpha[4 * hh + j];
-#pragma unroll
-      for (int m = 0; m < 3; m++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[m][j] *= al[j];
-      for (int t = 0; t < W; t++) {
-        const float lv = sm.lev[load_code(sm.vc + t * rb, bits, c)];
-        const int md = sm.mod[t];   // the same for every thread: a uniform branch around register-indexed sums
-        if (md == 0) {
-#pragma unroll
-          for (int j = 0; j < 4; j++) acc[0][j] = fmaf(sm.sc[4 * hh + j][t], lv, acc[0][j]);
-        } else if (md == 1) {
-#pragma unroll
-          for (int j = 0; j < 4; j++) acc[1][j] = fmaf(sm.sc[4 * hh + j][t], lv, acc[1][j]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; j++) acc[2][j] = fmaf(sm.sc[4 * hh + j][t], lv, acc[2][j]);
-        }
-      }
-    }
-    __syncthreads();
-  }
-  // R_m^T once per head, then the normalisation
-#pragma unroll
-  for (int m = 0; m < 3; m++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) sm.acc[m][4 * hh + j][c] = acc[m][j];
-  if (lane == 0) sm.linv[warp] = run_l > 0.f ? 1.0f / run_l : 0.f;
-  __syncthreads();
-  const float* Rset = R + (size_t)(n_R == 1 ? 0 : h) * 3 * D * D;
-  float o[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int m = 0; m < 3; m++)
-    for (int r = 0; r < D; r++) {
-      const float rv = __ldg(Rset + ((size_t)m * D + r) * D + c);
-#pragma unroll
-      for (int j = 0; j < 4; j++) o[j] = fmaf(rv, sm.acc[m][4 * hh + j][r], o[j]);
-    }
-#pragma unroll
-  for (int j = 0; j < 4; j++) {
-    const int head = 4 * hh + j;
-    if (head < G) out[((size_t)b * cv.n_q_heads + (size_t)h * G + head) * D + c] = o[j] * sm.linv[head];
-  }
-}
-
 // TurboQuant codec (Preliminaries, Eq. 2-3): norm, randomised Hadamard rotation, nearest level of the fixed codebook;
 // no window statistics, no modality rotation.  32 vectors per block of 128 threads.
 __global__ void __launch_bounds__(128) k_turboquant_encode(const __half* __restrict__ x, long long n, int bits,
@@ -516,15 +315,9 @@ okq_status okq_ladder_decode_attention(const okq_ladder_cache* cache, int32_t n_
   if (st != OKQ_OK) return st;
   if (!q || !signs || !R || !out || (n_R != 1 && n_R != cache->n_kv_heads)) return OKQ_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(signs) || !aligned16(R) || !aligned16(out)) return OKQ_ERR_ALIGNMENT;
-  static thread_local unsigned long long attr_mask = 0;
-  int attr_dev = 0;
-  if (attr_needed(attr_mask, attr_dev)) {
-    cudaError_t e = cudaFuncSetAttribute(k_ladder_decode, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecodeSmemL));
-    if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
-    attr_done(attr_mask, attr_dev);
-  }
-  k_ladder_decode<<<dim3(cache->n_kv_heads, cache->batch), LD_THREADS, sizeof(DecodeSmemL), static_cast<cudaStream_t>(stream)>>>(
-      ladder_view(cache), n_tokens, static_cast<const __half*>(q), sm_scale, signs, R, n_R, out);
+  const cudaError_t e = launch_ladder_decode(ladder_view(cache), n_tokens, static_cast<const __half*>(q), sm_scale, signs, R, n_R, out,
+                                             static_cast<cudaStream_t>(stream));
+  if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return launch_status();
 }
 
