@@ -7,6 +7,7 @@
 // cell, threshold = mid-point of neighbouring levels), held as constants.
 #include "../../include/okq_ladder.h"
 #include "okq_ladder.cuh"
+#include "okq_rotate.cuh"
 
 namespace okq {
 
@@ -32,67 +33,82 @@ __device__ __forceinline__ void pack_quarter(const unsigned char* cd, int bits, 
   for (int k = 0; k < nb; k++) dst[k] = (unsigned char)((k < 8 ? lo >> (8 * k) : hi >> (8 * (k - 8))) & 0xffu);
 }
 
-// code of channel c in a token's bit stream
-__device__ __forceinline__ unsigned load_code(const unsigned char* row, int bits, int c) {
-  const int pos = bits * c, byte = pos >> 3;
-  const unsigned w = (unsigned)row[byte] | ((unsigned)row[byte + ((pos & 7) + bits > 8 ? 1 : 0)] << 8);
-  return (w >> (pos & 7)) & ((1u << bits) - 1u);
+// Codes are integers k added to 1.5 * 2^23: the float's bits are MAGIC_BITS + k, and eight of them at 8 field positions sum to
+// the packed fields plus a constant (modulo 2^32).
+constexpr float MAGIC = 12582912.0f;
+constexpr uint32_t MAGIC_BITS = 0x4B400000u;
+template <int BITS> __host__ __device__ constexpr uint32_t magic_sum8() {
+  uint32_t s = 0;
+  for (int i = 0; i < 8; i++) s += MAGIC_BITS << (BITS * i);
+  return s;
+}
+// four groups of eight codes (8 BITS bits each) -> 4 * BITS bytes of the bit stream
+template <int BITS> __device__ __forceinline__ void store_groups(const uint32_t (&g8)[4], unsigned char* dst) {
+  uint32_t* d = reinterpret_cast<uint32_t*>(dst);
+  if constexpr (BITS == 4) *reinterpret_cast<uint4*>(d) = make_uint4(g8[0], g8[1], g8[2], g8[3]);
+  else if constexpr (BITS == 2) *reinterpret_cast<uint2*>(d) = make_uint2(g8[0] | g8[1] << 16, g8[2] | g8[3] << 16);
+  else {
+    d[0] = g8[0] | g8[1] << 24;
+    d[1] = g8[1] >> 8 | g8[2] << 16;
+    d[2] = g8[2] >> 16 | g8[3] << 8;
+  }
 }
 
 struct QuantSmem {
-  float z[W][D + 1];
-  unsigned char code[W][D];
-  unsigned char mod[W];
+  __align__(16) float z[W * ZS];       // rotated keys
+  __align__(16) float m[D], r[D];      // per channel: stored minimum, 1 / stored step (0 for a zero step)
 };
 
-// grid (windows, heads, batch), 128 threads
+// grid (windows, heads, batch), 128 threads.  Bound by issue slots, like the 2-bit key quantiser whose transform it shares;
+// a thread packs the 32 codes of a quarter of one token's row in registers.
+template <int BITS>
 __global__ void __launch_bounds__(128) k_ladder_keys(LadderView cv, const __half* __restrict__ k, long long sb, long long sh,
                                                      long long st, const float* __restrict__ signs) {
   __shared__ QuantSmem sm;
-  const int win = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const size_t u = cv.unit(b, h);
-  const float4 sg = *reinterpret_cast<const float4*>(signs + 4 * lane);
-  for (int kk = 0; kk < 8; kk++) {
-    const int i = warp * 8 + kk;
-    const float4 x = load_row4(k + b * sb + h * sh + (long long)(win * W + i) * st, lane);
-    float n = warp_norm(x);
-    const __half nh = __float2half_rn(n);
-    const float nf = __half2float(nh);
-    const float cinv = nf != 0.0f ? __fdiv_rn(RSQRT_D, nf) : 0.0f;
-    const float4 y = warp_fwht(make_float4(__fmul_rn(sg.x, x.x), __fmul_rn(sg.y, x.y), __fmul_rn(sg.z, x.z), __fmul_rn(sg.w, x.w)), lane);
-    // a zero vector (norm 0) has z = +0 in every coordinate
-    sm.z[i][4 * lane + 0] = nf != 0.0f ? __fmul_rn(y.x, cinv) : 0.0f; sm.z[i][4 * lane + 1] = nf != 0.0f ? __fmul_rn(y.y, cinv) : 0.0f;
-    sm.z[i][4 * lane + 2] = nf != 0.0f ? __fmul_rn(y.z, cinv) : 0.0f; sm.z[i][4 * lane + 3] = nf != 0.0f ? __fmul_rn(y.w, cinv) : 0.0f;
-    if (lane == 0) cv.k_norm[u * cv.capacity + (size_t)win * W + i] = nh;
-  }
+  const int win = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+  const size_t u = cv.unit(b, h), tok0 = u * cv.capacity + (size_t)win * W;
+  rotate_rows(k + b * sb + h * sh + (long long)win * W * st, st, W, signs, sm.z, [&](int i, __half nh) { cv.k_norm[tok0 + i] = nh; });
   __syncthreads();
+  constexpr float L = (float)((1 << BITS) - 1);
   {
-    const int c = tid;
-    const float L = (float)((1 << cv.bits) - 1);
-    float mn = sm.z[0][c], mx = mn;
-    for (int i = 1; i < W; i++) { const float v = sm.z[i][c]; mn = fminf(mn, v); mx = fmaxf(mx, v); }
+    const int c = tid, cp = zpos(c);
+    float mn = sm.z[cp], mx = mn;
+#pragma unroll 8
+    for (int i = 1; i < W; i++) { const float v = sm.z[i * ZS + cp]; mn = fminf(mn, v); mx = fmaxf(mx, v); }
     const __half mh = __float2half_rn(mn);
     const float mf = __half2float(mh);
     float range = __fsub_rn(mx, mf);
     range = range < 0.0f ? 0.0f : range;
     const __half s16 = __float2half_rn(__fdiv_rn(range, L));
     const float sf = __half2float(s16);
-    __half* meta = cv.k_meta + ((u * (cv.capacity / W) + win) * D + c) * 2;
-    meta[0] = mh; meta[1] = s16;
-    const float r = sf > 0.0f ? __fdiv_rn(1.0f, sf) : 0.0f;
-    for (int i = 0; i < W; i++) {
-      float q = rintf(__fmul_rn(__fsub_rn(sm.z[i][c], mf), r));
-      q = q < 0.0f ? 0.0f : (q > L ? L : q);
-      sm.code[i][c] = sf > 0.0f ? (unsigned char)q : (unsigned char)0;
-    }
+    reinterpret_cast<__half2*>(cv.k_meta)[(u * (cv.capacity / W) + win) * D + c] = __halves2half2(mh, s16);
+    sm.m[c] = mf;
+    sm.r[c] = sf > 0.0f ? __fdiv_rn(1.0f, sf) : 0.0f;
   }
   __syncthreads();
-  {
-    const int i = tid >> 2, part = tid & 3;
-    unsigned char* row = cv.k_codes + (u * cv.capacity + (size_t)win * W + i) * cv.row_bytes();
-    pack_quarter(&sm.code[i][32 * part], cv.bits, row + 4 * cv.bits * part);
+  // code = clamp(rint((z - m) / s), 0, L): clamping first gives the same integer, adding MAGIC rounds to nearest even.  A zero
+  // step has r = 0 and so code 0.
+  const int i = tid >> 2, part = tid & 3;
+  uint32_t g8[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    uint32_t w = 0;
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+      const int c = 32 * part + 8 * q + 4 * e;
+      const float4 z = *reinterpret_cast<const float4*>(&sm.z[i * ZS + zpos(c)]);
+      const float4 m = *reinterpret_cast<const float4*>(&sm.m[c]), r = *reinterpret_cast<const float4*>(&sm.r[c]);
+      const float zs[4] = {z.x, z.y, z.z, z.w}, ms[4] = {m.x, m.y, m.z, m.w}, rs[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+      for (int n = 0; n < 4; n++) {
+        const float x = fminf(fmaxf(__fmul_rn(__fsub_rn(zs[n], ms[n]), rs[n]), 0.0f), L);
+        w += __float_as_uint(__fadd_rn(x, MAGIC)) << (BITS * (4 * e + n));
+      }
+    }
+    g8[q] = w - magic_sum8<BITS>();
+    if (BITS < 4) g8[q] &= (1u << (8 * BITS % 32)) - 1u;
   }
+  store_groups<BITS>(g8, cv.k_codes + (tok0 + i) * (16 * BITS) + 4 * BITS * part);
 }
 
 struct ValueSmem {
@@ -196,54 +212,92 @@ namespace okq {
 namespace {
 
 // TurboQuant codec (Preliminaries, Eq. 2-3): norm, randomised Hadamard rotation, nearest level of the fixed codebook;
-// no window statistics, no modality rotation.  32 vectors per block of 128 threads.
-__global__ void __launch_bounds__(128) k_turboquant_encode(const __half* __restrict__ x, long long n, int bits,
-                                                           const float* __restrict__ signs, unsigned char* __restrict__ codes,
-                                                           __half* __restrict__ norms) {
-  __shared__ unsigned char code[W][D];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long base = (long long)blockIdx.x * W;
-  const float4 sg = *reinterpret_cast<const float4*>(signs + 4 * lane);
-  const float* th = c_thresholds[bits - 2];
-  const int nth = (1 << bits) - 1;
-  for (int kk = 0; kk < 8; kk++) {
-    const int i = warp * 8 + kk;
-    if (base + i >= n) break;
-    const float4 v = load_row4(x + (base + i) * D, lane);
-    const float nrm = warp_norm(v);
-    const __half nh = __float2half_rn(nrm);
-    const float nf = __half2float(nh);
-    const float cinv = nf != 0.0f ? __fdiv_rn(RSQRT_D, nf) : 0.0f;
-    const float4 y = warp_fwht(make_float4(__fmul_rn(sg.x, v.x), __fmul_rn(sg.y, v.y), __fmul_rn(sg.z, v.z), __fmul_rn(sg.w, v.w)), lane);
-    const float z[4] = {nf != 0.0f ? __fmul_rn(y.x, cinv) : 0.0f, nf != 0.0f ? __fmul_rn(y.y, cinv) : 0.0f,
-                        nf != 0.0f ? __fmul_rn(y.z, cinv) : 0.0f, nf != 0.0f ? __fmul_rn(y.w, cinv) : 0.0f};
+// no window statistics, no modality rotation.  32 vectors per block of 128 threads, eight threads per vector in the
+// transform (two in-register halves around one shared-memory exchange).  524288 vectors at 2 bits, encode and decode:
+// 300 us with one warp per vector (20 shuffles per transform) and byte-wise packing.
+
+// number of thresholds below z: compared one by one at 2 bits, at 3 and 4 bits a bit of the code at a time
+// (the threshold in the middle of what is left)
+template <int BITS> __device__ __forceinline__ uint32_t nearest_level(float z, const float* th) {
+  if constexpr (BITS == 2) return (uint32_t)(z > th[0]) + (uint32_t)(z > th[1]) + (uint32_t)(z > th[2]);
+  uint32_t code = 0;
 #pragma unroll
-    for (int k4 = 0; k4 < 4; k4++) {
-      int cd = 0;
-      for (int j = 0; j < nth; j++) cd += z[k4] > th[j];
-      code[i][4 * lane + k4] = (unsigned char)cd;
-    }
-    if (lane == 0) norms[base + i] = nh;
-  }
-  __syncthreads();
-  const int i = tid >> 2, part = tid & 3;
-  if (base + i < n) pack_quarter(&code[i][32 * part], bits, codes + (base + i) * 16 * bits + 4 * bits * part);
+  for (int step = 1 << (BITS - 1); step; step >>= 1)
+    if (z > th[code + step - 1]) code += step;
+  return code;
 }
 
-// x_hat = |x| H^T level[code], H^T y = diag(signs) Had y / sqrt(128); one warp per vector
+template <int BITS>
+__global__ void __launch_bounds__(128) k_turboquant_encode(const __half* __restrict__ x, long long n, const float* __restrict__ signs,
+                                                           unsigned char* __restrict__ codes, __half* __restrict__ norms) {
+  __shared__ __align__(16) float z[W * ZS];
+  __shared__ float th[16];
+  const int tid = threadIdx.x;
+  const long long base = (long long)blockIdx.x * W;
+  const int rows = (int)(n - base < W ? n - base : W);
+  if (tid < 16) th[tid] = c_thresholds[BITS - 2][tid];
+  rotate_rows(x + base * D, D, rows, signs, z, [&](int i, __half nh) { if (i < rows) norms[base + i] = nh; });
+  __syncthreads();
+  const int i = tid >> 2, part = tid & 3;
+  if (i >= rows) return;
+  uint32_t g8[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    uint32_t w = 0;
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+      const float4 v = *reinterpret_cast<const float4*>(&z[i * ZS + zpos(32 * part + 8 * q + 4 * e)]);
+      const float zs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; k++) w |= nearest_level<BITS>(zs[k], th) << (BITS * (4 * e + k));
+    }
+    g8[q] = w;
+  }
+  store_groups<BITS>(g8, codes + (base + i) * (16 * BITS) + 4 * BITS * part);
+}
+
+// x_hat = |x| H^T level[code], H^T y = diag(signs) Had y / sqrt(128)
+template <int BITS>
 __global__ void __launch_bounds__(128) k_turboquant_decode(const unsigned char* __restrict__ codes, const __half* __restrict__ norms,
-                                                           long long n, int bits, const float* __restrict__ signs,
-                                                           float* __restrict__ x_hat) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long i = (long long)blockIdx.x * 4 + warp;
-  if (i >= n) return;
-  const unsigned char* row = codes + i * 16 * bits;
-  const float* lv = c_levels[bits - 2];
-  const float4 y = warp_fwht(make_float4(lv[load_code(row, bits, 4 * lane + 0)], lv[load_code(row, bits, 4 * lane + 1)],
-                                         lv[load_code(row, bits, 4 * lane + 2)], lv[load_code(row, bits, 4 * lane + 3)]), lane);
-  const float4 sg = *reinterpret_cast<const float4*>(signs + 4 * lane);
-  const float f = RSQRT_D * __half2float(norms[i]);
-  *reinterpret_cast<float4*>(x_hat + i * D + 4 * lane) = make_float4(sg.x * y.x * f, sg.y * y.y * f, sg.z * y.z * f, sg.w * y.w * f);
+                                                           long long n, const float* __restrict__ signs, float* __restrict__ x_hat) {
+  __shared__ __align__(16) float z[16 * ZS];
+  __shared__ float lev[16];
+  const int tid = threadIdx.x, a = tid & 7, r = tid >> 3;
+  if (tid < 16) lev[tid] = c_levels[BITS - 2][tid];
+  __syncthreads();
+  uint64_t sg[8];   // signs of channels 16 u + 2 a, + 1
+#pragma unroll
+  for (int u = 0; u < 8; u++) sg[u] = *reinterpret_cast<const uint64_t*>(signs + 16 * u + 2 * a);
+#pragma unroll 1
+  for (int half = 0; half < 2; half++) {
+    const long long i = (long long)blockIdx.x * W + 16 * half + r;
+    const long long ir = i < n ? i : n - 1;
+    // 16 codes: 2 BITS bytes at byte 2 BITS a of the row
+    const unsigned char* src = codes + ir * (16 * BITS) + 2 * BITS * a;
+    uint32_t x[2];   // eight codes each
+    if constexpr (BITS == 4) { const uint2 v = *reinterpret_cast<const uint2*>(src); x[0] = v.x; x[1] = v.y; }
+    else if constexpr (BITS == 2) { const uint32_t v = *reinterpret_cast<const uint32_t*>(src); x[0] = v; x[1] = v >> 16; }
+    else {
+      const uint16_t* s2 = reinterpret_cast<const uint16_t*>(src);
+      const uint32_t v0 = s2[0], v1 = s2[1], v2 = s2[2];
+      x[0] = v0 | v1 << 16;
+      x[1] = v1 >> 8 | v2 << 8;
+    }
+    const float f = RSQRT_D * __half2float(norms[ir]);
+    uint64_t P[8], Q[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      const uint32_t w = x[q >> 2] >> (2 * BITS * (q & 3));
+      P[q] = pack2(lev[w & ((1u << BITS) - 1u)], lev[(w >> BITS) & ((1u << BITS) - 1u)]);
+    }
+    hadamard_eight(P, Q, z + r * ZS, a);
+    __syncwarp();   // (the row is written again in the next half)
+    if (i < n) {
+      const uint64_t f2 = pack2(f, f);
+#pragma unroll
+      for (int u = 0; u < 8; u++) *reinterpret_cast<uint64_t*>(x_hat + i * D + 16 * u + 2 * a) = mul2(mul2(sg[u], Q[u]), f2);
+    }
+  }
 }
 
 okq_status check_ladder(const okq_ladder_cache* c, int n_tokens) {
@@ -290,8 +344,13 @@ okq_status okq_ladder_quantize_keys(const okq_ladder_cache* cache, const void* k
   if (!aligned16(k_fp16) || !aligned16(signs) || strides[0] % 8 || strides[1] % 8 || strides[2] % 8) return OKQ_ERR_ALIGNMENT;
   if (n_tokens == 0) return OKQ_OK;
   const dim3 grid(n_tokens / W, cache->n_kv_heads, cache->batch);
-  k_ladder_keys<<<grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(ladder_view(cache), static_cast<const __half*>(k_fp16),
-                                                                     strides[0], strides[1], strides[2], signs);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(ladder_view(cache), static_cast<const __half*>(k_fp16), strides[0], strides[1],
+                                                                strides[2], signs);
+  };
+  if (cache->bits == 2) go(k_ladder_keys<2>);
+  else if (cache->bits == 3) go(k_ladder_keys<3>);
+  else go(k_ladder_keys<4>);
   return launch_status();
 }
 
@@ -303,6 +362,12 @@ okq_status okq_ladder_quantize_values(const okq_ladder_cache* cache, const void*
   if (!v_fp16 || !strides || !modality || !R || (n_R != 1 && n_R != cache->n_kv_heads)) return OKQ_ERR_INVALID_ARG;
   if (!aligned16(v_fp16) || !aligned16(R) || strides[0] % 8 || strides[1] % 8 || strides[2] % 8) return OKQ_ERR_ALIGNMENT;
   if (n_tokens == 0) return OKQ_OK;
+  // the tensor-core kernel, whose codes are the exact chain's; the chain kernel stays for strides that a tensor map cannot
+  // describe (zero, 2^40 bytes or more)
+  st = launch_ladder_values_tc(ladder_view(cache), static_cast<const __half*>(v_fp16), strides, modality, n_tokens, R, n_R, sm_count(),
+                               static_cast<cudaStream_t>(stream));
+  if (st == OKQ_OK) return launch_status();
+  if (st != OKQ_ERR_UNSUPPORTED) return st;
   const dim3 grid(n_tokens / W, cache->n_kv_heads, cache->batch);
   k_ladder_values<<<grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(ladder_view(cache), static_cast<const __half*>(v_fp16),
                                                                        strides[0], strides[1], strides[2], modality, n_tokens, R, n_R);
@@ -328,8 +393,13 @@ okq_status okq_turboquant_encode(const void* x_fp16, int64_t n_vectors, int32_t 
   if (!aligned16(x_fp16) || !aligned16(signs) || !aligned16(codes)) return OKQ_ERR_ALIGNMENT;
   if (n_vectors == 0) return OKQ_OK;
   if ((n_vectors + W - 1) / W > 0x7fffffffLL) return OKQ_ERR_CAPACITY;
-  k_turboquant_encode<<<(unsigned)((n_vectors + W - 1) / W), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const __half*>(x_fp16), n_vectors, bits, signs, codes, static_cast<__half*>(norms));
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)((n_vectors + W - 1) / W), 128, 0, static_cast<cudaStream_t>(stream)>>>(
+        static_cast<const __half*>(x_fp16), n_vectors, signs, codes, static_cast<__half*>(norms));
+  };
+  if (bits == 2) go(k_turboquant_encode<2>);
+  else if (bits == 3) go(k_turboquant_encode<3>);
+  else go(k_turboquant_encode<4>);
   return launch_status();
 }
 
@@ -340,8 +410,13 @@ okq_status okq_turboquant_decode(const uint8_t* codes, const void* norms, int64_
   if (!aligned16(codes) || !aligned16(signs) || !aligned16(x_hat)) return OKQ_ERR_ALIGNMENT;
   if (n_vectors == 0) return OKQ_OK;
   if ((n_vectors + 3) / 4 > 0x7fffffffLL) return OKQ_ERR_CAPACITY;
-  k_turboquant_decode<<<(unsigned)((n_vectors + 3) / 4), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-      codes, static_cast<const __half*>(norms), n_vectors, bits, signs, x_hat);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)((n_vectors + W - 1) / W), 128, 0, static_cast<cudaStream_t>(stream)>>>(
+        codes, static_cast<const __half*>(norms), n_vectors, signs, x_hat);
+  };
+  if (bits == 2) go(k_turboquant_decode<2>);
+  else if (bits == 3) go(k_turboquant_decode<3>);
+  else go(k_turboquant_decode<4>);
   return launch_status();
 }
 

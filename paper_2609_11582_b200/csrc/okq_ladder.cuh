@@ -40,4 +40,8 @@ struct LadderView {
 cudaError_t launch_ladder_decode(const LadderView& cv, int n_tokens, const __half* q, float sm_scale, const float* signs,
                                  const float* R, int n_R, float* out, cudaStream_t s);
 
+// value quantiser on the tensor cores (okq_quant_tc.cu); OKQ_ERR_UNSUPPORTED for strides a tensor map cannot describe
+okq_status launch_ladder_values_tc(const LadderView& lv, const __half* v, const int64_t strides[3], const unsigned char* modality,
+                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s);
+
 }  // namespace okq

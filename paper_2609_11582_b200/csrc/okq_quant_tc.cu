@@ -28,12 +28,19 @@
 // a time, with the exact fused-multiply-add chain of the reference arithmetic over the value row, read again from
 // global memory; the code in the record is then patched.  Codes and norms (exact summation tree) are therefore bit-identical to the exact path.
 //
+// The same kernel writes the value codes of the bit-width ladder (BITS = 2, 3 or 4: token-major bit streams): a table of 32
+// bins over the coordinate, each with at most one threshold of the codebook, gives (threshold, code below it) in one
+// look-up, the coordinates within the band go the same way as above, and a warp transposes its 32 x 32 codes through
+// shared memory and stores 4 BITS bytes per token.  8 sequences x 4 heads x 8192 tokens at 3 bits, keys and values:
+// 1282 us with one block per window evaluating the exact chain; see okq_ladder.cu for the figures of this form.
+//
 // Every wait on an mbarrier is bounded; on a timeout the kernel records OKQ_ERR_TIMEOUT in the
 // cache's status word, stops issuing work, frees its tensor memory and returns.
 #include <cuda.h>   // CUtensorMap and the type of cuTensorMapEncodeTiled only; the entry point is fetched at run time
 
 #include "okq_common.cuh"
 #include "okq_device.cuh"
+#include "okq_ladder.cuh"
 #include "okq_quant_tail.cuh"
 
 namespace okq {
@@ -70,11 +77,23 @@ struct FixItem {
   const __half* xrow;    // the token's value row (128 fp16)
   const float* rrow;     // row of the rotation matrix (128 fp32): output channel of the coordinate
   float inv;             // 1 / norm
-  int bit;               // bit position of the 2-bit field in the word
+  int bit;               // bit position of the field in the word
 };
-constexpr int FIX_MAX = 256;
 
-struct TcSmem {
+// bins of the code table: bin i covers [(i - 16.5) w, (i - 15.5) w); every width keeps all thresholds at least 0.13 w away
+// from the edges, so a coordinate within the band of a threshold is always looked up in that threshold's bin
+constexpr int BINS = 32;
+__host__ __device__ constexpr float bin_width(int bits) { return bits == 2 ? 0.0078875f : bits == 3 ? 0.0152875f : 0.02097845f; }
+
+template <int BITS> struct LadderSmem {
+  float2 bin[BINS];                                  // threshold in the bin (+inf: none), code below it (integer bits)
+  __align__(4) unsigned char code[16][W][36];        // per worker warp: [token][channel of its 32], 9-word rows
+};
+template <> struct LadderSmem<0> {};
+
+template <int BITS> struct TcSmem {
+  static constexpr int FIX_MAX = BITS ? 128 : 256;
+  LadderSmem<BITS> lad;
   __align__(1024) unsigned char a[2][TILE_BYTES];      // value tiles (double buffered)
   __align__(1024) unsigned char b[2][2][TILE_BYTES];   // two resident matrices, each as R_hi, R_lo
   __align__(16) float part[2][4][TILE];                // per token: sum of squares of channels [32 q, 32 q + 32)
@@ -130,7 +149,8 @@ __device__ __forceinline__ uint32_t vtile_off(int r, int kc) {
 // Bounded wait of a whole warp for one phase of an mbarrier (each try may suspend the thread for a short,
 // system-chosen time).  Gives up after about two seconds, or as soon as another role has given up; giving
 // up raises the abort flag.
-__device__ __forceinline__ bool mbar_wait(TcSmem& sm, unsigned long long* bar, uint32_t parity) {
+template <class SM>
+__device__ __forceinline__ bool mbar_wait(SM& sm, unsigned long long* bar, uint32_t parity) {
   const uint32_t mbar = smem_u32(bar);
   bool done = false;
   const long long t0 = clock64();
@@ -160,6 +180,21 @@ __device__ __forceinline__ bool mbar_drain(unsigned long long* bar, uint32_t par
 }
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// the reference arithmetic: one fused-multiply-add chain, input index ascending
+__device__ __noinline__ float exact_chain(const float* rrow, const __half* xrow) {
+  float a = 0.0f;
+#pragma unroll 4
+  for (int kc = 0; kc < 16; kc++) {
+    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(xrow) + kc);
+    const __half2* h2 = reinterpret_cast<const __half2*>(&raw);
+    const float4 r0 = __ldg(reinterpret_cast<const float4*>(rrow) + 2 * kc), r1 = __ldg(reinterpret_cast<const float4*>(rrow) + 2 * kc + 1);
+    const float2 x0 = __half22float2(h2[0]), x1 = __half22float2(h2[1]), x2 = __half22float2(h2[2]), x3 = __half22float2(h2[3]);
+    a = __fmaf_rn(r0.x, x0.x, a); a = __fmaf_rn(r0.y, x0.y, a); a = __fmaf_rn(r0.z, x1.x, a); a = __fmaf_rn(r0.w, x1.y, a);
+    a = __fmaf_rn(r1.x, x2.x, a); a = __fmaf_rn(r1.y, x2.y, a); a = __fmaf_rn(r1.z, x3.x, a); a = __fmaf_rn(r1.w, x3.y, a);
+  }
+  return a;
 }
 
 // The jobs of a tile, derived identically by the MMA warp and every worker warp from the tile's modality
@@ -225,14 +260,31 @@ struct Slots {
 // persistent grid, NT_ALL threads.  Tiles are numbered (b, h, tile-in-sequence), tile = 4 windows; a CTA
 // owns a contiguous range of them.  A "job" is one tile and at most two of the modalities present in it
 // (one accumulator of 128 columns each); jobs alternate between two accumulator sets in tensor memory.
-__global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_constant__ CUtensorMap vmap, CacheView cv, int layer,
+// BITS = 0: window records of `cv` (2 bits); 2, 3, 4: the canonical arrays of `lv` (cv: shape and modality only).
+template <int BITS>
+__global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_constant__ CUtensorMap vmap, CacheView cv, LadderView lv, int layer,
                                                              const unsigned char* __restrict__ modality, int n_tokens,
                                                              int n_win, const float* __restrict__ R, int n_R,
                                                              const __half* __restrict__ vrows, long long vs_b, long long vs_h,
                                                              long long vs_t, long long wait_limit, int skip_tile) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  TcSmem& sm = *reinterpret_cast<TcSmem*>(smem_raw);
+  using SM = TcSmem<BITS>;
+  constexpr int FIX_MAX = SM::FIX_MAX;
+  SM& sm = *reinterpret_cast<SM*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if constexpr (BITS != 0) {
+    if (tid < BINS) {
+      const float lo = ((float)tid - 16.5f) * bin_width(BITS), hi = lo + bin_width(BITS);
+      float th = INFINITY;
+      int below = 0;
+      for (int j = 0; j < (1 << BITS) - 1; j++) {
+        const float x = c_thresholds[BITS - 2][j];
+        if (x < lo) below++;
+        else if (x < hi) th = x;
+      }
+      sm.lad.bin[tid] = make_float2(th, __int_as_float(below));
+    }
+  }
   const int tiles_per_unit = (n_win + 3) / 4;   // n_win: windows to pack (the schedule may keep recent tokens raw)
   const int n_tiles_all = tiles_per_unit * cv.n_kv_heads * cv.batch;
   // contiguous tile range of this CTA
@@ -391,8 +443,9 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     const int eq = warp & 3, ewq = warp >> 2;
     // while the first tile is on its way: this CTA's share of the modality bytes and of the raw tail rows
     for (int bb = 0; bb < cv.batch; bb++) bulk_modality(cv, bb, modality, n_tokens, blockIdx.x * NT + tid, gridDim.x * NT);
-    for (int u = blockIdx.x; u < cv.batch * cv.n_kv_heads; u += gridDim.x)
-      bulk_tail_rows(cv, layer, u / cv.n_kv_heads, u % cv.n_kv_heads, vrows, vs_b, vs_h, vs_t, n_tokens, true, tid, NT);
+    if (BITS == 0)
+      for (int u = blockIdx.x; u < cv.batch * cv.n_kv_heads; u += gridDim.x)
+        bulk_tail_rows(cv, layer, u / cv.n_kv_heads, u % cv.n_kv_heads, vrows, vs_b, vs_h, vs_t, n_tokens, true, tid, NT);
     Slots slots;
     uint32_t jobidx = 0;
     bool dead = false;
@@ -425,6 +478,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         if (lane == 0) mbar_arrive(&sm.part_ready[buf]);
       }
       if (!mbar_wait(sm, &sm.part_ready[buf], par)) break;
+      [[maybe_unused]] unsigned nonzero = 0;   // tokens of the window that are not zero vectors
       if (ewq < wins) {
         // lane: norm of token `lane` of the window; the warp needs all 32 factors -1 / (3 T norm)
         const int tok = 32 * ewq + lane;
@@ -434,10 +488,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         n = n > 65504.0f ? 65504.0f : n;
         const __half nh16 = __float2half_rn(n);
         const float nf = __half2float(nh16);
-        if (eq == 0) reinterpret_cast<__half*>(cv.body(layer, cb, ch, cwin0 + ewq) + B_VNORM)[norm_pos(lane)] = nh16;
+        if (eq == 0) {
+          if (BITS == 0) reinterpret_cast<__half*>(cv.body(layer, cb, ch, cwin0 + ewq) + B_VNORM)[norm_pos(lane)] = nh16;
+          else lv.v_norm[lv.unit(cb, ch) * lv.capacity + (size_t)(cwin0 + ewq) * W + lane] = nh16;
+        }
         const float inv = nf != 0.0f ? __fdiv_rn(1.0f, nf) : 0.0f;
         sm.inv[warp][lane] = inv;
-        sm.c3[warp][lane] = __fmul_rn(inv, NEG_INV_3T);
+        sm.c3[warp][lane] = BITS == 0 ? __fmul_rn(inv, NEG_INV_3T) : inv * (1.0f / (BINS * bin_width(BITS)));
+        nonzero = __ballot_sync(0xffffffffu, nf != 0.0f);
       }
       __syncwarp();
       uint32_t wacc[4] = {0u, 0u, 0u, 0u};   // this channel's codes of the window, one word per t (sh = 0 position)
@@ -495,7 +553,50 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
                            "=r"(r[16]),"=r"(r[17]),"=r"(r[18]),"=r"(r[19]),"=r"(r[20]),"=r"(r[21]),"=r"(r[22]),"=r"(r[23]),"=r"(r[24]),"=r"(r[25]),"=r"(r[26]),"=r"(r[27]),"=r"(r[28]),"=r"(r[29]),"=r"(r[30]),"=r"(r[31])
                          : "r"(taddr) : "memory");
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-            // token i = 8*j + 2*t + e sits in word t at bit 16*e + 2*j (+ 8 for the second channel of the word)
+            if constexpr (BITS != 0) {
+              unsigned close = 0;   // tokens whose coordinate lies within the band of a threshold
+              unsigned char* codes = &sm.lad.code[warp][0][lane];
+              const float4* c3p = reinterpret_cast<const float4*>(sm.c3[warp]);
+              const float4* ivp = reinterpret_cast<const float4*>(sm.inv[warp]);
+#pragma unroll
+              for (int i4 = 0; i4 < 8; i4++) {
+                const float4 c4 = c3p[i4], v4 = ivp[i4];
+                const float cs[4] = {c4.x, c4.y, c4.z, c4.w}, iv[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                  const int tok = 4 * i4 + u;
+                  const float zr = __uint_as_float(r[tok]);
+                  float x, f;
+                  asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(x) : "f"(zr), "f"(cs[u]), "f"(16.5f / BINS));
+                  asm("fma.rm.f32 %0, %1, %2, %3;\n" : "=f"(f) : "f"(x), "f"((float)BINS - 0.0001f), "f"(FLOOR_MAGIC));
+                  const float2 bin = sm.lad.bin[__float_as_uint(f) & (BINS - 1)];
+                  const float d = fmaf(zr, iv[u], -bin.x);
+                  const int code = __float_as_int(bin.y) + (d > 0.0f ? 1 : 0);
+                  if (fabsf(d) <= BAND) close |= 1u << tok;
+                  if (keep == 0xffffffffu || ((keep >> tok) & 1u)) codes[tok * 36] = (unsigned char)code;
+                }
+              }
+              close &= keep & nonzero;   // (a zero vector's coordinates are exactly zero)
+              while (close) {
+                const int tok = __ffs(close) - 1, c = 32 * eq + lane;
+                close &= close - 1;
+                const __half* xrow = vrows + cb * vs_b + ch * vs_h + (long long)((cwin0 + ewq) * W + tok) * vs_t;
+                const float* rrow = R + (size_t)((n_R == 1 ? 0 : ch) * 3 + mods[mi]) * D * D + (size_t)c * D;
+                const int slot_i = atomicAdd(&sm.fix_count, 1);
+                if (slot_i < FIX_MAX) {
+                  FixItem& it = sm.fix[slot_i];
+                  it.word = reinterpret_cast<uint32_t*>(lv.v_codes + (lv.unit(cb, ch) * lv.capacity + (size_t)(cwin0 + ewq) * W + tok) * (16 * BITS)) +
+                            ((BITS * c) >> 5);
+                  it.xrow = xrow; it.rrow = rrow; it.inv = sm.inv[warp][tok]; it.bit = (BITS * c) & 31;
+                } else {
+                  const float z = __fmul_rn(exact_chain(rrow, xrow), sm.inv[warp][tok]);
+                  int code = 0;
+                  for (int j = 0; j < (1 << BITS) - 1; j++) code += z > c_thresholds[BITS - 2][j];
+                  codes[tok * 36] = (unsigned char)code;
+                }
+              }
+            } else {
+                        // token i = 8*j + 2*t + e sits in word t at bit 16*e + 2*j (+ 8 for the second channel of the word)
             uint32_t kaccA[4] = {0u, 0u, 0u, 0u}, kaccB[4] = {0u, 0u, 0u, 0u};
             const float4* c3p = reinterpret_cast<const float4*>(sm.c3[warp]);
 #pragma unroll
@@ -542,23 +643,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
                             vword_index((mu >> 2) * 128 + (4 * g + t) * 4 + (mu & 3));
                   it.xrow = xrow; it.rrow = rrow; it.inv = sm.inv[warp][tok]; it.bit = pos + 8 * sh;
                 } else {                  // the list is full: here and now
-                  float a = 0.0f;
-#pragma unroll 4
-                  for (int kc = 0; kc < 16; kc++) {
-                    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(xrow) + kc);
-                    const __half2* h2 = reinterpret_cast<const __half2*>(&raw);
-                    const float4 r0 = __ldg(reinterpret_cast<const float4*>(rrow) + 2 * kc), r1 = __ldg(reinterpret_cast<const float4*>(rrow) + 2 * kc + 1);
-                    const float2 x0 = __half22float2(h2[0]), x1 = __half22float2(h2[1]), x2 = __half22float2(h2[2]), x3 = __half22float2(h2[3]);
-                    a = __fmaf_rn(r0.x, x0.x, a); a = __fmaf_rn(r0.y, x0.y, a); a = __fmaf_rn(r0.z, x1.x, a); a = __fmaf_rn(r0.w, x1.y, a);
-                    a = __fmaf_rn(r1.x, x2.x, a); a = __fmaf_rn(r1.y, x2.y, a); a = __fmaf_rn(r1.z, x3.x, a); a = __fmaf_rn(r1.w, x3.y, a);
-                  }
-                  const float z = __fmul_rn(a, sm.inv[warp][tok]);
+                  const float z = __fmul_rn(exact_chain(rrow, xrow), sm.inv[warp][tok]);
                   const uint32_t code = (uint32_t)((z > -CB_THRESH) + (z > 0.0f) + (z > CB_THRESH));
                   codes = (codes & ~(3u << pos)) | (code << pos);
                 }
                 differ &= ~(3u << pos);
               }
               wacc[t] |= codes;
+            }
             }
           }
         }
@@ -568,7 +660,31 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         jobidx++;
       }
       if (dead) break;
-      if (ewq < wins) {
+      if (BITS != 0 && ewq < wins) {
+        if constexpr (BITS != 0) {
+          // lane = token: its 32 codes of this warp's channels are 4 BITS bytes of the token's row
+          __syncwarp();
+          const uint32_t* row = reinterpret_cast<const uint32_t*>(&sm.lad.code[warp][lane][0]);
+          uint32_t q4[8];
+#pragma unroll
+          for (int i = 0; i < 8; i++) {   // four codes of a byte each -> 4 BITS bits
+            const uint32_t x = row[i];
+            const uint32_t y = (x & 0x00ff00ffu) | ((x & 0xff00ff00u) >> (8 - BITS));
+            q4[i] = (y & 0xffffu) | (y >> (16 - 2 * BITS));
+          }
+          uint32_t* dst = reinterpret_cast<uint32_t*>(lv.v_codes + (lv.unit(cb, ch) * lv.capacity + (size_t)(cwin0 + ewq) * W + lane) * (16 * BITS) +
+                                                      4 * BITS * eq);
+          if constexpr (BITS == 4)
+            *reinterpret_cast<uint4*>(dst) = make_uint4(q4[0] | q4[1] << 16, q4[2] | q4[3] << 16, q4[4] | q4[5] << 16, q4[6] | q4[7] << 16);
+          else if constexpr (BITS == 2)
+            *reinterpret_cast<uint2*>(dst) = make_uint2(q4[0] | q4[1] << 8 | q4[2] << 16 | q4[3] << 24, q4[4] | q4[5] << 8 | q4[6] << 16 | q4[7] << 24);
+          else {
+            dst[0] = q4[0] | q4[1] << 12 | q4[2] << 24;
+            dst[1] = q4[2] >> 8 | q4[3] << 4 | q4[4] << 16 | q4[5] << 28;
+            dst[2] = q4[5] >> 4 | q4[6] << 8 | q4[7] << 20;
+          }
+        }
+      } else if (ewq < wins) {
         // join the two channels of each word (c and c ^ 8 are eight lanes apart) and store: channel
         // c = 16*mu + 8*sh + g writes the words t = 2*sh, 2*sh + 1 of (mu, g)
         const int c = 32 * eq + lane, mu = c >> 4, sh = (c >> 3) & 1, g = c & 7;
@@ -607,15 +723,27 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         a = __fmaf_rn(r1.x, x2.x, a); a = __fmaf_rn(r1.y, x2.y, a); a = __fmaf_rn(r1.z, x3.x, a); a = __fmaf_rn(r1.w, x3.y, a);
       }
       const float z = __fmul_rn(a, it.inv);
-      const uint32_t code = (uint32_t)((z > -CB_THRESH) + (z > 0.0f) + (z > CB_THRESH));
       if (lane == 0) {
-        atomicAnd(it.word, ~(3u << it.bit));
-        atomicOr(it.word, code << it.bit);
+        if constexpr (BITS == 0) {
+          const uint32_t code = (uint32_t)((z > -CB_THRESH) + (z > 0.0f) + (z > CB_THRESH));
+          atomicAnd(it.word, ~(3u << it.bit));
+          atomicOr(it.word, code << it.bit);
+        } else {
+          uint32_t code = 0;
+          for (int j = 0; j < (1 << BITS) - 1; j++) code += z > c_thresholds[BITS - 2][j];
+          const unsigned long long field = (unsigned long long)((1u << BITS) - 1u) << it.bit, val = (unsigned long long)code << it.bit;
+          atomicAnd(it.word, ~(uint32_t)field);
+          atomicOr(it.word, (uint32_t)val);
+          if (field >> 32) {   // a 3-bit code across two words
+            atomicAnd(it.word + 1, ~(uint32_t)(field >> 32));
+            atomicOr(it.word + 1, (uint32_t)(val >> 32));
+          }
+        }
       }
       __syncwarp();
     }
   }
-  if (tid == 0 && sm.abort) atomicCAS(cv.status, 0, (int)OKQ_ERR_TIMEOUT);
+  if (tid == 0 && sm.abort && cv.status) atomicCAS(cv.status, 0, (int)OKQ_ERR_TIMEOUT);
   if (warp == 0 && !sm.tmem_busy) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
 }
 
@@ -638,14 +766,16 @@ EncodeTiledFn encode_tiled() {
 
 }  // namespace
 
-okq_status launch_quantize_values_tc(const CacheView& cv, int layer, const __half* v, const int64_t strides[3],
+template <int BITS>
+static okq_status launch_values_tc(const CacheView& cv, const LadderView& lv, int layer, const __half* v, const int64_t strides[3],
                                      const unsigned char* modality, int n_tokens, int n_win, const float* R, int n_R,
                                      int n_sm, cudaStream_t s, long long wait_limit, int skip_tile) {
+  static_assert(sizeof(TcSmem<BITS>) + 1024 <= 227 * 1024, "shared memory of one block");
   static thread_local unsigned long long attr_mask = 0;
   int attr_dev = 0;
   if (attr_needed(attr_mask, attr_dev)) {
-    cudaError_t e = cudaFuncSetAttribute(k_quantize_values_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(TcSmem) + 1024);
+    cudaError_t e = cudaFuncSetAttribute(k_quantize_values_tc<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(TcSmem<BITS>) + 1024);
     if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
     attr_done(attr_mask, attr_dev);
   }
@@ -667,9 +797,26 @@ okq_status launch_quantize_values_tc(const CacheView& cv, int layer, const __hal
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) { set_last_cuda_error((int)cudaErrorInvalidValue); return OKQ_ERR_CUDA; }
   const int grid = (int)(n_tiles < n_sm ? n_tiles : n_sm);
-  k_quantize_values_tc<<<grid, NT_ALL, sizeof(TcSmem) + 1024, s>>>(vmap, cv, layer, modality, n_tokens, n_win, R, n_R, v, (long long)strides[0],
+  k_quantize_values_tc<BITS><<<grid, NT_ALL, sizeof(TcSmem<BITS>) + 1024, s>>>(vmap, cv, lv, layer, modality, n_tokens, n_win, R, n_R, v, (long long)strides[0],
                                                                    (long long)strides[1], (long long)strides[2], wait_limit > 0 ? wait_limit : WAIT_LIMIT_CLOCKS, skip_tile);
   return OKQ_OK;
+}
+
+okq_status launch_quantize_values_tc(const CacheView& cv, int layer, const __half* v, const int64_t strides[3],
+                                     const unsigned char* modality, int n_tokens, int n_win, const float* R, int n_R,
+                                     int n_sm, cudaStream_t s, long long wait_limit, int skip_tile) {
+  return launch_values_tc<0>(cv, LadderView{}, layer, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, wait_limit, skip_tile);
+}
+
+okq_status launch_ladder_values_tc(const LadderView& lv, const __half* v, const int64_t strides[3], const unsigned char* modality,
+                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s) {
+  CacheView cv{};   // shape and modality bytes; no status word: the ladder calls have none
+  cv.n_layers = 1; cv.batch = lv.batch; cv.n_kv_heads = lv.n_kv_heads; cv.n_q_heads = lv.n_q_heads; cv.capacity = lv.capacity;
+  cv.modality = lv.modality;
+  const int n_win = n_tokens / W;
+  return lv.bits == 2 ? launch_values_tc<2>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1)
+       : lv.bits == 3 ? launch_values_tc<3>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1)
+                      : launch_values_tc<4>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1);
 }
 
 }  // namespace okq
