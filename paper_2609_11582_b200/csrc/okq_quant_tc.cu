@@ -104,7 +104,7 @@ template <int BITS> struct TcSmem {
   __align__(8) unsigned long long empty[2];            // 16 arrivals: every worker warp is done with the buffer
   __align__(8) unsigned long long mma_done[2];         // 1 arrival (tcgen05.commit): accumulator set complete
   __align__(8) unsigned long long acc_free[2];         // 16 arrivals: every worker warp has read the accumulator set
-  __align__(8) unsigned long long part_ready[2];       // 16 arrivals: every worker warp has written its partial norms
+  __align__(8) unsigned long long part_ready[2][4];    // 4 arrivals: a window's four warps have written its partial norms
   __align__(8) unsigned long long slot_ready;          // 16 arrivals: every worker warp has written its share of a rotation matrix
   uint32_t tmem_slot;
   FixItem fix[FIX_MAX];
@@ -197,6 +197,33 @@ __device__ __noinline__ float exact_chain(const float* rrow, const __half* xrow)
   return a;
 }
 
+// R_m (fp32) as two fp16 operand tiles in slot `slot`, by the NT worker threads: all of a thread's loads in flight together
+template <int BITS>
+__device__ __forceinline__ void write_matrix(TcSmem<BITS>& sm, const float* Rm, int slot, int tid) {
+  constexpr int N = D * D / 8 / NT;
+  float4 x[N][2];
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    const float* src = Rm + (size_t)(tid + NT * i) * 8;
+    x[i][0] = __ldg(reinterpret_cast<const float4*>(src));
+    x[i][1] = __ldg(reinterpret_cast<const float4*>(src) + 1);
+  }
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    const int idx = tid + NT * i, n = idx >> 4, kc = idx & 15;
+    const float xs[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
+    __align__(16) __half hi[8], lo[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      hi[u] = __float2half_rn(xs[u]);
+      lo[u] = __float2half_rn(xs[u] - __half2float(hi[u]));
+    }
+    const uint32_t off = tile_off(n, kc * 8);
+    *reinterpret_cast<uint4*>(sm.b[slot][0] + off) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(sm.b[slot][1] + off) = *reinterpret_cast<const uint4*>(lo);
+  }
+}
+
 // The jobs of a tile, derived identically by the MMA warp and every worker warp from the tile's modality
 // bytes: `present` = modalities in the tile (bit m); a job takes at most two of them, so a tile with all
 // three needs two jobs.  winmask[m] = windows of the tile (bit w) that hold modality m.
@@ -217,41 +244,44 @@ __device__ __forceinline__ TileMods tile_mods(const unsigned char* mod, int lane
   }
   return t;
 }
-// modalities of job `jt` (0 or 1) of a tile: returns their count (0 = no such job)
-__device__ __forceinline__ int job_mods(unsigned present, int jt, int (&mods)[2]) {
-  int n = 0;
-  unsigned p = present;
-  if (jt == 1) {   // the third modality, if there is one
-    if (__popc(p) < 3) return 0;
-    mods[0] = 2;
-    return 1;
+// The tile's jobs in scalars (arrays indexed by a run-time value would live in local memory: 1000 cycles per tile and warp):
+// job 0 takes the first two modalities, job 1 the third one, if there is one.
+struct TileJobs {
+  int n_jobs, n0, m0, m1;
+  __device__ __forceinline__ explicit TileJobs(unsigned present) {
+    const unsigned rest = present & (present - 1u);
+    n_jobs = present == 0u ? 0 : (present == 7u ? 2 : 1);
+    n0 = rest ? 2 : 1;
+    m0 = __ffs(present) - 1;
+    m1 = __ffs(rest) - 1;
   }
-  while (p && n < 2) { mods[n++] = __ffs(p) - 1; p &= p - 1; }
-  return n;
-}
+  __device__ __forceinline__ int count(int jt) const { return jt ? 1 : n0; }
+  __device__ __forceinline__ int mod(int jt, int mi) const { return jt ? 2 : (mi ? m1 : m0); }
+};
 
 // The two resident rotation matrices (hi/lo pairs), tracked identically by the MMA warp and the worker warps.
 // plan() assigns the job's matrices to slots and says which have to be written first; a matrix goes to the
 // slot the job's other matrix does not use, else to the one that was not used last.
 struct Slots {
-  int key[2] = {-1, -1};   // (rotation set * 3 + modality) held by each slot
+  int k0 = -1, k1 = -1;   // (rotation set * 3 + modality) held by each slot
   int last = 0;
-  __device__ __forceinline__ bool plan(int nm, const int (&keys)[2], int (&slot)[2], bool (&need)[2]) {
-    for (int mi = 0; mi < 2; mi++) {
-      need[mi] = false;
-      slot[mi] = mi < nm ? (key[0] == keys[mi] ? 0 : (key[1] == keys[mi] ? 1 : -1)) : -1;
+  int sa = 0, sb = 0;     // slots of the planned job's matrices
+  bool na = false, nb = false;   // whether they have to be written
+  __device__ __forceinline__ bool plan(int nm, int ka, int kb) {
+    sa = k0 == ka ? 0 : (k1 == ka ? 1 : -1);
+    sb = nm == 2 ? (k0 == kb ? 0 : (k1 == kb ? 1 : -1)) : -1;
+    na = sa < 0;
+    nb = nm == 2 && sb < 0;
+    if (na) {
+      sa = (sb >= 0 ? sb : last) ^ 1;
+      if (sa) k1 = ka; else k0 = ka;
     }
-    bool any = false;
-    for (int mi = 0; mi < nm; mi++) {
-      if (slot[mi] >= 0) continue;
-      const int other = nm == 2 ? slot[mi ^ 1] : -1;
-      const int victim = other >= 0 ? (other ^ 1) : (last ^ 1);
-      key[victim] = keys[mi];
-      slot[mi] = victim;
-      need[mi] = any = true;
+    if (nb) {
+      sb = sa ^ 1;
+      if (sb) k1 = kb; else k0 = kb;
     }
-    last = slot[nm - 1];
-    return any;
+    last = nm == 2 ? sb : sa;
+    return na || nb;
   }
 };
 
@@ -298,7 +328,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;\n" ::"r"(smem_u32(&sm.empty[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&sm.mma_done[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;\n" ::"r"(smem_u32(&sm.acc_free[i])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;\n" ::"r"(smem_u32(&sm.part_ready[i])));
+      for (int w = 0; w < 4; w++) asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(&sm.part_ready[i][w])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 16;\n" ::"r"(smem_u32(&sm.slot_ready)));
     sm.abort = 0;
@@ -375,6 +405,11 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       step_coords();
       mod_cur = fetch_mod(i + 1);
     }
+    // with its tiles on their way: this CTA's share of the modality bytes and of the raw tail rows
+    for (int bb = 0; bb < cv.batch; bb++) bulk_modality(cv, bb, modality, n_tokens, blockIdx.x * 32 + lane, gridDim.x * 32);
+    if (BITS == 0)
+      for (int u = blockIdx.x; u < cv.batch * cv.n_kv_heads; u += gridDim.x)
+        bulk_tail_rows(cv, layer, u / cv.n_kv_heads, u % cv.n_kv_heads, vrows, vs_b, vs_h, vs_t, n_tokens, true, lane, 32);
     // after a timeout somewhere: no copy of this warp may still be landing when the block ends
     if (sm.abort)
       for (int i = max(0, armed - 2); i < armed; i++) mbar_drain(&sm.full[i & 1], (uint32_t)(i >> 1) & 1u);
@@ -387,17 +422,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       const int buf = i & 1;
       if (!mbar_wait(sm, &sm.full[buf], (uint32_t)(i >> 1) & 1u)) break;
       const TileMods tm = tile_mods(sm.mod[buf], lane);
-      for (int jt = 0; jt < 2; jt++) {
-        int mods[2] = {0, 0};
-        const int nm = job_mods(tm.present, jt, mods);
-        if (nm == 0) break;
+      const TileJobs jobs(tm.present);
+      for (int jt = 0; jt < jobs.n_jobs; jt++) {
+        const int nm = jobs.count(jt);
         const uint32_t a = jobidx & 1u;
         if (jobidx >= 2 && !mbar_wait(sm, &sm.acc_free[a], ((jobidx >> 1) - 1u) & 1u)) { dead = true; break; }
         // resident rotation matrices: the worker warps write a missing one and report on slot_ready
-        int slot[2];
-        bool need[2];
-        const int keys[2] = {(n_R == 1 ? 0 : ch) * 3 + mods[0], (n_R == 1 ? 0 : ch) * 3 + mods[1]};
-        if (slots.plan(nm, keys, slot, need)) {
+        const int key0 = (n_R == 1 ? 0 : ch) * 3;
+        if (slots.plan(nm, key0 + jobs.mod(jt, 0), key0 + jobs.mod(jt, 1))) {
           if (!mbar_wait(sm, &sm.slot_ready, refills & 1u)) { dead = true; break; }
           refills++;
         }
@@ -406,13 +438,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           for (int mi = 0; mi < nm; mi++) {
             // the windows [w_lo, w_hi] of the tile that hold this modality are the N extent of the MMAs
-            const unsigned wm = tm.winmask[mods[mi]];
+            const int mod = jobs.mod(jt, mi), slot = mi ? slots.sb : slots.sa;
+            const unsigned wm = mod == 0 ? tm.winmask[0] : (mod == 1 ? tm.winmask[1] : tm.winmask[2]);
             const int w_lo = __ffs(wm) - 1, w_hi = 31 - __clz(wm);
             const uint32_t n_ext = 32u * (uint32_t)(w_hi - w_lo + 1);
             const uint32_t idesc = (1u << 4) | ((n_ext >> 3) << 17) | ((128u >> 4) << 24);   // D fp32, A/B fp16 K-major, M = 128
             const uint32_t dcol = tmem + a * 256u + (uint32_t)mi * 128u + 32u * (uint32_t)w_lo;
-            const uint64_t da0 = make_desc(smem_u32(sm.b[slot[mi]][0]), 2048, 128);                   // R: M = output channel
-            const uint64_t da1 = make_desc(smem_u32(sm.b[slot[mi]][1]), 2048, 128);
+            const uint64_t da0 = make_desc(smem_u32(sm.b[slot][0]), 2048, 128);                   // R: M = output channel
+            const uint64_t da1 = make_desc(smem_u32(sm.b[slot][1]), 2048, 128);
             const uint64_t db0 = make_desc_sw128(smem_u32(sm.a[buf]) + 4096u * (uint32_t)w_lo);       // values: N = token
 #pragma unroll
             for (int k = 0; k < 16; k++) {
@@ -438,14 +471,9 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     if (jobidx >= 1 && !mbar_drain(&sm.mma_done[(jobidx - 1u) & 1u], ((jobidx - 1u) >> 1) & 1u)) sm.tmem_busy = 1;
   } else {
     // ------------------------------------------------------------------ worker warps
-    // norm role: token rows 32*eq + lane, channels [32 q, 32 q + 32); epilogue role: channels 32*eq + lane (the
-    // warp's tensor-memory lane quarter), window ewq
+    // window ewq of every tile, together with the three other warps of the window and nobody else: norm role: its token
+    // rows, channels [32 eq, 32 eq + 32); epilogue role: channels 32*eq + lane (the warp's tensor-memory lane quarter)
     const int eq = warp & 3, ewq = warp >> 2;
-    // while the first tile is on its way: this CTA's share of the modality bytes and of the raw tail rows
-    for (int bb = 0; bb < cv.batch; bb++) bulk_modality(cv, bb, modality, n_tokens, blockIdx.x * NT + tid, gridDim.x * NT);
-    if (BITS == 0)
-      for (int u = blockIdx.x; u < cv.batch * cv.n_kv_heads; u += gridDim.x)
-        bulk_tail_rows(cv, layer, u / cv.n_kv_heads, u % cv.n_kv_heads, vrows, vs_b, vs_h, vs_t, n_tokens, true, tid, NT);
     Slots slots;
     uint32_t jobidx = 0;
     bool dead = false;
@@ -454,13 +482,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       const uint32_t par = (uint32_t)(i >> 1) & 1u;
       if (!mbar_wait(sm, &sm.full[buf], par)) break;
       const TileMods tm = tile_mods(sm.mod[buf], lane);
+      const TileJobs jobs(tm.present);
       const unsigned mymod = sm.mod[buf][32 * ewq + lane];   // token `lane` of this warp's window
       const int wins = min(4, n_win - cwin0);
       {
         // Sum of squares with the exact adjacent-pair tree, split so that shared-memory reads are free of bank
         // conflicts: a 16-byte chunk (8 channels) is three levels of the tree, the warp's four chunks two more;
         // the last two levels (p0 + p1) + (p2 + p3) follow below.
-        const int row = 32 * eq + lane, q = ewq;
+        const int row = 32 * ewq + lane, q = eq;
         float part[4];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
@@ -475,9 +504,9 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         }
         sm.part[buf][q][row] = __fadd_rn(__fadd_rn(part[0], part[1]), __fadd_rn(part[2], part[3]));
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.part_ready[buf]);
+        if (lane == 0) mbar_arrive(&sm.part_ready[buf][ewq]);
       }
-      if (!mbar_wait(sm, &sm.part_ready[buf], par)) break;
+      if (!mbar_wait(sm, &sm.part_ready[buf][ewq], par)) break;
       [[maybe_unused]] unsigned nonzero = 0;   // tokens of the window that are not zero vectors
       if (ewq < wins) {
         // lane: norm of token `lane` of the window; the warp needs all 32 factors -1 / (3 T norm)
@@ -499,38 +528,17 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       }
       __syncwarp();
       uint32_t wacc[4] = {0u, 0u, 0u, 0u};   // this channel's codes of the window, one word per t (sh = 0 position)
-      for (int jt = 0; jt < 2; jt++) {
-        int mods[2] = {0, 0};
-        const int nm = job_mods(tm.present, jt, mods);
-        if (nm == 0) break;
+      for (int jt = 0; jt < jobs.n_jobs; jt++) {
+        const int nm = jobs.count(jt);
         const uint32_t a = jobidx & 1u;
         {
           // A rotation matrix this job needs is not resident: split R_m into fp16 hi + lo, laid out as the A
           // operand (row = output channel, K = input channel).  Every MMA issued so far has completed (this warp
           // has waited for each), and the job's own MMAs wait for slot_ready.
-          int slot[2];
-          bool need[2];
-          const int keys[2] = {(n_R == 1 ? 0 : ch) * 3 + mods[0], (n_R == 1 ? 0 : ch) * 3 + mods[1]};
-          if (slots.plan(nm, keys, slot, need)) {
-            for (int mi = 0; mi < nm; mi++) {
-              if (!need[mi]) continue;
-              const float* Rm = R + (size_t)keys[mi] * D * D;
-              for (int idx = tid; idx < D * D / 8; idx += NT) {
-                const int n = idx >> 4, kc = idx & 15;
-                const float4 x0 = __ldg(reinterpret_cast<const float4*>(Rm + n * D + kc * 8));
-                const float4 x1 = __ldg(reinterpret_cast<const float4*>(Rm + n * D + kc * 8 + 4));
-                const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-                __align__(16) __half hi[8], lo[8];
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                  hi[u] = __float2half_rn(xs[u]);
-                  lo[u] = __float2half_rn(xs[u] - __half2float(hi[u]));
-                }
-                const uint32_t off = tile_off(n, kc * 8);
-                *reinterpret_cast<uint4*>(sm.b[slot[mi]][0] + off) = *reinterpret_cast<const uint4*>(hi);
-                *reinterpret_cast<uint4*>(sm.b[slot[mi]][1] + off) = *reinterpret_cast<const uint4*>(lo);
-              }
-            }
+          const int key0 = (n_R == 1 ? 0 : ch) * 3;
+          if (slots.plan(nm, key0 + jobs.mod(jt, 0), key0 + jobs.mod(jt, 1))) {
+            if (slots.na) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 0)) * D * D, slots.sa, tid);
+            if (slots.nb) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 1)) * D * D, slots.sb, tid);
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // generic-proxy writes -> tensor-core reads
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.slot_ready);
@@ -538,13 +546,15 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         }
         if (!mbar_wait(sm, &sm.mma_done[a], (jobidx >> 1) & 1u)) { dead = true; break; }
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const bool last_job = jt == 1 || __popc(tm.present) < 3;
+        const bool last_job = jt + 1 == jobs.n_jobs;
         // the tile's MMAs are complete and this warp keeps what it needs of the buffer in registers (the rare exact
         // recomputation below reads its value row from global memory)
         if (last_job && lane == 0) mbar_arrive(&sm.empty[buf]);
         if (ewq < wins) {
+#pragma unroll 1
           for (int mi = 0; mi < nm; mi++) {
-            const unsigned keep = __ballot_sync(0xffffffffu, mymod == (unsigned)mods[mi]);   // bit i: token i
+            const int mod = jobs.mod(jt, mi);
+            const unsigned keep = __ballot_sync(0xffffffffu, mymod == (unsigned)mod);   // bit i: token i
             if (!keep) continue;
             uint32_t r[32];
             const uint32_t taddr = tmem + ((uint32_t)(eq * 32) << 16) + a * 256u + (uint32_t)mi * 128u + (uint32_t)ewq * 32u;
@@ -581,7 +591,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
                 const int tok = __ffs(close) - 1, c = 32 * eq + lane;
                 close &= close - 1;
                 const __half* xrow = vrows + cb * vs_b + ch * vs_h + (long long)((cwin0 + ewq) * W + tok) * vs_t;
-                const float* rrow = R + (size_t)((n_R == 1 ? 0 : ch) * 3 + mods[mi]) * D * D + (size_t)c * D;
+                const float* rrow = R + (size_t)((n_R == 1 ? 0 : ch) * 3 + mod) * D * D + (size_t)c * D;
                 const int slot_i = atomicAdd(&sm.fix_count, 1);
                 if (slot_i < FIX_MAX) {
                   FixItem& it = sm.fix[slot_i];
@@ -635,7 +645,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
                 const int tok = 8 * ((pos & 15) >> 1) + 2 * t + (pos >> 4);
                 const int c = 32 * eq + lane, mu = c >> 4, sh = (c >> 3) & 1, g = c & 7;
                 const __half* xrow = vrows + cb * vs_b + ch * vs_h + (long long)((cwin0 + ewq) * W + tok) * vs_t;
-                const float* rrow = R + (size_t)((n_R == 1 ? 0 : ch) * 3 + mods[mi]) * D * D + (size_t)c * D;
+                const float* rrow = R + (size_t)((n_R == 1 ? 0 : ch) * 3 + mod) * D * D + (size_t)c * D;
                 const int slot_i = atomicAdd(&sm.fix_count, 1);
                 if (slot_i < FIX_MAX) {   // later, by a whole warp (the code written now is one of the two neighbouring levels)
                   FixItem& it = sm.fix[slot_i];
