@@ -197,20 +197,23 @@ __device__ __noinline__ float exact_chain(const float* rrow, const __half* xrow)
   return a;
 }
 
-// R_m (fp32) as two fp16 operand tiles in slot `slot`, by the NT worker threads: all of a thread's loads in flight together
+// R_m (fp32) as two fp16 operand tiles in slot `slot`, by the NT worker threads: all of a thread's loads in flight together.
+// A warp takes 8 rows x 32 columns: 128-byte pieces of a row in global memory, eight consecutive 16-byte rows of a core
+// matrix per quarter-warp in shared memory (lanes along a row instead put eight stores on the same banks: 6000 cycles).
 template <int BITS>
 __device__ __forceinline__ void write_matrix(TcSmem<BITS>& sm, const float* Rm, int slot, int tid) {
   constexpr int N = D * D / 8 / NT;
   float4 x[N][2];
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const float* src = Rm + (size_t)(tid + NT * i) * 8;
+    const int item = (tid >> 5) + NT / 32 * i, n = 8 * (item >> 2) + (tid & 7), kc = 4 * (item & 3) + ((tid >> 3) & 3);
+    const float* src = Rm + n * D + kc * 8;
     x[i][0] = __ldg(reinterpret_cast<const float4*>(src));
     x[i][1] = __ldg(reinterpret_cast<const float4*>(src) + 1);
   }
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const int idx = tid + NT * i, n = idx >> 4, kc = idx & 15;
+    const int item = (tid >> 5) + NT / 32 * i, n = 8 * (item >> 2) + (tid & 7), kc = 4 * (item & 3) + ((tid >> 3) & 3);
     const float xs[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
     __align__(16) __half hi[8], lo[8];
 #pragma unroll
@@ -474,6 +477,9 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     // window ewq of every tile, together with the three other warps of the window and nobody else: norm role: its token
     // rows, channels [32 eq, 32 eq + 32); epilogue role: channels 32*eq + lane (the warp's tensor-memory lane quarter)
     const int eq = warp & 3, ewq = warp >> 2;
+    // the rotation matrices on their way to L2 before the first tile says which one it needs
+    for (int i = blockIdx.x * NT + tid; i < n_R * 3 * D * D / 32; i += gridDim.x * NT)
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(R + (size_t)i * 32));
     Slots slots;
     uint32_t jobidx = 0;
     bool dead = false;
