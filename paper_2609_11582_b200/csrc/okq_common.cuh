@@ -43,6 +43,32 @@ inline void attr_done(unsigned long long& mask, int dev) {
   if (dev >= 0 && dev < 64) mask |= 1ull << dev;
 }
 
+// Launch that may overlap the end of the kernel before it in the stream: its blocks are placed and set up as soon as that
+// kernel has let go (depend_wait below) or is through.  Every kernel launched this way calls depend_wait before it touches
+// global memory: it returns once the kernel before has completed and its writes are visible, whatever that kernel was.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void depend_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");   // the next kernel may be placed; it waits for this one's end
+}
+#endif
+
 inline okq_status launch_status() {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   const int unit = blockIdx.x / CS, rank = blockIdx.x % CS;
   const int h = unit % cv.n_kv_heads, e = unit / cv.n_kv_heads, b = e % cv.batch, li = e / cv.batch, layer = P.layer0 + li;
   const int G = P.group;
+  depend_wait();
   const int seq = cv.seq_len[layer * cv.batch + b];
   // tokens [0, v_pk) have packed values (and keys); of the rest, [v_pk, k_pk) have packed keys (captioning schedule only)
   const int v_pk = cv.v_packed(seq), k_pk = cv.k_packed(seq), nwin = v_pk / W, n_tail = seq - v_pk;
@@ -387,11 +388,7 @@ static int small_clusters() {
 
 template <int FMT, int CS>
 static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at;
-  small_config<FMT, CS>(cfg, at, units);
-  cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, k_decode_small<FMT, CS>, P);
+  return launch_dependent(k_decode_small<FMT, CS>, dim3(units * CS), NTHREADS, sizeof(SmallSmem<FMT, CS>), s, CS, P);
 }
 
 template <int FMT>

@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(128) k_quantize_keys(CacheView cv, int layer, 
                                                       const float* __restrict__ signs, int n_tokens) {
   __shared__ WindowSmem sm;
   const int win = (int)blockIdx.x - 1, h = blockIdx.y, b = blockIdx.z;
+  depend_wait();
   if (win < 0) {
     bulk_tail_rows(cv, layer, b, h, k, sb, sh, st, n_tokens, false, threadIdx.x, 128);
     return;
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(128) k_append(CacheView cv, int layer0, const 
   __shared__ WindowSmem sm;
   __shared__ int s_pos;
   int h = blockIdx.x, b = blockIdx.y, li = blockIdx.z, layer = layer0 + li;
+  depend_wait();
   // The n_kv_heads blocks of a (layer, sequence) all need the position before any of them may advance it.
   // Each block counts itself in the top byte of seq_len while reading it; the block that finds the others
   // already counted stores the new length (which also clears the count): by then every block has its copy.
@@ -441,7 +443,7 @@ okq_status okq_quantize_keys(const okq_cache* cache, int32_t layer, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __half* k = static_cast<const __half*>(k_fp16);
   const dim3 grid(cv.k_packed(n_tokens) / W + 1, cv.n_kv_heads, cv.batch);
-  k_quantize_keys<<<grid, 128, 0, s>>>(cv, layer, k, strides[0], strides[1], strides[2], signs, n_tokens);
+  launch_dependent(k_quantize_keys, grid, 128, 0, s, 1, cv, layer, k, strides[0], strides[1], strides[2], signs, n_tokens);
   return launch_status();
 }
 
@@ -509,8 +511,8 @@ okq_status okq_append(const okq_cache* cache, int32_t layer, int32_t layer_count
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the kernel counts a sequence's blocks in the top byte of its seq_len entry while it runs
   if (cache->capacity >= APPEND_ARRIVAL || cache->n_kv_heads > 127) return OKQ_ERR_UNSUPPORTED;
-  k_append<<<dim3(cv.n_kv_heads, cv.batch, layer_count), 128, 0, s>>>(
-      cv, layer, static_cast<const __half*>(k_new), static_cast<const __half*>(v_new), modality_new, signs, R, n_R);
+  launch_dependent(k_append, dim3(cv.n_kv_heads, cv.batch, layer_count), 128, 0, s, 1, cv, layer, static_cast<const __half*>(k_new),
+                   static_cast<const __half*>(v_new), modality_new, signs, R, n_R);
   return launch_status();
 }
 

@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = sm.tmem_slot;
+  depend_wait();
 
   // coordinates of the first tile; every role steps them without divisions afterwards
   int cb = 0, ch = 0, cwin0 = 0;
@@ -813,8 +814,10 @@ static okq_status launch_values_tc(const CacheView& cv, const LadderView& lv, in
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) { set_last_cuda_error((int)cudaErrorInvalidValue); return OKQ_ERR_CUDA; }
   const int grid = (int)(n_tiles < n_sm ? n_tiles : n_sm);
-  k_quantize_values_tc<BITS><<<grid, NT_ALL, sizeof(TcSmem<BITS>) + 1024, s>>>(vmap, cv, lv, layer, modality, n_tokens, n_win, R, n_R, v, (long long)strides[0],
-                                                                   (long long)strides[1], (long long)strides[2], wait_limit > 0 ? wait_limit : WAIT_LIMIT_CLOCKS, skip_tile);
+  const cudaError_t le = launch_dependent(k_quantize_values_tc<BITS>, dim3(grid), NT_ALL, sizeof(TcSmem<BITS>) + 1024, s, 1, vmap, cv, lv, layer,
+                                          modality, n_tokens, n_win, R, n_R, v, (long long)strides[0], (long long)strides[1], (long long)strides[2],
+                                          wait_limit > 0 ? wait_limit : WAIT_LIMIT_CLOCKS, skip_tile);
+  if (le != cudaSuccess) { set_last_cuda_error((int)le); return OKQ_ERR_CUDA; }
   return OKQ_OK;
 }
 
