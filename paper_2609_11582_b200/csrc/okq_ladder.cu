@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(128) k_ladder_keys(LadderView cv, const __half
   __shared__ QuantSmem sm;
   const int win = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
   const size_t u = cv.unit(b, h), tok0 = u * cv.capacity + (size_t)win * W;
+  depend_wait();
   rotate_rows(k + b * sb + h * sh + (long long)win * W * st, st, W, signs, sm.z, [&](int i, __half nh) { cv.k_norm[tok0 + i] = nh; });
   __syncthreads();
   constexpr float L = (float)((1 << BITS) - 1);
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(128) k_turboquant_encode(const __half* __restr
   const int tid = threadIdx.x;
   const long long base = (long long)blockIdx.x * W;
   const int rows = (int)(n - base < W ? n - base : W);
+  depend_wait();
   if (tid < 16) th[tid] = c_thresholds[BITS - 2][tid];
   rotate_rows(x + base * D, D, rows, signs, z, [&](int i, __half nh) { if (i < rows) norms[base + i] = nh; });
   __syncthreads();
@@ -263,6 +265,7 @@ __global__ void __launch_bounds__(128) k_turboquant_decode(const unsigned char* 
   __shared__ __align__(16) float z[16 * ZS];
   __shared__ float lev[16];
   const int tid = threadIdx.x, a = tid & 7, r = tid >> 3;
+  depend_wait();
   if (tid < 16) lev[tid] = c_levels[BITS - 2][tid];
   __syncthreads();
   uint64_t sg[8];   // signs of channels 16 u + 2 a, + 1
@@ -345,7 +348,7 @@ okq_status okq_ladder_quantize_keys(const okq_ladder_cache* cache, const void* k
   if (n_tokens == 0) return OKQ_OK;
   const dim3 grid(n_tokens / W, cache->n_kv_heads, cache->batch);
   auto go = [&](auto kernel) {
-    kernel<<<grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(ladder_view(cache), static_cast<const __half*>(k_fp16), strides[0], strides[1],
+    launch_dependent(kernel, dim3(grid), 128, 0, static_cast<cudaStream_t>(stream), 1, ladder_view(cache), static_cast<const __half*>(k_fp16), strides[0], strides[1],
                                                                 strides[2], signs);
   };
   if (cache->bits == 2) go(k_ladder_keys<2>);
@@ -394,7 +397,7 @@ okq_status okq_turboquant_encode(const void* x_fp16, int64_t n_vectors, int32_t 
   if (n_vectors == 0) return OKQ_OK;
   if ((n_vectors + W - 1) / W > 0x7fffffffLL) return OKQ_ERR_CAPACITY;
   auto go = [&](auto kernel) {
-    kernel<<<(unsigned)((n_vectors + W - 1) / W), 128, 0, static_cast<cudaStream_t>(stream)>>>(
+    launch_dependent(kernel, dim3((unsigned)((n_vectors + W - 1) / W)), 128, 0, static_cast<cudaStream_t>(stream), 1, 
         static_cast<const __half*>(x_fp16), n_vectors, signs, codes, static_cast<__half*>(norms));
   };
   if (bits == 2) go(k_turboquant_encode<2>);
@@ -411,7 +414,7 @@ okq_status okq_turboquant_decode(const uint8_t* codes, const void* norms, int64_
   if (n_vectors == 0) return OKQ_OK;
   if ((n_vectors + 3) / 4 > 0x7fffffffLL) return OKQ_ERR_CAPACITY;
   auto go = [&](auto kernel) {
-    kernel<<<(unsigned)((n_vectors + W - 1) / W), 128, 0, static_cast<cudaStream_t>(stream)>>>(
+    launch_dependent(kernel, dim3((unsigned)((n_vectors + W - 1) / W)), 128, 0, static_cast<cudaStream_t>(stream), 1, 
         codes, static_cast<const __half*>(norms), n_vectors, signs, x_hat);
   };
   if (bits == 2) go(k_turboquant_decode<2>);

@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
   const int n_win = n_tokens / W;
   const size_t u = cv.unit(b, h);
   WarpL<BITS>& ws = sm.w[warp];
+  depend_wait();
 
   // ---- this warp's windows, the first ones on their way
   const int cnt = (n_win + cs * NW - 1) / (cs * NW);
@@ -462,17 +463,8 @@ cudaError_t launch(const LadderView& cv, int cs, int n_tokens, const __half* q, 
     if (e != cudaSuccess) return e;
     attr_done(attr_mask, dev);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(cv.batch * cv.n_kv_heads * cs));
-  cfg.blockDim = dim3(NT_L);
-  cfg.dynamicSmemBytes = sizeof(BlockL<BITS>);
-  cfg.stream = s;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cs; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_ladder_decode<BITS>, cv, n_tokens, q, sm_scale, signs, R, n_R, out);
+  return launch_dependent(k_ladder_decode<BITS>, dim3((unsigned)(cv.batch * cv.n_kv_heads * cs)), NT_L, sizeof(BlockL<BITS>), s, cs, cv,
+                          n_tokens, q, sm_scale, signs, R, n_R, out);
 }
 
 }  // namespace
