@@ -228,7 +228,7 @@ okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t l
  *   - Limit: the tensor-core path's scratch of the largest launch (this is not okq_decode_workspace_bytes(),
  *     which also covers okq_decode_attention_simt and can be larger when num_splits is given), i.e.
  *     (layer_count * batch * n_kv_heads + number of CTAs) * 12736 bytes of per-CTA partials plus
- *     (layer_count * batch * n_kv_heads + 8 * number of CTAs) * 12832 bytes of per-warp-pair pieces,
+ *     (layer_count * batch * n_kv_heads + 8 * number of CTAs) * 12832 bytes of per-warp pieces,
  *     must fit in the scratch: about 1950 (sequence, KV head) pairs per launch with the automatic grid;
  *     anything larger returns OKQ_ERR_WORKSPACE and launches nothing (use
  *     okq_decode_attention with your own buffer).
@@ -268,8 +268,8 @@ void okq_profile_events(void* before, void* after);
 
 /*
  * Choice of the split-K kernel behind okq_decode_attention (the paper has no counterpart; for cross-checks and
- * timing comparisons).  1 (default): the mma.sync warp-pair kernel; 0: the tcgen05 kernel with the unpacked codes
- * in tensor memory (fp16 metadata only; a cache with MXFP4 metadata always takes the warp-pair kernel).  Both fill
+ * timing comparisons).  1 (default): the mma.sync kernels; 0: the tcgen05 kernel with the unpacked codes
+ * in tensor memory (fp16 metadata only; a cache with MXFP4 metadata always takes the mma.sync kernels).  Both fill
  * the same partial records for the same combine kernel.  Process-wide; not to be changed while a decode call is
  * being issued on another thread.  Returns the previous value; a value other than 0 or 1 changes nothing.
  */

@@ -52,11 +52,11 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
                              void* workspace, size_t workspace_bytes, float* C_out, void* stream);
 
 /*
- * Eigen-decomposition of one symmetric 128 x 128 matrix (cyclic Jacobi in fp64, one thread block) and
+ * Eigen-decomposition of one symmetric 128 x 128 matrix (cyclic Jacobi in fp64, one thread-block cluster) and
  * R = H U^T with the ordering and sign convention stated above.
  *   C  float [128][128] (symmetric; only read), signs  float [128] (+-1)
  *   R_out  float [128][128] (row = rotated coordinate), lambda_out  float [128] (descending)
- *   workspace: 128 KB of the workspace (fp64 eigenvector matrix).
+ *   workspace: at least 128 KB (checked; the solver keeps everything in shared memory).
  * The device status convention of okq.h does not apply: the iteration has a fixed sweep limit (30), which
  * a symmetric matrix does not reach; `sweeps_out` (device int32, may be null) receives the sweeps used.
  */

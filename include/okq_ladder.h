@@ -11,9 +11,9 @@
  *          code = index of the nearest of the 2^b Lloyd-Max levels of N(0, 1/128);
  *   decode (Eq. 1)         scores in the rotated space against one rotated query per head, online softmax,
  *          value sums in each modality's rotated basis, R_m^T once per head.
- * This is a plain CUDA-core implementation over a canonical cache (no fragment-order records, no tensor
- * cores: with eight or sixteen non-uniform value levels the bit-plane identity of the 2-bit decode kernel
- * does not apply, the levels come from a table); it exists for parity with the ladder and is not tuned.
+ * Key codes and split weights meet on the tensor cores, value sums are fp32 multiply-adds, the value rotation is the
+ * tensor-core product of the 2-bit path with the coordinates near a threshold recomputed exactly.  The calls have no
+ * status word: a bounded wait of the value quantiser that ran out would leave codes unwritten.
  *
  * Cache layout (all buffers caller-owned, 16-byte aligned; n_tokens must be a multiple of 32: no raw tail):
  *   k_codes, v_codes  uint8 [batch][n_kv_heads][capacity][16 * bits]: per token a little-endian bit stream,
@@ -60,7 +60,7 @@ okq_status okq_ladder_quantize_values(const okq_ladder_cache* cache, const void*
                                       void* stream);
 
 /* Eq. 1 over the first n_tokens tokens of every sequence.  q: device fp16 [batch][n_q_heads][128];
- * out: device float [batch][n_q_heads][128]; one thread block per (sequence, KV head). */
+ * out: device float [batch][n_q_heads][128]; a cluster of one to eight thread blocks per (sequence, KV head). */
 okq_status okq_ladder_decode_attention(const okq_ladder_cache* cache, int32_t n_tokens, const void* q,
                                        float sm_scale, const float* signs, const float* R, int32_t n_R,
                                        float* out, void* stream);

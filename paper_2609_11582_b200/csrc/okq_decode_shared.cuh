@@ -79,7 +79,7 @@ __device__ inline int block_prefix(const CacheView& cv, int layer0, int n_entrie
 
 // tcgen05 split-K kernel (fp16 metadata): fills partials_f exactly where launch_decode_mma's own split kernel would
 okq_status launch_decode_tc(const DecodeParams& P, int n_cta, cudaStream_t s);
-// which split-K kernel launch_decode_mma uses: 0 = the tcgen05 kernel (fp16 metadata), 1 = the mma.sync warp-pair kernel
+// which split-K kernel launch_decode_mma uses: 0 = the tcgen05 kernel (fp16 metadata), 1 = the mma.sync kernel
 extern int g_decode_impl;
 
 // one-launch form for few (sequence, head) units: cluster size it would use for a call (0: not applicable), launch

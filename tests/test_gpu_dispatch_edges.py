@@ -1,0 +1,146 @@
+"""Edges of the kernels and of the rules that choose between them: cluster sizes of the one-launch decode and of the ladder
+decode, strides of the value quantisers, query tiles of the calibration weights, degenerate matrices of the eigen solver."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import okq_calib_oracle as CO
+from paper_2609_11582_b200 import binding as B
+from paper_2609_11582_b200 import workloads as WL
+from tests import harness as Hn
+from tests.test_gpu_ladder import LadderCase
+
+pytestmark = pytest.mark.gpu
+D, W = 128, 32
+
+
+# (sequences, KV heads): units at which the cluster goes 16 -> 8 -> 4 -> split-K kernel; tokens: fewer windows than warps, one
+# window, no window at all, a full and an empty raw tail
+@pytest.mark.parametrize("batch,heads", [(1, 1), (2, 4), (15, 1), (33, 1), (17, 2)])
+@pytest.mark.parametrize("n", [31, 32, 32 * 13 + 31])
+def test_one_launch_decode_at_its_edges(batch, heads, n):
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=7 * heads, prefix_text=40, video_chunk=70, audio_chunk=21)
+    c = Hn.Case(w, n_tokens=n, meta_format=B.META_MXFP4 if batch % 2 else B.META_FP16)
+    # the CUDA-core kernels are within 1e-6 of the definition, so the bound is the tensor-core path's own
+    Hn.assert_attention_close(c.gpu_decode(0)[0], c.gpu_decode(0, simt=True)[0])
+
+
+@pytest.mark.parametrize("meta", [B.META_FP16, B.META_MXFP4])
+@pytest.mark.parametrize("n", [100, 128, 128 + 159, 1024 + 127])
+def test_one_launch_decode_captioning_schedule(meta, n):
+    """Up to four packed windows and 127 raw keys among the raw values; against the split-K pair."""
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=2)
+    dev = torch.device("cuda")
+    cache = B.Cache(1, 2, w.n_kv_heads, w.n_q_heads, 1280, device=dev, meta_format=meta, schedule=B.SCHEDULE_CAPTION)
+    k, v = WL.gen_kv(w, 0, n_tokens=n)
+    signs, R = WL.gen_signs(w, 0).to(dev), WL.gen_rotations(w, 0)[None].contiguous().to(dev)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(2, 1).contiguous().to(dev)
+    B.quantize_keys(cache, 0, k.to(dev), signs)
+    B.quantize_values(cache, 0, v.to(dev), mod, R)
+    q = WL.gen_queries(w, 0).to(dev)
+    outs = []
+    for splits in (0, 2):
+        ws = torch.empty(B.decode_workspace_bytes(cache, 1, splits), dtype=torch.uint8, device=dev)
+        out = torch.full((1, 2, w.n_q_heads, D), float("nan"), device=dev)
+        B.decode_attention(cache, 0, 1, q, signs, R, ws, out, num_splits=splits)
+        outs.append(out.cpu().numpy().astype(np.float64))
+    Hn.assert_attention_close(outs[0], outs[1])
+
+
+# clusters of 1, 2, 4 and 8 blocks (by units and windows); one window; more warps than windows
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("batch,n", [(1, 32), (1, 32 * 9), (12, 32 * 20), (38, 32 * 3)])
+def test_ladder_cache_and_decode_over_cluster_sizes(bits, batch, n):
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, prefix_text=5, video_chunk=45, audio_chunk=19)
+    c = LadderCase(w, bits, n)
+    got = c.gpu_attention()
+    # fp32 sums of scores of size up to 2^5 (log2 domain) over 8 tensor-core steps, truncated: 2^5 * 8 * 2^-24 = 1.5e-5 per
+    # numerator at the very worst; sums over tokens average it.  The worst (sequence, head) vector may be short: ten times that.
+    rel, worst, mx = Hn.attention_errors(got, c.oracle_attention())
+    assert rel < 1.5e-5 and worst < 1.5e-4, (rel, worst, mx)
+    if batch == 1:
+        c.check_cache()
+
+
+@pytest.mark.parametrize("bulk", [False, True])
+def test_value_quantiser_strides(bulk):
+    """Heads inside tokens and a broadcast (zero-stride) head: the same records as from a contiguous copy; the default entry
+    point takes what a tensor map cannot describe, the bulk one reports it."""
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=2)
+    n, dev = 32 * 5 + 7, torch.device("cuda")
+    _, v = WL.gen_kv(w, 0, n_tokens=n)
+    v = v.to(dev)
+    R = WL.gen_rotations(w, 0)[None].contiguous().to(dev)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(2, 1).contiguous().to(dev)
+
+    def records(x):
+        cache = B.Cache(1, 2, w.n_kv_heads, w.n_q_heads, 192, device=dev)
+        B.quantize_values(cache, 0, x, mod, R, bulk=bulk)
+        return cache.records.clone(), cache.v_tail.clone(), cache.modality.clone(), cache.seq_len.clone()
+
+    inner = v.transpose(1, 2).contiguous().transpose(1, 2)
+    assert all(torch.equal(a, b) for a, b in zip(records(inner), records(v)))
+    shared = v[:, :1].expand(2, w.n_kv_heads, n, D)
+    if bulk:
+        with pytest.raises(B.OkqError) as e:
+            records(shared)
+        assert e.value.status == B.ERR_UNSUPPORTED
+    else:
+        assert all(torch.equal(a, b) for a, b in zip(records(shared), records(shared.contiguous())))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_ladder_values_with_a_broadcast_head(bits):
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=1)
+    _, v = WL.gen_kv(w, 0, n_tokens=96)
+    R = WL.gen_rotations(w, 0)[None].contiguous().cuda()
+    mod = WL.modality_layout(w, 96).unsqueeze(0).contiguous().cuda()
+    shared = v.cuda()[:, :1].expand(1, w.n_kv_heads, 96, D)
+    caches = [B.LadderCache(1, w.n_kv_heads, w.n_q_heads, 96, bits) for _ in range(2)]
+    for c, x in zip(caches, (shared, shared.contiguous())):
+        B.ladder_quantize_values(c, x, mod, R)
+    assert torch.equal(caches[0].v_codes, caches[1].v_codes) and torch.equal(caches[0].v_norm, caches[1].v_norm)
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 193])
+@pytest.mark.parametrize("scale", [D ** -0.5, 0.0, -0.05])
+def test_calibration_weights_at_tile_edges(n, scale):
+    """One more and one fewer than the 128-query and 64-key tiles; a zero and a negative softmax scale."""
+    g = torch.Generator().manual_seed(n)
+    q = torch.randn(3, n, D, generator=g).half()
+    k = torch.randn(n, D, generator=g).half()
+    w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(3, n), sm_scale=scale).cpu().double().numpy()
+    s = q.double() @ k.double().T * scale
+    s = s.masked_fill(torch.ones(n, n).triu(1).bool(), -float("inf"))
+    ref = s.softmax(-1).square().sum((0, 1)).numpy()
+    # fp32 scores of size up to 2^3: 2^3 * 2^-21 in the exponent, twice for the square
+    assert np.abs(w - ref).max() <= 1e-5 * ref.max()
+
+
+def _matrices():
+    g = torch.Generator().manual_seed(3)
+    q = torch.linalg.qr(torch.randn(D, D, generator=g, dtype=torch.float64))[0]
+    yield "zero", torch.zeros(D, D)
+    yield "identity", torch.eye(D)
+    yield "rank one", torch.ones(D, D)
+    yield "repeated", (q * torch.tensor([5.0] * 40 + [1.0] * 48 + [0.0] * 40, dtype=torch.float64)) @ q.T
+    yield "indefinite", (q * torch.linspace(-3, 3, D, dtype=torch.float64)) @ q.T
+    yield "zero diagonal", torch.ones(D, D) - torch.eye(D)
+    yield "tiny", 1e-30 * ((q * torch.linspace(0, 1, D, dtype=torch.float64)) @ q.T)
+
+
+@pytest.mark.parametrize("name,C", list(_matrices()), ids=[n for n, _ in _matrices()])
+def test_eigen_solver_on_degenerate_matrices(name, C):
+    C = (0.5 * (C + C.T)).float().contiguous()
+    signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0)
+    R, lam, sweeps = B.calib_rotation(C.cuda(), signs.cuda(), B.calib_workspace(1, 1))
+    R, lam = R.cpu().double().numpy(), lam.cpu().double().numpy()
+    Cd = C.double().numpy()
+    top = max(np.abs(Cd).sum(1).max(), 1e-300)
+    assert 0 <= int(sweeps.item()) < 30
+    # fp32 outputs of an fp64 solution: 128 products of 2^-24 each
+    assert np.abs(R @ R.T - np.eye(D)).max() < 1e-5
+    assert (np.diff(lam) <= 0).all()
+    assert np.abs(lam - np.sort(np.linalg.eigvalsh(Cd))[::-1]).max() <= 1e-6 * top
+    H = CO.hadamard_matrix(signs.numpy())
+    assert np.abs(R @ Cd @ R.T - (H * lam) @ H.T).max() <= 1e-5 * top
