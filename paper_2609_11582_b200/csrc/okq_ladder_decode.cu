@@ -76,7 +76,8 @@ template <int BITS> struct Pairs {
   static constexpr uint32_t ONES = (BITS == 2 ? 0x3u : BITS == 3 ? 0x7u : 0xfu) * 0x00010001u;
 };
 
-template <int BITS>
+// NH: heads whose value sums are formed, the group rounded up to 2, 5, 7 or 8 (the scores' m16 tile holds eight either way)
+template <int BITS, int NH>
 __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_tokens, const __half* __restrict__ q,
                                                           float sm_scale, const float* __restrict__ signs,
                                                           const float* __restrict__ R, int n_R, float* __restrict__ out) {
@@ -157,9 +158,9 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
   const float fsc = sm.fsc[g];
 
   const int hw = lane >> 4, l16 = lane & 15;   // value sums: token parity, channels 8 l16 .. 8 l16 + 7
-  float acc[GP][8];
+  float acc[NH][8];
 #pragma unroll
-  for (int j = 0; j < GP; j++)
+  for (int j = 0; j < NH; j++)
 #pragma unroll
     for (int c = 0; c < 8; c++) acc[j][c] = 0.f;
   float run_m = -INFINITY, run_l = 0.f;
@@ -173,7 +174,8 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
       float v[8];
 #pragma unroll
       for (int c = 0; c < 8; c++) {
-        const float give = hw ? acc[j][c] : acc[j + 4][c], keep = hw ? acc[j + 4][c] : acc[j][c];
+        const float lo = j < NH ? acc[j < NH ? j : 0][c] : 0.f, hi = j + 4 < NH ? acc[j + 4 < NH ? j + 4 : 0][c] : 0.f;
+        const float give = hw ? lo : hi, keep = hw ? hi : lo;
         v[c] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
       }
       float4* dst = reinterpret_cast<float4*>(row + (4 * hw + j) * D);
@@ -188,7 +190,7 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
     }
     held |= 1 << cur_mod;
 #pragma unroll
-    for (int j = 0; j < GP; j++)
+    for (int j = 0; j < NH; j++)
 #pragma unroll
       for (int c = 0; c < 8; c++) acc[j][c] = 0.f;
   };
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
 #pragma unroll
       for (int j = 0; j < GP; j++) al[j] = __shfl_sync(0xffffffffu, alpha, 4 * j);
 #pragma unroll
-      for (int j = 0; j < GP; j++)
+      for (int j = 0; j < NH; j++)
 #pragma unroll
         for (int c = 0; c < 8; c++) acc[j][c] *= al[j];
       for (int m = 0; m < 3; m++)
@@ -316,11 +318,13 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
         const uint32_t* r = reinterpret_cast<const uint32_t*>(row) + ((3 * l16) >> 2);
         x = __funnelshift_r(r[0], r[1], 8 * ((3 * l16) & 3));   // (the second word may lie behind the row: not used then)
       }
-      const float4 pa = *reinterpret_cast<const float4*>(&ws.p[tok][0]), pb = *reinterpret_cast<const float4*>(&ws.p[tok][4]);
+      const float4 pa = *reinterpret_cast<const float4*>(&ws.p[tok][0]);
+      float4 pb = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (NH > 4) pb = *reinterpret_cast<const float4*>(&ws.p[tok][4]);
       float pv[GP] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
       if (masked && !((sel >> tok) & 1u)) {
 #pragma unroll
-        for (int j = 0; j < GP; j++) pv[j] = 0.f;
+        for (int j = 0; j < NH; j++) pv[j] = 0.f;
       }
       const char* lev = reinterpret_cast<const char*>(sm.lev);
 #pragma unroll
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
         const uint32_t off = (sh < 0 ? x << 2 : x >> sh) & (((1u << BITS) - 1u) << 2);
         const float lv = *reinterpret_cast<const float*>(lev + off);
 #pragma unroll
-        for (int j = 0; j < GP; j++) acc[j][c] = fmaf(pv[j], lv, acc[j][c]);
+        for (int j = 0; j < NH; j++) acc[j][c] = fmaf(pv[j], lv, acc[j][c]);
       }
     };
     const unsigned mine = __ballot_sync(0xffffffffu, mymod == cur_mod);
@@ -452,19 +456,26 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
   }
 }
 
-template <int BITS>
-cudaError_t launch(const LadderView& cv, int cs, int n_tokens, const __half* q, float sm_scale, const float* signs, const float* R,
+template <int BITS, int NH>
+cudaError_t launch_heads(const LadderView& cv, int cs, int n_tokens, const __half* q, float sm_scale, const float* signs, const float* R,
                    int n_R, float* out, cudaStream_t s) {
   static_assert(sizeof(BlockL<BITS>) <= 227 * 1024, "shared memory of one block");
   static thread_local unsigned long long attr_mask = 0;
   int dev = 0;
   if (attr_needed(attr_mask, dev)) {
-    const cudaError_t e = cudaFuncSetAttribute(k_ladder_decode<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockL<BITS>));
+    const cudaError_t e = cudaFuncSetAttribute(k_ladder_decode<BITS, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockL<BITS>));
     if (e != cudaSuccess) return e;
     attr_done(attr_mask, dev);
   }
-  return launch_dependent(k_ladder_decode<BITS>, dim3((unsigned)(cv.batch * cv.n_kv_heads * cs)), NT_L, sizeof(BlockL<BITS>), s, cs, cv,
+  return launch_dependent(k_ladder_decode<BITS, NH>, dim3((unsigned)(cv.batch * cv.n_kv_heads * cs)), NT_L, sizeof(BlockL<BITS>), s, cs, cv,
                           n_tokens, q, sm_scale, signs, R, n_R, out);
+}
+
+template <int BITS, class... A>
+cudaError_t launch(const LadderView& cv, A... args) {
+  const int G = cv.n_q_heads / cv.n_kv_heads;
+  return G <= 2 ? launch_heads<BITS, 2>(cv, args...) : G <= 5 ? launch_heads<BITS, 5>(cv, args...)
+       : G <= 7 ? launch_heads<BITS, 7>(cv, args...) : launch_heads<BITS, 8>(cv, args...);
 }
 
 }  // namespace
