@@ -342,37 +342,53 @@ constexpr int NBLK = NPOS * (NPOS - 1) / 2;        // 2 x 2 blocks above the dia
 constexpr int ROUNDS = D - 1;
 constexpr int V_CTAS = 4, V_COLS = D / V_CTAS;     // blocks that carry the eigenvectors, columns of each
 
-// Cyclic Jacobi on a symmetric 128 x 128 matrix in fp64, one cluster of 1 + V_CTAS blocks.
+// Cyclic Jacobi on a symmetric 128 x 128 matrix, one cluster of 1 + V_CTAS blocks; the result is fp64-converged.
 //
 // The round-robin pairing is kept as a ring (Brent and Luk): after every round each index moves one place, so the pair
 // k of a round is always positions (top k, bottom k) and a sweep of 127 rounds brings everybody home.  Block 0 holds the
 // matrix in position order, upper half only, as 2 x 2 blocks (pair k, pair l), one plane per block element: a thread owns
 // two blocks, reads them at fixed addresses, applies its rows' and its columns' rotation in registers and stores the
-// results where the move takes them, at fixed addresses of a second buffer.  Per round that is 128 KB of shared-memory
-// traffic and two block barriers; with the matrix in place, rows first and columns then, it was 512 KB, the
-// eigenvectors' rows through L2 and three barriers (5.2 us per round).
+// results where the move takes them, at fixed addresses of a second buffer.  A pair's next off-diagonal element comes out
+// of one such block, so 64 threads work out the next round's angles while everybody applies this round: one block barrier
+// per round.  (With the matrix in place, rows first and columns then, it was 512 KB of shared-memory traffic per round,
+// the eigenvectors' rows through L2 and three barriers: 5.2 us per round, 7.2 ms per matrix; now about 1.05 us, 1.48 ms.)
 // The rotations of a sweep go to the other blocks, which apply them to V^T (row = eigenvector estimate, V_COLS columns
 // each) while block 0 works on the next sweep.
-// The angle is taken in fp32 (the residual element is computed, not assumed zero, so that only costs a factor 1e-7 per
-// visit); cosine and sine are orthonormal to fp64 by two Newton steps.  Stops after a sweep whose largest tangent was
-// below 1e-8: what is left is quadratically smaller.
+// A round is bound by the chain of its angle threads (loads queued behind the other warps', about 1200 cycles in fp32, 1900
+// in fp64) and by block 0's shared-memory traffic, so the first sweeps run on an fp32 copy of the
+// matrix, at half the traffic: they only choose the angles.  The eigenvectors take the same rotations with fp64 cosines and
+// stay orthogonal to fp64; V A V^T is then formed in fp64 from the original matrix and the fp64 sweeps finish on that.
+// Angles are taken in fp32 throughout (the residual element is computed, not assumed zero, so that only costs a factor 1e-7
+// per visit); cosine and sine of the fp64 rotations are orthonormal to fp64 by two Newton steps.  Stops after a sweep whose
+// largest tangent was below 1e-8: what is left is quadratically smaller.
 // Then: eigenvalues in descending order, every eigenvector with its largest-magnitude component positive, R = H U^T with
 // H = Had_128 diag(signs) / sqrt(128), a Hadamard transform per column.
-struct EigA {
-  double buf[2][4 * NBLK + NPOS + D];   // off-diagonal planes [2 * row part + column part][block], pairs' elements, diagonal
-  double2 cs[NPOS];
-  double red[32];
-  unsigned maxt;                        // largest |tangent| of the sweep (float bits); 0: nothing rotated
+constexpr int CHUNK = 32;               // rounds whose rotations are worked out together
+template <class T> struct __align__(2 * sizeof(T)) Pair2 { T x, y; };
+template <class T> struct EigA {
+  T buf[2][4 * NBLK];                   // off-diagonal planes [2 * row part + column part][block]
+  __align__(16) Pair2<T> cs[2][NPOS];   // rotations of this round and of the next
+  T dg[2][D];                           // diagonal, by position, after the rotations of the round (before its move)
+  T own[NPOS];                          // the pairs' own off-diagonal elements at the start of a phase
+  float tmax[2];                        // largest |tangent| of the sweep, per angle warp; 0: nothing rotated
 };
 struct EigV {
   double v[D][V_COLS];                  // V^T, rows by index
-  double t[2][ROUNDS * NPOS];           // tangents of a sweep, written by block 0
+  union {
+    double t[2][ROUNDS * NPOS];         // tangents of a sweep, written by block 0
+    double other[V_CTAS - 1][D][V_COLS];   // between the phases: the other slices of V^T, then this slice's part of V A
+  };
+  union {
+    double a[D][V_COLS];                // between the phases: this slice's columns of the matrix
+    Pair2<double> cs[CHUNK][NPOS];      // rotations of the rounds being applied
+  };
   double lam[D];
   double best[V_CTAS][D];               // per slice and eigenvector: the slice's component of largest magnitude
   int done[2];
   int order[D];
 };
-constexpr int EIG_SMEM = sizeof(EigA) > sizeof(EigV) ? (int)sizeof(EigA) : (int)sizeof(EigV);
+constexpr int EIG_SMEM = sizeof(EigA<double>) > sizeof(EigV) ? (int)sizeof(EigA<double>) : (int)sizeof(EigV);
+constexpr int FP32_SWEEPS = 7;                     // at most; of 11 to 13 in all
 static_assert(EIG_SMEM <= 227 * 1024, "shared memory of one block");
 
 // position 2 k: top of pair k, 2 k + 1: bottom
@@ -392,168 +408,285 @@ __device__ __forceinline__ int eig_index(int pos, int r) {
 __device__ __forceinline__ int eig_block(int k, int l) {
   return k < NPOS / 2 ? k * (NPOS - 1) + l - k - 1 : (NPOS - 1 - k) * (NPOS - 1) + k + (l - k - 1);
 }
-// where the element of positions (a, b) is kept
+// where the element of positions (a, b) of different pairs is kept
 __device__ __forceinline__ int eig_slot(int a, int b) {
-  if ((a >> 1) == (b >> 1)) return 4 * NBLK + (a >> 1);
   if ((a >> 1) > (b >> 1)) { const int x = a; a = b; b = x; }
   return (2 * (a & 1) + (b & 1)) * NBLK + eig_block(a >> 1, b >> 1);
 }
-__device__ __forceinline__ double2 eig_cos_sin(double t) {   // c = 1 / sqrt(1 + t^2) to fp64, s = t c
+// position of index i in round 0
+__device__ __forceinline__ int eig_home(int i) { return i < NPOS ? 2 * i : 2 * (D - 1 - i) + 1; }
+__device__ __forceinline__ Pair2<double> eig_cos_sin(double t) {   // c = 1 / sqrt(1 + t^2) to fp64, s = t c
   const double x = fma(t, t, 1.0), hx = 0.5 * x;
   double y = (double)rsqrtf((float)x);
   y = y * fma(-hx * y, y, 1.5);
   y = y * fma(-hx * y, y, 1.5);
-  return make_double2(y, t * y);
+  return {y, t * y};
+}
+__device__ __forceinline__ Pair2<float> eig_cos_sin(float t) {
+  const float y = rsqrtf(fmaf(t, t, 1.0f));
+  return {y, t * y};
 }
 
-__global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __restrict__ C, const float* __restrict__ signs,
-                                                           float* __restrict__ R, float* __restrict__ lambda,
-                                                           int* __restrict__ sweeps_out) {
-  extern __shared__ __align__(16) unsigned char eig_raw[];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x;
-  EigV& sv = *reinterpret_cast<EigV*>(eig_raw);
-  cluster.sync();   // every block runs before its shared memory is written from outside
-  if (rank == 0) {
-    EigA& sa = *reinterpret_cast<EigA*>(eig_raw);
-    // largest magnitude (the matrix is scaled by a power of two to at most 1) and trace
-    double mx = 0.0, tr = 0.0;
-    for (int i = tid; i < D * D; i += EIG_THREADS) mx = fmax(mx, fabs((double)C[i]));
-    if (tid < D) tr = fabs((double)C[tid * D + tid]);
-    for (int d = 16; d; d >>= 1) {
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-      tr += __shfl_xor_sync(0xffffffffu, tr, d);
+// Block 0: sweeps on the matrix in sa (buf[0], own, dg[0] = diagonal by position) until the largest tangent of a sweep is at
+// most `stop` or `max_sweeps` are done; an element is rotated if its magnitude exceeds `tiny` and its square `rel2` times the
+// product of its diagonal elements.  Returns the number of sweeps that rotated something; *diag: the buffer of dg that holds
+// the rotated diagonal of the last round.  One cluster barrier per sweep.
+template <class T>
+__device__ int eig_sweeps(cg::cluster_group& cluster, EigA<T>& sa, EigV& sv, T tiny, T rel2, float stop, int max_sweeps, int* diag) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // this thread's two blocks: where they are read, the rows' and columns' pairs, where their elements go.  Elements that
+  // become a pair's own are worked out by its angle thread instead and dropped here (slot -1).
+  int rd[2], pk[2], pl[2], wr[2][4];
+#pragma unroll
+  for (int u = 0; u < 2; u++) {
+    const int j = lane + 32 * u;
+    const bool first = j < NPOS - 1 - warp;
+    pk[u] = first ? warp : NPOS - 1 - warp;
+    pl[u] = first ? warp + 1 + j : NPOS - warp + (j - (NPOS - 1 - warp));
+    rd[u] = warp * (NPOS - 1) + j;
+    if (j >= NPOS - 1) { rd[u] = -1; pk[u] = 0; pl[u] = 1; }
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const int pa = eig_move(2 * pk[u] + (e >> 1)), pb = eig_move(2 * pl[u] + (e & 1));
+      wr[u][e] = (pa >> 1) == (pb >> 1) ? -1 : eig_slot(pa, pb);
     }
-    if (lane == 0) sa.red[warp] = mx;
-    __syncthreads();
-    for (int i = 0; i < 32; i++) mx = fmax(mx, sa.red[i]);
-    __syncthreads();
-    if (lane == 0 && warp < 4) sa.red[warp] = tr;
-    __syncthreads();
-    int ex = 0;
-    if (mx > 0.0) frexp(mx, &ex);   // mx < 2^ex
-    const double scale = ldexp(1.0, -ex);
-    // the size below which an off-diagonal element is left alone
-    const double tiny = fmax(((sa.red[0] + sa.red[1]) + (sa.red[2] + sa.red[3])) * scale * 1e-18, 1e-30);
-    for (int i = tid; i < D * D; i += EIG_THREADS) {
-      const int a = i / D, b = i % D;
-      if (a > b) continue;
-      const int ia = eig_index(a, 0), ib = eig_index(b, 0);
-      const double x = 0.5 * ((double)C[ia * D + ib] + (double)C[ib * D + ia]) * scale;
-      if (a == b) sa.buf[0][4 * NBLK + NPOS + a] = x;
-      else sa.buf[0][eig_slot(a, b)] = x;
-    }
-    // this thread's two blocks: where they are read, the rows' and columns' pairs, where their elements go
-    int rd[2], pk[2], pl[2], wr[2][4];
-#pragma unroll
-    for (int u = 0; u < 2; u++) {
-      const int j = lane + 32 * u;
-      const bool first = j < NPOS - 1 - warp;
-      pk[u] = first ? warp : NPOS - 1 - warp;
-      pl[u] = first ? warp + 1 + j : NPOS - warp + (j - (NPOS - 1 - warp));
-      rd[u] = warp * (NPOS - 1) + j;
-      if (j >= NPOS - 1) { rd[u] = -1; pk[u] = 0; pl[u] = 1; }
-#pragma unroll
-      for (int e = 0; e < 4; e++) wr[u][e] = eig_slot(eig_move(2 * pk[u] + (e >> 1)), eig_move(2 * pl[u] + (e & 1)));
-    }
-    const int dk = tid & (NPOS - 1);
-    const int d_off = eig_slot(eig_move(2 * dk), eig_move(2 * dk + 1));
-    const int d_top = 4 * NBLK + NPOS + eig_move(2 * dk), d_bot = 4 * NBLK + NPOS + eig_move(2 * dk + 1);
-    double* t_remote[V_CTAS];
-#pragma unroll
-    for (int r = 0; r < V_CTAS; r++) t_remote[r] = cluster.map_shared_rank(&sv.t[0][0], r + 1);
-    if (tid == 0) sa.maxt = 0;
-    __syncthreads();
-    int cur = 0, sweeps = 0, sweep = 0;
-    for (;; sweep++) {
-      const int tbase = (sweep & 1) * ROUNDS * NPOS;
-#pragma unroll 1
-      for (int round = 0; round < ROUNDS; round++) {
-        const double* in = sa.buf[cur];
-        double* out = sa.buf[cur ^ 1];
-        if (tid < NPOS) {
-          const double app = in[4 * NBLK + NPOS + 2 * dk], aqq = in[4 * NBLK + NPOS + 2 * dk + 1], apq = in[4 * NBLK + dk];
-          double t = 0.0, res = apq;
-          double2 cs = make_double2(1.0, 0.0);
-          if (fabs(apq) > tiny && apq * apq > 1e-34 * fabs(app * aqq)) {
-            const float tau = __fdividef((float)(aqq - app), 2.0f * (float)apq);
-            const float tf = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
-            t = (double)tf;
-            cs = eig_cos_sin(t);
-            res = cs.x * cs.x * fma(1.0 - t * t, apq, t * (app - aqq));
-            atomicMax(&sa.maxt, __float_as_uint(fabsf(tf)));
-          }
-          sa.cs[dk] = cs;
-          out[d_top] = app - t * (apq + res);
-          out[d_bot] = aqq + t * (apq + res);
-          out[d_off] = res;
-#pragma unroll
-          for (int r = 0; r < V_CTAS; r++) t_remote[r][tbase + round * NPOS + dk] = t;
-        }
-        double x[2][4];
-#pragma unroll
-        for (int u = 0; u < 2; u++)
-          if (rd[u] >= 0)
-#pragma unroll
-            for (int e = 0; e < 4; e++) x[u][e] = in[e * NBLK + rd[u]];
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 2; u++)
-          if (rd[u] >= 0) {
-            const double2 ck = sa.cs[pk[u]], cl = sa.cs[pl[u]];
-            const double r00 = ck.x * x[u][0] - ck.y * x[u][2], r01 = ck.x * x[u][1] - ck.y * x[u][3];
-            const double r10 = ck.y * x[u][0] + ck.x * x[u][2], r11 = ck.y * x[u][1] + ck.x * x[u][3];
-            out[wr[u][0]] = cl.x * r00 - cl.y * r01;
-            out[wr[u][1]] = cl.y * r00 + cl.x * r01;
-            out[wr[u][2]] = cl.x * r10 - cl.y * r11;
-            out[wr[u][3]] = cl.y * r10 + cl.x * r11;
-          }
-        __syncthreads();
-        cur ^= 1;
-      }
-      const float mt = __uint_as_float(sa.maxt);
-      if (mt > 0.0f) sweeps++;
-      const bool done = mt <= 1e-8f || sweep + 1 >= MAX_SWEEPS;
-      if (tid < V_CTAS) cluster.map_shared_rank(&sv.done[0], tid + 1)[sweep & 1] = done;
-      __syncthreads();
-      if (tid == 0) sa.maxt = 0;
-      cluster.sync();   // the sweep's tangents are in place; the sweep before has been applied
-      if (done) break;
-    }
-    if (tid == 0 && sweeps_out) *sweeps_out = sweeps;
-    if (tid < D) {
-      const double l = sa.buf[cur][4 * NBLK + NPOS + tid] * ldexp(1.0, ex);
-      const int idx = eig_index(tid, 0);
-      for (int r = 0; r < V_CTAS; r++) cluster.map_shared_rank(&sv.lam[0], r + 1)[idx] = l;
-    }
-    cluster.sync();   // eigenvalues are out
-    cluster.sync();   // (the other blocks exchange their slices' largest components)
-    return;
   }
-  const int col0 = (rank - 1) * V_COLS;
-  for (int i = tid; i < D * V_COLS; i += EIG_THREADS) sv.v[i / V_COLS][i % V_COLS] = i / V_COLS == col0 + i % V_COLS ? 1.0 : 0.0;
+  // Angle threads: thread dk < 64 has pair dk.  Of the round under way it knows the tangent t, the rotated pair's own
+  // off-diagonal element res (moved like any other) and, through dg, the rotated diagonal.
+  const int dk = tid & (NPOS - 1);
+  const int d_off = eig_slot(eig_move(2 * dk), eig_move(2 * dk + 1));
+  // positions that move to (top dk, bottom dk); always of two different pairs, the first one lower
+  const int pa = dk == 0 ? 0 : (dk == 1 ? 1 : 2 * (dk - 1)), pb = dk == NPOS - 1 ? 2 * (NPOS - 1) : 2 * (dk + 1) + 1;
+  const int src = eig_block(pa >> 1, pb >> 1);
+  double* t_remote[V_CTAS];
+#pragma unroll
+  for (int r = 0; r < V_CTAS; r++) t_remote[r] = cluster.map_shared_rank(&sv.t[0][0], r + 1);
+  T t = 0, res = 0;
+  float tmax = 0.f;
+  auto angle = [&](T app, T aqq, T apq, int to) {
+    Pair2<T> cs = {1, 0};
+    t = 0; res = apq;
+    if ((apq < 0 ? -apq : apq) > tiny && apq * apq > rel2 * (app * aqq < 0 ? -(app * aqq) : app * aqq)) {
+      const float tau = __fdividef((float)(aqq - app), 2.0f * (float)apq);
+      float root;
+      asm("sqrt.approx.ftz.f32 %0, %1;\n" : "=f"(root) : "f"(fmaf(tau, tau, 1.0f)));
+      t = (T)__fdividef(copysignf(1.0f, tau), fabsf(tau) + root);
+      cs = eig_cos_sin(t);
+      res = cs.x * cs.x * ((1 - t * t) * apq + t * (app - aqq));
+    }
+    sa.cs[to][dk] = cs;
+    sa.dg[to][2 * dk] = app - t * (apq + res);
+    sa.dg[to][2 * dk + 1] = aqq + t * (apq + res);
+  };
+  __syncthreads();
+  T app = 0, aqq = 0;
+  if (tid < NPOS) { app = sa.dg[0][2 * dk]; aqq = sa.dg[0][2 * dk + 1]; angle(app, aqq, sa.own[dk], 0); }
+  __syncthreads();
+  int cur = 0, sweeps = 0, sweep = 0;
+  for (;; sweep++) {
+    const int tbase = (sweep & 1) * ROUNDS * NPOS;
+#pragma unroll 1
+    for (int round = 0; round < ROUNDS; round++) {
+      const T* in = sa.buf[cur];
+      T* out = sa.buf[cur ^ 1];
+      const Pair2<T>* cs = sa.cs[cur];
+      if (tid < NPOS) {
+        out[d_off] = res;
+        tmax = fmaxf(tmax, fabsf((float)t));
+#pragma unroll
+        for (int r = 0; r < V_CTAS; r++) t_remote[r][tbase + round * NPOS + dk] = (double)t;
+        // the next round's pair: rows (c, -s) of a top, (s, c) of a bottom
+        const Pair2<T> ca = cs[pa >> 1], cb = cs[pb >> 1];
+        const T u0 = (pa & 1) ? ca.y : ca.x, u1 = (pa & 1) ? ca.x : -ca.y;
+        const T w0 = (pb & 1) ? cb.y : cb.x, w1 = (pb & 1) ? cb.x : -cb.y;
+        const T m0 = w0 * in[src] + w1 * in[NBLK + src], m1 = w0 * in[2 * NBLK + src] + w1 * in[3 * NBLK + src];
+        angle(sa.dg[cur][pa], sa.dg[cur][pb], u0 * m0 + u1 * m1, cur ^ 1);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; u++)
+        if (rd[u] >= 0) {
+          T x[4];
+#pragma unroll
+          for (int e = 0; e < 4; e++) x[e] = in[e * NBLK + rd[u]];
+          const Pair2<T> ck = cs[pk[u]], cl = cs[pl[u]];
+          const T r00 = ck.x * x[0] - ck.y * x[2], r01 = ck.x * x[1] - ck.y * x[3];
+          const T r10 = ck.y * x[0] + ck.x * x[2], r11 = ck.y * x[1] + ck.x * x[3];
+          const T y[4] = {cl.x * r00 - cl.y * r01, cl.y * r00 + cl.x * r01, cl.x * r10 - cl.y * r11, cl.y * r10 + cl.x * r11};
+#pragma unroll
+          for (int e = 0; e < 4; e++)
+            if (wr[u][e] >= 0) out[wr[u][e]] = y[e];
+        }
+      __syncthreads();
+      cur ^= 1;
+    }
+    if (warp < 2) {
+      for (int d = 16; d; d >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, d));
+      if (lane == 0) sa.tmax[warp] = tmax;
+      tmax = 0.f;
+    }
+    __syncthreads();
+    const float mt = fmaxf(sa.tmax[0], sa.tmax[1]);
+    if (mt > 0.0f) sweeps++;
+    const bool done = !(mt > stop) || sweep + 1 >= max_sweeps;
+    if (tid < V_CTAS) cluster.map_shared_rank(&sv.done[0], tid + 1)[sweep & 1] = done;
+    cluster.sync();   // the sweep's tangents are in place; the sweep before has been applied
+    if (done) break;
+  }
+  *diag = cur ^ 1;    // dg[cur] already has the rotations of a round that does not happen
+  return sweeps;
+}
+
+// the other blocks: the sweeps of one phase applied to this slice of V^T
+__device__ __forceinline__ void eig_apply(cg::cluster_group& cluster, EigV& sv) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int sweep = 0;; sweep++) {
     cluster.sync();
     const double* ts = sv.t[sweep & 1];
-    for (int round = 0; round < ROUNDS; round++) {
-      // a warp takes two pairs, a lane one column
+    for (int r0 = 0; r0 < ROUNDS; r0 += CHUNK) {
+      const int nr = min(CHUNK, ROUNDS - r0);
+      // each rotation once per block (every warp for itself: 900 cycles per round)
+      for (int i = threadIdx.x; i < nr * NPOS; i += EIG_THREADS) (&sv.cs[0][0])[i] = eig_cos_sin(ts[r0 * NPOS + i]);
+      __syncthreads();
+      for (int round = r0; round < r0 + nr; round++) {
+        // a warp takes two pairs, a lane one column
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const int k = warp + 32 * u;
-        const double t = ts[round * NPOS + k];
-        if (t != 0.0) {
-          const double2 cs = eig_cos_sin(t);
+        for (int u = 0; u < 2; u++) {
+          const int k = warp + 32 * u;
+          const Pair2<double> cs = sv.cs[round - r0][k];
           double* vp = &sv.v[eig_index(2 * k, round)][lane];
           double* vq = &sv.v[eig_index(2 * k + 1, round)][lane];
           const double a = *vp, b = *vq;
           *vp = cs.x * a - cs.y * b;
           *vq = cs.y * a + cs.x * b;
         }
+        __syncthreads();
       }
-      __syncthreads();
     }
     if (sv.done[sweep & 1]) break;
   }
+}
+
+__global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __restrict__ C, const float* __restrict__ signs,
+                                                           float* __restrict__ R, float* __restrict__ lambda,
+                                                           int* __restrict__ sweeps_out) {
+  extern __shared__ __align__(16) unsigned char eig_raw[];
+  __shared__ double red[32];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x;
+  EigV& sv = *reinterpret_cast<EigV*>(eig_raw);
+  EigA<double>& sd = *reinterpret_cast<EigA<double>*>(eig_raw);
+  EigA<float>& sf = *reinterpret_cast<EigA<float>*>(eig_raw);
+  cluster.sync();   // every block runs before its shared memory is written from outside
+  // largest magnitude (the matrix is scaled by a power of two to at most 1) and trace
+  double mx = 0.0, tr = 0.0;
+  for (int i = tid; i < D * D; i += EIG_THREADS) mx = fmax(mx, fabs((double)C[i]));
+  if (tid < D) tr = fabs((double)C[tid * D + tid]);
+  for (int d = 16; d; d >>= 1) {
+    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+    tr += __shfl_xor_sync(0xffffffffu, tr, d);
+  }
+  if (lane == 0) red[warp] = mx;
+  __syncthreads();
+  for (int i = 0; i < 32; i++) mx = fmax(mx, red[i]);
+  __syncthreads();
+  if (lane == 0 && warp < 4) red[warp] = tr;
+  __syncthreads();
+  int ex = 0;
+  if (mx > 0.0) frexp(mx, &ex);   // mx < 2^ex
+  const double scale = ldexp(1.0, -ex);
+  auto element = [&](int i, int j) { return 0.5 * ((double)C[i * D + j] + (double)C[j * D + i]) * scale; };
+  if (rank == 0) {
+    for (int i = tid; i < D * D; i += EIG_THREADS) {
+      const int a = i / D, b = i % D;
+      if (a > b) continue;
+      const float x = (float)element(eig_index(a, 0), eig_index(b, 0));
+      if (a == b) sf.dg[0][a] = x;
+      else if ((a >> 1) == (b >> 1)) sf.own[a >> 1] = x;
+      else sf.buf[0][eig_slot(a, b)] = x;
+    }
+    int diag;
+    // fp32: elements below the rounding noise of the largest or of their diagonal are left to the second phase
+    int sweeps = eig_sweeps<float>(cluster, sf, sv, 1e-8f, 1e-13f, 1e-3f, FP32_SWEEPS, &diag);
+    cluster.sync();   // V^T is complete
+    cluster.sync();   // the products are ready
+    for (int r = 0; r < V_CTAS; r++) cluster.sync();   // ... and added up here, slice by slice
+    // the size below which an off-diagonal element is left alone
+    const double tiny = fmax(((red[0] + red[1]) + (red[2] + red[3])) * scale * 1e-18, 1e-30);
+    sweeps += eig_sweeps<double>(cluster, sd, sv, tiny, 1e-34, 1e-8f, MAX_SWEEPS - FP32_SWEEPS, &diag);
+    if (tid == 0 && sweeps_out) *sweeps_out = sweeps;
+    if (tid < D) {
+      const double l = sd.dg[diag][tid] * ldexp(1.0, ex);
+      const int idx = eig_index(tid, ROUNDS - 1);   // who sat there in the last round
+      for (int r = 0; r < V_CTAS; r++) cluster.map_shared_rank(&sv.lam[0], r + 1)[idx] = l;
+    }
+    cluster.sync();   // eigenvalues are out
+    cluster.sync();   // (the other blocks exchange their slices' largest components)
+    return;
+  }
+  const int slice = rank - 1, col0 = slice * V_COLS;
+  for (int i = tid; i < D * V_COLS; i += EIG_THREADS) {
+    sv.v[i / V_COLS][i % V_COLS] = i / V_COLS == col0 + i % V_COLS ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  eig_apply(cluster, sv);
+  cluster.sync();     // V^T is complete
+  {
+    // this slice's columns of V^T A: all of V^T (the other slices from their blocks) times the slice's columns of A
+    for (int i = tid; i < D * V_COLS; i += EIG_THREADS) sv.a[i / V_COLS][i % V_COLS] = element(i / V_COLS, col0 + i % V_COLS);
+    for (int o = 1; o < V_CTAS; o++) {
+      const double* src = cluster.map_shared_rank(&sv.v[0][0], (slice + o) % V_CTAS + 1);
+      for (int i = tid; i < D * V_COLS; i += EIG_THREADS) (&sv.other[o - 1][0][0])[i] = src[i];
+    }
+    __syncthreads();
+    double z[4] = {0.0, 0.0, 0.0, 0.0};   // rows l = warp + 32 i, column lane
+    for (int o = 0; o < V_CTAS; o++) {
+      const double (*v)[V_COLS] = o == 0 ? sv.v : sv.other[o - 1];
+      const int i0 = (slice + o) % V_CTAS * V_COLS;
+      for (int i = 0; i < V_COLS; i++) {
+        const double x = sv.a[i0 + i][lane];
+#pragma unroll
+        for (int q = 0; q < 4; q++) z[q] = fma(v[warp + 32 * q][i], x, z[q]);
+      }
+    }
+    cluster.sync();   // every slice has been read: the space is free for the products
+    double (*zs)[V_COLS] = sv.other[0];
+#pragma unroll
+    for (int q = 0; q < 4; q++) zs[warp + 32 * q][lane] = z[q];
+    __syncthreads();
+    // this slice's share of V^T A V: rows l = warp + 32 i, columns m = lane + 32 k
+    double p[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int k = 0; k < 4; k++) p[i][k] = 0.0;
+    for (int jj = 0; jj < V_COLS; jj++) {
+      const int j = (jj + lane) & (V_COLS - 1);   // (a column of V^T per step would put all lanes on one bank pair)
+      double vm[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) vm[k] = sv.v[lane + 32 * k][j];
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const double x = zs[warp + 32 * i][j];
+#pragma unroll
+        for (int k = 0; k < 4; k++) p[i][k] = fma(x, vm[k], p[i][k]);
+      }
+    }
+    EigA<double>& dst = *cluster.map_shared_rank(&sd, 0);
+    for (int r = 0; r < V_CTAS; r++) {   // added up in block 0, in slice order
+      if (r == slice)
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+          for (int k = 0; k < 4; k++) {
+            const int a = eig_home(warp + 32 * i), b = eig_home(lane + 32 * k);
+            if (a > b) continue;
+            double* at = a == b ? &dst.dg[0][a] : (a >> 1) == (b >> 1) ? &dst.own[a >> 1] : &dst.buf[0][eig_slot(a, b)];
+            *at = r == 0 ? p[i][k] : *at + p[i][k];
+          }
+      cluster.sync();
+    }
+  }
+  eig_apply(cluster, sv);
   cluster.sync();   // eigenvalues are here
   if (tid < D) {    // the slice's component of largest magnitude (the first of equals), to all slices
     double best = 0.0, val = 0.0;
