@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
   const int G = P.group, Hkv = cv.n_kv_heads;
   const int n_entries = P.layer_count * cv.batch;
 
+  depend_wait();
   // ---- partition of the flattened window axis
   const int total = block_prefix(cv, P.layer0, n_entries, sm.prefix);
   const int per = (total + gridDim.x - 1) / gridDim.x;
@@ -177,13 +178,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
       const int pa = mg.pa[su], np = mg.pb[su] - pa + 1;
       if (np <= 0) continue;
       const int inc0 = su + pa - mg.pa[0], hsel = 2 * (L & 3);
+      // all the pieces' rows on their way together (they come from L2: one after another they were a third of a call with
+      // few windows per warp)
+      float4 x[NWARP];
+#pragma unroll
+      for (int q = 0; q < NWARP; q++) {
+        x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q < np && ((mg.mask[inc0 + (q < np ? q : 0)] >> m) & 1))   // (else: no such warp / no token of this modality)
+          x[q] = __ldcg(&P.pieces[(size_t)(ub + su) + (size_t)blockIdx.x * NWARP + pa + q].frag[m][rg][L]);
+      }
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < NWARP; q++) {
-        if (q >= np || !((mg.mask[inc0 + q] >> m) & 1)) continue;   // no such warp / no token of this modality
-        const float fe = mg.fac[inc0 + q][hsel], fo = mg.fac[inc0 + q][hsel + 1];
-        const float4 x = __ldcg(&P.pieces[(size_t)(ub + su) + (size_t)blockIdx.x * NWARP + pa + q].frag[m][rg][L]);
-        v.x = fmaf(x.x, fe, v.x); v.y = fmaf(x.y, fo, v.y); v.z = fmaf(x.z, fe, v.z); v.w = fmaf(x.w, fo, v.w);
+        const float2 f = *reinterpret_cast<const float2*>(&mg.fac[inc0 + (q < np ? q : 0)][hsel]);
+        v.x = fmaf(x[q].x, f.x, v.x); v.y = fmaf(x[q].y, f.y, v.y); v.z = fmaf(x[q].z, f.x, v.z); v.w = fmaf(x[q].w, f.y, v.w);
       }
       // in units of the bit-plane form, whose weight sums are zero here
       constexpr float F = LEVEL_UNIT * 16.0f / PARTIAL_ACC_SCALE;
@@ -263,6 +271,7 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   const int bb = live ? b : 0;
   const int G = P.group, Hkv = cv.n_kv_heads;
   const int n_entries = P.layer_count * cv.batch;
+  depend_wait();
   const int seq = live ? cv.seq_len[layer * cv.batch + bb] : 0;
   // tokens [0, v_pk) have packed values (and keys): they are in the split-K partials; tokens [v_pk, seq) have raw
   // values; of those, [v_pk, k_pk) have packed keys (captioning schedule only), the rest raw keys
@@ -704,7 +713,7 @@ static cudaError_t combine_attr() {
 template <bool CAPTION, int NS, int SEQ>
 static void combine_launch(const DecodeParams& P, int n_cta, cudaStream_t s) {
   const dim3 grid(P.cv.n_kv_heads * NS, (P.cv.batch + SEQ - 1) / SEQ, P.layer_count);
-  k_combine_mma<CAPTION, NS, SEQ><<<grid, SEQ * 128, sizeof(CombineSmem<CAPTION, SEQ>), s>>>(P, n_cta);
+  launch_dependent(k_combine_mma<CAPTION, NS, SEQ>, grid, SEQ * 128, sizeof(CombineSmem<CAPTION, SEQ>), s, 1, P, n_cta);
 }
 
 template <bool CAPTION>
@@ -751,8 +760,8 @@ okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, c
   if (P.cv.fmt == FMT_FP16 && g_decode_impl == 0) {
     const okq_status st = launch_decode_tc(P, n_cta, s);
     if (st != OKQ_OK) return st;
-  } else if (P.cv.fmt == FMT_MXFP4) k_decode_mma<FMT_MXFP4><<<n_cta, NTHREADS, sizeof(MmaSmem<FMT_MXFP4>), s>>>(P);
-  else k_decode_mma<FMT_FP16><<<n_cta, NTHREADS, sizeof(MmaSmem<FMT_FP16>), s>>>(P);
+  } else if (P.cv.fmt == FMT_MXFP4) launch_dependent(k_decode_mma<FMT_MXFP4>, dim3(n_cta), NTHREADS, sizeof(MmaSmem<FMT_MXFP4>), s, 1, P);
+  else launch_dependent(k_decode_mma<FMT_FP16>, dim3(n_cta), NTHREADS, sizeof(MmaSmem<FMT_FP16>), s, 1, P);
   if (after) cudaEventRecord(after, s);
   if (P.cv.sched == SCHED_CAPTION) combine_dispatch<true>(P, n_cta, s);
   else combine_dispatch<false>(P, n_cta, s);
