@@ -82,8 +82,7 @@ okq_status launch_decode_tc(const DecodeParams& P, int n_cta, cudaStream_t s);
 // which split-K kernel launch_decode_mma uses: 0 = the tcgen05 kernel (fp16 metadata), 1 = the mma.sync kernel
 extern int g_decode_impl;
 
-// one-launch form for few (sequence, head) units: cluster size it would use for a call (0: not applicable), launch
-constexpr int SMALL_WINDOWS_PER_WARP = 16;
+// one-launch form for few (sequence, head) units: cluster size it would use for a call (0: the split-K pair), launch
 int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta);
 okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s);
 

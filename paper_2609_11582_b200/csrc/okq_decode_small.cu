@@ -2,7 +2,7 @@
 //
 // The split-K kernel and its combine kernel are a chain of launch, prefix, partials through memory, launch, prefix,
 // merge; with a handful of windows per warp that chain is the whole time (35 + 20 us for one layer of 4 sequences at
-// 4096 tokens).  Here a thread-block cluster owns one unit: its CS x 12 warps walk the unit's windows (the same code as
+// 4096 tokens).  Here a thread-block cluster (or one block) owns one unit: its CS x 12 warps walk the unit's windows (the same code as
 // the split-K kernel), leave their sums as pieces in global memory (L2), and after one cluster barrier every CTA merges
 // 1 / CS of the rotated channels over all pieces.  The merged sums are pushed into every CTA's shared memory, and after
 // the second barrier each CTA applies R_m^T for 1 / CS of the output columns.  The raw tail is scored by every CTA (its
@@ -30,10 +30,11 @@ template <int FMT, int CS> struct SmallSmem {
   static constexpr int NP = CS * NWARP;         // pieces of a unit
   static constexpr int KS = 2 * NTHREADS / C;   // row slices of the product (a thread takes two columns)
   static constexpr int TAIL = CAPTION_V_SLOTS;
+  static constexpr bool STAGED = CS >= 2;       // matrices and raw value rows in shared memory (a single block: from L2)
   // what takes the record ring's place once every warp of the CTA has walked its range
   struct After {
-    __align__(16) float R[3 * D][C];            // this CTA's columns of the three matrices
-    __align__(16) __half v[TAIL][C];            // and of the raw value rows
+    __align__(16) float R[STAGED ? 3 * D : 1][C];   // this CTA's columns of the three matrices
+    __align__(16) __half v[STAGED ? TAIL : 1][C];   // and of the raw value rows
     __align__(16) __half k[CAPTION_K_GROUP - W][KROW];   // raw key rows behind the first 32
     __align__(16) unsigned char img[PC_MAX][KIMG];
     __align__(16) float tsc[TAIL][GP];          // tail scores (log2 domain), then numerators
@@ -175,12 +176,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     }
   }
   cp_async_commit();
-  for (int i = tid; i < n_tail * (C / 8); i += NTHREADS)
-    cp_async16(&af.v[i / (C / 8)][8 * (i % (C / 8))], vt + cv.v_slot(v_pk + i / (C / 8)) * D + rank * C + 8 * (i % (C / 8)));
-  {
-    const float* R = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D + rank * C;
-    for (int i = tid; i < 3 * D * (C / 4); i += NTHREADS)
-      cp_async16(&af.R[i / (C / 4)][4 * (i % (C / 4))], R + (size_t)(i / (C / 4)) * D + 4 * (i % (C / 4)));
+  const float* Rsl = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D + rank * C;
+  if (SM::STAGED)
+    for (int i = tid; i < n_tail * (C / 8); i += NTHREADS)
+      cp_async16(&af.v[i / (C / 8)][8 * (i % (C / 8))], vt + cv.v_slot(v_pk + i / (C / 8)) * D + rank * C + 8 * (i % (C / 8)));
+  for (int i = tid; i < 3 * D * (C / 4); i += NTHREADS) {
+    if (SM::STAGED) cp_async16(&af.R[i / (C / 4)][4 * (i % (C / 4))], Rsl + (size_t)(i / (C / 4)) * D + 4 * (i % (C / 4)));
+    else if (i % 8 == 0) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Rsl + 4 * i));
   }
   cp_async_commit();
 
@@ -273,45 +275,52 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   // ---- merge of the pieces for channels [rank * C, rank * C + C): item = (modality, m-tile, lane), a float4 of the piece
   // = channels g and g + 8 of the tile for heads 2 t and 2 t + 1 (clusters of 16: half a tile, one of the two channels)
   {
-    constexpr int MT = C >= 16 ? C / 16 : 1, ITEMS = 3 * MT * 32, SHARES = NTHREADS / ITEMS;
-    static_assert(NTHREADS % ITEMS == 0, "whole shares");
-    const int share = tid / ITEMS, it = tid % ITEMS;
-    const int L32 = it & 31, mt = (it >> 5) % MT, m = it / (32 * MT);
-    const int mu = C >= 16 ? rank * MT + mt : rank / 2;
-    const int j0 = 2 * (L32 & 3);
+    constexpr int MT = C >= 16 ? C / 16 : 1, ITEMS = 3 * MT * 32, SHARES = ITEMS < NTHREADS ? NTHREADS / ITEMS : 1;
+    static_assert(NTHREADS % ITEMS == 0 || ITEMS % NTHREADS == 0, "whole shares");
+    const int share = tid / ITEMS;
     const int used = cnt > 0 ? (nwin + cnt - 1) / cnt : 0;   // pieces beyond have no windows
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    constexpr int IN_FLIGHT = 12;   // loads of a thread fetched together: the pieces come from L2
-    for (int p0 = share; p0 < used; p0 += IN_FLIGHT * SHARES) {
-      float4 x[IN_FLIGHT];
 #pragma unroll
-      for (int i = 0; i < IN_FLIGHT; i++) {
-        const int p = p0 + i * SHARES;
-        const bool have = p < used && ((sm.meta[p < used ? p : 0].held >> m) & 1);
-        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (have) x[i] = __ldcg(&pieces[p].frag[m][mu][L32]);
-      }
+    for (int it0 = 0; it0 < ITEMS; it0 += NTHREADS) {        // (one round, two for a single block)
+      const int it = ITEMS < NTHREADS ? tid % ITEMS : tid + it0;
+      const int L32 = it & 31, mt = (it >> 5) % MT, m = it / (32 * MT);
+      const int mu = C >= 16 ? rank * MT + mt : rank / 2;
+      const int j0 = 2 * (L32 & 3);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      constexpr int IN_FLIGHT = 12;   // loads of a thread fetched together: the pieces come from L2
+      for (int p0 = share; p0 < used; p0 += IN_FLIGHT * SHARES) {
+        float4 x[IN_FLIGHT];
 #pragma unroll
-      for (int i = 0; i < IN_FLIGHT; i++) {
-        const int p = min(p0 + i * SHARES, used - 1);
-        const float2 f = *reinterpret_cast<const float2*>(&af.fac[p][j0]);
-        v.x = fmaf(x[i].x, f.x, v.x); v.y = fmaf(x[i].y, f.y, v.y); v.z = fmaf(x[i].z, f.x, v.z); v.w = fmaf(x[i].w, f.y, v.w);
+        for (int i = 0; i < IN_FLIGHT; i++) {
+          const int p = p0 + i * SHARES;
+          const bool have = p < used && ((sm.meta[p < used ? p : 0].held >> m) & 1);
+          x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (have) x[i] = __ldcg(&pieces[p].frag[m][mu][L32]);
+        }
+#pragma unroll
+        for (int i = 0; i < IN_FLIGHT; i++) {
+          const int p = min(p0 + i * SHARES, used - 1);
+          const float2 f = *reinterpret_cast<const float2*>(&af.fac[p][j0]);
+          v.x = fmaf(x[i].x, f.x, v.x); v.y = fmaf(x[i].y, f.y, v.y); v.z = fmaf(x[i].z, f.x, v.z); v.w = fmaf(x[i].w, f.y, v.w);
+        }
       }
-    }
-    af.part[tid] = v;
-    __syncthreads();
-    if (tid < ITEMS) {
-      for (int s = 1; s < SHARES; s++) {
-        const float4 x = af.part[s * ITEMS + tid];
-        v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+      if (SHARES > 1) {
+        af.part[tid] = v;
+        __syncthreads();
+        if (tid < ITEMS)
+          for (int q = 1; q < SHARES; q++) {
+            const float4 x = af.part[q * ITEMS + tid];
+            v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+          }
       }
-      constexpr float F = LEVEL_UNIT * 16.0f;   // numerators carry 2^P_LOG2 = 1/16
-      static_assert(P_LOG2 == -4.0f, "");
-      const int ch = 16 * mu + (L32 >> 2);
-      for (int r = 0; r < CS; r++) {   // to every CTA of the cluster
-        float* dst = cluster.map_shared_rank(&af.vec[0][0], r);
-        if (C >= 16 || (rank & 1) == 0) *reinterpret_cast<float2*>(dst + (m * D + ch) * GP + j0) = make_float2(v.x * F, v.y * F);
-        if (C >= 16 || (rank & 1) == 1) *reinterpret_cast<float2*>(dst + (m * D + ch + 8) * GP + j0) = make_float2(v.z * F, v.w * F);
+      if (SHARES == 1 || tid < ITEMS) {
+        constexpr float F = LEVEL_UNIT * 16.0f;   // numerators carry 2^P_LOG2 = 1/16
+        static_assert(P_LOG2 == -4.0f, "");
+        const int ch = 16 * mu + (L32 >> 2);
+        for (int r = 0; r < CS; r++) {   // to every CTA of the cluster
+          float* dst = CS == 1 ? &af.vec[0][0] : cluster.map_shared_rank(&af.vec[0][0], r);
+          if (C >= 16 || (rank & 1) == 0) *reinterpret_cast<float2*>(dst + (m * D + ch) * GP + j0) = make_float2(v.x * F, v.y * F);
+          if (C >= 16 || (rank & 1) == 1) *reinterpret_cast<float2*>(dst + (m * D + ch + 8) * GP + j0) = make_float2(v.z * F, v.w * F);
+        }
       }
     }
   }
@@ -333,10 +342,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
 #pragma unroll
       for (int j = 0; j < GP; j++) { o[j].x = fmaf(x.x, wj[j], o[j].x); o[j].y = fmaf(x.y, wj[j], o[j].y); }
     };
+    if (SM::STAGED) {
 #pragma unroll 8
-    for (int r = ks * ROWS; r < (ks + 1) * ROWS; r++) add_row(*reinterpret_cast<const float2*>(&af.R[r][c]), af.vec[r]);
-    for (int i = ks; i < n_tail; i += KS)   // raw value rows
-      add_row(__half22float2(*reinterpret_cast<const __half2*>(&af.v[i][c])), af.tsc[i]);
+      for (int r = ks * ROWS; r < (ks + 1) * ROWS; r++) add_row(*reinterpret_cast<const float2*>(&af.R[r][c]), af.vec[r]);
+      for (int i = ks; i < n_tail; i += KS)   // raw value rows
+        add_row(__half22float2(*reinterpret_cast<const __half2*>(&af.v[i][c])), af.tsc[i]);
+    } else {
+#pragma unroll 16
+      for (int r = ks * ROWS; r < (ks + 1) * ROWS; r++) add_row(__ldg(reinterpret_cast<const float2*>(Rsl + (size_t)r * D + c)), af.vec[r]);
+#pragma unroll 4
+      for (int i = ks; i < n_tail; i += KS)
+        add_row(__half22float2(*reinterpret_cast<const __half2*>(vt + cv.v_slot(v_pk + i) * D + c)), af.tsc[i]);
+    }
 #pragma unroll
     for (int j = 0; j < GP; j++) *reinterpret_cast<float2*>(&af.prod[ks][j][c]) = o[j];
     __syncthreads();
@@ -391,23 +408,30 @@ static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s
   return launch_dependent(k_decode_small<FMT, CS>, dim3(units * CS), NTHREADS, sizeof(SmallSmem<FMT, CS>), s, CS, P);
 }
 
+// Cluster size for a call, 0 if the split-K pair should take it: whichever of the estimates below is least.  A cluster per
+// unit, in waves of as many as run at once (on this GPU 7 clusters of 16, 15 of 8, 33 of 4, 74 of 2, 148 blocks: a cluster
+// stays inside one of eight groups of SMs): 11.5 us a wave and 2.1 us per window of a warp.  The pair: 31 us, 2 us per window
+// of a warp with the windows balanced over all warps, 0.04 us per unit in the combine kernel.  Fitted to calls of 1 to 28
+// layers, 1 to 16 sequences, 1 to 8 heads and 200 to 131072 tokens; the host knows the capacity, not the lengths, and takes
+// sequences to be full: a cache mostly empty goes the way it would go full.
 template <int FMT>
-static int small_cluster(long long units, int n_cta) {
-  if (units * 16 <= n_cta && units <= small_clusters<FMT, 16>()) return 16;
-  if (units * 8 <= n_cta && units <= small_clusters<FMT, 8>()) return 8;
-  if (units * 4 <= n_cta && units <= small_clusters<FMT, 4>()) return 4;
-  return 0;
+static int small_cluster(long long units, long long windows, int n_cta) {
+  const int fit[5] = {small_clusters<FMT, 1>(), small_clusters<FMT, 2>(), small_clusters<FMT, 4>(), small_clusters<FMT, 8>(), small_clusters<FMT, 16>()};
+  int best = 0;
+  double best_cost = 31.0 + 2.0 * (double)units * (double)windows / (148.0 * NWARP) + 0.04 * (double)units;
+  for (int i = 4; i >= 0; i--) {   // (of equals the largest cluster)
+    // the warps' pieces have to fit the scratch, which is laid out for `units` and NWARP per CTA of the split-K kernel
+    if (fit[i] <= 0 || (units << i) * NWARP > units + (long long)NWARP * n_cta) continue;
+    const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * (1 << i) - 1) / (NWARP * (1 << i)));
+    const double cost = waves * (11.5 + 2.1 * walk);
+    if (cost < best_cost) { best_cost = cost; best = 1 << i; }
+  }
+  return best;
 }
 
-// Cluster size for a call, 0 if the split-K kernel should take it.  The clusters of all units have to be resident at once
-// (7 clusters of 16, 15 of 8, 33 of 4 on this GPU: a cluster stays inside one of its eight groups of SMs), and a warp's
-// share of the longest possible sequence has to be short: the units are not balanced against one another, and with fewer
-// CTAs than SMs a long walk costs more than the second launch saves.
 int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta) {
-  const long long units = (long long)layer_count * cv.batch * cv.n_kv_heads;
-  if (units * 4 > n_cta || cv.capacity / W > 16 * NWARP * SMALL_WINDOWS_PER_WARP) return 0;
-  const int cs = cv.fmt == FMT_MXFP4 ? small_cluster<FMT_MXFP4>(units, n_cta) : small_cluster<FMT_FP16>(units, n_cta);
-  return cv.capacity / W <= cs * NWARP * SMALL_WINDOWS_PER_WARP ? cs : 0;
+  const long long units = (long long)layer_count * cv.batch * cv.n_kv_heads, windows = cv.capacity / W;
+  return cv.fmt == FMT_MXFP4 ? small_cluster<FMT_MXFP4>(units, windows, n_cta) : small_cluster<FMT_FP16>(units, windows, n_cta);
 }
 
 template <int CS>
@@ -417,7 +441,8 @@ static cudaError_t small_format(const DecodeParams& P, int units, cudaStream_t s
 
 okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s) {
   const int units = P.layer_count * P.cv.batch * P.cv.n_kv_heads;
-  const cudaError_t e = cs == 16 ? small_format<16>(P, units, s) : cs == 8 ? small_format<8>(P, units, s) : small_format<4>(P, units, s);
+  const cudaError_t e = cs == 16 ? small_format<16>(P, units, s) : cs == 8 ? small_format<8>(P, units, s)
+                      : cs == 4 ? small_format<4>(P, units, s) : cs == 2 ? small_format<2>(P, units, s) : small_format<1>(P, units, s);
   if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return OKQ_OK;
 }
