@@ -418,6 +418,16 @@ static size_t mma_workspace(const okq_cache* c, int layer_count, int num_splits)
              sizeof(WarpPiece);
 }
 
+// What okq_decode_workspace_bytes asks for beyond the least a call accepts: room for the pieces of the one-launch kernel where
+// that is estimated to be the faster way (several waves of single blocks; a call given less takes the split-K pair).
+static size_t small_workspace(const okq_cache* c, int layer_count, int num_splits) {
+  if (num_splits != 0 || c->batch > MAX_ENTRIES) return 0;
+  const int per_launch = MAX_ENTRIES / c->batch, lc = layer_count < per_launch ? layer_count : per_launch;
+  const int cs = decode_small_cluster(make_view(c), lc, (long long)1 << 40);
+  return cs == 0 ? 0 : mma_partials_bytes(c, layer_count, num_splits) +
+                           (size_t)lc * c->batch * c->n_kv_heads * cs * DECODE_WARPS * sizeof(WarpPiece);
+}
+
 // Grid of the no-allocation form: what is accepted is fixed (the documented limit: one 12736-byte and one 12832-byte record
 // per unit and CTA resp. eighth of a CTA must fit the scratch); of the asked number of CTAs as many run as have room for
 // their warps' pieces.  0: too large.
@@ -441,7 +451,8 @@ static okq_status check_decode(const okq_cache* cache, int32_t layer, int32_t la
   if (n_R != 1 && n_R != cache->n_kv_heads) return OKQ_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(signs) || !aligned16(R) || !aligned16(workspace) || !aligned16(out))
     return OKQ_ERR_ALIGNMENT;
-  if (workspace_bytes < okq_decode_workspace_bytes(cache, layer_count, num_splits)) return OKQ_ERR_WORKSPACE;
+  const size_t simt = simt_workspace(cache, layer_count, num_splits), mma = mma_workspace(cache, layer_count, num_splits);
+  if (workspace_bytes < (simt > mma ? simt : mma)) return OKQ_ERR_WORKSPACE;
   return OKQ_OK;
 }
 
@@ -453,7 +464,7 @@ static DecodeParams make_params(const okq_cache* cache, int32_t layer, int32_t l
   P.layer0 = layer; P.layer_count = layer_count; P.n_splits = num_splits;
   P.group = cache->n_q_heads / cache->n_kv_heads;
   P.q = static_cast<const __half*>(q); P.signs = signs; P.R = R; P.n_R = n_R; P.sm_scale = sm_scale;
-  P.partials = nullptr; P.partials_f = nullptr; P.pieces = nullptr; P.out = out;
+  P.partials = nullptr; P.partials_f = nullptr; P.pieces = nullptr; P.piece_slots = 0; P.out = out;
   return P;
 }
 
@@ -476,8 +487,9 @@ int32_t okq_decode_select(int32_t impl) {
 
 size_t okq_decode_workspace_bytes(const okq_cache* cache, int32_t layer_count, int32_t num_splits) {
   if (check_cache(cache, false) != OKQ_OK || layer_count <= 0 || num_splits < 0) return 0;
-  size_t a = simt_workspace(cache, layer_count, num_splits), b = mma_workspace(cache, layer_count, num_splits);
-  return a > b ? a : b;
+  const size_t a = simt_workspace(cache, layer_count, num_splits), b = mma_workspace(cache, layer_count, num_splits);
+  const size_t c = small_workspace(cache, layer_count, num_splits), ab = a > b ? a : b;
+  return ab > c ? ab : c;
 }
 
 okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t layer_count, const void* q,
@@ -496,6 +508,7 @@ okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t l
                                  signs + (size_t)l0 * D, R + (size_t)l0 * n_R * 3 * D * D, n_R, out + l0 * q_stride, num_splits);
     P.partials_f = static_cast<PartialF*>(workspace);
     P.pieces = reinterpret_cast<WarpPiece*>(static_cast<unsigned char*>(workspace) + mma_partials_bytes(cache, lc, num_splits));
+    P.piece_slots = (long long)((workspace_bytes - mma_partials_bytes(cache, lc, num_splits)) / sizeof(WarpPiece));
     const int n_cta = mma_ctas(cache, lc, num_splits);
     st = launch_decode_mma(P, n_cta, s, g_ev_before, g_ev_after);
     if (st != OKQ_OK) return st;
@@ -528,6 +541,8 @@ okq_status okq_decode_attention_noalloc(const okq_cache* cache, int32_t layer, i
     P.partials_f = static_cast<PartialF*>(scratch);
     const int n_cta = noalloc_ctas(cache, lc, num_splits);
     P.pieces = reinterpret_cast<WarpPiece*>(P.partials_f + (size_t)lc * cache->batch * cache->n_kv_heads + n_cta);
+    P.piece_slots = (long long)(((size_t)OKQ_NOALLOC_SCRATCH_BYTES - ((size_t)lc * cache->batch * cache->n_kv_heads + n_cta) * sizeof(PartialF)) /
+                                sizeof(WarpPiece));
     st = launch_decode_mma(P, n_cta, s, nullptr, nullptr);
     if (st != OKQ_OK) return st;
   }

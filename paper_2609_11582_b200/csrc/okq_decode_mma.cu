@@ -731,7 +731,7 @@ int g_decode_impl = 1;
 
 okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, cudaEvent_t before, cudaEvent_t after) {
   if (P.n_splits == 0 && g_decode_impl == 1) {   // the library's own choice of the grid
-    const int cs = decode_small_cluster(P.cv, P.layer_count, n_cta);
+    const int cs = decode_small_cluster(P.cv, P.layer_count, P.piece_slots);
     if (cs > 0) {
       if (before) cudaEventRecord(before, s);
       const okq_status st = launch_decode_small(P, cs, s);

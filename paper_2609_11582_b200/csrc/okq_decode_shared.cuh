@@ -47,7 +47,8 @@ struct DecodeParams {
   float sm_scale;
   Partial* partials;   // CUDA-core path: [layer_count*batch*n_kv_heads][n_splits]
   PartialF* partials_f;  // tensor-core path: [n_units + n_cta]
-  WarpPiece* pieces;     // tensor-core path: [n_units + DECODE_WARPS * n_cta]
+  WarpPiece* pieces;     // tensor-core path: [n_units + DECODE_WARPS * n_cta] at least
+  long long piece_slots; // how many there is room for
   float* out;          // [layer_count][batch][n_q_heads][128]
 };
 
@@ -83,7 +84,7 @@ okq_status launch_decode_tc(const DecodeParams& P, int n_cta, cudaStream_t s);
 extern int g_decode_impl;
 
 // one-launch form for few (sequence, head) units: cluster size it would use for a call (0: the split-K pair), launch
-int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta);
+int decode_small_cluster(const CacheView& cv, int layer_count, long long piece_slots);
 okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s);
 
 // launches the tensor-core split kernel (bracketed by the optional events) and its combine kernel

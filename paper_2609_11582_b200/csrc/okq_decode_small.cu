@@ -415,13 +415,12 @@ static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s
 // layers, 1 to 16 sequences, 1 to 8 heads and 200 to 131072 tokens; the host knows the capacity, not the lengths, and takes
 // sequences to be full: a cache mostly empty goes the way it would go full.
 template <int FMT>
-static int small_cluster(long long units, long long windows, int n_cta) {
+static int small_cluster(long long units, long long windows, long long piece_slots) {
   const int fit[5] = {small_clusters<FMT, 1>(), small_clusters<FMT, 2>(), small_clusters<FMT, 4>(), small_clusters<FMT, 8>(), small_clusters<FMT, 16>()};
   int best = 0;
   double best_cost = 31.0 + 2.0 * (double)units * (double)windows / (148.0 * NWARP) + 0.04 * (double)units;
   for (int i = 4; i >= 0; i--) {   // (of equals the largest cluster)
-    // the warps' pieces have to fit the scratch, which is laid out for `units` and NWARP per CTA of the split-K kernel
-    if (fit[i] <= 0 || (units << i) * NWARP > units + (long long)NWARP * n_cta) continue;
+    if (fit[i] <= 0 || (units << i) * NWARP > piece_slots) continue;   // the warps' pieces have to fit the scratch
     const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * (1 << i) - 1) / (NWARP * (1 << i)));
     const double cost = waves * (11.5 + 2.1 * walk);
     if (cost < best_cost) { best_cost = cost; best = 1 << i; }
@@ -429,9 +428,9 @@ static int small_cluster(long long units, long long windows, int n_cta) {
   return best;
 }
 
-int decode_small_cluster(const CacheView& cv, int layer_count, int n_cta) {
+int decode_small_cluster(const CacheView& cv, int layer_count, long long piece_slots) {
   const long long units = (long long)layer_count * cv.batch * cv.n_kv_heads, windows = cv.capacity / W;
-  return cv.fmt == FMT_MXFP4 ? small_cluster<FMT_MXFP4>(units, windows, n_cta) : small_cluster<FMT_FP16>(units, windows, n_cta);
+  return cv.fmt == FMT_MXFP4 ? small_cluster<FMT_MXFP4>(units, windows, piece_slots) : small_cluster<FMT_FP16>(units, windows, piece_slots);
 }
 
 template <int CS>
