@@ -46,7 +46,7 @@ __device__ __forceinline__ float ex2f(float x) {
 // running maximum and sum of its own columns per lane; the four lanes of a row meet once at the end.  Keys pass through
 // two cp.async buffers.  What bounds it: the products' dispatch (8.6 cycles of a sub-partition each) and one exponential
 // per score.  8192 tokens x 7 heads, both passes: 1.29 ms with 16 rows per warp, unbuffered tiles, scalar fragment loads and
-// expf of every score with a shuffle reduction per tile; see below for this form.
+// expf of every score with a shuffle reduction per tile, 0.57 ms in this form.
 // Block order: longest first, every other wave of blocks reversed, so that an SM's blocks add up to about the same.
 template <int PASS>
 __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict__ q, const __half* __restrict__ k, int G, int n,
