@@ -194,8 +194,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_mma(DecodeParams P) {
         v.x = fmaf(x[q].x, f.x, v.x); v.y = fmaf(x[q].y, f.y, v.y); v.z = fmaf(x[q].z, f.x, v.z); v.w = fmaf(x[q].w, f.y, v.w);
       }
       // in units of the bit-plane form, whose weight sums are zero here
-      constexpr float F = LEVEL_UNIT * 16.0f / PARTIAL_ACC_SCALE;
-      static_assert(P_LOG2 == -4.0f, "the factor 16 above is 2^-P_LOG2");
+      constexpr float F = LEVEL_UNIT / PARTIAL_ACC_SCALE;
       PartialF* out = P.partials_f + (size_t)(ub + su) + blockIdx.x;
       out->frag[m][4 * rg][L] = v.x * F; out->frag[m][4 * rg + 1][L] = v.y * F;
       out->frag[m][4 * rg + 2][L] = v.z * F; out->frag[m][4 * rg + 3][L] = v.w * F;

@@ -32,7 +32,7 @@ constexpr float PARTIAL_ACC_SCALE = (CB_OUTER - CB_INNER) * 262144.0f;  // (b - 
 constexpr int DECODE_WARPS = 12;    // warps per CTA
 struct WarpPiece {
   float4 frag[3][8][32];   // [modality][m-tile][lane]: the tile's four accumulator registers
-  float wm[GP], wl[GP];    // reference maximum (log2 domain) of everything in the piece, sum of exp2(score - maximum)
+  float wm[GP], wl[GP];    // reference (log2 domain) of everything in the piece, sum of exp2(score - reference)
   int mask;                // modalities the piece holds (bit m); the other modalities' sums are not written
   int pad[3];
 };

@@ -313,8 +313,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
           }
       }
       if (SHARES == 1 || tid < ITEMS) {
-        constexpr float F = LEVEL_UNIT * 16.0f;   // numerators carry 2^P_LOG2 = 1/16
-        static_assert(P_LOG2 == -4.0f, "");
+        constexpr float F = LEVEL_UNIT;
         const int ch = 16 * mu + (L32 >> 2);
         for (int r = 0; r < CS; r++) {   // to every CTA of the cluster
           float* dst = CS == 1 ? &af.vec[0][0] : cluster.map_shared_rank(&af.vec[0][0], r);

@@ -16,10 +16,20 @@ constexpr int PREFETCH = 3;                     // windows copied ahead of the o
 constexpr int NSLOT = PREFETCH + 1;             // record ring per warp
 constexpr int BATCH = 8;                        // windows whose bias sums come out of one set of products
 constexpr int M_PITCH = 256 + 16;               // bytes between the m planes of a batch: eight rows over all banks
-// Numerators are 2^(P_LOG2 + score - reference maximum) * vnorm in fp16: they start at 2^-4 when the reference maximum
-// moves and may grow to 2^7 before it has to move again
-constexpr float RESCALE_LOG2 = 11.0f, P_LOG2 = -4.0f;
-constexpr float REBASE_LOG2 = 60.0f;            // range of a piece's numbers above its own reference maximum
+// Numerators are p * vnorm in fp16, p = 2^(score - reference).  The reference is chosen by the numerators themselves and not by
+// the scores: when it moves, the largest numerator of the window gets a p that is a power of two (so it is exact) and lies in
+// [2^TOP_LOG2, 2^(TOP_LOG2 + 1)); it moves again when one exceeds NUM_MAX.  That leaves 25 binary digits below the largest one
+// whatever the values' scale is, and whatever mass a token with a small value takes.  Error against 64 bits, 16384 tokens, first
+// token 20 bits above the others with a zero value, values of norm 0.004: 2.4e-2 with the reference at the largest score and 2^-4
+// there, 1.4e-4 now; generator's inputs, 8192 tokens, MXFP4: 1.6e-4 and 0.6e-4.  A limit 16 to 32 times the top instead of 8 to
+// 16 measured 0.5 % less time and 1.3 times the error.  step7b 508 -> 517 us.
+constexpr int TOP_LOG2 = 11;
+constexpr float NUM_MAX = 32768.0f;
+// p itself only enters the fp32 weight sum: a token with next to no value may have a large one, up to 2^P_LOG2_MAX when the
+// reference moves; a window whose sum exceeds SUM_MAX moves it.  (Where no token of a window has a value, that is where the
+// reference goes: the next value brings it to where it belongs.)
+constexpr float P_LOG2_MAX = 60.0f, SUM_MAX = 0x1p80f;
+constexpr float REBASE_LOG2 = 30.0f;            // range of a piece's numbers above its own reference
 constexpr int FLUSH = 32;                       // windows a warp accumulates in registers at most
 constexpr int SWITCH_AFTER = 3;                 // pure windows of another modality in a row before the registers change over
 
@@ -34,7 +44,7 @@ template <int FMT> struct WarpSmem {
   __align__(16) unsigned char slot[NSLOT][Slot<FMT>::BYTES];
   __align__(16) float bias[BATCH][GP];         // bias sums of a batch of windows
   __align__(16) unsigned char mod[2][BATCH * W];   // modality bytes of two batches: in use, on its way
-  float rebase[2][32];                         // per lane, rarely used: 1 / fsc, reference maximum of the piece
+  float rebase[32];                            // per lane, rarely used: reference of the piece
   // m planes of a batch of windows: as copied (fp16 metadata) or as decoded (MXFP4)
   __align__(16) unsigned char m[BATCH * M_PITCH];
   __align__(16) unsigned char s[FMT == FMT_FP16 ? 16 : BATCH * 256];                      // MXFP4: decoded s planes of the batch
@@ -142,7 +152,7 @@ __device__ __forceinline__ void window_scores_mma(const unsigned char* st, const
 
 // what a warp ends a range with, besides the piece's sums: lane (g, t) of head g
 struct WalkEnd {
-  float m, l;      // reference maximum of everything in the piece (log2 domain), sum of exp2(score - maximum)
+  float m, l;      // reference of everything in the piece (log2 domain), sum of exp2(score - reference)
   unsigned held;   // modalities the piece holds something of (bit per modality)
 };
 
@@ -203,7 +213,6 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
   uint32_t qh[16];
   float fsc;
   queries(qh, fsc);
-  ws.rebase[0][lane] = 1.0f / fsc;
   const F2 fsc2 = f2(fsc, fsc);
 
   float acc[8][4];
@@ -212,15 +221,15 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
 #pragma unroll
     for (int i = 0; i < 4; i++) acc[mu][i] = 0.f;
   F2 run_l = f2(0.f, 0.f);
-  float run_m = -INFINITY, thr = -INFINITY;   // thr: the largest score / fsc the reference maximum run_m allows
-  F2 noff = f2(0.f, 0.f);                     // P_LOG2 - run_m
+  F2 noff = f2(INFINITY, INFINITY);           // minus the reference: the first window exceeds every limit
+  auto run_m = [&]() { return -un2(noff).x; };
   int cur_mod = -1, since = 0, streak = 0;
   unsigned held = 0;                          // modalities the piece already holds something of
 
   auto piece_row = [&](int m) { return &sg.piece->frag[m][0][lane]; };
-  // adds four-register rows to the piece (the first ones of a modality are stored), brought to its reference maximum
+  // adds four-register rows to the piece (the first ones of a modality are stored), brought to its reference
   auto put = [&](int m, const float (*o)[4], int mu0, int n) {
-    const float f = ex2(run_m - ws.rebase[1][lane]);
+    const float f = ex2(run_m() - ws.rebase[lane]);
     const float f_lo = __shfl_sync(0xffffffffu, f, 8 * t), f_hi = __shfl_sync(0xffffffffu, f, 8 * t + 4);
     float4* dst = piece_row(m) + 32 * mu0;
 #pragma unroll
@@ -315,6 +324,90 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
     a[2] = prmt(x1, LEVEL_LO, 0x1404u); a[3] = prmt(x1, LEVEL_LO, 0x3424u);
   };
 
+  // ---- online softmax (log2 domain): scores of the window staged at `st` from its products, then its numerators in fp16
+  // (operand pairs of tokens nu and nu + 2, parity e, for the value product) and the sum of their p; true if this lane's
+  // exceed what the reference allows
+  auto scores = [&](const unsigned char* st, float bias, F2 (&sc)[4]) {
+    const uint4 kn4 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_KNORM + 16 * t);
+    const uint32_t knu[4] = {kn4.x, kn4.y, kn4.z, kn4.w};
+    const F2 bb = f2(bias, bias);
+#pragma unroll
+    for (int nu = 0; nu < 4; nu++)
+      sc[nu] = mul2(add2(add2(f2(d[nu][0], d[nu][1]), f2(d[nu][2], d[nu][3])), bb), half2_to_f2(knu[nu]));
+  };
+  auto numerators = [&](const unsigned char* st, const F2 (&sc)[4], uint32_t (&pb)[2][2], F2& ps) {
+    const uint4 vn4 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_VNORM + 16 * t);
+    const uint32_t vnu[4] = {vn4.x, vn4.y, vn4.z, vn4.w};
+    float2 pn[4];
+    float mx = 0.f;
+#pragma unroll
+    for (int nu = 0; nu < 4; nu++) {
+      const float2 x = un2(fma2(sc[nu], fsc2, noff));
+      const F2 p = f2(ex2(x.x), ex2(x.y));
+      ps = nu == 0 ? p : add2(ps, p);
+      pn[nu] = un2(mul2(p, half2_to_f2(vnu[nu])));
+      mx = fmaxf(mx, fmaxf(pn[nu].x, pn[nu].y));
+    }
+#pragma unroll
+    for (int jp = 0; jp < 2; jp++) {
+      pb[jp][0] = pack_sat(pn[jp].x, pn[jp + 2].x);
+      pb[jp][1] = pack_sat(pn[jp].y, pn[jp + 2].y);
+    }
+    const float2 s2 = un2(ps);
+    return mx > NUM_MAX || s2.x > SUM_MAX || s2.y > SUM_MAX;
+  };
+  // The reference moves for every head, to where the window's largest numerator has its place.  That one is found by
+  // score + log2(vnorm), the logarithm taken as the straight line between powers of two: biased exponent and mantissa, read as
+  // one number (a zero norm counts as 2^-127).
+  auto move = [&](const unsigned char* st, const F2 (&sc)[4], bool first) {
+    const uint4 vn4 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_VNORM + 16 * t);
+    const uint32_t vnu[4] = {vn4.x, vn4.y, vn4.z, vn4.w};
+    float top = -INFINITY, top_u = 0.f, hi = -INFINITY;
+    uint32_t top_v = 0;
+#pragma unroll
+    for (int nu = 0; nu < 4; nu++) {
+      const float2 s = un2(mul2(sc[nu], fsc2)), v = un2(half2_to_f2(vnu[nu]));
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        const float u = e ? s.y : s.x;
+        const uint32_t vb = __float_as_uint(e ? v.y : v.x);
+        const float lg = fmaf(__uint_as_float(0x4B000000u | (vb >> 9)), 0x1p-14f, u - 639.0f);   // 2^23 + 2^14 (exponent + mantissa)
+        hi = fmaxf(hi, u);
+        if (lg > top) { top = lg; top_u = u; top_v = vb; }
+      }
+    }
+    float ref = top_u + (float)((int)(top_v >> 23) - 127 - TOP_LOG2);
+#pragma unroll
+    for (int dl = 1; dl < 4; dl <<= 1) {   // over the head's four lanes, of equals the higher reference
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, dl));
+      const float ot = __shfl_xor_sync(0xffffffffu, top, dl), oref = __shfl_xor_sync(0xffffffffu, ref, dl);
+      if (ot > top || (ot == top && oref > ref)) { top = ot; ref = oref; }
+    }
+    const float m_new = fmaxf(fmaxf(ref, hi - P_LOG2_MAX), run_m());
+    if (first) ws.rebase[lane] = m_new;
+    const float alpha = ex2(run_m() - m_new);     // 0 on the first window
+    noff = f2(-m_new, -m_new);
+    run_l = mul2(run_l, f2(alpha, alpha));
+    const float a_lo = __shfl_sync(0xffffffffu, alpha, 8 * t), a_hi = __shfl_sync(0xffffffffu, alpha, 8 * t + 4);
+#pragma unroll
+    for (int mu = 0; mu < 8; mu++) { acc[mu][0] *= a_lo; acc[mu][1] *= a_hi; acc[mu][2] *= a_lo; acc[mu][3] *= a_hi; }
+    const float piece_m = ws.rebase[lane];
+    if (__any_sync(0xffffffffu, m_new - piece_m > REBASE_LOG2)) {   // the piece follows before its numbers could overflow
+      const float f = ex2(piece_m - m_new);
+      const float f_lo = __shfl_sync(0xffffffffu, f, 8 * t), f_hi = __shfl_sync(0xffffffffu, f, 8 * t + 4);
+      ws.rebase[lane] = m_new;
+#pragma unroll 1
+      for (int m = 0; m < 3; m++)
+        if ((held >> m) & 1u)
+#pragma unroll 1
+          for (int mu = 0; mu < 8; mu++) {
+            float4* p = piece_row(m) + 32 * mu;
+            const float4 v = __ldcg(p);
+            __stcg(p, make_float4(v.x * f_lo, v.y * f_hi, v.z * f_lo, v.w * f_hi));
+          }
+    }
+  };
+
   const unsigned char* st = slots;                     // slot of window k
   const unsigned char* stn = slots;                    // slot of window k + 1
   auto s_plane = [&](int k) {
@@ -328,67 +421,15 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
 
   for (int k = k_first; k < k_end; k++) {
     st = stn;
-    // ---- online softmax (log2 domain) of window k.  The reference maximum moves only when a score exceeds it by more
-    // than 2^RESCALE_LOG2, so nothing but this lane's own maximum is looked at in the common case.
-    F2 sc[4];
-    {
-      const uint4 kn4 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_KNORM + 16 * t);
-      const uint32_t knu[4] = {kn4.x, kn4.y, kn4.z, kn4.w};
-      const F2 bb = f2(bias, bias);
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++)
-        sc[nu] = mul2(add2(add2(f2(d[nu][0], d[nu][1]), f2(d[nu][2], d[nu][3])), bb), half2_to_f2(knu[nu]));
-    }
-    float mx = -INFINITY;
-#pragma unroll
-    for (int nu = 0; nu < 4; nu++) { const float2 v = un2(sc[nu]); mx = fmaxf(mx, fmaxf(v.x, v.y)); }
-    if (__any_sync(0xffffffffu, mx > thr)) {
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      if (k == k_first) ws.rebase[1][lane] = mx * fsc;
-      const float m_new = fmaxf(mx * fsc, run_m);   // every head moves to its maximum so far
-      const float alpha = ex2(run_m - m_new);       // 0 on the first window
-      run_m = m_new;
-      thr = (run_m + RESCALE_LOG2) * ws.rebase[0][lane];
-      noff = f2(P_LOG2 - run_m, P_LOG2 - run_m);
-      run_l = mul2(run_l, f2(alpha, alpha));
-      const float a_lo = __shfl_sync(0xffffffffu, alpha, 8 * t), a_hi = __shfl_sync(0xffffffffu, alpha, 8 * t + 4);
-#pragma unroll
-      for (int mu = 0; mu < 8; mu++) { acc[mu][0] *= a_lo; acc[mu][1] *= a_hi; acc[mu][2] *= a_lo; acc[mu][3] *= a_hi; }
-      const float piece_m = ws.rebase[1][lane];
-      if (__any_sync(0xffffffffu, run_m - piece_m > REBASE_LOG2)) {   // the piece follows before its numbers could overflow
-        const float f = ex2(piece_m - run_m);
-        const float f_lo = __shfl_sync(0xffffffffu, f, 8 * t), f_hi = __shfl_sync(0xffffffffu, f, 8 * t + 4);
-        ws.rebase[1][lane] = run_m;
-#pragma unroll 1
-        for (int m = 0; m < 3; m++)
-          if ((held >> m) & 1u)
-#pragma unroll 1
-            for (int mu = 0; mu < 8; mu++) {
-              float4* p = piece_row(m) + 32 * mu;
-              const float4 v = __ldcg(p);
-              __stcg(p, make_float4(v.x * f_lo, v.y * f_hi, v.z * f_lo, v.w * f_hi));
-            }
-      }
-    }
-    // numerators times value norms, fp16: operand pairs (tokens nu and nu + 2, parity e) for the value product
+    // (the numerators' check is part of the test for the common case below)
     uint32_t pb[2][2];
+    F2 ps;
+    const float bias_k = bias;
+    bool over;
     {
-      const uint4 vn4 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_VNORM + 16 * t);
-      const uint32_t vnu[4] = {vn4.x, vn4.y, vn4.z, vn4.w};
-      float2 pn[4];
-#pragma unroll
-      for (int nu = 0; nu < 4; nu++) {
-        const float2 x = un2(fma2(sc[nu], fsc2, noff));
-        const F2 p = f2(ex2(x.x), ex2(x.y));
-        run_l = add2(run_l, p);
-        pn[nu] = un2(mul2(p, half2_to_f2(vnu[nu])));
-      }
-#pragma unroll
-      for (int jp = 0; jp < 2; jp++) {
-        pb[jp][0] = pack_sat(pn[jp].x, pn[jp + 2].x);
-        pb[jp][1] = pack_sat(pn[jp].y, pn[jp + 2].y);
-      }
+      F2 sc[4];
+      scores(st, bias_k, sc);
+      over = numerators(st, sc, pb, ps);
     }
     const int mymod = ws.mod[(k / BATCH) & 1][(k & (BATCH - 1)) * W + lane];
     const uint4 vc0 = *reinterpret_cast<const uint4*>(st + SL::BODY + B_VCODE + 16 * vpiece_slot(lane));
@@ -402,7 +443,17 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
     score_load(stn);
     const unsigned char* sp = s_plane(k + 1);
 
-    unsigned mine = __ballot_sync(0xffffffffu, mymod == cur_mod);
+    unsigned mine = __ballot_sync(0xffffffffu, mymod == cur_mod && !over);
+    if (mine != 0xffffffffu) {
+      if (__any_sync(0xffffffffu, over)) {   // the reference moves and the numerators are taken again
+        F2 sc[4];
+        scores(st, bias_k, sc);
+        move(st, sc, k == k_first);
+        numerators(st, sc, pb, ps);
+        mine = __ballot_sync(0xffffffffu, mymod == cur_mod);
+      }
+    }
+    run_l = add2(run_l, ps);
     if (mine != 0xffffffffu) {
       const int first = __shfl_sync(0xffffffffu, mymod, 0);
       const bool pure = __all_sync(0xffffffffu, mymod == first);
@@ -468,8 +519,8 @@ __device__ __forceinline__ WalkEnd walk_segment(WarpSmem<FMT>& ws, const uint4 (
   cp_async_wait<0>();
   if (since > 0) deposit();
   const float2 l2 = un2(run_l);
-  const float piece_m = ws.rebase[1][lane];
-  float l = (l2.x + l2.y) * ex2(run_m - piece_m - P_LOG2);
+  const float piece_m = ws.rebase[lane];
+  float l = (l2.x + l2.y) * ex2(run_m() - piece_m);
   l += __shfl_xor_sync(0xffffffffu, l, 1);
   l += __shfl_xor_sync(0xffffffffu, l, 2);
   return WalkEnd{piece_m, l, held};

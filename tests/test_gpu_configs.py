@@ -247,3 +247,45 @@ def test_layer_offset_and_many_sequences():
     for i, l in enumerate((1, 2)):
         ref, _ = c.oracle_attention(l)
         Hn.assert_attention_close(got[i], ref)
+
+
+# (share of the first token's score above the others', in bits; scale of its value; scale of all values; softmax scale)
+@pytest.mark.parametrize("sink_bits,sink_value,value_scale,sm_scale", [
+    (None, 1.0, 2.0 ** -15, None), (None, 1.0, 2048.0, None), (None, 1.0, 1.0, -D ** -0.5),
+    (14, 0.05, 1.0, None), (14, 0.003, 1 / 256, None), (20, 0.0, 0.1, None), (30, 0.3, 3.0, None), (45, 0.0, 1.0, None)])
+@pytest.mark.parametrize("meta_format", [B.META_FP16, B.META_MXFP4])
+def test_numerators_keep_their_digits(sink_bits, sink_value, value_scale, sm_scale, meta_format):
+    """The fp16 numerators p * |v| of the decode kernels have full precision whatever the values' scale is and however much of
+    the mass a token with a small or zero value takes (the first tokens of real models), in the one-launch and the split-K
+    kernel.  One block of the latter gives a warp ranges of 16384 / 12 tokens; the bound is the rounding of the numerators."""
+    n, G = 16384, 7
+    g = torch.Generator().manual_seed(11)
+    w = WL.scaled(WL.WORKLOADS["tiny"], n_tokens=n)
+    q = torch.randn(1, 1, G, D, generator=g)
+    k = torch.randn(1, 1, n, D, generator=g)
+    v = torch.randn(1, 1, n, D, generator=g)
+    if sink_bits is None:
+        q *= 3          # scores with a deviation of 4 bits: a few tokens count
+    else:
+        base = torch.randn(D, generator=g)
+        q += base
+        k[0, 0, 0] = base * sink_bits / (1.4427 * D ** -0.5 * base.square().sum())
+        v[0, 0, 0] *= sink_value
+    v *= value_scale
+    signs, R = WL.gen_signs(w, 0).cuda(), WL.gen_rotations(w, 0)[None].contiguous().cuda()
+    mod = WL.modality_layout(w, n)[None].contiguous().cuda()
+    cache = B.Cache(1, 1, 1, G, n, meta_format=meta_format)
+    B.quantize_keys(cache, 0, k.half().cuda(), signs)
+    B.quantize_values(cache, 0, v.half().cuda(), mod, R)
+    q = q.half().cuda()
+
+    def decode(splits, simt=False):
+        ws = torch.empty(B.decode_workspace_bytes(cache, 1, splits), dtype=torch.uint8, device="cuda")
+        out = torch.full((1, 1, G, D), float("nan"), device="cuda")
+        B.decode_attention(cache, 0, 1, q, signs, R, ws, out, sm_scale=sm_scale, num_splits=splits, simt=simt)
+        return out[0].cpu().numpy().astype(np.float64)
+
+    ref = decode(4, simt=True)   # fp32 throughout
+    for splits in (0, 1):
+        rel, worst, _ = Hn.attention_errors(decode(splits), ref)
+        assert rel < Hn.REL_L2_TOL and worst < Hn.REL_L2_TOL, (splits, rel, worst)
