@@ -218,3 +218,14 @@ def test_error_table_from_the_gpu_caches():
     for i in range(3):
         assert rows["OmniKVQuant K2V2"][i] < rows["TurboQuant K2/V2"][i]
     assert rows["OmniKVQuant K2V2"][0] < rows["TurboQuant K3/V2"][0] < rows["TurboQuant K2/V2"][0]
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("n", [640, 8192])
+def test_decode_is_as_exact_as_fp32(bits, n):
+    """Scores with deviations of 4 bits (four channels of ten times the size).  The products keep 2^-23 of each of 128 weights:
+    as independent errors in scores of up to 2^4, 2^4 * 2^-23 / sqrt(3) * ln 2 = 0.8e-6 of a numerator; twice that over a tensor,
+    ten times that for the worst of its vectors."""
+    c = LadderCase(WL.scaled(WL.WORKLOADS["layer7b"], batch=1), bits, n)
+    rel, worst, _ = Hn.attention_errors(c.gpu_attention(), c.oracle_attention())
+    assert rel < 1.6e-6 and worst < 8e-6, (rel, worst)
