@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(NT_L, 1) k_ladder_decode(LadderView cv, int n_
     for (int d = 1; d < 32; d <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
     int ex = 0;
     if (mx > 0.f) frexpf(mx, &ex);          // mx < 2^ex
-    const int kh = 14 - ex;                 // |q'| * 2^kh < 2^14
+    const int kh = 13 - ex;                 // |q'| * 2^kh < 2^13; times the largest step (2 sqrt(128) / 3) still an fp16 number
     const float up = exp2f((float)kh);
     *reinterpret_cast<float4*>(&sm.q[warp][4 * lane]) = make_float4(x.x * up, x.y * up, x.z * up, x.w * up);
     if (lane == 0) sm.fsc[warp] = exp2f((float)-kh) * sm_scale * 1.4426950408889634f;

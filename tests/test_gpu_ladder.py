@@ -229,3 +229,20 @@ def test_decode_is_as_exact_as_fp32(bits, n):
     c = LadderCase(WL.scaled(WL.WORKLOADS["layer7b"], batch=1), bits, n)
     rel, worst, _ = Hn.attention_errors(c.gpu_attention(), c.oracle_attention())
     assert rel < 1.6e-6 and worst < 8e-6, (rel, worst)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_decode_with_the_largest_steps(bits):
+    """Keys whose norm exceeds fp16 and that lie along one rotated coordinate, in both directions: z = +-sqrt(128) there, the
+    largest step there is, against queries that are largest in that coordinate.  (Scores are a few units: the keys are large,
+    the queries small.)"""
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=1)
+    signs = WL.gen_signs(w, 0)
+    k, v = WL.gen_kv(w, 0, n_tokens=64)
+    k[:, :, 0], k[:, :, 1] = (65504 * signs).half(), (-65504 * signs).half()   # row 0 of the Hadamard matrix is all ones
+    c = LadderCase(w, bits, 64, k=k, v=v)
+    g = torch.Generator().manual_seed(1)
+    c.q = (3e-6 * torch.randn(1, w.n_q_heads, D, generator=g) + 6e-6 * signs).half()
+    got, ref = c.gpu_attention(), c.oracle_attention()
+    rel, worst, _ = Hn.attention_errors(got, ref)
+    assert np.isfinite(got).all() and rel < 1e-5 and worst < 1e-4, (rel, worst)
