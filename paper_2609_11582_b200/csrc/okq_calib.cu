@@ -40,8 +40,10 @@ __device__ __forceinline__ float ex2f(float x) {
 }
 
 // One pass over the key tiles of a 128-query block of one head; scores in the log2 domain, s = (q . k) * scale2.
-//   PASS 0: rowstat[g * n + i] = -2 (m_i + log2 l_i), m_i = max_j s_ij, l_i = sum_j 2^(s_ij - m_i)
-//   PASS 1: column sums of alpha^2 = 2^(2 s + rowstat) over the block's queries -> partial[(itile * G + g) * n + j]
+//   PASS 0: rowstat[g * n + i] = (-2 m_i, 1 / l_i^2), m_i = max_j s_ij, l_i = sum_j 2^(s_ij - m_i)
+//   PASS 1: column sums of alpha^2 = 2^(2 s - 2 m_i) / l_i^2 over the block's queries -> partial[(itile * G + g) * n + j]
+// (The exponent is one fused multiply-add with a number that is exact: with m_i + log2 l_i in one number its rounding, 2^-24 of
+// it, was an error of every weight of the row, 3e-6 at scores of 2^5.)
 // A warp owns 32 query rows (its fragments stay in registers, so each key fragment serves two products) and keeps the
 // running maximum and sum of its own columns per lane; the four lanes of a row meet once at the end.  Keys pass through
 // two cp.async buffers.  What bounds it: the products' dispatch (8.6 cycles of a sub-partition each) and one exponential
@@ -50,7 +52,7 @@ __device__ __forceinline__ float ex2f(float x) {
 // Block order: longest first, every other wave of blocks reversed, so that an SM's blocks add up to about the same.
 template <int PASS>
 __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict__ q, const __half* __restrict__ k, int G, int n,
-                                                      float scale2, int causal, int n_sm, float* __restrict__ rowstat,
+                                                      float scale2, int causal, int n_sm, float2* __restrict__ rowstat,
                                                       float* __restrict__ partial) {
   __shared__ __align__(16) __half ks[2][TK * KS_STRIDE];
   __shared__ float colsum[4][TK];
@@ -81,13 +83,14 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
         qa[mt][s][e] = i < n && !no_q ? *reinterpret_cast<const uint32_t*>(qh + (size_t)i * D + c) ^ flip : 0u;
       }
   }
-  float m[2][2], l[2][2];   // PASS 0: running maximum and sum; PASS 1: l = rowstat
+  float m[2][2], l[2][2];   // PASS 0: running maximum and sum; PASS 1: rowstat
 #pragma unroll
   for (int mt = 0; mt < 2; mt++)
 #pragma unroll
     for (int hf = 0; hf < 2; hf++) {
-      m[mt][hf] = -INFINITY;
-      l[mt][hf] = PASS == 0 ? 0.f : (row[mt][hf] < n ? rowstat[(size_t)head * n + row[mt][hf]] : -INFINITY);
+      const float2 st = PASS == 1 && row[mt][hf] < n ? rowstat[(size_t)head * n + row[mt][hf]] : make_float2(-INFINITY, 0.f);
+      m[mt][hf] = st.x;
+      l[mt][hf] = st.y;
     }
   const int n_jt = causal ? min((n + TK - 1) / TK, (itile * TQ + TQ - 1) / TK + 1) : (n + TK - 1) / TK;
   auto fetch = [&](int jt) {
@@ -165,8 +168,8 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
         for (int nt = 0; nt < 4; nt++)
 #pragma unroll
           for (int e = 0; e < 2; e++)
-            c[2 * nt + e] = (ex2f(fmaf(d[0][nt][e], two, l[0][0])) + ex2f(fmaf(d[0][nt][2 + e], two, l[0][1]))) +
-                            (ex2f(fmaf(d[1][nt][e], two, l[1][0])) + ex2f(fmaf(d[1][nt][2 + e], two, l[1][1])));
+            c[2 * nt + e] = fmaf(ex2f(fmaf(d[0][nt][e], two, m[0][0])), l[0][0], ex2f(fmaf(d[0][nt][2 + e], two, m[0][1])) * l[0][1]) +
+                            fmaf(ex2f(fmaf(d[1][nt][e], two, m[1][0])), l[1][0], ex2f(fmaf(d[1][nt][2 + e], two, m[1][1])) * l[1][1]);
         // over the eight row groups, each lane ending with one column: n-tile bits 1, 0 and e by lane bits 4, 3, 2
 #pragma unroll
         for (int w = 4, bit = 16; w >= 1; w >>= 1, bit >>= 1) {
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
           ll = (mm == -INFINITY ? 0.f : ll * ex2f(mm - mn)) + (mo == -INFINITY ? 0.f : lo * ex2f(mo - mn));
           mm = mn;
         }
-        if (t == 0 && row[mt][hf] < n) rowstat[(size_t)head * n + row[mt][hf]] = -2.0f * (mm + log2f(ll));
+        if (t == 0 && row[mt][hf] < n) rowstat[(size_t)head * n + row[mt][hf]] = make_float2(-2.0f * mm, 1.0f / (ll * ll));
       }
   }
 }
@@ -764,8 +767,8 @@ okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, i
   if (!aligned16(q_fp16) || !aligned16(k_fp16) || !aligned16(workspace) || !aligned16(w_out)) return OKQ_ERR_ALIGNMENT;
   if (workspace_bytes < attn_bytes(group, n)) return OKQ_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  float* rowstat = static_cast<float*>(workspace);
-  float* partial = rowstat + (size_t)group * n * 2;
+  float2* rowstat = static_cast<float2*>(workspace);
+  float* partial = reinterpret_cast<float*>(rowstat + (size_t)group * n);
   const int grid = (n + TQ - 1) / TQ * group, n_sm = sm_count();
   const __half* q = static_cast<const __half*>(q_fp16);
   const __half* k = static_cast<const __half*>(k_fp16);

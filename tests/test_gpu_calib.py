@@ -108,3 +108,13 @@ def test_end_to_end_calibration_reduces_error():
         e_cal, e_had = mse(vb, R.cpu().numpy()), mse(vb, H)
         print(f"modality {m}: calibrated {e_cal:.4f}  hadamard {e_had:.4f}")
         assert e_cal < e_had
+
+
+def test_attention_weights_of_large_scores():
+    """Scores of several hundred (log2): nearly every query attends to one key, whose weight is 2^0 / l^2 with l close to 1.  What
+    is left is the rounding of sums over some hundred queries: 2^-20 of the weights' norm."""
+    q, k, v, mod, signs = _case(1000)
+    q = (40 * q.float()).half()
+    w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(q.shape[0], 1000)).cpu().numpy().astype(np.float64)
+    ref = CO.attention_weights(q.numpy().view(np.uint16), k.numpy().view(np.uint16), causal=True)
+    assert np.linalg.norm(w - ref) <= 2.0 ** -20 * np.linalg.norm(ref), np.linalg.norm(w - ref) / np.linalg.norm(ref)
