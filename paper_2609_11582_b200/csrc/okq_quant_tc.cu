@@ -27,6 +27,8 @@
 // coordinates in the band (about 1e-4 of them) are listed and recomputed at the end of the kernel, one per warp at
 // a time, with the exact fused-multiply-add chain of the reference arithmetic over the value row, read again from
 // global memory; the code in the record is then patched.  Codes and norms (exact summation tree) are therefore bit-identical to the exact path.
+// The band is good for rotations.  If a matrix row is longer than 2 (the errors grow with it, and entries may not even fit fp16)
+// or a value longer than fp16 can say, the block takes all its coordinates through the exact chain at the end.
 //
 // The same kernel writes the value codes of the bit-width ladder (BITS = 2, 3 or 4: token-major bit streams): a table of 32
 // bins over the coordinate, each with at most one threshold of the codebook, gives (threshold, code below it) in one
@@ -58,6 +60,8 @@ constexpr float TWO_THIRDS = 2.0f / 3.0f;          // rounds up: a zero coordina
 // threshold and is recomputed with the exact fused-multiply-add chain of the reference arithmetic.
 constexpr float BAND = 0x1p-18f;
 constexpr float BAND_V = BAND / (3.0f * CB_THRESH);
+constexpr float NORM_MAX = 65504.0f;               // of a stored norm; the value itself may be sqrt(128) times as long
+constexpr float ROW_SQ_MAX = 4.0f;                 // squared length of the matrix rows that BAND is good for
 constexpr float FLOOR_MAGIC = 12582912.0f;         // 1.5 * 2^23: unit in the last place 1, bits 0x4B400000
 // sum over the eight fields (bit 16*e + 2*j) of a word of the magic bits shifted to the field, modulo 2^32
 constexpr uint32_t magic_sum() {
@@ -109,6 +113,7 @@ template <int BITS> struct TcSmem {
   uint32_t tmem_slot;
   FixItem fix[FIX_MAX];
   int fix_count;
+  int redo;                                            // BAND was not good for one of the block's matrices or values
   long long limit;                                     // SM clocks a wait may take
   volatile int abort;                                  // set by a role whose bounded wait ran out
   volatile int tmem_busy;                              // set if products may still be in flight at the end (tensor memory is then not released)
@@ -198,7 +203,7 @@ __device__ __noinline__ float exact_chain(const float* rrow, const __half* xrow)
 }
 
 // R_m (fp32) as two fp16 operand tiles in slot `slot`, by the NT worker threads: all of a thread's loads in flight together.
-// A warp takes 8 rows x 32 columns: 128-byte pieces of a row in global memory, eight consecutive 16-byte rows of a core
+// A warp takes 8 rows, 32 columns at a time: 128-byte pieces of a row in global memory, eight consecutive 16-byte rows of a core
 // matrix per quarter-warp in shared memory (lanes along a row instead put eight stores on the same banks: 6000 cycles).
 template <int BITS>
 __device__ __forceinline__ void write_matrix(TcSmem<BITS>& sm, const float* Rm, int slot, int tid) {
@@ -206,18 +211,21 @@ __device__ __forceinline__ void write_matrix(TcSmem<BITS>& sm, const float* Rm, 
   float4 x[N][2];
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const int item = (tid >> 5) + NT / 32 * i, n = 8 * (item >> 2) + (tid & 7), kc = 4 * (item & 3) + ((tid >> 3) & 3);
+    const int n = 8 * (tid >> 5) + (tid & 7), kc = 4 * i + ((tid >> 3) & 3);
     const float* src = Rm + n * D + kc * 8;
     x[i][0] = __ldg(reinterpret_cast<const float4*>(src));
     x[i][1] = __ldg(reinterpret_cast<const float4*>(src) + 1);
   }
+  static_assert(N == 4 && NT / 32 == D / 8, "a warp has whole rows");
+  float sq = 0.0f;
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const int item = (tid >> 5) + NT / 32 * i, n = 8 * (item >> 2) + (tid & 7), kc = 4 * (item & 3) + ((tid >> 3) & 3);
+    const int n = 8 * (tid >> 5) + (tid & 7), kc = 4 * i + ((tid >> 3) & 3);
     const float xs[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
     __align__(16) __half hi[8], lo[8];
 #pragma unroll
     for (int u = 0; u < 8; u++) {
+      sq = fmaf(xs[u], xs[u], sq);
       hi[u] = __float2half_rn(xs[u]);
       lo[u] = __float2half_rn(xs[u] - __half2float(hi[u]));
     }
@@ -225,6 +233,9 @@ __device__ __forceinline__ void write_matrix(TcSmem<BITS>& sm, const float* Rm, 
     *reinterpret_cast<uint4*>(sm.b[slot][0] + off) = *reinterpret_cast<const uint4*>(hi);
     *reinterpret_cast<uint4*>(sm.b[slot][1] + off) = *reinterpret_cast<const uint4*>(lo);
   }
+  sq += __shfl_xor_sync(0xffffffffu, sq, 8);
+  sq += __shfl_xor_sync(0xffffffffu, sq, 16);
+  if (!(sq <= ROW_SQ_MAX)) sm.redo = 1;   // (not a number either)
 }
 
 // The jobs of a tile, derived identically by the MMA warp and every worker warp from the tile's modality
@@ -337,6 +348,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     sm.abort = 0;
     sm.tmem_busy = 0;
     sm.fix_count = 0;
+    sm.redo = 0;
     sm.limit = wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -521,7 +533,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         const float sum = __fadd_rn(__fadd_rn(sm.part[buf][0][tok], sm.part[buf][1][tok]),
                                     __fadd_rn(sm.part[buf][2][tok], sm.part[buf][3][tok]));
         float n = __fsqrt_rn(sum);
-        n = n > 65504.0f ? 65504.0f : n;
+        if (n > NORM_MAX) { n = NORM_MAX; sm.redo = 1; }
         const __half nh16 = __float2half_rn(n);
         const float nf = __half2float(nh16);
         if (eq == 0) {
@@ -721,8 +733,25 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
   __syncthreads();
   // ---- the listed coordinates, one per warp at a time: the two rows go through the warp's corner of the (idle) first
   // tile buffer, every lane evaluates the same chain (input index ascending, one rounding per step), lane 0 patches
+  auto patch = [&](uint32_t* word, int bit, float z) {   // the code of coordinate z in place of what is there
+    if constexpr (BITS == 0) {
+      const uint32_t code = (uint32_t)((z > -CB_THRESH) + (z > 0.0f) + (z > CB_THRESH));
+      atomicAnd(word, ~(3u << bit));
+      atomicOr(word, code << bit);
+    } else {
+      uint32_t code = 0;
+      for (int j = 0; j < (1 << BITS) - 1; j++) code += z > c_thresholds[BITS - 2][j];
+      const unsigned long long field = (unsigned long long)((1u << BITS) - 1u) << bit, val = (unsigned long long)code << bit;
+      atomicAnd(word, ~(uint32_t)field);
+      atomicOr(word, (uint32_t)val);
+      if (field >> 32) {   // a 3-bit code across two words
+        atomicAnd(word + 1, ~(uint32_t)(field >> 32));
+        atomicOr(word + 1, (uint32_t)(val >> 32));
+      }
+    }
+  };
   {
-    const int n_fix = min(sm.fix_count, FIX_MAX);
+    const int n_fix = sm.redo ? 0 : min(sm.fix_count, FIX_MAX);
     unsigned char* scr = sm.a[0] + warp * 1024;
     for (int i = warp; i < n_fix && !sm.abort; i += NT_ALL / 32) {
       const FixItem it = sm.fix[i];
@@ -740,24 +769,37 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
         a = __fmaf_rn(r1.x, x2.x, a); a = __fmaf_rn(r1.y, x2.y, a); a = __fmaf_rn(r1.z, x3.x, a); a = __fmaf_rn(r1.w, x3.y, a);
       }
       const float z = __fmul_rn(a, it.inv);
-      if (lane == 0) {
-        if constexpr (BITS == 0) {
-          const uint32_t code = (uint32_t)((z > -CB_THRESH) + (z > 0.0f) + (z > CB_THRESH));
-          atomicAnd(it.word, ~(3u << it.bit));
-          atomicOr(it.word, code << it.bit);
-        } else {
-          uint32_t code = 0;
-          for (int j = 0; j < (1 << BITS) - 1; j++) code += z > c_thresholds[BITS - 2][j];
-          const unsigned long long field = (unsigned long long)((1u << BITS) - 1u) << it.bit, val = (unsigned long long)code << it.bit;
-          atomicAnd(it.word, ~(uint32_t)field);
-          atomicOr(it.word, (uint32_t)val);
-          if (field >> 32) {   // a 3-bit code across two words
-            atomicAnd(it.word + 1, ~(uint32_t)(field >> 32));
-            atomicOr(it.word + 1, (uint32_t)(val >> 32));
-          }
-        }
-      }
+      if (lane == 0) patch(it.word, it.bit, z);
       __syncwarp();
+    }
+  }
+  // ---- or all of the block's coordinates, one per thread: a warp has 32 channels of a token
+  if (sm.redo && !sm.abort) {
+    for (int i = 0; i < my_tiles; i++) {
+      const int tile = tile_begin + i, b = tile / (tiles_per_unit * cv.n_kv_heads), h = tile / tiles_per_unit % cv.n_kv_heads;
+      const int win0 = tile % tiles_per_unit * 4, n_tok = min(TILE, (n_win - win0) * W);
+      for (int idx = tid; idx < n_tok * D; idx += NT_ALL) {
+        const int tok = win0 * W + idx / D, c = idx % D;
+        unsigned m = modality[(size_t)b * n_tokens + tok];
+        m = m > 2 ? 0 : m;
+        float nf;
+        uint32_t* word;
+        int bit;
+        if constexpr (BITS == 0) {
+          unsigned char* body = cv.body(layer, b, h, tok / W);
+          nf = __half2float(reinterpret_cast<const __half*>(body + B_VNORM)[norm_pos(tok % W)]);
+          int w;
+          vcode_pos(tok % W, c, w, bit);
+          word = reinterpret_cast<uint32_t*>(body + B_VCODE) + w;
+        } else {
+          const size_t t = lv.unit(b, h) * lv.capacity + tok;
+          nf = __half2float(lv.v_norm[t]);
+          word = reinterpret_cast<uint32_t*>(lv.v_codes + t * (16 * BITS)) + ((BITS * c) >> 5);
+          bit = (BITS * c) & 31;
+        }
+        const float a = exact_chain(R + ((size_t)((n_R == 1 ? 0 : h) * 3 + m) * D + c) * D, vrows + b * vs_b + h * vs_h + (long long)tok * vs_t);
+        patch(word, bit, __fmul_rn(a, nf != 0.0f ? __fdiv_rn(1.0f, nf) : 0.0f));
+      }
     }
   }
   if (tid == 0 && sm.abort && cv.status) atomicCAS(cv.status, 0, (int)OKQ_ERR_TIMEOUT);

@@ -144,3 +144,27 @@ def test_eigen_solver_on_degenerate_matrices(name, C):
     assert np.abs(lam - np.sort(np.linalg.eigvalsh(Cd))[::-1]).max() <= 1e-6 * top
     H = CO.hadamard_matrix(signs.numpy())
     assert np.abs(R @ Cd @ R.T - (H * lam) @ H.T).max() <= 1e-5 * top
+
+
+@pytest.mark.parametrize("bits", [0, 2, 3, 4])
+@pytest.mark.parametrize("row,value", [(1e-6, 1.0), (30.0, 1.0), (1e3, 1.0), (1e6, 1.0), (1.0, 4000.0), (1.0, 12000.0)])
+def test_value_codes_for_any_matrix(bits, row, value):
+    """Matrices with rows shorter and longer than 1, entries beyond fp16, values whose norm fp16 holds just and not at all: the
+    codes of the exact chain (which a broadcast head gets), from the hot path's quantiser (0) and the ladder's."""
+    n = 32 * 64 + (7 if bits == 0 else 0)
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=1, n_kv_heads=2, n_q_heads=14)
+    g = torch.Generator().manual_seed(5)
+    shared = (value * torch.randn(1, 1, n, D, generator=g)).clamp(-65504, 65504).half().cuda().expand(1, 2, n, D)
+    R = row * WL.gen_rotations(w, 0)[None].contiguous().cuda()
+    mod = WL.modality_layout(w, n).unsqueeze(0).contiguous().cuda()
+
+    def quantised(v):
+        if bits:
+            c = B.LadderCache(1, 2, 14, n, bits)
+            B.ladder_quantize_values(c, v, mod, R)
+            return c.v_codes, c.v_norm
+        c = B.Cache(1, 1, 2, 14, n + 25)
+        B.quantize_values(c, 0, v, mod, R)
+        return c.records, c.v_tail
+
+    assert all(torch.equal(a, b) for a, b in zip(quantised(shared), quantised(shared.contiguous())))
