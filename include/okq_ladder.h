@@ -13,7 +13,8 @@
  *          value sums in each modality's rotated basis, R_m^T once per head.
  * Key codes and split weights meet on the tensor cores, value sums are fp32 multiply-adds, the value rotation is the
  * tensor-core product of the 2-bit path with the coordinates near a threshold recomputed exactly.  The calls have no
- * status word: a bounded wait of the value quantiser that ran out would leave codes unwritten.
+ * status word: where a bounded wait of the value quantiser runs out, the norms of the tokens whose codes are not complete
+ * become NaN, and so do the outputs of a decode call that reads them.
  *
  * Cache layout (all buffers caller-owned, 16-byte aligned; n_tokens must be a multiple of 32: no raw tail):
  *   k_codes, v_codes  uint8 [batch][n_kv_heads][capacity][16 * bits]: per token a little-endian bit stream,
@@ -58,6 +59,12 @@ okq_status okq_ladder_quantize_keys(const okq_ladder_cache* cache, const void* k
 okq_status okq_ladder_quantize_values(const okq_ladder_cache* cache, const void* v_fp16, const int64_t strides[3],
                                       int32_t n_tokens, const uint8_t* modality, const float* R, int32_t n_R,
                                       void* stream);
+
+/* Testing aid for the bounded waits of okq_ladder_quantize_values (the paper has no counterpart), as okq_debug_bulk_timeout
+ * is for the 2-bit path: the first 128-token tile is never delivered and every wait limited to `limit_clocks` SM clocks. */
+okq_status okq_debug_ladder_timeout(const okq_ladder_cache* cache, const void* v_fp16, const int64_t strides[3],
+                                    int32_t n_tokens, const uint8_t* modality, const float* R, int32_t n_R,
+                                    int64_t limit_clocks, void* stream);
 
 /* Eq. 1 over the first n_tokens tokens of every sequence.  q: device fp16 [batch][n_q_heads][128];
  * out: device float [batch][n_q_heads][128]; a cluster of one to eight thread blocks per (sequence, KV head). */

@@ -114,6 +114,8 @@ def lib():
         L.okq_ladder_quantize_values.restype = C.c_int
         L.okq_ladder_quantize_values.argtypes = [C.POINTER(okq_ladder_cache), C.c_void_p, C.POINTER(C.c_int64), C.c_int32,
                                                  C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p]
+        L.okq_debug_ladder_timeout.restype = C.c_int
+        L.okq_debug_ladder_timeout.argtypes = list(L.okq_ladder_quantize_values.argtypes[:-1]) + [C.c_int64, C.c_void_p]
         L.okq_ladder_decode_attention.restype = C.c_int
         L.okq_ladder_decode_attention.argtypes = [C.POINTER(okq_ladder_cache), C.c_int32, C.c_void_p, C.c_float, C.c_void_p,
                                                   C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]
@@ -132,7 +134,7 @@ def exported_symbols():
             "okq_decode_attention_noalloc", "okq_quantize_values_bulk", "okq_debug_bulk_timeout", "okq_cache_export_mx",
             "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_calib_moments", "okq_calib_rotation",
             "okq_ladder_codebook", "okq_ladder_quantize_keys", "okq_ladder_quantize_values",
-            "okq_ladder_decode_attention", "okq_turboquant_encode", "okq_turboquant_decode"]
+            "okq_debug_ladder_timeout", "okq_ladder_decode_attention", "okq_turboquant_encode", "okq_turboquant_decode"]
 
 
 def _ptr(t) -> int:
@@ -378,6 +380,16 @@ def ladder_quantize_values(cache: LadderCache, v: torch.Tensor, modality: torch.
     n_R = R.shape[0] if R.dim() == 4 else 1
     _check(lib().okq_ladder_quantize_values(C.byref(cache.c), _ptr(v), strides, v.shape[2], _ptr(modality), _ptr(R), n_R,
                                             _stream(stream)), "okq_ladder_quantize_values")
+
+
+def debug_ladder_timeout(cache: LadderCache, v: torch.Tensor, modality: torch.Tensor, R: torch.Tensor,
+                         limit_clocks: int = 20_000_000, stream=None):
+    """okq_debug_ladder_timeout: the ladder's value quantiser with its first tile withheld and every wait limited to
+    `limit_clocks` SM clocks; the norms of the tokens concerned become NaN (testing aid)."""
+    strides = (C.c_int64 * 3)(v.stride(0), v.stride(1), v.stride(2))
+    n_R = R.shape[0] if R.dim() == 4 else 1
+    _check(lib().okq_debug_ladder_timeout(C.byref(cache.c), _ptr(v), strides, v.shape[2], _ptr(modality), _ptr(R), n_R, limit_clocks,
+                                          _stream(stream)), "okq_debug_ladder_timeout")
 
 
 def ladder_decode_attention(cache: LadderCache, n_tokens: int, q, signs, R, out, sm_scale=None, stream=None):

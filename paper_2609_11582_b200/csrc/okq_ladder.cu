@@ -377,6 +377,18 @@ okq_status okq_ladder_quantize_values(const okq_ladder_cache* cache, const void*
   return launch_status();
 }
 
+okq_status okq_debug_ladder_timeout(const okq_ladder_cache* cache, const void* v_fp16, const int64_t strides[3], int32_t n_tokens,
+                                    const uint8_t* modality, const float* R, int32_t n_R, int64_t limit_clocks, void* stream) {
+  okq_status st = check_ladder(cache, n_tokens);
+  if (st != OKQ_OK) return st;
+  if (!v_fp16 || !strides || !modality || !R || (n_R != 1 && n_R != cache->n_kv_heads) || limit_clocks <= 0) return OKQ_ERR_INVALID_ARG;
+  if (!aligned16(v_fp16) || !aligned16(R) || strides[0] % 8 || strides[1] % 8 || strides[2] % 8) return OKQ_ERR_ALIGNMENT;
+  if (n_tokens == 0) return OKQ_OK;
+  st = launch_ladder_values_tc(ladder_view(cache), static_cast<const __half*>(v_fp16), strides, modality, n_tokens, R, n_R, sm_count(),
+                               static_cast<cudaStream_t>(stream), (long long)limit_clocks, 0);
+  return st != OKQ_OK ? st : launch_status();
+}
+
 okq_status okq_ladder_decode_attention(const okq_ladder_cache* cache, int32_t n_tokens, const void* q, float sm_scale,
                                        const float* signs, const float* R, int32_t n_R, float* out, void* stream) {
   okq_status st = check_ladder(cache, n_tokens);

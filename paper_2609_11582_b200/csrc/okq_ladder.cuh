@@ -42,6 +42,7 @@ cudaError_t launch_ladder_decode(const LadderView& cv, int n_tokens, const __hal
 
 // value quantiser on the tensor cores (okq_quant_tc.cu); OKQ_ERR_UNSUPPORTED for strides a tensor map cannot describe
 okq_status launch_ladder_values_tc(const LadderView& lv, const __half* v, const int64_t strides[3], const unsigned char* modality,
-                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s);
+                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s, long long wait_limit = 0,
+                                   int skip_tile = -1);
 
 }  // namespace okq

@@ -37,7 +37,8 @@
 // 1282 us with one block per window evaluating the exact chain, 146 us now.
 //
 // Every wait on an mbarrier is bounded; on a timeout the kernel records OKQ_ERR_TIMEOUT in the
-// cache's status word, stops issuing work, frees its tensor memory and returns.
+// cache's status word (the ladder, which has none: NaN in the value norms of the block's tokens, which decode hands on), stops
+// issuing work, frees its tensor memory and returns.
 #include <cuda.h>   // CUtensorMap and the type of cuTensorMapEncodeTiled only; the entry point is fetched at run time
 
 #include "okq_common.cuh"
@@ -802,6 +803,12 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       }
     }
   }
+  if (BITS != 0 && sm.abort) {   // the ladder's calls have no status word: the tokens of the block's tiles get norms that are no numbers
+    for (int i = tid; i < my_tiles * TILE; i += NT_ALL) {
+      const int tile = tile_begin + i / TILE, tok = tile % tiles_per_unit * TILE + i % TILE;
+      if (tok < n_win * W) lv.v_norm[(size_t)(tile / tiles_per_unit) * lv.capacity + tok] = __ushort_as_half(0x7fff);
+    }
+  }
   if (tid == 0 && sm.abort && cv.status) atomicCAS(cv.status, 0, (int)OKQ_ERR_TIMEOUT);
   if (warp == 0 && !sm.tmem_busy) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
 }
@@ -870,14 +877,14 @@ okq_status launch_quantize_values_tc(const CacheView& cv, int layer, const __hal
 }
 
 okq_status launch_ladder_values_tc(const LadderView& lv, const __half* v, const int64_t strides[3], const unsigned char* modality,
-                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s) {
+                                   int n_tokens, const float* R, int n_R, int n_sm, cudaStream_t s, long long wait_limit, int skip_tile) {
   CacheView cv{};   // shape and modality bytes; no status word: the ladder calls have none
   cv.n_layers = 1; cv.batch = lv.batch; cv.n_kv_heads = lv.n_kv_heads; cv.n_q_heads = lv.n_q_heads; cv.capacity = lv.capacity;
   cv.modality = lv.modality;
   const int n_win = n_tokens / W;
-  return lv.bits == 2 ? launch_values_tc<2>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1)
-       : lv.bits == 3 ? launch_values_tc<3>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1)
-                      : launch_values_tc<4>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, 0, -1);
+  return lv.bits == 2 ? launch_values_tc<2>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, wait_limit, skip_tile)
+       : lv.bits == 3 ? launch_values_tc<3>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, wait_limit, skip_tile)
+                      : launch_values_tc<4>(cv, lv, 0, v, strides, modality, n_tokens, n_win, R, n_R, n_sm, s, wait_limit, skip_tile);
 }
 
 }  // namespace okq

@@ -116,3 +116,27 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     ea, eb = B.cache_export(cache, 0), B.cache_export(exact, 0)
     npk = (n // W) * W
     assert torch.equal(ea["v_codes"][:, :, :npk], eb["v_codes"][:, :, :npk]) and torch.equal(ea["v_norm"][:, :, :npk], eb["v_norm"][:, :, :npk])
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_ladder_wait_that_runs_out_leaves_a_mark(bits):
+    """The ladder's value quantiser has no status word: with its first tile withheld, the tokens of the blocks that gave up have
+    NaN norms, decode hands them on, and the same call without the handicap gives finite outputs again."""
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=2)
+    n, dev = 1024, torch.device("cuda")
+    k, v = WL.gen_kv(w, 0, n_tokens=n)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(w.batch, 1).contiguous().to(dev)
+    R, signs, q = WL.gen_rotations(w, 0)[None].contiguous().to(dev), WL.gen_signs(w, 0).to(dev), WL.gen_queries(w, 0).to(dev)
+    cache = B.LadderCache(w.batch, w.n_kv_heads, w.n_q_heads, n + 32, bits, device=dev)
+    B.ladder_quantize_keys(cache, k.to(dev), signs)
+    out = torch.empty(w.batch, w.n_q_heads, D, device=dev)
+    B.debug_ladder_timeout(cache, v.to(dev), mod, R, limit_clocks=20_000_000)
+    torch.cuda.synchronize()                      # returns: the kernel ended by itself
+    marked = cache.v_norm.isnan()
+    # 64 tiles of 128 tokens, one per block: the first block's tokens are marked, the others' are complete
+    assert marked[0, 0, :128].all() and not marked[0, 0, 128:].any() and not marked[:, 1:].any() and not marked[1].any()
+    B.ladder_decode_attention(cache, n, q, signs, R, out)
+    assert out[0, :w.group].isnan().all() and out[0, w.group:].isfinite().all() and out[1].isfinite().all()
+    B.ladder_quantize_values(cache, v.to(dev), mod, R)
+    B.ladder_decode_attention(cache, n, q, signs, R, out)
+    assert out.isfinite().all() and not cache.v_norm.isnan().any()
