@@ -88,15 +88,47 @@ class Case:
         torch.cuda.synchronize()
         return e
 
-    def gpu_decode(self, layer, layer_count=1, num_splits=0, simt=False):
+    def gpu_decode(self, layer, layer_count=1, num_splits=0, simt=False, least_workspace=False):
+        """Output of one call.  Afterwards `self.split_k` says whether the split-K pair took it (else the one-launch kernel)."""
         c = self.cache
-        ws = torch.empty(max(16, B.decode_workspace_bytes(c, layer_count, num_splits)), dtype=torch.uint8, device=c.device)
-        out = torch.full((layer_count, c.batch, c.n_q_heads, D), float("nan"), dtype=torch.float32, device=c.device)
-        B.decode_attention(c, layer, layer_count, self.d_q[layer:layer + layer_count].contiguous(),
-                           self.d_signs[layer:layer + layer_count].contiguous(),
-                           self.d_R[layer:layer + layer_count].contiguous(), ws, out, num_splits=num_splits, simt=simt)
-        torch.cuda.synchronize()
+        q, signs, R = (x[layer:layer + layer_count].contiguous() for x in (self.d_q, self.d_signs, self.d_R))
+
+        def call(ws):
+            out = torch.full((layer_count, c.batch, c.n_q_heads, D), float("nan"), dtype=torch.float32, device=c.device)
+            B.decode_attention(c, layer, layer_count, q, signs, R, ws, out, num_splits=num_splits, simt=simt)
+            torch.cuda.synchronize()
+            return out
+
+        ws = decode_workspace(c, layer_count, num_splits, call if least_workspace else None)
+        out = call(ws)
+        self.split_k = ran_split_k(ws)
         return out.cpu().numpy().astype(np.float64)
+
+
+def decode_workspace(cache, layer_count, num_splits=0, call=None):
+    """A workspace for a decode call, filled with a pattern: of the size the library asks for, or, given `call(workspace)`, the
+    smallest one that the call accepts.  That one holds the split-K kernel's pieces and no more, so calls whose one-launch kernel
+    needs more of them take the split-K pair, with its automatic grid."""
+    size = max(16, B.decode_workspace_bytes(cache, layer_count, num_splits))
+    if call is not None:
+        lo = 0                                # sizes in units of 16 bytes: lo is refused, size accepted
+        size = (size + 15) // 16
+        while size - lo > 1:
+            mid = (lo + size) // 2
+            try:
+                call(torch.empty(16 * mid, dtype=torch.uint8, device=cache.device))
+                size = mid
+            except B.OkqError as e:
+                assert e.status == B.ERR_WORKSPACE
+                lo = mid
+        size *= 16
+    return torch.full((size,), 0xA5, dtype=torch.uint8, device=cache.device)
+
+
+def ran_split_k(ws: torch.Tensor) -> bool:
+    """Whether a call that was given `ws` (from decode_workspace) ran the split-K kernel: its first partial, at the start of the
+    workspace, is written by every launch with a packed window; the one-launch kernel leaves that place alone."""
+    return bool((ws[:64] != 0xA5).any())
 
 
 def compare_cache(case: Case, layer: int, exp: dict, kq: dict, vq: dict):

@@ -2,7 +2,7 @@
 
   * 30B-A3B shape (GQA group 8, video 400 / audio 100 chunks), reduced layers and context;
   * long-context decode (batch 1, many CTAs per (sequence, head));
-  * long single-modality ranges per warp pair, and thousands of two-window units in one launch;
+  * long single-modality ranges per warp, and thousands of two-window units in one launch;
   * the full 7B decode step (28 layers x batch 8 x 16384 tokens, one append + one decode call
     over all layers, inputs drawn on the GPU exactly as bench.py does), checked on sampled
     (layer, sequence) pairs the oracle can afford, plus properties that hold at any size.
@@ -26,10 +26,12 @@ def test_group8_30b_shape():
     for l in range(2):
         kq, vq, _, _ = c.oracle_quantize(l)
         Hn.compare_cache(c, l, c.gpu_export(l), kq, vq)
-    got = c.gpu_decode(0, layer_count=2)
-    for l in range(2):
-        ref, _ = c.oracle_attention(l)
-        print("30B shape layer", l, Hn.assert_attention_close(got[l], ref))
+    for splits in (9, 0):                    # the split-K pair on 144 blocks, then the library's choice
+        got = c.gpu_decode(0, layer_count=2, num_splits=splits)
+        assert c.split_k == (splits > 0)
+        for l in range(2):
+            ref, _ = c.oracle_attention(l)
+            print("30B shape layer", l, Hn.assert_attention_close(got[l], ref))
     simt = c.gpu_decode(0, layer_count=2, simt=True)
     assert np.abs(simt - got).max() < 1e-3
 
@@ -38,14 +40,14 @@ def test_long_context_batch1():
     w = WL.scaled(WL.WORKLOADS["long7b"], n_layers=1, n_tokens=32768 + 31)
     c = Hn.Case(w)
     ref, _ = c.oracle_attention(0)
-    got = c.gpu_decode(0)[0]                 # 148 CTAs over 4 (sequence, head) units: 37 partials each
-    print("long context", Hn.assert_attention_close(got, ref))
-    got4 = c.gpu_decode(0, num_splits=3)[0]
-    Hn.assert_attention_close(got4, ref)
+    for splits in (0, 37, 3):                # the library's choice (clusters), 148 CTAs over 4 units: 37 partials each, 12 CTAs
+        got = c.gpu_decode(0, num_splits=splits)[0]
+        assert c.split_k == (splits > 0)
+        print("long context, splits", splits, Hn.assert_attention_close(got, ref))
 
 
 def test_one_modality_long_ranges():
-    """One warp pair covers 256 windows of a single modality (one CTA per (sequence, head), no modality change
+    """One warp covers 171 windows of a single modality (one CTA per (sequence, head), no modality change
     that would move the register sums out): the value sums must not drift with the length of the range.  The
     tensor cores accumulate without rounding to nearest, so a long chain into one register is biased; the
     kernel bounds the chain, and this case fails (worst head above the tolerance) if it does not."""
@@ -61,38 +63,45 @@ def test_one_modality_long_ranges():
 
 @pytest.mark.parametrize("meta_format", [B.META_FP16, B.META_MXFP4])
 def test_middle_sized_grid(meta_format):
-    """64 (head, four-sequence group, layer) blocks: fewer than SMs but too many for four column slices each, the
-    case in which the combine kernel runs one sequence per block over all columns."""
+    """64 (head, four-sequence group, layer) combine blocks: fewer than SMs but too many for four column slices each, the
+    case in which the combine kernel runs one sequence per block over all columns.  The split-K pair takes the call when the
+    workspace is the least it accepts; with the one the library asks for, one block per unit does (256 of them)."""
     w = WL.scaled(WL.WORKLOADS["step7b"], n_layers=8, n_tokens=1024 + 7)
     c = Hn.Case(w, meta_format=meta_format)
-    got = c.gpu_decode(0, layer_count=w.n_layers)
-    for l in (0, 3, 7):
-        ref, _ = c.oracle_attention(l)
-        Hn.assert_attention_close(got[l], ref)
+    refs = {l: c.oracle_attention(l)[0] for l in (0, 3, 7)}
+    for least in (True, False):
+        got = c.gpu_decode(0, layer_count=w.n_layers, least_workspace=least)
+        assert c.split_k == least
+        for l, ref in refs.items():
+            Hn.assert_attention_close(got[l], ref)
 
 
 def test_one_head_over_every_cta():
-    """A single (sequence, head) unit of 129 windows: every CTA of the split-K kernel holds one window of it, so the
-    combine kernel merges 129 partials for one head group, more than its table of precomputed factors holds."""
+    """A single (sequence, head) unit of 129 windows.  With 148 blocks asked for every CTA of the split-K kernel holds one window
+    of it, so the combine kernel merges 129 partials for one head group, more than its table of precomputed factors holds; the
+    library's own choice is a cluster of 16."""
     w = WL.scaled(WL.WORKLOADS["tiny"], n_tokens=4128 + 5, n_chunks=0)
     c = Hn.Case(w)
     ref, _ = c.oracle_attention(0)
-    got = c.gpu_decode(0)[0]
-    print("one head over every CTA", Hn.assert_attention_close(got, ref))
+    for splits in (148, 0):
+        got = c.gpu_decode(0, num_splits=splits)[0]
+        assert c.split_k == (splits > 0)
+        print("one head over every CTA, splits", splits, Hn.assert_attention_close(got, ref))
 
 
 def test_decode_is_deterministic():
-    """No atomics and a fixed partition: two calls on the same cache give bit-identical outputs (both grids)."""
+    """A fixed partition, and sums of one address in one warp's order: two calls on the same cache give bit-identical outputs
+    (clusters, then the split-K pair)."""
     w = WL.scaled(WL.WORKLOADS["step7b"], n_layers=2, batch=3, n_tokens=2048 + 17)
     c = Hn.Case(w)
     for splits in (0, 2):
         a = c.gpu_decode(0, layer_count=2, num_splits=splits)
         b = c.gpu_decode(0, layer_count=2, num_splits=splits)
-        assert np.array_equal(a, b)
+        assert np.array_equal(a, b) and c.split_k == (splits > 0)
 
 
 def test_many_short_units_per_cta():
-    """8192 (sequence, head) units of two windows each in one launch: every warp pair crosses several unit
+    """8192 (sequence, head) units of two windows each in one launch: every warp crosses several unit
     boundaries and every CTA merges ~55 units, more than one batch of its end-of-launch merge."""
     w = WL.Workload("short", 5, 8, 128, 16, 8, 64 + 5, 16, 20, 12, 0)
     c = Hn.Case(w)
@@ -188,13 +197,13 @@ def test_every_window_holds_all_three_modalities(meta_format):
     ea, eb = c.gpu_export(0), b.gpu_export(0)
     assert b.cache.device_status() == 0
     assert torch.equal(ea["v_norm"], eb["v_norm"])
-    assert torch.equal(ea["v_codes"], eb["v_codes"])               # the bulk path fixes up coordinates near a threshold
+    assert torch.equal(ea["v_codes"], eb["v_codes"])               # both entry points: coordinates near a threshold are fixed up
     Hn.assert_attention_close(b.gpu_decode(0)[0], ref)
 
 
 def test_ragged_batch_lengths():
-    """Sequences of different lengths in one decode call (lengths set per sequence, tails filled to match):
-    the persistent kernel's partition follows the per-sequence window counts."""
+    """Sequences of different lengths in one decode call (lengths set per sequence, tails filled to match): the clusters'
+    ranges and the persistent kernel's partition follow the per-sequence window counts."""
     w = WL.scaled(WL.WORKLOADS["layer7b"], batch=4, n_layers=2, n_tokens=1500)
     c = Hn.Case(w, capacity=1536)
     dev = c.cache.device
@@ -210,12 +219,15 @@ def test_ragged_batch_lengths():
                 vt[l, b, :, : n - npk] = c.v[l][b, :, npk:n].to(dev)
     c.cache.seq_len.copy_(torch.from_numpy(lengths.reshape(-1).astype(np.int32)).to(dev))
     got = c.gpu_decode(0, layer_count=2)
+    assert not c.split_k
+    got_pair = c.gpu_decode(0, layer_count=2, num_splits=5)   # 160 CTAs over 32 units
+    assert c.split_k
     got_simt = c.gpu_decode(0, layer_count=2, simt=True)
     for l in range(2):
         for b in range(w.batch):
             n = int(lengths[l, b])
             if n == 0:
-                assert (got[l, b] == 0).all() and (got_simt[l, b] == 0).all()
+                assert (got[l, b] == 0).all() and (got_pair[l, b] == 0).all() and (got_simt[l, b] == 0).all()
                 continue
             kb = Hn.u16(c.k[l][b, :, :n]); vb = Hn.u16(c.v[l][b, :, :n])
             mod = c.mod_b[b, :n].numpy()
@@ -225,6 +237,7 @@ def test_ragged_batch_lengths():
             ref, _ = O.attention(1, q, kq, vq, mod, kb[:, npk:], vb[:, npk:], c.signs[l].numpy(), c.R[l].numpy())
             ref = ref.reshape(w.n_q_heads, D)
             Hn.assert_attention_close(got[l, b], ref)
+            Hn.assert_attention_close(got_pair[l, b], ref)
             Hn.assert_attention_close(got_simt[l, b], ref)
 
 

@@ -14,35 +14,40 @@ pytestmark = pytest.mark.gpu
 D, W = 128, 32
 
 
-# (sequences, KV heads): units at which the cluster goes 16 -> 8 -> 4 -> split-K kernel; tokens: fewer windows than warps, one
-# window, no window at all, a full and an empty raw tail
-@pytest.mark.parametrize("batch,heads", [(1, 1), (2, 4), (15, 1), (33, 1), (17, 2)])
+# (sequences, KV heads), units around the steps of the rule: a cluster of 16; the most clusters of 8 and of 4 that run at once
+# (15, 33); clusters of 2 up to the most of them (74); single blocks in one wave (75, 76, 148) and in two (149); the split-K pair
+# (448 units would be a fourth wave); tokens: fewer windows than warps, one window, no window at all, a full and an empty raw tail
+@pytest.mark.parametrize("batch,heads", [(1, 1), (2, 4), (15, 1), (33, 1), (17, 2), (74, 1), (75, 1), (76, 1), (37, 4), (149, 1), (112, 4)])
 @pytest.mark.parametrize("n", [31, 32, 32 * 13 + 31])
 def test_one_launch_decode_at_its_edges(batch, heads, n):
     w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=7 * heads, prefix_text=40, video_chunk=70, audio_chunk=21)
     c = Hn.Case(w, n_tokens=n, meta_format=B.META_MXFP4 if batch % 2 else B.META_FP16)
     # the CUDA-core kernels are within 1e-6 of the definition, so the bound is the tensor-core path's own
-    Hn.assert_attention_close(c.gpu_decode(0)[0], c.gpu_decode(0, simt=True)[0])
+    got = c.gpu_decode(0)[0]
+    assert c.split_k == (batch * heads == 448 and n >= W)
+    Hn.assert_attention_close(got, c.gpu_decode(0, simt=True)[0])
 
 
 @pytest.mark.parametrize("meta", [B.META_FP16, B.META_MXFP4])
 @pytest.mark.parametrize("n", [100, 128, 128 + 159, 1024 + 127])
-def test_one_launch_decode_captioning_schedule(meta, n):
+@pytest.mark.parametrize("batch", [2, 40])   # clusters of 8, single blocks
+def test_one_launch_decode_captioning_schedule(meta, n, batch):
     """Up to four packed windows and 127 raw keys among the raw values; against the split-K pair."""
-    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=2)
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch)
     dev = torch.device("cuda")
-    cache = B.Cache(1, 2, w.n_kv_heads, w.n_q_heads, 1280, device=dev, meta_format=meta, schedule=B.SCHEDULE_CAPTION)
+    cache = B.Cache(1, batch, w.n_kv_heads, w.n_q_heads, 1280, device=dev, meta_format=meta, schedule=B.SCHEDULE_CAPTION)
     k, v = WL.gen_kv(w, 0, n_tokens=n)
     signs, R = WL.gen_signs(w, 0).to(dev), WL.gen_rotations(w, 0)[None].contiguous().to(dev)
-    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(2, 1).contiguous().to(dev)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(batch, 1).contiguous().to(dev)
     B.quantize_keys(cache, 0, k.to(dev), signs)
     B.quantize_values(cache, 0, v.to(dev), mod, R)
     q = WL.gen_queries(w, 0).to(dev)
     outs = []
     for splits in (0, 2):
-        ws = torch.empty(B.decode_workspace_bytes(cache, 1, splits), dtype=torch.uint8, device=dev)
-        out = torch.full((1, 2, w.n_q_heads, D), float("nan"), device=dev)
+        ws = Hn.decode_workspace(cache, 1, splits)
+        out = torch.full((1, batch, w.n_q_heads, D), float("nan"), device=dev)
         B.decode_attention(cache, 0, 1, q, signs, R, ws, out, num_splits=splits)
+        assert Hn.ran_split_k(ws) == (splits > 0 and n >= 128 + W)
         outs.append(out.cpu().numpy().astype(np.float64))
     Hn.assert_attention_close(outs[0], outs[1])
 

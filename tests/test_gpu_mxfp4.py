@@ -85,8 +85,7 @@ def test_bulk_value_quantiser_writes_the_same_bodies():
     b = Hn.Case(w, n_tokens=8 * W, meta_format=MX, bulk_values=True)
     ea, eb = a.gpu_export(0), b.gpu_export(0)
     assert torch.equal(ea["v_norm"], eb["v_norm"]) and torch.equal(ea["k_mx"], eb["k_mx"])
-    # the tensor-core rotation may move a value across a codebook threshold it sits on
-    assert (ea["v_codes"] != eb["v_codes"]).sum().item() <= 4
+    assert torch.equal(ea["v_codes"], eb["v_codes"])
 
 
 def test_import_is_refused_and_formats_agree_on_bodies():

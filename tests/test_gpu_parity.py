@@ -213,7 +213,7 @@ def test_bulk_value_quantiser_on_tensor_cores():
     # decode over the bulk-built cache matches the oracle
     ref, _ = c.oracle_attention(0)
     Hn.assert_attention_close(c.gpu_decode(0)[0], ref)
-    # raw tail and modality as in the exact path
+    # raw tail
     U = w.batch * w.n_kv_heads
     assert (Hn.u16(c.cache.v_tail).reshape(U, W, D)[:, :19] == Hn.u16(c.v[0]).reshape(U, c.n, D)[:, 2048 + 64:]).all()
     # a signed permutation is rotated exactly by any arithmetic: codes must then be identical

@@ -4,8 +4,10 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import okq_oracle as O
 from paper_2609_11582_b200 import binding as B
 from paper_2609_11582_b200 import workloads as WL
+from tests import harness as Hn
 
 pytestmark = pytest.mark.gpu
 D, W = 128, 32
@@ -52,7 +54,7 @@ def test_guard_words_and_determinism():
     for l in range(L):
         k, v = WL.gen_kv(w, l, device=dev)
         B.quantize_keys(cache, l, k, signs[l])
-        B.quantize_values(cache, l, v, mod, R[l], bulk=(l == 1))     # one layer through each value path
+        B.quantize_values(cache, l, v, mod, R[l], bulk=(l == 1))     # one layer through each value entry point
     for s in range(3):                                               # crosses a window boundary: one flush
         kn, vn, mn = WL.gen_new_token(w, 0, s, device=dev)
         kn = kn.unsqueeze(0).expand(L, -1, -1, -1).contiguous(); vn = vn.unsqueeze(0).expand(L, -1, -1, -1).contiguous()
@@ -93,7 +95,7 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     """The tensor-core value quantiser with its first tile withheld and every wait limited to about ten milliseconds:
     each role's wait for that tile runs out, the kernel returns by itself and the device status word says
     ERR_TIMEOUT.  Nothing faults: the context stays usable, and the same call without the handicap then gives the
-    codes of the exact quantiser."""
+    oracle's codes."""
     w = WL.scaled(WL.WORKLOADS["layer7b"], batch=2)
     n = 1024 + 40
     dev = torch.device("cuda")
@@ -110,12 +112,12 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     B.quantize_values(cache, 0, vd, mod, R, bulk=True)
     torch.cuda.synchronize()
     assert cache.device_status() == 0
-    exact = B.Cache(1, w.batch, w.n_kv_heads, w.n_q_heads, 1088, device=dev)
-    B.quantize_values(exact, 0, vd, mod, R)
-    torch.cuda.synchronize()
-    ea, eb = B.cache_export(cache, 0), B.cache_export(exact, 0)
-    npk = (n // W) * W
-    assert torch.equal(ea["v_codes"][:, :, :npk], eb["v_codes"][:, :, :npk]) and torch.equal(ea["v_norm"][:, :, :npk], eb["v_norm"][:, :, :npk])
+    e = B.cache_export(cache, 0)
+    npk, U = (n // W) * W, w.batch * w.n_kv_heads
+    _, vq, _ = O.quantize_batch(Hn.u16(k).reshape(U, n, D), Hn.u16(v).reshape(U, n, D), mod.cpu().numpy(), WL.gen_signs(w, 0).numpy(),
+                                R[0].cpu().numpy(), unit_seq=np.repeat(np.arange(w.batch), w.n_kv_heads))
+    assert (e["v_codes"].cpu().numpy().reshape(U, -1, 32)[:, :npk] == vq["codes"]).all()
+    assert (Hn.u16(e["v_norm"]).reshape(U, -1)[:, :npk] == vq["norm"]).all()
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])

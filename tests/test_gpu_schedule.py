@@ -61,7 +61,7 @@ def test_bulk_prefill_then_decode(n, meta_format):
     cache = B.Cache(1, w.batch, w.n_kv_heads, w.n_q_heads, ((n + 31) // 32 + 2) * 32, meta_format=meta_format, schedule=CAP)
     modb = mod[None].repeat(w.batch, 1).contiguous().cuda()
     B.quantize_keys(cache, 0, k.cuda(), signs.cuda())
-    B.quantize_values(cache, 0, v.cuda(), modb, R.cuda()[None], bulk=(n % 2 == 0))   # both value quantisers
+    B.quantize_values(cache, 0, v.cuda(), modb, R.cuda()[None], bulk=(n % 2 == 0))   # both value entry points
     torch.cuda.synchronize()
     assert cache.device_status() == 0 and cache.seq_len.cpu().tolist() == [n] * w.batch
     got = _decode(cache, w, q, signs, R)
@@ -115,8 +115,8 @@ def test_append_equals_bulk_and_decode_at_every_step():
 
 @pytest.mark.parametrize("schedule", [B.SCHEDULE_WINDOW, CAP])
 def test_full_size_batched_call_equals_per_layer_calls(schedule):
-    """The 28-layer call runs the combine kernel in its four-sequences-per-block configuration, a single-layer call
-    in the one-sequence configuration (which the small cases above reach and check against the oracle).  Both must
+    """The 28-layer call runs the split-K pair with the combine kernel in its four-sequences-per-block configuration, a
+    single-layer call (8 sequences x 4 heads, about 512 windows each) whichever kernel the library takes for it.  Both must
     give the same attention output up to the rounding of a different split of the windows; repeated a few steps so
     that a timing-dependent fault between the sequence groups of a block would show (non-finite or far-off values)."""
     w = WL.WORKLOADS["step7b"]
@@ -179,7 +179,8 @@ def _check_sampled(cache, w, samples, kept, q, signs, R, mod_row, n, out, meta_f
 def test_middle_sized_grid_caption(meta_format):
     """Captioning schedule with 64 (head, four-sequence group, layer) combine blocks: fewer than SMs but too many for
     four column slices each, so the combine kernel runs one sequence per block over all output columns; every
-    sequence holds packed keys whose values are still raw, raw keys and raw values.  Against the oracle."""
+    sequence holds packed keys whose values are still raw, raw keys and raw values.  The split-K pair takes the call when the
+    workspace is the least it accepts; with the one the library asks for, one block per unit does.  Against the oracle."""
     w = WL.scaled(WL.WORKLOADS["step7b"], n_layers=8, n_tokens=1024 + 77)
     n, L, dev = w.n_tokens, w.n_layers, torch.device("cuda")
     cache = B.Cache(L, w.batch, w.n_kv_heads, w.n_q_heads, ((n + 31) // 32 + 2) * 32, device=dev, meta_format=meta_format, schedule=CAP)
@@ -198,14 +199,20 @@ def test_middle_sized_grid_caption(meta_format):
         for (sl, sb) in samples:
             if sl == l:
                 kept[(sl, sb)] = (k[sb], v[sb])
-    ws = torch.empty(B.decode_workspace_bytes(cache, L, 0), dtype=torch.uint8, device=dev)
-    out = torch.full((L, w.batch, w.n_q_heads, D), float("nan"), dtype=torch.float32, device=dev)
-    B.decode_attention(cache, 0, L, q.to(dev), d_signs, d_R, ws, out)
-    torch.cuda.synchronize()
-    assert cache.device_status() == 0
-    o = out.cpu().numpy().astype(np.float64)
-    assert np.isfinite(o).all()
-    _check_sampled(cache, w, samples, kept, q, signs, R, mod_cpu.numpy(), n, o, meta_format)
+    d_q = q.to(dev)
+
+    def call(ws):
+        out = torch.full((L, w.batch, w.n_q_heads, D), float("nan"), dtype=torch.float32, device=dev)
+        B.decode_attention(cache, 0, L, d_q, d_signs, d_R, ws, out)
+        torch.cuda.synchronize()
+        return out
+
+    for least in (True, False):
+        ws = Hn.decode_workspace(cache, L, 0, call if least else None)
+        o = call(ws).cpu().numpy().astype(np.float64)
+        assert Hn.ran_split_k(ws) == least and cache.device_status() == 0
+        assert np.isfinite(o).all()
+        _check_sampled(cache, w, samples, kept, q, signs, R, mod_cpu.numpy(), n, o, meta_format)
 
 
 @pytest.mark.parametrize("meta_format", [B.META_FP16, B.META_MXFP4])
