@@ -242,17 +242,6 @@ struct CombineSmem {
   int prefix[MAX_ENTRIES + 1];
 };
 
-// (stored m, s) at position p of a window's (m, s) planes, from its metadata in either format; the fp16 format's
-// m carries its position scale, the MXFP4 format decodes to the plain value
-__device__ __forceinline__ float2 window_meta_pos(const unsigned char* meta, int fmt, int p) {
-  if (fmt == FMT_FP16)
-    return make_float2(__half2float(reinterpret_cast<const __half*>(meta + OFF_KM)[p]),
-                       __half2float(reinterpret_cast<const __half*>(meta + OFF_KS)[p]));
-  const unsigned mn = (meta[p >> 1] >> (4 * (p & 1))) & 15u, sn = (meta[64 + (p >> 1)] >> (4 * (p & 1))) & 15u;
-  const int blk = (p >> 3) & 3;
-  return make_float2(mx_decode(mn, (int)meta[128 + blk] - 127), mx_decode(sn, (int)meta[132 + blk] - 127));
-}
-
 // NS: CTAs that share one (head, sequence group): each computes D / NS output columns (used when the grid
 // would otherwise leave most SMs idle; the merge is repeated by every slice, the matrix streaming is split)
 template <bool CAPTION, int NS, int SEQ>

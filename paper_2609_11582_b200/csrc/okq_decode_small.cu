@@ -417,7 +417,7 @@ template <int FMT>
 static int small_cluster(long long units, long long windows, long long piece_slots) {
   const int fit[5] = {small_clusters<FMT, 1>(), small_clusters<FMT, 2>(), small_clusters<FMT, 4>(), small_clusters<FMT, 8>(), small_clusters<FMT, 16>()};
   int best = 0;
-  double best_cost = 31.0 + 2.0 * (double)units * (double)windows / (148.0 * NWARP) + 0.04 * (double)units;
+  double best_cost = 31.0 + 2.0 * (double)units * (double)windows / ((double)sm_count() * NWARP) + 0.04 * (double)units;
   for (int i = 4; i >= 0; i--) {   // (of equals the largest cluster)
     if (fit[i] <= 0 || (units << i) * NWARP > piece_slots) continue;   // the warps' pieces have to fit the scratch
     const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * (1 << i) - 1) / (NWARP * (1 << i)));
