@@ -35,10 +35,10 @@ METRIC = "2-bit KV decode-attention effective HBM GB/s (packed-KV bytes per deco
 W_TOKENS = 32                      # tokens per window: one step in 32 packs a window ("flush")
 BYTES_PER_TOKEN_HEAD = 84          # 32 B key codes + 2 B key norm + 16 B (m, s) + 32 B value codes + 2 B value norm
 # dram__bytes_read.sum + dram__bytes_write.sum of one split-K decode launch, measured with ncu on a
-# 4-layer slice of the workload (176 MB of records, larger than L2) and divided by its token-heads;
-# traffic grows in proportion to the token-heads.  To be re-measured whenever the split-K kernel changes.
-NCU_DRAM_BYTES_PER_TOKEN_HEAD = 86.36
-NCU_DRAM_BYTES_PER_TOKEN_HEAD_MX = 74.82   # same capture with --meta mxfp4
+# 5-layer slice of the workload (220 MB of records, larger than L2; fewer layers take the one-launch kernel) and divided by
+# its token-heads; traffic grows in proportion to the token-heads.  To be re-measured whenever the split-K kernel changes.
+NCU_DRAM_BYTES_PER_TOKEN_HEAD = 87.75
+NCU_DRAM_BYTES_PER_TOKEN_HEAD_MX = 75.99   # same capture with --meta mxfp4
 
 
 def measured_peaks():
@@ -209,7 +209,7 @@ def run_prefill(args, w, B, dev, rank, emit=True):
 def run_ladder(args, B, dev, rank, emit=True):
     """Secondary measurement: the bit-width ladder entry points (K2V2 / K3V3 / K4V4 over the canonical bit-stream
     cache; a thread-block cluster per (sequence, KV head) in decode) and the TurboQuant codec,
-    on 256 sequences x 4 KV heads x 8192 tokens of the 7B layer shape (1024 thread blocks in decode).  GB/s of packed bytes read per decode."""
+    on 256 sequences x 4 KV heads x 8192 tokens of the 7B layer shape.  GB/s of packed bytes read per decode."""
     w = WL.scaled(WL.WORKLOADS["layer7b"], batch=256, name="layer7b[batch=256]")
     Bn, H, Hq, N = w.batch, w.n_kv_heads, w.n_q_heads, w.n_tokens
     k, v = WL.gen_kv(w, 0, device=dev)

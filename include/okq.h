@@ -150,14 +150,15 @@ okq_status okq_quantize_values(const okq_cache* cache, int32_t layer, const void
                                const float* R, int32_t n_R, void* stream);
 
 /*
- * Bulk (prefill) form of okq_quantize_values with the rotation z = R_m v on the tensor cores
- * (Eq. 6 as a dense [tokens x 128] x [128 x 128] product per modality; tcgen05.mma with R split
- * into two fp16 matrices and fp32 accumulation in tensor memory).  Same arguments, same stored
- * norms and the same stored codes, bit for bit: a coordinate that the tensor-core product leaves
- * within 2^-18 of a codebook threshold is recomputed with the fused-multiply-add chain of
- * okq_quantize_values before its code is taken.  If the tensor-core pipeline does not answer within a
- * bounded wait the device status word becomes OKQ_ERR_TIMEOUT and the remaining tiles are
- * skipped.
+ * Bulk (prefill) form of okq_quantize_values: the same kernel, which has the rotation z = R_m v on the
+ * tensor cores (Eq. 6 as a dense [tokens x 128] x [128 x 128] product per modality; tcgen05.mma with R split
+ * into two fp16 matrices and fp32 accumulation in tensor memory) and recomputes a coordinate within 2^-18
+ * of a codebook threshold, or all of them where R is no rotation, with the fused-multiply-add chain above:
+ * the stored norms and codes are those of the chain, bit for bit.  The difference is in strides that a
+ * tensor map cannot describe (zero, 2^40 bytes or more): okq_quantize_values then evaluates the chain
+ * itself, this call returns OKQ_ERR_UNSUPPORTED.  If the tensor-core pipeline does not answer within a
+ * bounded wait, in either call, the device status word becomes OKQ_ERR_TIMEOUT and the remaining tiles
+ * are skipped.
  */
 okq_status okq_quantize_values_bulk(const okq_cache* cache, int32_t layer, const void* v_fp16,
                                     const int64_t strides[3], int32_t n_tokens,
@@ -203,11 +204,15 @@ okq_status okq_append(const okq_cache* cache, int32_t layer, int32_t layer_count
  *   sm_scale   softmax scale, normally 1/sqrt(128)
  *   signs, R   as for okq_append
  *   workspace  device scratch of at least okq_decode_workspace_bytes(cache, layer_count, num_splits)
- *   num_splits 0 = one persistent CTA per SM, each owning an equal slice of the flattened
- *              (layer, sequence, head, window) axis; n > 0 = n CTAs per (sequence, KV head)
- *              on average (at most 1024 in total)
+ *   num_splits n > 0 = a split-K kernel with n CTAs per (sequence, KV head) on average (at most 1024 in
+ *              total), each owning an equal slice of the flattened (layer, sequence, head, window) axis, and a
+ *              combine kernel; 0 = the library's choice: that pair with one persistent CTA per SM, or, where it is
+ *              estimated to be faster, one launch in which a cluster of 1 to 16 CTAs has a (sequence, KV head)
  *   out        device float [layer_count][batch][n_q_heads][128]
  * A sequence with seq_len 0 yields zeros.
+ * With num_splits 0 the choice depends on the shape, the cache's capacity (not on the lengths) and, since the
+ * one launch needs room for its own partial sums, on workspace_bytes.  The ways differ in rounding: outputs are
+ * the same bit for bit from call to call with the same workspace size, capacity and lengths.
  */
 okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t layer_count,
                                 const void* q, float sm_scale, const float* signs, const float* R,
@@ -218,8 +223,8 @@ okq_status okq_decode_attention(const okq_cache* cache, int32_t layer, int32_t l
  * okq_decode_attention for callers that have no scratch buffer to give and no way to get
  * one: code running where cudaMalloc is off limits (inside a serving loop whose memory was
  * carved up at start-up, under a caching allocator that must not be bypassed, in a plugin
- * that is only handed its inputs and outputs).  The paper has no counterpart; this is the
- * same kernel pair with its split-K partials kept in a fixed OKQ_NOALLOC_SCRATCH_BYTES
+ * that is only handed its inputs and outputs).  The paper has no counterpart; these are the
+ * same kernels, chosen in the same way, with their partials kept in a fixed OKQ_NOALLOC_SCRATCH_BYTES
  * (64 MiB) array that is part of the library's device image, so every GPU that loads the
  * library carries those 64 MiB until the process exits.  The call allocates nothing: no
  * cudaMalloc, no cudaFree, no allocating library routine.
@@ -261,7 +266,8 @@ okq_status okq_decode_attention_simt(const okq_cache* cache, int32_t layer, int3
  * Profiling aid (the paper has no counterpart): until cleared with two nulls, every
  * okq_decode_attention call made by the calling thread records `before` on its stream
  * just ahead of the split-K kernel and `after` just behind it (ahead of the combine
- * kernel), so a benchmark can time the dominant kernel alone.  Both are cudaEvent_t
+ * kernel), so a benchmark can time the dominant kernel alone; around all of a call that
+ * takes one launch.  Both are cudaEvent_t
  * handles passed as void*, owned by the caller.
  */
 void okq_profile_events(void* before, void* after);

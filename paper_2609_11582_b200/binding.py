@@ -259,7 +259,7 @@ def decode_attention(cache: Cache, layer: int, layer_count: int, q, signs, R, wo
 
 def decode_attention_noalloc(cache: Cache, layer: int, layer_count: int, q, signs, R, out, n_R=1, sm_scale=None,
                              num_splits=0, stream=None):
-    """okq_decode_attention_noalloc: same result as decode_attention, scratch held inside the library
+    """okq_decode_attention_noalloc: decode_attention (bit for bit where the same kernel takes the call), scratch held inside the library
     (64 MiB per GPU, shared by all calls on that GPU; overlapping calls race).  Allocates nothing."""
     scale = HEAD_DIM ** -0.5 if sm_scale is None else sm_scale
     _check(lib().okq_decode_attention_noalloc(C.byref(cache.c), layer, layer_count, _ptr(q), scale, _ptr(signs),
@@ -268,12 +268,13 @@ def decode_attention_noalloc(cache: Cache, layer: int, layer_count: int, q, sign
 
 
 def decode_select(impl: int) -> int:
-    """Choose the split-K kernel of later decode calls (0: tcgen05, 1: mma.sync warp pairs, the default); returns the previous choice."""
+    """Choose the split-K kernel of later decode calls (0: tcgen05, 1: mma.sync, the default); returns the previous choice."""
     return lib().okq_decode_select(impl)
 
 
 def profile_events(before=None, after=None):
-    """Record two torch.cuda.Event objects around the split-K kernel of later decode calls (None clears)."""
+    """Record two torch.cuda.Event objects around the split-K kernel of later decode calls, or around all of a call that takes
+    one launch (None clears)."""
     lib().okq_profile_events(None if before is None else before.cuda_event, None if after is None else after.cuda_event)
 
 

@@ -22,12 +22,12 @@
 // A warp's registers hold the value sums of one modality in its rotated basis; tokens of another
 // modality inside its range are "visitors", whose products are added straight to the warp's piece
 // in global memory (vector reductions), as are the registers every FLUSH windows.
-// What bounds it: dispatch slots.  Per window a warp issues about 600 instructions (53 of them products); LOP3, PRMT,
+// What bounds it: dispatch slots.  Per window a warp issues about 650 instructions (53 of them products); LOP3, PRMT,
 // IMAD and HFMA2 take two dispatch cycles of an SM sub-partition each, a product 8.6 by itself and about 10 with the
 // masks that feed it, so more warps do not help: 12 per CTA with 168 registers each is where the accumulators, both
 // operand sets and the next window's scores fit without spills.  step7b (28 layers x 8 x 16384 tokens, 1.233 GB of
 // records), whole call: 570 us with a score and a value warp per window pair and two bit-plane products per 16 x 16
-// codes, 515 us in this form.  Two windows per turn (8 warps, 233 registers) measured 541 us, an unrolled pair of turns
+// codes, 517 us in this form.  Two windows per turn (8 warps, 233 registers) measured 541 us, an unrolled pair of turns
 // 594 us (the loop outgrows the instruction cache).
 // The grid is persistent: CTA i owns an equal slice of the flattened (layer, sequence, head,
 // window) axis, each of its warps an equal part of that slice, which the warp walks without any

@@ -1,7 +1,9 @@
 // OmniKVQuant at 2, 3 and 4 bits per code over a canonical cache (the bit-width ladder: K2V2 / K3V3 / K4V4).
-// Plain CUDA-core kernels that follow the 2-bit path's arithmetic with the number of levels changed:
+// The 2-bit path's arithmetic with the number of levels changed:
 //   k_ladder_keys    Eq. 2 + Eq. 4: one block per 32-token window of one (sequence, KV head)
-//   k_ladder_values  Eq. 6 + Eq. 3: likewise, the rotation as one fused-multiply-add chain per coordinate
+//   k_ladder_values  Eq. 6 + Eq. 3: likewise, the rotation as one fused-multiply-add chain per coordinate; only for strides that
+//                    a tensor map cannot describe, everything else takes the tensor-core kernel (okq_quant_tc.cu)
+//   k_turboquant_encode, k_turboquant_decode   the baseline codec
 // (decode attention: okq_ladder_decode.cu)
 // The value levels are the Lloyd-Max quantiser of N(0, 1/128) with 2^b levels (fixed point of: level = mean of its
 // cell, threshold = mid-point of neighbouring levels), held as constants.
