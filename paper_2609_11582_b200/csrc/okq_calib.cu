@@ -11,6 +11,7 @@
 
 #include "../../include/okq_calib.h"
 #include "okq_common.cuh"
+#include "okq_eigen.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -571,7 +572,7 @@ __device__ __forceinline__ void eig_apply(cg::cluster_group& cluster, EigV& sv) 
 
 __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __restrict__ C, const float* __restrict__ signs,
                                                            float* __restrict__ R, float* __restrict__ lambda,
-                                                           int* __restrict__ sweeps_out) {
+                                                           int* __restrict__ sweeps_out, const int* __restrict__ left) {
   extern __shared__ __align__(16) unsigned char eig_raw[];
   __shared__ double red[32];
   cg::cluster_group cluster = cg::this_cluster();
@@ -579,6 +580,8 @@ __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __rest
   EigV& sv = *reinterpret_cast<EigV*>(eig_raw);
   EigA<double>& sd = *reinterpret_cast<EigA<double>*>(eig_raw);
   EigA<float>& sf = *reinterpret_cast<EigA<float>*>(eig_raw);
+  depend_wait();
+  if (*left == 0) return;   // the direct solver has done it
   cluster.sync();   // every block runs before its shared memory is written from outside
   // largest magnitude (the matrix is scaled by a power of two to at most 1) and trace
   double mx = 0.0, tr = 0.0;
@@ -743,7 +746,6 @@ size_t attn_bytes(int group, int n) {
   return ((size_t)group * n * 2 + n_it * group * n) * sizeof(float);
 }
 size_t moments_bytes() { return (size_t)MAX_CHUNKS * 3 * D * D * sizeof(float) + 16; }
-constexpr size_t EIGEN_BYTES = (size_t)D * D * sizeof(double);
 
 }  // namespace
 }  // namespace okq
@@ -807,18 +809,13 @@ okq_status okq_calib_rotation(const float* C, const float* signs, void* workspac
     if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
     attr_done(attr_mask, attr_dev);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1 + V_CTAS);
-  cfg.blockDim = dim3(EIG_THREADS);
-  cfg.dynamicSmemBytes = EIG_SMEM;
-  cfg.stream = static_cast<cudaStream_t>(stream);
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = 1 + V_CTAS; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, k_calib_eigen, C, signs, R_out, lambda_out, sweeps_out);
-  if (le != cudaSuccess) { set_last_cuda_error((int)le); return OKQ_ERR_CUDA; }
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  double* ws = static_cast<double*>(workspace);
+  cudaError_t e = launch_calib_spectrum(C, signs, ws, R_out, lambda_out, sweeps_out, st);
+  if (e == cudaSuccess)
+    e = launch_dependent(k_calib_eigen, dim3(1 + V_CTAS), EIG_THREADS, EIG_SMEM, st, 1 + V_CTAS, C, signs, R_out, lambda_out, sweeps_out,
+                         reinterpret_cast<const int*>(ws + EIGEN_LEFT));
+  if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return launch_status();
 }
 
