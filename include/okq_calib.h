@@ -41,6 +41,12 @@ okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, i
                                        float sm_scale, int32_t causal, void* workspace, size_t workspace_bytes,
                                        float* w_out, void* stream);
 
+/* Testing aid for the bounded waits of okq_calib_attention_weights (the paper has no counterpart), as okq_debug_bulk_timeout is
+ * for the value quantiser: from 257 tokens on every block's first score tile is never delivered and every wait limited to
+ * `limit_clocks` SM clocks; scale 1 / sqrt(128), causal.  The weights of the blocks that gave up are NaN. */
+okq_status okq_debug_calib_timeout(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n, void* workspace,
+                                   size_t workspace_bytes, float* w_out, int64_t limit_clocks, void* stream);
+
 /*
  * C_m = sum_{j: modality_j = m} w_j v_j^T v_j for m = 0 (text), 1 (audio), 2 (video); ids > 2 count as text.
  *   v_fp16  fp16 [n][128], w  float [n] (>= 0), modality  uint8 [n], C_out  float [3][128][128]
@@ -52,13 +58,14 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
                              void* workspace, size_t workspace_bytes, float* C_out, void* stream);
 
 /*
- * Eigen-decomposition of one symmetric 128 x 128 matrix (cyclic Jacobi in fp64, one thread-block cluster) and
+ * Eigen-decomposition of one symmetric 128 x 128 matrix in fp64 (reduction to tridiagonal form, its eigenvalues and vectors,
+ * Newton-Schulz steps towards orthogonality; cyclic Jacobi where equal eigenvalues leave the vectors undetermined) and
  * R = H U^T with the ordering and sign convention stated above.
  *   C  float [128][128] (symmetric; only read), signs  float [128] (+-1)
  *   R_out  float [128][128] (row = rotated coordinate), lambda_out  float [128] (descending)
- *   workspace: at least 128 KB (checked; the solver keeps everything in shared memory).
- * The device status convention of okq.h does not apply: the iteration has a fixed sweep limit (30), which
- * a symmetric matrix does not reach; `sweeps_out` (device int32, may be null) receives the sweeps used.
+ *   workspace: at least 128 KB (checked).
+ * The device status convention of okq.h does not apply: the iterations have fixed limits (8 steps, 30 sweeps), which
+ * a symmetric matrix does not reach; `sweeps_out` (device int32, may be null) receives the steps or sweeps used.
  */
 okq_status okq_calib_rotation(const float* C, const float* signs, void* workspace, size_t workspace_bytes,
                               float* R_out, float* lambda_out, int32_t* sweeps_out, void* stream);

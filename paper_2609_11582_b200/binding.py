@@ -98,6 +98,9 @@ def lib():
         L.okq_calib_attention_weights.restype = C.c_int
         L.okq_calib_attention_weights.argtypes = [C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_float, C.c_int32,
                                                   C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p]
+        L.okq_debug_calib_timeout.restype = C.c_int
+        L.okq_debug_calib_timeout.argtypes = [C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_size_t, C.c_void_p,
+                                              C.c_int64, C.c_void_p]
         L.okq_calib_moments.restype = C.c_int
         L.okq_calib_moments.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t,
                                         C.c_void_p, C.c_void_p]
@@ -132,7 +135,7 @@ def exported_symbols():
             "okq_quantize_keys", "okq_quantize_values", "okq_append", "okq_decode_attention", "okq_cache_export",
             "okq_cache_import", "okq_profile_events", "okq_decode_select", "okq_decode_attention_simt",
             "okq_decode_attention_noalloc", "okq_quantize_values_bulk", "okq_debug_bulk_timeout", "okq_cache_export_mx",
-            "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_calib_moments", "okq_calib_rotation",
+            "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_debug_calib_timeout", "okq_calib_moments", "okq_calib_rotation",
             "okq_ladder_codebook", "okq_ladder_quantize_keys", "okq_ladder_quantize_values",
             "okq_debug_ladder_timeout", "okq_ladder_decode_attention", "okq_turboquant_encode", "okq_turboquant_decode"]
 
@@ -318,6 +321,15 @@ def calib_attention_weights(q, k, workspace, sm_scale=None, causal=True, stream=
     scale = HEAD_DIM ** -0.5 if sm_scale is None else sm_scale
     _check(lib().okq_calib_attention_weights(_ptr(q), _ptr(k), group, n, scale, 1 if causal else 0, _ptr(workspace),
                                              workspace.numel(), _ptr(w), _stream(stream)), "okq_calib_attention_weights")
+    return w
+
+
+def debug_calib_timeout(q, k, workspace, limit_clocks, stream=None):
+    """okq_debug_calib_timeout: the attention weights with every block's first tile withheld and waits limited to
+    `limit_clocks` SM clocks."""
+    w = torch.empty(q.shape[1], dtype=torch.float32, device=q.device)
+    _check(lib().okq_debug_calib_timeout(_ptr(q), _ptr(k), q.shape[0], q.shape[1], _ptr(workspace), workspace.numel(), _ptr(w),
+                                         limit_clocks, _stream(stream)), "okq_debug_calib_timeout")
     return w
 
 

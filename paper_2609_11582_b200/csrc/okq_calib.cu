@@ -10,6 +10,7 @@
 #include <cooperative_groups.h>
 
 #include "../../include/okq_calib.h"
+#include "okq_calib_scores.cuh"
 #include "okq_common.cuh"
 #include "okq_eigen.cuh"
 
@@ -762,23 +763,39 @@ size_t okq_calib_workspace_bytes(int32_t group, int32_t n) {
   return (b + 255) & ~(size_t)255;
 }
 
-okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n,
-                                       float sm_scale, int32_t causal, void* workspace, size_t workspace_bytes,
-                                       float* w_out, void* stream) {
+static okq_status attention_weights(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n, float sm_scale, int32_t causal,
+                                    void* workspace, size_t workspace_bytes, float* w_out, long long wait_limit, int skip_step, void* stream) {
   if (!q_fp16 || !k_fp16 || !w_out || !workspace || group <= 0 || n <= 0) return OKQ_ERR_INVALID_ARG;
   if (!aligned16(q_fp16) || !aligned16(k_fp16) || !aligned16(workspace) || !aligned16(w_out)) return OKQ_ERR_ALIGNMENT;
   if (workspace_bytes < attn_bytes(group, n)) return OKQ_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  float2* rowstat = static_cast<float2*>(workspace);
-  float* partial = reinterpret_cast<float*>(rowstat + (size_t)group * n);
-  const int grid = (n + TQ - 1) / TQ * group, n_sm = sm_count();
+  const int n_sm = sm_count();
   const __half* q = static_cast<const __half*>(q_fp16);
   const __half* k = static_cast<const __half*>(k_fp16);
   const float scale2 = sm_scale * 1.4426950408889634f;
+  if (n >= SCORE_MIN_TOKENS && scale2 > 0.f) {   // (a zero or negative scale: the kernels that take any)
+    const cudaError_t e = launch_calib_scores(q, k, group, n, scale2, causal, n_sm, workspace, w_out, wait_limit, skip_step, s);
+    if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
+    return OKQ_OK;
+  }
+  float2* rowstat = static_cast<float2*>(workspace);
+  float* partial = reinterpret_cast<float*>(rowstat + (size_t)group * n);
+  const int grid = (n + TQ - 1) / TQ * group;
   k_calib_pass<0><<<grid, 128, 0, s>>>(q, k, group, n, scale2, causal, n_sm, rowstat, partial);
   k_calib_pass<1><<<grid, 128, 0, s>>>(q, k, group, n, scale2, causal, n_sm, rowstat, partial);
   k_calib_wsum<<<(n + 31) / 32, 256, 0, s>>>(partial, group, n, causal, w_out);
   return launch_status();
+}
+
+okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n,
+                                       float sm_scale, int32_t causal, void* workspace, size_t workspace_bytes,
+                                       float* w_out, void* stream) {
+  return attention_weights(q_fp16, k_fp16, group, n, sm_scale, causal, workspace, workspace_bytes, w_out, 0, -1, stream);
+}
+
+okq_status okq_debug_calib_timeout(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n, void* workspace,
+                                   size_t workspace_bytes, float* w_out, int64_t limit_clocks, void* stream) {
+  return attention_weights(q_fp16, k_fp16, group, n, 0.08838834764831845f, 1, workspace, workspace_bytes, w_out, limit_clocks, 0, stream);
 }
 
 okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* modality, int32_t n,

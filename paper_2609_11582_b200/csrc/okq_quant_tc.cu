@@ -39,12 +39,11 @@
 // Every wait on an mbarrier is bounded; on a timeout the kernel records OKQ_ERR_TIMEOUT in the
 // cache's status word (the ladder, which has none: NaN in the value norms of the block's tokens, which decode hands on), stops
 // issuing work, frees its tensor memory and returns.
-#include <cuda.h>   // CUtensorMap and the type of cuTensorMapEncodeTiled only; the entry point is fetched at run time
-
 #include "okq_common.cuh"
 #include "okq_device.cuh"
 #include "okq_ladder.cuh"
 #include "okq_quant_tail.cuh"
+#include "okq_tc.cuh"
 
 namespace okq {
 
@@ -72,7 +71,6 @@ constexpr uint32_t magic_sum() {
   return s;
 }
 constexpr uint32_t MAGIC_SUM = magic_sum();
-constexpr long long WAIT_LIMIT_CLOCKS = 4000000000ll;   // about two seconds of SM clocks
 
 // A coordinate too close to a threshold for the tensor-core product to decide: recomputed with the reference
 // arithmetic at the end of the kernel (its code is patched in the record), so that the tile pipeline never waits for
@@ -120,13 +118,6 @@ template <int BITS> struct TcSmem {
   volatile int tmem_busy;                              // set if products may still be in flight at the end (tensor memory is then not released)
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred = 0;
-  asm volatile("{\n\t.reg .b32 rx;\n\t.reg .pred px;\n\telect.sync rx|px, 0xffffffff;\n\tselp.u32 %0, 1, 0, px;\n\t}\n" : "=r"(pred));
-  return pred != 0;
-}
-
 // shared-memory matrix descriptor: no swizzle, K-major; core matrices of 8 rows x 16 bytes,
 // `lbo` bytes between the two 8-element K chunks of one MMA, `sbo` bytes between 8-row groups
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
@@ -139,53 +130,10 @@ __device__ __forceinline__ uint32_t tile_off(int r, int k) {
   return (uint32_t)((k >> 3) * 2048 + (r >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
-// shared-memory matrix descriptor of a TMA-written tile: K-major, 128-byte swizzle (rows of 64 fp16 = 128
-// bytes, 8-row groups 1024 bytes apart; the leading-dimension field is not used by this layout)
-__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3fff) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-
 // byte offset of the 16-byte chunk holding channels [8 kc, 8 kc + 8) of token row r in a TMA-written value
 // tile: two halves of 64 channels, 128 bytes per row, chunk index xor-ed with the row inside its 8-row group
 __device__ __forceinline__ uint32_t vtile_off(int r, int kc) {
   return (uint32_t)((kc >> 3) * (TILE_BYTES / 2) + r * 128 + (((kc & 7) ^ (r & 7)) << 4));
-}
-
-// Bounded wait of a whole warp for one phase of an mbarrier (each try may suspend the thread for a short,
-// system-chosen time).  Gives up after about two seconds, or as soon as another role has given up; giving
-// up raises the abort flag.
-template <class SM>
-__device__ __forceinline__ bool mbar_wait(SM& sm, unsigned long long* bar, uint32_t parity) {
-  const uint32_t mbar = smem_u32(bar);
-  bool done = false;
-  const long long t0 = clock64();
-  while (!done) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-                 : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
-    done = ok != 0;
-    if (!done && (sm.abort || clock64() - t0 > sm.limit)) break;
-  }
-  if (!done) sm.abort = 1;
-  return __all_sync(0xffffffffu, done);   // called by whole warps: one answer per warp
-}
-// After a timeout: wait, again with a limit and whatever the abort flag says, for a phase that this warp's own
-// asynchronous work (bulk copies, tensor-core products) will complete.  Returns false if it did not.
-__device__ __forceinline__ bool mbar_drain(unsigned long long* bar, uint32_t parity) {
-  const uint32_t mbar = smem_u32(bar);
-  bool done = false;
-  const long long t0 = clock64();
-  while (!done && clock64() - t0 < WAIT_LIMIT_CLOCKS / 8) {   // a quarter of a second, whatever the caller's limit
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-                 : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
-    done = ok != 0;
-  }
-  return __all_sync(0xffffffffu, done);
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // the reference arithmetic: one fused-multiply-add chain, input index ascending
@@ -812,25 +760,6 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
   if (tid == 0 && sm.abort && cv.status) atomicCAS(cv.status, 0, (int)OKQ_ERR_TIMEOUT);
   if (warp == 0 && !sm.tmem_busy) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
 }
-
-namespace {
-
-using EncodeTiledFn = decltype(&cuTensorMapEncodeTiled);
-
-// cuTensorMapEncodeTiled, looked up through the runtime (no link against the driver library)
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-}  // namespace
 
 template <int BITS>
 static okq_status launch_values_tc(const CacheView& cv, const LadderView& lv, int layer, const __half* v, const int64_t strides[3],
