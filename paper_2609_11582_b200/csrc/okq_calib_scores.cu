@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
     P2 acc[16];                                // pass 1: sums of this thread's columns over the lane's queries
 #pragma unroll
     for (int i = 0; i < 16; i++) acc[i] = pk(0.f, 0.f);
+    float tot = 0.f;                           // ... of earlier steps, one column per lane
     int items = 0;
     auto row_stat = [&]() -> float2 {          // pass 1: of this lane's query in the current step
       const int i = cur.qtile() * TS + 32 * eq + lane;
@@ -255,14 +256,14 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
         const float mn = fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2);
         if (!edge || mn != -INFINITY) {
           const P2 neg = pk(-mn, -mn);
-          P2 s[2] = {pk(l * ex2a(m - mn), 0.f), pk(0.f, 0.f)};   // (0 for the first finite maximum)
+          P2 s[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};   // (on their own: a long sum takes one rounding per tile)
 #pragma unroll
           for (int c = 0; c < 16; c++) {
             const float2 x = up(pfma(pk(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), one2, neg));
             s[c & 1] = padd(s[c & 1], pk(ex2a(x.x), ex2a(x.y)));
           }
           const float2 u = up(padd(s[0], s[1]));
-          l = u.x + u.y;
+          l = fmaf(l, ex2a(m - mn), u.x + u.y);     // (a factor 0 for the first finite maximum)
           m = mn;
         }
         if (last) {
@@ -289,8 +290,9 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
           const float2 x = up(pfma(pk(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), two2, m2));
           acc[c] = pfma(pk(ex2a(x.x), ex2a(x.y)), c2, acc[c]);
         }
-        if (last) {
-          // over the lanes, each ending with one column: bits 4..0 of the column by lane bits 4..0
+        // over the lanes, each ending with one column: bits 4..0 of the column by lane bits 4..0.  Every 16 steps: the exchange is
+        // hidden behind the exponentials, and sums of 98 terms in one register cost a factor two in the error.
+        if (last || (i & 15) == 15) {
           float v[32];
 #pragma unroll
           for (int c = 0; c < 16; c++) { const float2 x = up(acc[c]); v[2 * c] = x.x; v[2 * c + 1] = x.y; acc[c] = pk(0.f, 0.f); }
@@ -304,7 +306,11 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
                 v[c] = keep + __shfl_xor_sync(0xffffffffu, give, w);
               }
           }
-          sm.col[items & 1][eq][32 * wq + lane] = v[0];
+          tot += v[0];
+        }
+        if (last) {
+          sm.col[items & 1][eq][32 * wq + lane] = tot;
+          tot = 0.f;
           asm volatile("bar.sync 1, %0;\n" ::"n"(NT) : "memory");
           const int c = 32 * wq + lane, j = t * TS + c;
           if (eq == 0 && j < n) {
