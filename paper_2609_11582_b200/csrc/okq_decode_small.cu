@@ -23,6 +23,20 @@ constexpr int KROW = D + 8;                     // halfs per staged raw key row:
 constexpr int KIMG = OFF_VCODE + 144;           // key part of a window record (+ its MXFP4 metadata bytes)
 constexpr int PC_MAX = 4;                       // packed windows among the raw-value tokens (captioning schedule)
 
+// What a CTA's block index and its sequence's length say, worked out in front of the windows' walk and read back from shared memory
+// behind it: the walk needs every register there is, and what lives across it is spilled in its loop (4 % of a call with several
+// windows per warp).
+struct __align__(16) Place {
+  int unit, rank, h, b, li, layer;
+  // tokens [0, v_pk) have packed values (and keys); of the rest, [v_pk, k_pk) have packed keys (captioning schedule only)
+  int v_pk, k_pk, nwin, n_tail, npc, n_rawk;
+  // The windows make `used` pieces of at most cnt windows, dealt out evenly over the CTAs (this one has [piece0, piece1)): one CTA
+  // filled after the other, 64 windows over 192 warps were one for every warp of five CTAs, three to a sub-partition's dispatch, and
+  // nothing for the rest (13.6 -> 11.6 us).  Fewer windows per piece, spread over all warps, is no better: what a warp does once,
+  // whatever its windows, is dispatch of the same SM.
+  int cnt, used, piece0, piece1;
+};
+
 struct PieceMeta { float m[GP], l[GP]; int held; };
 
 template <int FMT, int CS> struct SmallSmem {
@@ -53,6 +67,7 @@ template <int FMT, int CS> struct SmallSmem {
   // query fragments of the unit in mma A order, high and low parts: [kq][lane][r & 3], and the heads' scales
   __align__(16) uint32_t qhi[4][32][4], qlo[4][32][4];
   float fsc[GP];
+  Place at;
 };
 
 // Rotated query of head g as fragments in shared memory, by one warp with four channels per lane: the transform of
@@ -99,65 +114,82 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   const CacheView& cv = P.cv;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int unit = blockIdx.x / CS, rank = blockIdx.x % CS;
-  const int h = unit % cv.n_kv_heads, e = unit / cv.n_kv_heads, b = e % cv.batch, li = e / cv.batch, layer = P.layer0 + li;
   const int G = P.group;
   depend_wait();
-  const int seq = cv.seq_len[layer * cv.batch + b];
-  // tokens [0, v_pk) have packed values (and keys); of the rest, [v_pk, k_pk) have packed keys (captioning schedule only)
-  const int v_pk = cv.v_packed(seq), k_pk = cv.k_packed(seq), nwin = v_pk / W, n_tail = seq - v_pk;
-  const int npc = (k_pk - v_pk) / W, n_rawk = seq - k_pk;
-  const __half* qbase = P.q + (((size_t)li * cv.batch + b) * cv.n_q_heads + (size_t)h * G) * D;
-  const float* signs = P.signs + (size_t)li * D;
-  const __half* kt = cv.k_tail + cv.k_tail_off(layer, b, h);
-  const __half* vt = cv.v_tail + cv.v_tail_off(layer, b, h);
-
-  // ---- on their way from the start: queries and the first raw keys
-  for (int i = tid; i < G * (D / 8); i += NTHREADS) cp_async16(&sm.q[i / (D / 8)][8 * (i % (D / 8))], qbase + 8 * i);
-  for (int i = tid; i < min(W, n_rawk) * (D / 8); i += NTHREADS)
-    cp_async16(&sm.k0[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(k_pk + i / (D / 8)) * D + 8 * (i % (D / 8)));
-  cp_async_commit();
-
-  cluster.barrier_arrive();   // every CTA of the cluster runs before its shared memory is written from outside
-  // ---- this warp's windows
-  const int cnt = (nwin + CS * NWARP - 1) / (CS * NWARP);
-  const int gw = rank * NWARP + warp, w0 = min(nwin, gw * cnt), w1 = min(nwin, w0 + cnt);
-  WarpPiece* const pieces = P.pieces + (size_t)unit * (CS * NWARP);
   WalkEnd we{-INFINITY, 0.f, 0u};
-  auto queries = [&]() {   // the CTA's first eight warps, then everyone waits
-    if (warp < GP) head_fragments(qbase + warp * D, signs, P.sm_scale, warp, warp < G, lane, sm.qhi, sm.qlo, sm.fsc);
-    asm volatile("bar.sync 1, %0;\n" ::"n"(NTHREADS) : "memory");
-  };
-  if (w1 > w0) {
-    Segment sg;
-    sg.rec0 = cv.unit(layer, b, h);
-    sg.mod0 = cv.modality + (size_t)b * cv.capacity;
-    sg.w0 = w0;
-    sg.n_my = w1 - w0;
-    sg.piece = pieces + gw;
-    we = walk_segment<FMT>(sm.w[warp], reinterpret_cast<const uint4(*)[32]>(sm.qlo), sg, lane, [&](uint32_t (&qh)[16], float& fsc) {
-      queries();
-      fsc = sm.fsc[lane >> 2];
+  auto pieces_of = [](const Place& a) { return a.cnt > 1 ? (a.nwin + a.cnt - 1) / a.cnt : a.nwin; };
+  Place at;
+  {
+    at.unit = blockIdx.x / CS; at.rank = blockIdx.x % CS;
+    const int e = at.unit / cv.n_kv_heads;
+    at.h = at.unit % cv.n_kv_heads; at.b = e % cv.batch; at.li = e / cv.batch; at.layer = P.layer0 + at.li;
+    const int seq = cv.seq_len[at.layer * cv.batch + at.b];
+    at.v_pk = cv.v_packed(seq); at.k_pk = cv.k_packed(seq); at.nwin = at.v_pk / W; at.n_tail = seq - at.v_pk;
+    at.npc = (at.k_pk - at.v_pk) / W; at.n_rawk = seq - at.k_pk;
+    at.cnt = (at.nwin + CS * NWARP - 1) / (CS * NWARP);
+    at.used = CS > 1 ? pieces_of(at) : 0;   // (a single block's division can wait)
+    at.piece0 = at.used * at.rank / CS; at.piece1 = CS > 1 ? at.used * (at.rank + 1) / CS : NWARP;
+    if (CS > 1 && tid == 0) sm.at = at;
+    const __half* qbase = P.q + (((size_t)at.li * cv.batch + at.b) * cv.n_q_heads + (size_t)at.h * G) * D;
+    const float* signs = P.signs + (size_t)at.li * D;
+    const __half* kt = cv.k_tail + cv.k_tail_off(at.layer, at.b, at.h);
+
+    // ---- on their way from the start: queries and the first raw keys
+    for (int i = tid; i < G * (D / 8); i += NTHREADS) cp_async16(&sm.q[i / (D / 8)][8 * (i % (D / 8))], qbase + 8 * i);
+    for (int i = tid; i < min(W, at.n_rawk) * (D / 8); i += NTHREADS)
+      cp_async16(&sm.k0[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(at.k_pk + i / (D / 8)) * D + 8 * (i % (D / 8)));
+    cp_async_commit();
+
+    cluster.barrier_arrive();   // every CTA of the cluster runs before its shared memory is written from outside
+    // ---- this warp's windows
+    auto queries = [&]() {   // the CTA's first eight warps, then everyone waits
+      if (warp < GP) head_fragments(qbase + warp * D, signs, P.sm_scale, warp, warp < G, lane, sm.qhi, sm.qlo, sm.fsc);
+      asm volatile("bar.sync 1, %0;\n" ::"n"(NTHREADS) : "memory");
+    };
+    const int piece = at.piece0 + warp;
+    if (CS > 1 ? piece < at.piece1 : piece * at.cnt < at.nwin) {
+      Segment sg;
+      sg.rec0 = cv.unit(at.layer, at.b, at.h);
+      sg.mod0 = cv.modality + (size_t)at.b * cv.capacity;
+      sg.w0 = piece * at.cnt;
+      sg.n_my = min(at.cnt, at.nwin - sg.w0);
+      sg.piece = P.pieces + (size_t)at.unit * (CS * NWARP) + piece;
+      we = walk_segment<FMT>(sm.w[warp], reinterpret_cast<const uint4(*)[32]>(sm.qlo), sg, lane, [&](uint32_t (&qh)[16], float& fsc) {
+        queries();
+        fsc = sm.fsc[lane >> 2];
 #pragma unroll
-      for (int kq = 0; kq < 4; kq++) {
-        const uint4 x = *reinterpret_cast<const uint4*>(sm.qhi[kq][lane]);
-        qh[4 * kq] = x.x; qh[4 * kq + 1] = x.y; qh[4 * kq + 2] = x.z; qh[4 * kq + 3] = x.w;
-      }
-    });
+        for (int kq = 0; kq < 4; kq++) {
+          const uint4 x = *reinterpret_cast<const uint4*>(sm.qhi[kq][lane]);
+          qh[4 * kq] = x.x; qh[4 * kq + 1] = x.y; qh[4 * kq + 2] = x.z; qh[4 * kq + 3] = x.w;
+        }
+      });
+    } else {
+      queries();
+    }
+  }
+  if (CS > 1) {                    // (a single block, with less to keep: as they are)
+    asm volatile("" ::: "memory");   // (written in front of the warps' common barrier for the queries)
+    at = sm.at;
   } else {
-    queries();
+    at.used = at.piece1 = pieces_of(at);
   }
   cluster.barrier_wait();
   // ---- the piece's header goes to every CTA of the cluster
-  for (int r = 0; r < CS; r++) {
-    PieceMeta* pm = cluster.map_shared_rank(&sm.meta[gw], r);
-    if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
-    if (lane == 0) pm->held = (int)we.held;
-  }
+  if (at.piece0 + warp < at.piece1)
+    for (int r = 0; r < CS; r++) {
+      PieceMeta* pm = cluster.map_shared_rank(&sm.meta[at.piece0 + warp], r);
+      if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
+      if (lane == 0) pm->held = (int)we.held;
+    }
   cluster.barrier_arrive();   // (release: the pieces and their headers)
   cp_async_wait<0>();
   __syncthreads();            // the record rings are idle: their space holds the rest from here on
 
+  const int rank = at.rank, h = at.h, b = at.b, li = at.li, layer = at.layer;
+  const int v_pk = at.v_pk, k_pk = at.k_pk, nwin = at.nwin, n_tail = at.n_tail, npc = at.npc, n_rawk = at.n_rawk, used = at.used;
+  const __half* kt = cv.k_tail + cv.k_tail_off(layer, b, h);
+  const __half* vt = cv.v_tail + cv.v_tail_off(layer, b, h);
+  WarpPiece* const pieces = P.pieces + (size_t)at.unit * (CS * NWARP);
   // ---- rest of the tail, value rows and matrices
   for (int i = tid; i < (n_rawk - W) * (D / 8); i += NTHREADS)
     cp_async16(&af.k[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(k_pk + W + i / (D / 8)) * D + 8 * (i % (D / 8)));
@@ -240,7 +272,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   {
     const int j = tid & (GP - 1), stripe = tid / GP;
     float M = -INFINITY;
-    for (int p = stripe; p < SM::NP; p += NTHREADS / GP) M = fmaxf(M, sm.meta[p].m[j]);
+    for (int p = stripe; p < used; p += NTHREADS / GP) M = fmaxf(M, sm.meta[p].m[j]);
     for (int i = stripe; i < n_tail; i += NTHREADS / GP) M = fmaxf(M, af.tsc[i][j]);
     M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
     M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
@@ -251,7 +283,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     for (int w = 1; w < NWARP; w++) M = fmaxf(M, af.red[w][j]);
     __syncthreads();
     float L = 0.f;
-    for (int p = stripe; p < SM::NP; p += NTHREADS / GP) {
+    for (int p = stripe; p < used; p += NTHREADS / GP) {
       const float pm = sm.meta[p].m[j];
       const float f = pm == -INFINITY ? 0.f : exp2f(pm - M);
       af.fac[p][j] = f;
@@ -278,7 +310,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     constexpr int MT = C >= 16 ? C / 16 : 1, ITEMS = 3 * MT * 32, SHARES = ITEMS < NTHREADS ? NTHREADS / ITEMS : 1;
     static_assert(NTHREADS % ITEMS == 0 || ITEMS % NTHREADS == 0, "whole shares");
     const int share = tid / ITEMS;
-    const int used = cnt > 0 ? (nwin + cnt - 1) / cnt : 0;   // pieces beyond have no windows
 #pragma unroll
     for (int it0 = 0; it0 < ITEMS; it0 += NTHREADS) {        // (one round, two for a single block)
       const int it = ITEMS < NTHREADS ? tid % ITEMS : tid + it0;
