@@ -242,7 +242,9 @@ constexpr int MAX_CHUNKS = 64;     // token ranges (blocks) per modality
 // exponent e with 2^e >= max_j w_j (0 when all weights are 0): the weights are used as w_j * 2^-e <= 1
 __global__ void k_calib_wmax(const float* __restrict__ w, int n, int* __restrict__ e_out) {
   __shared__ float red[32];
+  depend_wait();
   float mx = 0.f;
+#pragma unroll 8
   for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, w[j]);
   for (int d = 16; d; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
@@ -256,7 +258,10 @@ __global__ void k_calib_wmax(const float* __restrict__ w, int n, int* __restrict
 }
 
 // grid (n_chunks, 3), 256 threads: block (chunk, m) adds the tokens of modality m in its token range into
-// a 128 x 128 partial moment matrix.  Warp w owns rows 16 w .. 16 w + 15 (all 128 columns).
+// a 128 x 128 partial moment matrix.  Warp w owns rows 16 w .. 16 w + 15 (all 128 columns).  A tile without a token of the modality
+// is left out: modalities come in runs, so a tile is mostly one block's.  Staging puts a tile's 32 tokens on the lanes, whose
+// transposed halves are then 64 contiguous bytes (channels on the lanes instead were sixteen stores on one bank).
+// 8192 tokens, the three kernels: 55 -> 23 us.
 __global__ void __launch_bounds__(256) k_calib_moments(const __half* __restrict__ v, const float* __restrict__ w,
                                                       const unsigned char* __restrict__ modality, int n, int n_chunks,
                                                       const int* __restrict__ w_exp, float* __restrict__ partial) {
@@ -265,6 +270,7 @@ __global__ void __launch_bounds__(256) k_calib_moments(const __half* __restrict_
   __shared__ __align__(16) __half xl[D * VT_STRIDE];    // w v, low fp16 term
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int chunk = blockIdx.x, m = blockIdx.y;
+  depend_wait();
   const int n_tiles = (n + MT - 1) / MT;
   const int per = (n_tiles + n_chunks - 1) / n_chunks;
   const int t_begin = chunk * per, t_end = min(n_tiles, t_begin + per);
@@ -275,16 +281,21 @@ __global__ void __launch_bounds__(256) k_calib_moments(const __half* __restrict_
 #pragma unroll
     for (int e = 0; e < 4; e++) acc[nt][e] = 0.f;
   for (int tile = t_begin; tile < t_end; tile++) {
+    const int j = tile * MT + lane;
+    bool mine = false;
+    if (j < n) {
+      unsigned mm = modality[j];
+      mm = mm > 2 ? 0 : mm;
+      mine = (int)mm == m;
+    }
+    if (!__any_sync(0xffffffffu, mine)) continue;   // (the same in every warp)
+    const float wj = mine ? w[j] * wscale : 0.f;
     __syncthreads();
-    for (int idx = tid; idx < MT * (D / 8); idx += 256) {
-      const int r = idx >> 4, c8 = idx & 15, j = tile * MT + r;
+#pragma unroll
+    for (int i = 0; i < D / 64; i++) {
+      const int r = lane, c8 = warp + 8 * i;
       uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-      float wj = 0.f;
-      if (j < n) {
-        unsigned mm = modality[j];
-        mm = mm > 2 ? 0 : mm;
-        if ((int)mm == m) { raw = *reinterpret_cast<const uint4*>(v + (size_t)j * D + c8 * 8); wj = w[j] * wscale; }
-      }
+      if (mine) raw = *reinterpret_cast<const uint4*>(v + (size_t)j * D + c8 * 8);
       const __half* hv = reinterpret_cast<const __half*>(&raw);
 #pragma unroll
       for (int u = 0; u < 8; u++) {
@@ -321,21 +332,32 @@ __global__ void __launch_bounds__(256) k_calib_moments(const __half* __restrict_
   }
 }
 
-// C = 2^e * (sum of the partial matrices in chunk order), made exactly symmetric.  One thread per element pair.
-__global__ void k_calib_csum(const float* __restrict__ partial, int n_chunks, const int* __restrict__ w_exp,
-                             float* __restrict__ C) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 3 * D * D) return;
-  const int m = idx / (D * D), a = (idx / D) % D, b = idx % D;
-  if (b < a) return;
+// C = 2^e * (sum of the partial matrices in chunk order), made exactly symmetric.  Block = a 32 x 32 tile on or above the diagonal of
+// one matrix, and its mirror image; 1024 threads, an element of each.
+__global__ void __launch_bounds__(1024) k_calib_csum(const float* __restrict__ partial, int n_chunks, const int* __restrict__ w_exp,
+                                                    float* __restrict__ C) {
+  __shared__ float mirror[32][33];
+  depend_wait();
+  const int m = blockIdx.y, r = threadIdx.x >> 5, c = threadIdx.x & 31;
+  int ta = 0, tb = blockIdx.x;                 // tile (ta, tb), ta <= tb
+  while (tb >= D / 32 - ta) { tb -= D / 32 - ta; ta++; }
+  tb += ta;
+  const float* p0 = partial + (size_t)m * D * D + (32 * ta + r) * D + 32 * tb + c;
+  const float* p1 = partial + (size_t)m * D * D + (32 * tb + r) * D + 32 * ta + c;
   float s0 = 0.f, s1 = 0.f;
-  for (int c = 0; c < n_chunks; c++) {
-    s0 += partial[((size_t)c * 3 + m) * D * D + a * D + b];
-    s1 += partial[((size_t)c * 3 + m) * D * D + b * D + a];
+#pragma unroll 8
+  for (int k = 0; k < n_chunks; k++) {
+    s0 += p0[(size_t)k * 3 * D * D];
+    s1 += p1[(size_t)k * 3 * D * D];
   }
-  const float val = 0.5f * (s0 + s1) * exp2f((float)*w_exp);
-  C[(size_t)m * D * D + a * D + b] = val;
-  C[(size_t)m * D * D + b * D + a] = val;
+  mirror[r][c] = s1;
+  __syncthreads();
+  const float val = 0.5f * (s0 + mirror[c][r]) * exp2f((float)*w_exp);
+  if (ta < tb || r <= c) C[(size_t)m * D * D + (32 * ta + r) * D + 32 * tb + c] = val;
+  __syncthreads();
+  mirror[r][c] = val;
+  __syncthreads();
+  if (ta < tb || r > c) C[(size_t)m * D * D + (32 * tb + r) * D + 32 * ta + c] = mirror[c][r];
 }
 
 // ---------------------------------------------------------------- eigenbasis and rotation
@@ -808,9 +830,12 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
   int* w_exp = reinterpret_cast<int*>(partial + (size_t)MAX_CHUNKS * 3 * D * D);
   const int n_tiles = (n + MT - 1) / MT;
   const int n_chunks = n_tiles < MAX_CHUNKS ? n_tiles : MAX_CHUNKS;
-  k_calib_wmax<<<1, 1024, 0, s>>>(w, n, w_exp);
-  k_calib_moments<<<dim3(n_chunks, 3), 256, 0, s>>>(static_cast<const __half*>(v_fp16), w, modality, n, n_chunks, w_exp, partial);
-  k_calib_csum<<<(3 * D * D + 255) / 256, 256, 0, s>>>(partial, n_chunks, w_exp, C_out);
+  cudaError_t e = launch_dependent(k_calib_wmax, dim3(1), 1024, 0, s, 1, w, n, w_exp);
+  if (e == cudaSuccess)
+    e = launch_dependent(k_calib_moments, dim3(n_chunks, 3), 256, 0, s, 1, static_cast<const __half*>(v_fp16), w, modality, n, n_chunks, w_exp, partial);
+  constexpr int TILES = D / 32 * (D / 32 + 1) / 2;
+  if (e == cudaSuccess) e = launch_dependent(k_calib_csum, dim3(TILES, 3), 1024, 0, s, 1, partial, n_chunks, w_exp, C_out);
+  if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return launch_status();
 }
 
