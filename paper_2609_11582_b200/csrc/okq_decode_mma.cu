@@ -211,6 +211,24 @@ constexpr int MRG_MAX = 8;                // partials per (sequence, head) whose
 constexpr int CB_CHUNK = 16;              // rows of a rotation matrix staged per step
 constexpr int CB_NBUF = 4;                // staged slices in flight (three ahead of the one in use)
 
+// the bf16 terms of two numbers, largest first: x = sum of the low halves, y = sum of the high halves, to 24 bits
+__device__ __forceinline__ void bf16_terms(float x, float y, uint32_t (&tm)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(tm[i]) : "f"(y), "f"(x));
+    x -= __uint_as_float(tm[i] << 16);
+    y -= __uint_as_float(tm[i] & 0xffff0000u);
+  }
+}
+__device__ __forceinline__ void mma16816_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
 // CAPTION: the captioning schedule keeps up to 159 raw values (and up to 127 raw keys) per sequence, and
 // the keys of the raw values' tokens may already be packed
 // SEQ: sequences per CTA (4 for full grids: the matrices are streamed once per four sequences; 1 when the
@@ -221,19 +239,21 @@ struct CombineSmem {
   static constexpr int TAIL = CAPTION ? CAPTION_V_SLOTS : W;   // most raw-value tokens of a sequence
   // ring of 16-row slices of the rotation matrices; with one sequence per block it is large enough for a quarter
   // of the columns of all three matrices, which the four-slice configuration fetches whole at the start
-  static constexpr int RBUF_FLOATS = SEQ == 1 ? 3 * D * (D / 4) : CB_NBUF * CB_CHUNK * D;
-  __align__(16) float Rbuf[RBUF_FLOATS];
+  static constexpr bool SPLIT = SEQ == CB_SEQ_MAX;   // the product with R_m^T on the tensor cores, from three bf16 terms
+  __align__(16) float Rbuf[SPLIT ? 4 : 3 * D * (D / 4)];
   // per partial and head: rescale factor, weight sums of the modalities (one-sequence blocks have room for the
   // partials of a long single sequence, which is spread over many CTAs of the split-K kernel)
   static constexpr int MRG_TAB = SEQ == 1 ? 64 : MRG_MAX;
   __align__(16) float mrg[CB_SEQ][MRG_TAB][GP][4];
-  __align__(16) float vec[3][CB_ROWS][D];     // merged rotated-basis sums, [modality][row][rotated channel]
+  __align__(16) float vec[SPLIT ? 1 : 3][SPLIT ? 1 : CB_ROWS][D];   // merged rotated-basis sums, [modality][row][rotated channel]
+  // or their terms, [term][row][modality * 128 + rotated channel]: rows of 784 bytes, an odd number of 16-byte columns
+  static constexpr int XP = 3 * D + 8, OUT_PITCH = D + 4;
+  __align__(16) unsigned short xs[SPLIT ? 3 : 1][SPLIT ? CB_ROWS : 1][XP];
+  static_assert(!SPLIT || 2 * CB_ROWS * OUT_PITCH * 4 <= (int)sizeof(xs), "the products of the two halves take the terms' place");
   __align__(16) float rawv[CB_ROWS][D];       // raw-tail contribution, [row][channel]
   // tail scores (log2 domain), then softmax numerators, [sequence][token][head]: blocks of several sequences keep
-  // them in the matrix ring, which is idle until the rotated sums are complete
-  static constexpr bool TSC_IN_RING = SEQ != 1;
-  static_assert(!TSC_IN_RING || CB_SEQ * TAIL * GP <= RBUF_FLOATS, "tail scores must fit the matrix ring");
-  __align__(16) float tsc_own[TSC_IN_RING ? 4 : CB_SEQ * TAIL * GP];
+  // them behind the tail scratch, where the terms of the rotated sums are written later
+  __align__(16) float tsc_own[SPLIT ? 4 : CB_SEQ * TAIL * GP];
   float Ms[CB_SEQ][GP], Ls[CB_SEQ][GP];
   float red[CB_SEQ][4][GP];   // per warp of a sequence: partial maxima / sums of the softmax bookkeeping
   // one-sequence blocks: the headers (m, l, weight sums) of the sequence's first MRG_TAB partials, fetched early
@@ -249,7 +269,12 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   constexpr int CB_SEQ = SEQ, CB_ROWS = SEQ * GP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CombineSmem<CAPTION, SEQ>& sm = *reinterpret_cast<CombineSmem<CAPTION, SEQ>*>(smem_raw);
-  float* const tsc_base = sm.TSC_IN_RING ? &sm.Rbuf[0] : &sm.tsc_own[0];
+  constexpr bool SPLIT = CombineSmem<CAPTION, SEQ>::SPLIT;
+  constexpr int KROW = D + 8;                              // halfs per staged key row
+  constexpr int KSM_FLOATS = W * KROW / 2, QSM_FLOATS = GP * D / 2;
+  float* const scratch = SPLIT ? reinterpret_cast<float*>(&sm.xs[0][0][0]) : &sm.vec[0][0][0];
+  float* const tsc_base = SPLIT ? scratch + CB_SEQ * (KSM_FLOATS + QSM_FLOATS) : &sm.tsc_own[0];
+  static_assert(!SPLIT || 4 * (CB_SEQ * (KSM_FLOATS + QSM_FLOATS) + CB_SEQ * sm.TAIL * GP) <= (int)sizeof(sm.xs), "tail scratch and scores must fit");
   auto tsc = [&](int b_, int i_) -> float* { return tsc_base + ((size_t)b_ * sm.TAIL + i_) * GP; };   // one token's eight heads
   const CacheView& cv = P.cv;
   const int h = blockIdx.x / NS, sl = blockIdx.x % NS, li = blockIdx.z, layer = P.layer0 + li;
@@ -272,11 +297,9 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   // tail (272-byte rows: 16-byte reads of 32 different rows hit different banks) or, under the captioning
   // schedule, the key parts of the up to four packed windows among the raw-value tokens; then the group's query
   // rows.  Everything is fetched with cp.async so that all the loads are in flight together.
-  constexpr int KROW = D + 8;                              // halfs per staged key row
-  constexpr int KSM_FLOATS = W * KROW / 2, QSM_FLOATS = GP * D / 2;
   constexpr int KIMG = OFF_VCODE + 144;                    // key part of a window record (+ its MXFP4 metadata bytes)
-  static_assert(CB_SEQ * (KSM_FLOATS + QSM_FLOATS) <= 3 * CB_ROWS * D && 4 * KIMG <= KSM_FLOATS * 4, "tail scratch must fit");
-  __half* ksm = reinterpret_cast<__half*>(&sm.vec[0][0][0] + bs * (KSM_FLOATS + QSM_FLOATS));
+  static_assert((SPLIT || CB_SEQ * (KSM_FLOATS + QSM_FLOATS) <= 3 * CB_ROWS * D) && 4 * KIMG <= KSM_FLOATS * 4, "tail scratch must fit");
+  __half* ksm = reinterpret_cast<__half*>(scratch + bs * (KSM_FLOATS + QSM_FLOATS));
   __half* qsm = ksm + W * KROW;
   unsigned char* kimg = reinterpret_cast<unsigned char*>(ksm);
   const int npc = CAPTION ? (k_pk - v_pk) / W : 0;   // packed windows among the raw-value tokens: the first chunks
@@ -573,11 +596,93 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
     }
 #pragma unroll
     for (int jj = 0; jj < 4; jj++) {
-      sm.vec[0][bs * GP + jg + jj][c] = vacc[jj][0];
-      sm.vec[1][bs * GP + jg + jj][c] = vacc[jj][1];
-      sm.vec[2][bs * GP + jg + jj][c] = vacc[jj][2];
+#pragma unroll
+      for (int m = 0; m < 3; m++) {
+        if constexpr (SPLIT) {
+          uint32_t tm[3];
+          bf16_terms(vacc[jj][m], 0.f, tm);
+#pragma unroll
+          for (int i = 0; i < 3; i++) sm.xs[i][bs * GP + jg + jj][m * D + c] = (unsigned short)tm[i];
+        } else {
+          sm.vec[m][bs * GP + jg + jj][c] = vacc[jj][m];
+        }
+      }
       sm.rawv[bs * GP + jg + jj][c] = araw[jg + jj];
     }
+  }
+
+  if constexpr (SPLIT) {
+    // out[row][c] = raw[row][c] + sum_m sum_r R_m[r][c] * vec[m][row][r] on the tensor cores: both factors as three bf16 terms (24
+    // bits, the exponents of fp32), the six products whose terms' orders add up to at most four.  A warp takes all 32 rows, 16
+    // columns and half of the 384 rotated channels; its share of the matrices comes straight from L2, a step ahead.  On CUDA cores the
+    // product was bound by shared memory (a 4 x 4 tile per thread: two multiply-adds per number read) at 24000 cycles a block;
+    // about half now.  28 layers x 8 sequences x 4 heads at 300 tokens, the whole call: 81.5 -> 68.8 us; 28 x 16 x 8 at 64: 180 -> 139.
+    __syncthreads();   // the terms are complete
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int kh = warp >> 3, n0 = 16 * (warp & 7);
+    const float* Rset = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D;
+    constexpr int KS = 3 * D / 16 / 2;   // 16-channel steps of a half
+    float acc[2][2][4];
+#pragma unroll
+    for (int m = 0; m < 2; m++)
+#pragma unroll
+      for (int n = 0; n < 2; n++)
+#pragma unroll
+        for (int i = 0; i < 4; i++) acc[m][n][i] = 0.f;
+    float rn[2][4];
+    auto fetch = [&](int ks) {
+#pragma unroll
+      for (int n = 0; n < 2; n++) {
+        const float* p = Rset + (size_t)(16 * ks + 2 * t) * D + n0 + 8 * n + g;
+        rn[n][0] = __ldg(p); rn[n][1] = __ldg(p + D); rn[n][2] = __ldg(p + 8 * D); rn[n][3] = __ldg(p + 9 * D);
+      }
+    };
+    fetch(kh * KS);
+    const unsigned short* arow = &sm.xs[0][lane & 15][8 * (lane >> 4)];
+    for (int ks = kh * KS; ks < (kh + 1) * KS; ks++) {
+      uint32_t b[2][2][3];
+#pragma unroll
+      for (int n = 0; n < 2; n++) {
+        bf16_terms(rn[n][0], rn[n][1], b[n][0]);
+        bf16_terms(rn[n][2], rn[n][3], b[n][1]);
+      }
+      if (ks + 1 < (kh + 1) * KS) fetch(ks + 1);
+#pragma unroll
+      for (int ta = 2; ta >= 0; ta--) {
+        uint32_t a[2][4];
+#pragma unroll
+        for (int m = 0; m < 2; m++) ldsm_x4(a[m], arow + (ta * CB_ROWS + 16 * m) * sm.XP + 16 * ks);
+#pragma unroll
+        for (int tb = 2 - ta; tb >= 0; tb--)
+#pragma unroll
+          for (int m = 0; m < 2; m++)
+#pragma unroll
+            for (int n = 0; n < 2; n++) mma16816_bf16(acc[m][n], a[m], b[n][0][tb], b[n][1][tb]);
+      }
+    }
+    __syncthreads();   // everyone has read the terms
+    float* half_out = reinterpret_cast<float*>(&sm.xs[0][0][0]) + kh * CB_ROWS * sm.OUT_PITCH;
+#pragma unroll
+    for (int m = 0; m < 2; m++)
+#pragma unroll
+      for (int n = 0; n < 2; n++)
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+          *reinterpret_cast<float2*>(&half_out[(16 * m + g + 8 * i) * sm.OUT_PITCH + n0 + 8 * n + 2 * t]) = make_float2(acc[m][n][2 * i], acc[m][n][2 * i + 1]);
+    __syncthreads();
+    const float* sums = reinterpret_cast<const float*>(&sm.xs[0][0][0]);
+    for (int i = threadIdx.x; i < CB_ROWS * D / 4; i += SEQ * 128) {
+      const int row = i / (D / 4), cl = 4 * (i % (D / 4)), ob = blockIdx.y * CB_SEQ + row / GP, j = row % GP;
+      if (ob >= cv.batch || j >= G) continue;
+      const float L = sm.Ls[row / GP][j];
+      const float inv = L > 0.f ? 1.0f / L : 0.f;
+      const float4 x = *reinterpret_cast<const float4*>(&sums[row * sm.OUT_PITCH + cl]);
+      const float4 y = *reinterpret_cast<const float4*>(&sums[(CB_ROWS + row) * sm.OUT_PITCH + cl]);
+      const float4 rv = *reinterpret_cast<const float4*>(&sm.rawv[row][cl]);
+      *reinterpret_cast<float4*>(&P.out[(((size_t)li * cv.batch + ob) * cv.n_q_heads + h * G + j) * D + cl]) =
+          make_float4((x.x + y.x + rv.x) * inv, (x.y + y.y + rv.y) * inv, (x.z + y.z + rv.z) * inv, (x.w + y.w + rv.w) * inv);
+    }
+    return;
   }
 
   // out[row][c] = raw[row][c] + sum_m sum_r R_m[r][c] * vec[m][row][r].  The first half of the threads compute
@@ -613,7 +718,6 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
     cp_async_wait<0>();
     __syncthreads();   // the matrices have landed and vec is complete
   } else {
-    if (sm.TSC_IN_RING) __syncthreads();   // everyone has read its softmax numerators: the ring takes matrices now
     if (!comp)
       for (int pre = 0; pre < CB_NBUF - 1; pre++) stage(pre);
   }
