@@ -810,12 +810,14 @@ static void combine_launch(const DecodeParams& P, int n_cta, cudaStream_t s) {
 
 template <bool CAPTION>
 static void combine_dispatch(const DecodeParams& P, int n_cta, cudaStream_t s) {
-  // full grids: four sequences per block, so that a layer's matrices are streamed once per four sequences;
-  // fewer such blocks than SMs: one sequence per block; a handful (e.g. a single-layer call): one sequence
-  // and a quarter of the output columns per block
+  // Four sequences per block, whose product runs on the tensor cores, wherever there are so many: 28 layers x 4 sequences x 4 heads at
+  // 2000 / 8192 tokens 89 / 163 us against 125 / 193 with one per block, 14 x 4 x 4 at 16384 163 against 167.  Two sequences fill half
+  // of such a block: worth it once there are blocks for half of the SMs (28 x 2 x 4 at 16384 tokens 160 against 167, 12 x 2 x 4 at
+  // 30000 138 against 134).  A single sequence per block otherwise, and a handful of blocks (e.g. a single-layer call) share it, a
+  // quarter of the output columns each.
   const int n_blocks = P.cv.n_kv_heads * ((P.cv.batch + CB_SEQ_MAX - 1) / CB_SEQ_MAX) * P.layer_count;
   if (4 * n_blocks <= n_cta) combine_launch<CAPTION, 4, 1>(P, n_cta, s);
-  else if (n_blocks <= n_cta) combine_launch<CAPTION, 1, 1>(P, n_cta, s);
+  else if (P.cv.batch < 2 || (P.cv.batch == 2 && 2 * n_blocks < n_cta)) combine_launch<CAPTION, 1, 1>(P, n_cta, s);
   else combine_launch<CAPTION, 1, CB_SEQ_MAX>(P, n_cta, s);
 }
 

@@ -118,3 +118,106 @@ def test_attention_weights_of_large_scores():
     w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(q.shape[0], 1000)).cpu().numpy().astype(np.float64)
     ref = CO.attention_weights(q.numpy().view(np.uint16), k.numpy().view(np.uint16), causal=True)
     assert np.linalg.norm(w - ref) <= 2.0 ** -20 * np.linalg.norm(ref), np.linalg.norm(w - ref) / np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,G,causal", [(256, 2, True), (257, 1, True), (383, 2, False), (384, 7, True), (385, 17, True), (640, 3, True),
+                                        (1025, 1, False), (2047, 1, True)])
+def test_attention_weights_at_the_edges_of_the_tiles(n, G, causal):
+    """Around the fewest tokens of the tensor-core form (257), whole and ragged tiles of 128, ranges of steps that cut query and key
+    tiles into pieces; the workspace is exactly as long as documented and nothing behind it is written.  A weight's error is that of
+    sums of a few hundred fp32 numbers: 2^-20 of the weights' norm."""
+    q, k, _, _, _ = _case(n, group=G)
+    nb = B.lib().okq_calib_workspace_bytes(G, n)
+    buf = torch.full((nb + 4096,), 0x5a, dtype=torch.uint8, device="cuda")
+    w = B.calib_attention_weights(q.cuda(), k.cuda(), buf[:nb], causal=causal)
+    again = B.calib_attention_weights(q.cuda(), k.cuda(), buf[:nb], causal=causal)
+    assert (buf[nb:] == 0x5a).all() and (w == again).all()
+    ref = CO.attention_weights(q.numpy().view(np.uint16), k.numpy().view(np.uint16), causal=causal)
+    assert np.linalg.norm(w.cpu().numpy() - ref) <= 2.0 ** -20 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("scale", [-0.05, 0.0, 0.3])
+def test_attention_weights_for_any_scale(scale):
+    q, k, _, _, _ = _case(300, group=2)
+    w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(2, 300), sm_scale=scale).cpu().numpy()
+    ref = CO.attention_weights(q.numpy().view(np.uint16), k.numpy().view(np.uint16), sm_scale=scale)
+    assert np.linalg.norm(w - ref) <= 2.0 ** -20 * np.linalg.norm(ref)
+
+
+def test_attention_weights_wait_that_runs_out_leaves_a_mark():
+    """With every block's first tile withheld the kernels return by themselves and the weights are NaN; the same call without the
+    handicap gives finite weights."""
+    q, k, _, _, _ = _case(1000)
+    ws = B.calib_workspace(q.shape[0], 1000)
+    w = B.debug_calib_timeout(q.cuda(), k.cuda(), ws, limit_clocks=20_000_000)
+    torch.cuda.synchronize()                      # returns: the kernels ended by themselves
+    assert w.isnan().all()
+    assert B.calib_attention_weights(q.cuda(), k.cuda(), ws).isfinite().all()
+
+
+def _matrices():
+    rng = np.random.default_rng(11)
+    had = np.array([[1.0]])
+    while had.shape[0] < D:
+        had = np.block([[had, had], [had, -had]])
+    Q, _ = np.linalg.qr(rng.standard_normal((D, D)))
+    x = rng.standard_normal((D, D))
+    low = rng.standard_normal((D, 9))
+    half = rng.standard_normal((64, 64))
+    spectrum = np.logspace(1, -2, D)
+    cluster = spectrum.copy()
+    cluster[40:60] = cluster[40]
+    off = np.eye(D, k=1) + np.eye(D, k=-1)
+    return {"definite": x @ x.T, "indefinite": x + x.T, "low rank": low @ low.T, "low rank + identity": low @ low.T + 2 * np.eye(D),
+            "zero": np.zeros((D, D)), "identity": np.eye(D), "diagonal, repeated": np.diag(rng.integers(0, 5, D).astype(float)),
+            "two equal blocks": np.kron(np.eye(2), half @ half.T), "cluster": (Q * cluster) @ Q.T, "graded": (Q * np.logspace(0, -30, D)) @ Q.T,
+            "tiny": x @ x.T * 1e-33, "huge": x @ x.T * 1e33, "ones": np.ones((D, D)), "pairs": np.diag(np.abs(np.arange(D) - 63.5)) + off,
+            "two eigenvalues": had, "one element": np.diag([3.0] + [0.0] * (D - 1))}
+
+
+@pytest.mark.parametrize("kind", list(_matrices()))
+def test_rotation_of_matrices_that_are_hard_for_a_solver(kind):
+    """Repeated and clustered eigenvalues (the direct solver leaves some of these to the Jacobi one), exhausted reductions, extreme
+    scales.  What is unique of the result - eigenvalues, residuals, orthogonality - to a few roundings of the fp32 outputs."""
+    C32 = torch.from_numpy(_matrices()[kind]).float().contiguous()
+    signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0)
+    ws = torch.empty(D * D * 8, dtype=torch.uint8, device="cuda")     # the documented 128 KB
+    R, lam, _ = B.calib_rotation(C32.cuda(), signs.cuda(), ws)
+    Cm = C32.numpy().astype(np.float64)
+    Cm = 0.5 * (Cm + Cm.T)
+    U = CO.hadamard_matrix(signs.numpy()).T @ R.cpu().numpy().astype(np.float64)      # rows: eigenvectors
+    lam = lam.cpu().numpy().astype(np.float64)
+    ref = np.linalg.eigvalsh(Cm)[::-1]
+    size = max(np.abs(ref).max(), 1e-300)
+    assert (np.diff(lam) <= 0).all()
+    assert np.abs(lam - ref).max() <= 2.0 ** -22 * size
+    assert np.abs(U @ U.T - np.eye(D)).max() <= 1e-6
+    assert np.abs(U @ Cm - lam[:, None] * U).max() <= 1e-6 * size
+
+
+def test_rotation_of_numbers_that_are_none_ends():
+    signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0).cuda()
+    ws = torch.empty(D * D * 8, dtype=torch.uint8, device="cuda")
+    for bad in (float("nan"), float("inf")):
+        C = torch.eye(D, device="cuda")
+        C[3, 4] = C[4, 3] = bad
+        B.calib_rotation(C, signs, ws)
+    R, lam, _ = B.calib_rotation(torch.eye(D, device="cuda"), signs, ws)
+    assert (lam == 1).all() and R.isfinite().all()
+
+
+@pytest.mark.parametrize("n,kind", [(31, "one"), (33, "alternating"), (64, "runs"), (2049, "runs"), (4133, "ids beyond two")])
+def test_moments_of_tiles_with_and_without_a_modality(n, kind):
+    _, _, v, mod, _ = _case(n)
+    if kind == "one":
+        mod = torch.full_like(mod, 2)
+    elif kind == "alternating":
+        mod = (torch.arange(n) % 3).to(torch.uint8)
+    elif kind == "ids beyond two":
+        mod = torch.where(torch.arange(n) % 700 < 350, torch.full_like(mod, 7), mod)
+    w = torch.linspace(0.0, 3.0, n)
+    C = B.calib_moments(v.cuda(), w.cuda(), mod.cuda(), B.calib_workspace(1, n)).cpu().numpy().astype(np.float64)
+    ref = CO.weighted_moments(v.numpy().view(np.uint16), w.numpy().astype(np.float64), mod.numpy())
+    for m in range(3):   # fp32 sums of n products of numbers split to 22 bits
+        assert np.abs(C[m] - ref[m]).max() <= 1e-5 * max(np.abs(ref[m]).max(), 1e-30)
+        assert (C[m] == C[m].T).all()

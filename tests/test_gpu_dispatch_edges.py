@@ -52,6 +52,32 @@ def test_one_launch_decode_captioning_schedule(meta, n, batch):
     Hn.assert_attention_close(outs[0], outs[1])
 
 
+# blocks of four sequences (more than 148 of them), the last one partly filled; no packed window, one, several; a full raw tail.
+# The matrices may be of any size: the combine kernel's product takes them as they are.
+@pytest.mark.parametrize("schedule", [B.SCHEDULE_WINDOW, B.SCHEDULE_CAPTION])
+@pytest.mark.parametrize("batch,group,n,size", [(5, 5, 31, 1.0), (6, 8, 32 * 9 + 31, 1.0), (7, 1, 32 * 12, 1e20), (8, 7, 32 * 9 + 1, 1e-20)])
+def test_combine_blocks_of_several_sequences(schedule, batch, group, n, size):
+    layers, heads, dev = 38, 2, torch.device("cuda")
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=heads * group, prefix_text=40, video_chunk=70, audio_chunk=21)
+    cache = B.Cache(layers, batch, heads, heads * group, 32 * 14, device=dev, schedule=schedule)
+    k, v = WL.gen_kv(w, 0, n_tokens=n)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(batch, 1).contiguous().to(dev)
+    signs = torch.stack([WL.gen_signs(w, l) for l in range(layers)]).to(dev)
+    R = torch.stack([WL.gen_rotations(w, l) for l in range(layers)])[:, None].contiguous().to(dev)
+    for l in range(layers):
+        B.quantize_keys(cache, l, k.to(dev).roll(l, dims=2), signs[l])
+        B.quantize_values(cache, l, v.to(dev).roll(l, dims=2), mod, R[l])
+    q = torch.stack([WL.gen_queries(w, l) for l in range(layers)]).to(dev)
+    out, ref = (torch.full((layers, batch, heads * group, D), float("nan"), device=dev) for _ in range(2))
+    B.decode_attention(cache, 0, layers, q, signs, size * R, Hn.decode_workspace(cache, layers, 2), out, num_splits=2)
+    one = Hn.decode_workspace(cache, 1)
+    for l in range(layers):   # the one-launch kernel, whose product is on CUDA cores
+        B.decode_attention(cache, l, 1, q[l], signs[l], size * R[l], one, ref[l])
+    outs = [x.cpu().numpy().astype(np.float64) for x in (out, ref)]
+    top = np.abs(outs[1]).max()
+    Hn.assert_attention_close(outs[0] / top, outs[1] / top)
+
+
 # clusters of 1, 2, 4 and 8 blocks (by units and windows); one window; more warps than windows
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("batch,n", [(1, 32), (1, 32 * 9), (12, 32 * 20), (38, 32 * 3)])
