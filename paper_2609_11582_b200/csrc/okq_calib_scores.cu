@@ -13,8 +13,9 @@
 // worker warps, four to each quarter of the lanes, 32 columns each.  The (tile, head) steps of a pass are numbered and cut
 // into equal ranges, one per block; what a range holds of a query or key tile is a piece, pieces are put together in order.
 //
-// What bounds it: one exponential per score and pass (16 per cycle and SM; 8192 tokens x 7 heads, causal: 51 us a pass), behind
-// it the workers' issue slots; the tensor pipe is a third busy.
+// What bounds it: one exponential per score and pass (16 per cycle and SM; 8192 tokens x 7 heads, causal: 51 us a pass), the units
+// for which are busy 73 % of the time; the tensor pipe is a third busy.  8192 tokens x 7 heads 578 -> 195 us against the mma.sync
+// kernels of okq_calib.cu, 512 x 7 39 -> 21 (most of it the four launches).
 #include "okq_calib_scores.cuh"
 #include "okq_tc.cuh"
 

@@ -7,9 +7,9 @@
 // 1 / CS of the rotated channels over all pieces.  The merged sums are pushed into every CTA's shared memory, and after
 // the second barrier each CTA applies R_m^T for 1 / CS of the output columns.  The raw tail is scored by every CTA (its
 // rows are staged at the start) while the first barrier is on its way.
-// What bounds it: latency (launch, query rotation, 4 to 10 windows per warp, two cluster barriers, L2 round trips of the
-// merge).  One sequence, one head group of seven, 2048 tokens: 59 -> 14 us per call; one layer of 4 sequences x 4 heads at
-// 4111 tokens 32 -> 18.5 us against the split-K pair.
+// What bounds it: latency (launch, query rotation, the first window of a warp, two cluster barriers, L2 round trips of the
+// merge).  One sequence, one head group of seven, 2048 tokens: 59 -> 11.3 us per call; one layer of 4 sequences x 4 heads at
+// 4111 tokens 32 -> 16.8 us against the split-K pair.
 #include <cooperative_groups.h>
 #include "okq_decode_walk.cuh"
 
@@ -40,7 +40,8 @@ struct __align__(16) Place {
 struct PieceMeta { float m[GP], l[GP]; int held; };
 
 template <int FMT, int CS> struct SmallSmem {
-  static constexpr int C = D / CS;              // output columns (and merged channels) of a CTA
+  static constexpr int MS = CS == 6 ? 4 : CS;   // CTAs that merge and write: the largest power of two
+  static constexpr int C = D / MS;              // output columns (and merged channels) of one of them
   static constexpr int NP = CS * NWARP;         // pieces of a unit
   static constexpr int KS = 2 * NTHREADS / C;   // row slices of the product (a thread takes two columns)
   static constexpr int TAIL = CAPTION_V_SLOTS;
@@ -107,7 +108,7 @@ __device__ __forceinline__ void head_fragments(const __half* qrow, const float* 
 template <int FMT, int CS>
 __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   using SM = SmallSmem<FMT, CS>;
-  constexpr int C = SM::C;
+  constexpr int C = SM::C, MS = SM::MS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SM& sm = *reinterpret_cast<SM*>(smem_raw);
   typename SM::After& af = sm.a;
@@ -174,14 +175,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     at.used = at.piece1 = pieces_of(at);
   }
   cluster.barrier_wait();
-  // ---- the piece's header goes to every CTA of the cluster
+  // ---- the piece's header goes to every merging CTA of the cluster
   if (at.piece0 + warp < at.piece1)
-    for (int r = 0; r < CS; r++) {
+    for (int r = 0; r < MS; r++) {
       PieceMeta* pm = cluster.map_shared_rank(&sm.meta[at.piece0 + warp], r);
       if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
       if (lane == 0) pm->held = (int)we.held;
     }
   cluster.barrier_arrive();   // (release: the pieces and their headers)
+  if (MS < CS && at.rank >= MS) {   // the rest is the merging CTAs'
+    cp_async_wait<0>();
+    cluster.barrier_wait();
+    cluster.sync();
+    return;
+  }
   cp_async_wait<0>();
   __syncthreads();            // the record rings are idle: their space holds the rest from here on
 
@@ -346,7 +353,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
       if (SHARES == 1 || tid < ITEMS) {
         constexpr float F = LEVEL_UNIT;
         const int ch = 16 * mu + (L32 >> 2);
-        for (int r = 0; r < CS; r++) {   // to every CTA of the cluster
+        for (int r = 0; r < MS; r++) {   // to every merging CTA of the cluster
           float* dst = CS == 1 ? &af.vec[0][0] : cluster.map_shared_rank(&af.vec[0][0], r);
           if (C >= 16 || (rank & 1) == 0) *reinterpret_cast<float2*>(dst + (m * D + ch) * GP + j0) = make_float2(v.x * F, v.y * F);
           if (C >= 16 || (rank & 1) == 1) *reinterpret_cast<float2*>(dst + (m * D + ch + 8) * GP + j0) = make_float2(v.z * F, v.w * F);
@@ -439,23 +446,27 @@ static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s
 }
 
 // Cluster size for a call, 0 if the split-K pair should take it: whichever of the estimates below is least.  A cluster per
-// unit, in waves of as many as run at once (on this GPU 7 clusters of 16, 15 of 8, 33 of 4, 74 of 2, 148 blocks: a cluster
+// unit, in waves of as many as run at once (on this GPU 7 clusters of 16, 15 of 8, 22 of 6, 33 of 4, 74 of 2, 148 blocks: a cluster
 // stays inside one of eight groups of SMs): 11.5 us a wave and 2.1 us per window of a warp.  The pair: 31 us, 2 us per window
 // of a warp with the windows balanced over all warps, 0.04 us per unit in the combine kernel.  Fitted to calls of 1 to 28
 // layers, 1 to 16 sequences, 1 to 8 heads and 200 to 32768 tokens.  Where a unit's windows spread over many blocks the pair costs
 // more than this says, its combine kernel merging that many partials per unit (one unit of 131072 tokens: 36 us estimated, 214
 // measured; four units: 50 and 75).  The host knows the capacity, not the lengths, and takes sequences to be full: a cache mostly
 // empty goes the way it would go full.
+// Clusters of six are for the 16 units of a layer of 4 sequences x 4 heads and a few more, one too many for clusters of eight: all six
+// blocks walk, four of them merge.
 template <int FMT>
 static int small_cluster(long long units, long long windows, long long piece_slots) {
-  const int fit[5] = {small_clusters<FMT, 1>(), small_clusters<FMT, 2>(), small_clusters<FMT, 4>(), small_clusters<FMT, 8>(), small_clusters<FMT, 16>()};
+  constexpr int SIZES = 6;
+  const int size[SIZES] = {1, 2, 4, 6, 8, 16};
+  const int fit[SIZES] = {small_clusters<FMT, 1>(), small_clusters<FMT, 2>(), small_clusters<FMT, 4>(), small_clusters<FMT, 6>(), small_clusters<FMT, 8>(), small_clusters<FMT, 16>()};
   int best = 0;
   double best_cost = 31.0 + 2.0 * (double)units * (double)windows / ((double)sm_count() * NWARP) + 0.04 * (double)units;
-  for (int i = 4; i >= 0; i--) {   // (of equals the largest cluster)
-    if (fit[i] <= 0 || (units << i) * NWARP > piece_slots) continue;   // the warps' pieces have to fit the scratch
-    const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * (1 << i) - 1) / (NWARP * (1 << i)));
+  for (int i = SIZES - 1; i >= 0; i--) {   // (of equals the largest cluster)
+    if (fit[i] <= 0 || units * size[i] * NWARP > piece_slots) continue;   // the warps' pieces have to fit the scratch
+    const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * size[i] - 1) / (NWARP * size[i]));
     const double cost = waves * (11.5 + 2.1 * walk);
-    if (cost < best_cost) { best_cost = cost; best = 1 << i; }
+    if (cost < best_cost) { best_cost = cost; best = size[i]; }
   }
   return best;
 }
@@ -472,7 +483,7 @@ static cudaError_t small_format(const DecodeParams& P, int units, cudaStream_t s
 
 okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s) {
   const int units = P.layer_count * P.cv.batch * P.cv.n_kv_heads;
-  const cudaError_t e = cs == 16 ? small_format<16>(P, units, s) : cs == 8 ? small_format<8>(P, units, s)
+  const cudaError_t e = cs == 16 ? small_format<16>(P, units, s) : cs == 8 ? small_format<8>(P, units, s) : cs == 6 ? small_format<6>(P, units, s)
                       : cs == 4 ? small_format<4>(P, units, s) : cs == 2 ? small_format<2>(P, units, s) : small_format<1>(P, units, s);
   if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return OKQ_OK;

@@ -14,7 +14,9 @@
 // left to the Jacobi solver, which needs no gaps: it runs behind this kernel and returns at once when there is nothing to do.
 //
 // Why: cyclic Jacobi is 11 to 13 sweeps of 127 dependent rounds of about a microsecond, whatever the number of SMs; the
-// reduction is 126 dependent steps of half a microsecond, and everything behind it is parallel over the vectors.
+// reduction is 126 dependent steps of 0.9 us, and everything behind it is parallel over the vectors.  One matrix 1506 -> 203 us
+// (cycles: reduction 214 000, eigenvalues 82 000, tridiagonal vectors 20 000, reflectors 40 000, Newton-Schulz 19 000, the rest 12 000);
+// a matrix that is left to the Jacobi solver pays both.
 #include <cooperative_groups.h>
 #include <type_traits>
 

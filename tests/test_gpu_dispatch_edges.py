@@ -28,6 +28,28 @@ def test_one_launch_decode_at_its_edges(batch, heads, n):
     Hn.assert_attention_close(got, c.gpu_decode(0, simt=True)[0])
 
 
+# 16 to 22 units: clusters of six, of which four blocks merge.  No window, one, fewer than the 72 warps, one more, several per warp
+@pytest.mark.parametrize("schedule", [B.SCHEDULE_WINDOW, B.SCHEDULE_CAPTION])
+@pytest.mark.parametrize("batch,heads,n", [(16, 1, 31), (5, 4, 32), (11, 2, 32 * 13 + 31), (4, 4, 32 * 73), (9, 2, 32 * 200 + 5)])
+def test_one_launch_decode_in_clusters_of_six(schedule, batch, heads, n):
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=7 * heads, prefix_text=40, video_chunk=70, audio_chunk=21)
+    dev = torch.device("cuda")
+    cache = B.Cache(1, batch, heads, 7 * heads, (n + W - 1) // W * W, device=dev, schedule=schedule,
+                    meta_format=B.META_MXFP4 if batch % 2 else B.META_FP16)
+    k, v = WL.gen_kv(w, 0, n_tokens=n)
+    signs, R = WL.gen_signs(w, 0).to(dev), WL.gen_rotations(w, 0)[None].contiguous().to(dev)
+    mod = WL.modality_layout(w, n).unsqueeze(0).repeat(batch, 1).contiguous().to(dev)
+    B.quantize_keys(cache, 0, k.to(dev), signs)
+    B.quantize_values(cache, 0, v.to(dev), mod, R)
+    q = WL.gen_queries(w, 0).to(dev)
+    outs = []
+    for splits in (0, 2):   # against the split-K pair
+        out = torch.full((1, batch, 7 * heads, D), float("nan"), device=dev)
+        B.decode_attention(cache, 0, 1, q, signs, R, Hn.decode_workspace(cache, 1, splits), out, num_splits=splits)
+        outs.append(out.cpu().numpy().astype(np.float64))
+    Hn.assert_attention_close(outs[0], outs[1])
+
+
 @pytest.mark.parametrize("meta", [B.META_FP16, B.META_MXFP4])
 @pytest.mark.parametrize("n", [100, 128, 128 + 159, 1024 + 127])
 @pytest.mark.parametrize("batch", [2, 40])   # clusters of 8, single blocks
