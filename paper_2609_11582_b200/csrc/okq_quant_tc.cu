@@ -194,8 +194,7 @@ struct TileMods {
   unsigned present;
   unsigned winmask[3];
 };
-__device__ __forceinline__ TileMods tile_mods(const unsigned char* mod, int lane) {
-  const uint32_t m4 = reinterpret_cast<const uint32_t*>(mod)[lane];   // 4 tokens per lane, window lane >> 3
+__device__ __forceinline__ TileMods tile_mods(uint32_t m4) {   // 4 tokens per lane, window lane >> 3
   TileMods t;
   t.present = 0;
 #pragma unroll
@@ -206,6 +205,9 @@ __device__ __forceinline__ TileMods tile_mods(const unsigned char* mod, int lane
     if (bal) t.present |= 1u << mm;
   }
   return t;
+}
+__device__ __forceinline__ TileMods tile_mods(const unsigned char* mod, int lane) {
+  return tile_mods(reinterpret_cast<const uint32_t*>(mod)[lane]);
 }
 // The tile's jobs in scalars (arrays indexed by a run-time value would live in local memory: 1000 cycles per tile and warp):
 // job 0 takes the first two modalities, job 1 the third one, if there is one.
@@ -324,25 +326,25 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     if (cwin0 >= tiles_per_unit * 4) { cwin0 = 0; if (++ch == cv.n_kv_heads) { ch = 0; cb++; } }
   };
 
+  // modality bytes of the current tile's tokens 4 lane .. 4 lane + 3 (255: no token)
+  auto tile_modality = [&]() -> uint32_t {
+    const int rows = min(TILE, (n_win - cwin0) * W);
+    uint32_t packed = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const int tok = 4 * lane + u;
+      unsigned m = 255;
+      if (tok < rows) { m = modality[(size_t)cb * n_tokens + (size_t)cwin0 * W + tok]; m = m > 2 ? 0 : m; }
+      packed |= m << (8 * u);
+    }
+    return packed;
+  };
+
   if (warp == 17) {
     // ------------------------------------------------------------------ loader warp
     // tile i of the range goes to buffer i & 1 once the buffer's previous tile (i - 2) has been released.
     // A lane carries the modality bytes of the tokens 4*lane .. 4*lane+3, fetched one tile ahead.
-    auto fetch_mod = [&](int i) -> uint32_t {
-      uint32_t packed = 0xffffffffu;
-      if (i < my_tiles) {
-        const int rows = min(TILE, (n_win - cwin0) * W);
-        packed = 0;
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-          const int tok = 4 * lane + u;
-          unsigned m = 255;
-          if (tok < rows) { m = modality[(size_t)cb * n_tokens + (size_t)cwin0 * W + tok]; m = m > 2 ? 0 : m; }
-          packed |= m << (8 * u);
-        }
-      }
-      return packed;
-    };
+    auto fetch_mod = [&](int i) -> uint32_t { return i < my_tiles ? tile_modality() : 0xffffffffu; };
     uint32_t mod_cur = fetch_mod(0);
     int armed = 0;   // tiles whose copies have been issued
     for (int i = 0; i < my_tiles; i++) {
@@ -445,6 +447,22 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
     Slots slots;
     uint32_t jobidx = 0;
     bool dead = false;
+    // A rotation matrix that a job needs is not resident: split R_m into fp16 hi + lo, laid out as the A
+    // operand (row = output channel, K = input channel).  Every MMA issued so far has completed (this warp
+    // has waited for each), and the job's own MMAs wait for slot_ready.
+    auto bring_matrices = [&](const TileJobs& jobs, int jt) {
+      const int key0 = (n_R == 1 ? 0 : ch) * 3;
+      if (slots.plan(jobs.count(jt), key0 + jobs.mod(jt, 0), key0 + jobs.mod(jt, 1))) {
+        if (slots.na) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 0)) * D * D, slots.sa, tid);
+        if (slots.nb) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 1)) * D * D, slots.sb, tid);
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // generic-proxy writes -> tensor-core reads
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.slot_ready);
+      }
+    };
+    // the first job's matrices before anything else: they are the longest way of a block's start (15000 of 70000 cycles for seven
+    // tiles), and behind the first tile's arrival and norms they came 5000 cycles later
+    if (my_tiles > 0) bring_matrices(TileJobs(tile_mods(tile_modality()).present), 0);
     for (int i = 0; i < my_tiles && !dead; i++) {
       const int buf = i & 1;
       const uint32_t par = (uint32_t)(i >> 1) & 1u;
@@ -499,19 +517,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_quantize_values_tc(const __grid_c
       for (int jt = 0; jt < jobs.n_jobs; jt++) {
         const int nm = jobs.count(jt);
         const uint32_t a = jobidx & 1u;
-        {
-          // A rotation matrix this job needs is not resident: split R_m into fp16 hi + lo, laid out as the A
-          // operand (row = output channel, K = input channel).  Every MMA issued so far has completed (this warp
-          // has waited for each), and the job's own MMAs wait for slot_ready.
-          const int key0 = (n_R == 1 ? 0 : ch) * 3;
-          if (slots.plan(nm, key0 + jobs.mod(jt, 0), key0 + jobs.mod(jt, 1))) {
-            if (slots.na) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 0)) * D * D, slots.sa, tid);
-            if (slots.nb) write_matrix<BITS>(sm, R + (size_t)(key0 + jobs.mod(jt, 1)) * D * D, slots.sb, tid);
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // generic-proxy writes -> tensor-core reads
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.slot_ready);
-          }
-        }
+        if (i > 0 || jt > 0) bring_matrices(jobs, jt);
         if (!mbar_wait(sm, &sm.mma_done[a], (jobidx >> 1) & 1u)) { dead = true; break; }
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const bool last_job = jt + 1 == jobs.n_jobs;
