@@ -2,11 +2,13 @@
 //
 //   k_calib_pass<0>, <1>          alpha = softmax(q k^T * scale) in 128 x 64 tiles on the tensor cores
 //                                 (mma.sync, fp16 products, fp32 sums): first the row maximum and
-//                                 normaliser, then the column sums of alpha^2
+//                                 normaliser, then the column sums of alpha^2; sequences of up to 256 tokens and
+//                                 scales that are not positive (the others: okq_calib_scores.cu)
 //   k_calib_wsum                  w_j: fixed-order sum of the per-(query tile, head) column sums
 //   k_calib_wmax, k_calib_moments C_m = sum w_j v_j^T v_j, tensor cores, values staged transposed
 //   k_calib_csum                  fixed-order sum of the per-chunk partial moments
-//   k_calib_eigen                 cyclic Jacobi (fp64, one cluster), ordering, signs, R = H U^T
+//   k_calib_eigen                 cyclic Jacobi (fp64, one cluster), ordering, signs, R = H U^T, for the matrices
+//                                 that the direct solver (okq_eigen.cu) leaves
 #include <cooperative_groups.h>
 
 #include "../../include/okq_calib.h"

@@ -171,12 +171,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   if (CS > 1) {                    // (a single block, with less to keep: as they are)
     asm volatile("" ::: "memory");   // (written in front of the warps' common barrier for the queries)
     at = sm.at;
-  } else {
-    at.used = at.piece1 = pieces_of(at);
   }
   cluster.barrier_wait();
   // ---- the piece's header goes to every merging CTA of the cluster
-  if (at.piece0 + warp < at.piece1)
+  if (CS == 1 || at.piece0 + warp < at.piece1)   // (a single block: all of its warps, those without windows too)
     for (int r = 0; r < MS; r++) {
       PieceMeta* pm = cluster.map_shared_rank(&sm.meta[at.piece0 + warp], r);
       if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
@@ -193,7 +191,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   __syncthreads();            // the record rings are idle: their space holds the rest from here on
 
   const int rank = at.rank, h = at.h, b = at.b, li = at.li, layer = at.layer;
-  const int v_pk = at.v_pk, k_pk = at.k_pk, nwin = at.nwin, n_tail = at.n_tail, npc = at.npc, n_rawk = at.n_rawk, used = at.used;
+  const int v_pk = at.v_pk, k_pk = at.k_pk, nwin = at.nwin, n_tail = at.n_tail, npc = at.npc, n_rawk = at.n_rawk, n_meta = CS == 1 ? SM::NP : at.used;
   const __half* kt = cv.k_tail + cv.k_tail_off(layer, b, h);
   const __half* vt = cv.v_tail + cv.v_tail_off(layer, b, h);
   WarpPiece* const pieces = P.pieces + (size_t)at.unit * (CS * NWARP);
@@ -279,7 +277,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   {
     const int j = tid & (GP - 1), stripe = tid / GP;
     float M = -INFINITY;
-    for (int p = stripe; p < used; p += NTHREADS / GP) M = fmaxf(M, sm.meta[p].m[j]);
+    for (int p = stripe; p < n_meta; p += NTHREADS / GP) M = fmaxf(M, sm.meta[p].m[j]);
     for (int i = stripe; i < n_tail; i += NTHREADS / GP) M = fmaxf(M, af.tsc[i][j]);
     M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));
     M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
@@ -290,7 +288,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     for (int w = 1; w < NWARP; w++) M = fmaxf(M, af.red[w][j]);
     __syncthreads();
     float L = 0.f;
-    for (int p = stripe; p < used; p += NTHREADS / GP) {
+    for (int p = stripe; p < n_meta; p += NTHREADS / GP) {
       const float pm = sm.meta[p].m[j];
       const float f = pm == -INFINITY ? 0.f : exp2f(pm - M);
       af.fac[p][j] = f;
@@ -317,6 +315,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
     constexpr int MT = C >= 16 ? C / 16 : 1, ITEMS = 3 * MT * 32, SHARES = ITEMS < NTHREADS ? NTHREADS / ITEMS : 1;
     static_assert(NTHREADS % ITEMS == 0 || ITEMS % NTHREADS == 0, "whole shares");
     const int share = tid / ITEMS;
+    const int used = CS == 1 ? pieces_of(at) : at.used;
 #pragma unroll
     for (int it0 = 0; it0 < ITEMS; it0 += NTHREADS) {        // (one round, two for a single block)
       const int it = ITEMS < NTHREADS ? tid % ITEMS : tid + it0;
