@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
     for (int i = 0; i < 16; i++) acc[i] = pk(0.f, 0.f);
     float tot = 0.f;                           // ... of earlier steps, one column per lane
     int items = 0;
+    const int ragged = n % TS ? n / TS : -1;   // the tile that is not full
     auto row_stat = [&]() -> float2 {          // pass 1: of this lane's query in the current step
       const int i = cur.qtile() * TS + 32 * eq + lane;
       return i < n ? __ldcg(&stat[(size_t)cur.head * n + i]) : make_float2(0.f, 0.f);
@@ -239,11 +240,11 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.acc_free[a]);
-      // scores that do not count: keys after the query, rows of no token
-      const bool edge = (causal && qt == kt) || (PASS == 0 && (kt + 1) * TS > n);
+      // scores that do not count: keys after the query, rows of no token (zero queries, whose products with infinite keys are NaN)
+      const bool edge = (causal && qt == kt) || (PASS == 0 ? kt : qt) == ragged;
       if (edge) {
         const int row = qt * TS + 32 * eq + lane, j0 = kt * TS + 32 * wq;
-        const int seen = min(causal ? row + 1 : n, n) - j0;
+        const int seen = (row < n ? (causal ? row + 1 : n) : 0) - j0;
 #pragma unroll
         for (int c = 0; c < 32; c++)
           if (c >= seen) r[c] = 0xff800000u;   // -inf
@@ -256,7 +257,8 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
         for (int c = 4; c < 32; c++) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(r[c]));
         const float mn = fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2);
         if (!edge || mn != -INFINITY) {
-          const P2 neg = pk(-mn, -mn);
+          const float at = mn == -INFINITY ? 0.f : mn;   // (whole tiles of infinite keys: every term is 0)
+          const P2 neg = pk(-at, -at);
           P2 s[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};   // (on their own: a long sum takes one rounding per tile)
 #pragma unroll
           for (int c = 0; c < 16; c++) {
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
             s[c & 1] = padd(s[c & 1], pk(ex2a(x.x), ex2a(x.y)));
           }
           const float2 u = up(padd(s[0], s[1]));
-          l = fmaf(l, ex2a(m - mn), u.x + u.y);     // (a factor 0 for the first finite maximum)
+          l = fmaf(l, ex2a(m - at), u.x + u.y);     // (a factor 0 for the first finite maximum)
           m = mn;
         }
         if (last) {

@@ -144,6 +144,24 @@ def test_attention_weights_for_any_scale(scale):
     assert np.linalg.norm(w - ref) <= 2.0 ** -20 * np.linalg.norm(ref)
 
 
+def infinite_keys(n, G):
+    """Queries whose channel 5 is negative, keys 64 .. 127 infinite in it: their scores are -inf and they get no weight."""
+    g = torch.Generator().manual_seed(n)
+    q, k = torch.randn(G, n, D, generator=g).half(), torch.randn(n, D, generator=g).half()
+    q[..., 5] = -q[..., 5].abs() - 0.01
+    k[64:128, 5] = float("inf")
+    return q, k
+
+
+@pytest.mark.parametrize("n,causal", [(257, False), (300, True), (512, True), (640, False)])
+def test_attention_weights_of_infinite_keys(n, causal):
+    q, k = infinite_keys(n, 3)
+    w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(3, n), causal=causal).cpu().numpy()
+    ref = CO.attention_weights(q.numpy().view(np.uint16), k.numpy().view(np.uint16), causal=causal)
+    assert (w[64:128] == 0).all()
+    assert np.linalg.norm(w - ref) <= 2.0 ** -20 * np.linalg.norm(ref)
+
+
 def test_attention_weights_wait_that_runs_out_leaves_a_mark():
     """With every block's first tile withheld the kernels return by themselves and the weights are NaN; the same call without the
     handicap gives finite weights."""
