@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
     asm volatile("cp.async.wait_group 1;\n" ::);
     __syncthreads();
     const __half* kt = ks[jt & 1];
-    // masks matter on the last tiles only
-    const bool edge = (jt + 1) * TK > n || (causal && (jt + 1) * TK - 1 > itile * TQ + warp * 32);
+    // masks matter on the last tiles only (and in rows of no token: their zero queries times infinite keys are NaN)
+    const bool edge = (jt + 1) * TK > n || itile * TQ + warp * 32 + 32 > n || (causal && (jt + 1) * TK - 1 > itile * TQ + warp * 32);
 #pragma unroll
     for (int half = 0; half < 2; half++) {   // 32 keys at a time
       float d[2][4][4];

@@ -153,7 +153,7 @@ def infinite_keys(n, G):
     return q, k
 
 
-@pytest.mark.parametrize("n,causal", [(257, False), (300, True), (512, True), (640, False)])
+@pytest.mark.parametrize("n,causal", [(200, True), (133, False), (256, True), (257, False), (300, True), (512, True), (640, False)])
 def test_attention_weights_of_infinite_keys(n, causal):
     q, k = infinite_keys(n, 3)
     w = B.calib_attention_weights(q.cuda(), k.cuda(), B.calib_workspace(3, n), causal=causal).cpu().numpy()
