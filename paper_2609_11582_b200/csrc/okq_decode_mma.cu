@@ -614,9 +614,12 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   if constexpr (SPLIT) {
     // out[row][c] = raw[row][c] + sum_m sum_r R_m[r][c] * vec[m][row][r] on the tensor cores: both factors as three bf16 terms (24
     // bits, the exponents of fp32), the six products whose terms' orders add up to at most four.  A warp takes all 32 rows, 16
-    // columns and half of the 384 rotated channels; its share of the matrices comes straight from L2, a step ahead.  On CUDA cores the
+    // columns and half of the 384 rotated channels; its share of the matrices comes straight from L2, a step ahead.  The products of
+    // a step of 16 channels are summed on the tensor cores, small ones first, the steps with rounded additions: the tensor cores cut
+    // their sums off, and one accumulator for all 72 products was 6.6e-7 too small (error 8.1e-7 of the output's norm; 8e-8 this way,
+    // 2.1e-7 a chain of fp32 multiply-adds), for 1 to 2 % of a small call.  On CUDA cores the
     // product was bound by shared memory (a 4 x 4 tile per thread: two multiply-adds per number read) at 24000 cycles a block;
-    // about half now.  28 layers x 8 sequences x 4 heads at 300 tokens, the whole call: 81.5 -> 68.8 us; 28 x 16 x 8 at 64: 180 -> 139.
+    // about half now.  28 layers x 8 sequences x 4 heads at 300 tokens, the whole call: 81.9 -> 70.6 us; 28 x 16 x 8 at 64: 181 -> 142.
     __syncthreads();   // the terms are complete
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int kh = warp >> 3, n0 = 16 * (warp & 7);
@@ -648,16 +651,25 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
       }
       if (ks + 1 < (kh + 1) * KS) fetch(ks + 1);
 #pragma unroll
-      for (int ta = 2; ta >= 0; ta--) {
-        uint32_t a[2][4];
+      for (int m = 0; m < 2; m++) {
+        float part[2][4];
 #pragma unroll
-        for (int m = 0; m < 2; m++) ldsm_x4(a[m], arow + (ta * CB_ROWS + 16 * m) * sm.XP + 16 * ks);
+        for (int n = 0; n < 2; n++)
 #pragma unroll
-        for (int tb = 2 - ta; tb >= 0; tb--)
+          for (int i = 0; i < 4; i++) part[n][i] = 0.f;
 #pragma unroll
-          for (int m = 0; m < 2; m++)
+        for (int ta = 2; ta >= 0; ta--) {
+          uint32_t a[4];
+          ldsm_x4(a, arow + (ta * CB_ROWS + 16 * m) * sm.XP + 16 * ks);
 #pragma unroll
-            for (int n = 0; n < 2; n++) mma16816_bf16(acc[m][n], a[m], b[n][0][tb], b[n][1][tb]);
+          for (int tb = 2 - ta; tb >= 0; tb--)
+#pragma unroll
+            for (int n = 0; n < 2; n++) mma16816_bf16(part[n], a, b[n][0][tb], b[n][1][tb]);
+        }
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+#pragma unroll
+          for (int i = 0; i < 4; i++) acc[m][n][i] += part[n][i];
       }
     }
     __syncthreads();   // everyone has read the terms

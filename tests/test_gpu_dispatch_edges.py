@@ -100,6 +100,38 @@ def test_combine_blocks_of_several_sequences(schedule, batch, group, n, size):
     Hn.assert_attention_close(outs[0] / top, outs[1] / top)
 
 
+# The combine kernel's product with R_m^T by itself: from the outputs with identity matrices and with none (the raw tail alone) follow the
+# rotated sums, and from those in 64 bits the outputs for any other matrices.  Bound: four units in the last place of fp32, norm over
+# norm; a chain of rounded fp32 multiply-adds has 2.1e-7 of it, a lost third bf16 term would be 2^-17.
+@pytest.mark.parametrize("schedule,batch,group,layers,mod_id", [(B.SCHEDULE_WINDOW, 6, 7, 38, 0), (B.SCHEDULE_WINDOW, 3, 8, 56, 1),
+                                                               (B.SCHEDULE_CAPTION, 6, 7, 38, 2)])
+def test_combine_product_in_blocks_of_several_sequences(schedule, batch, group, layers, mod_id):
+    heads, n, dev = 2, 32 * 12 + 17, torch.device("cuda")
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=heads * group)
+    cache = B.Cache(layers, batch, heads, heads * group, 32 * 14, device=dev, schedule=schedule)
+    k, v = (x.to(dev) for x in WL.gen_kv(w, 0, n_tokens=n))
+    mod = torch.full((batch, n), mod_id, dtype=torch.uint8, device=dev)
+    signs = torch.stack([WL.gen_signs(w, l) for l in range(layers)]).to(dev)
+    R = torch.stack([WL.gen_rotations(w, l) for l in range(layers)])[:, None].contiguous().to(dev)
+    for l in range(layers):
+        B.quantize_keys(cache, l, k.roll(l, dims=2), signs[l])
+        B.quantize_values(cache, l, v.roll(l, dims=2), mod, R[l])
+    q = torch.stack([WL.gen_queries(w, l) for l in range(layers)]).to(dev)
+
+    def call(ws, mats=R):
+        out = torch.full((layers, batch, heads * group, D), float("nan"), device=dev)
+        B.decode_attention(cache, 0, layers, q, signs, mats, ws, out)
+        torch.cuda.synchronize()
+        return out.double()
+
+    ws = Hn.decode_workspace(cache, layers, 0, call)   # no room for the one-launch kernel's pieces
+    raw = call(ws, torch.zeros_like(R))
+    sums = call(ws, torch.eye(D, device=dev).expand_as(R).contiguous()) - raw
+    assert Hn.ran_split_k(ws)
+    ref = torch.einsum("lbhr,lrc->lbhc", sums, R[:, 0, mod_id].double())
+    assert (call(ws) - raw - ref).norm() <= 2.0 ** -22 * ref.norm()
+
+
 # clusters of 1, 2, 4 and 8 blocks (by units and windows); one window; more warps than windows
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("batch,n", [(1, 32), (1, 32 * 9), (12, 32 * 20), (38, 32 * 3)])
