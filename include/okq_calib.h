@@ -59,7 +59,8 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
 
 /*
  * Eigen-decomposition of one symmetric 128 x 128 matrix in fp64 (reduction to tridiagonal form, its eigenvalues and vectors,
- * Newton-Schulz steps towards orthogonality; cyclic Jacobi where equal eigenvalues leave the vectors undetermined) and
+ * Newton-Schulz steps towards orthogonality; cyclic Jacobi where equal eigenvalues leave the vectors undetermined, and for
+ * matrices with diagonal elements below 2^-20 of the largest, whose small eigenvalues it keeps to fp32) and
  * R = H U^T with the ordering and sign convention stated above.
  *   C  float [128][128] (symmetric; only read), signs  float [128] (+-1)
  *   R_out  float [128][128] (row = rotated coordinate), lambda_out  float [128] (descending)

@@ -213,6 +213,39 @@ def test_rotation_of_matrices_that_are_hard_for_a_solver(kind):
     assert np.abs(U @ Cm - lam[:, None] * U).max() <= 1e-6 * size
 
 
+@pytest.mark.parametrize("decades", [0, 2, 3, 4, 5, 6])
+def test_rotation_keeps_small_eigenvalues_of_graded_matrices(decades):
+    """Channels whose scales differ by up to 10^6: every eigenvalue to a few roundings of fp32, relative to itself.  Reference: singular
+    values of the Cholesky factor by one-sided Jacobi rotations, which are exact to fp64 for such factors."""
+    from scipy.linalg import cholesky, lapack
+    rng = np.random.default_rng(5)
+    x = rng.standard_normal((D, 4 * D))
+    scale = np.logspace(0, -decades, D)[rng.permutation(D)]
+    C32 = torch.from_numpy(x @ x.T / (4 * D) * scale[:, None] * scale).float()
+    C32 = (C32 + C32.T) / 2
+    Cm = C32.double().numpy()
+    root = np.sqrt(np.diag(Cm))
+    sv, _, _, _, _, info = lapack.dgejsv((cholesky(Cm / root[:, None] / root, lower=True) * root[:, None]).T)
+    assert info == 0
+    ref = np.sort(sv ** 2)[::-1]
+    ws = torch.empty(D * D * 8, dtype=torch.uint8, device="cuda")
+    R, lam, _ = B.calib_rotation(C32.cuda(), torch.ones(D, device="cuda"), ws)
+    assert (np.abs(lam.double().cpu().numpy() - ref) <= 2.0 ** -23 * ref).all()
+    U = CO.hadamard_matrix(np.ones(D)).T @ R.double().cpu().numpy()
+    assert np.abs(U @ U.T - np.eye(D)).max() <= 1e-6
+
+
+def test_rotation_of_channels_without_values():
+    """Channels that are zero have eigenvalues that are."""
+    rng = np.random.default_rng(6)
+    x = rng.standard_normal((D, 4 * D))
+    x[1::9] = 0
+    _, lam, _ = B.calib_rotation(torch.from_numpy(x @ x.T).float().cuda(), torch.ones(D, device="cuda"),
+                                 torch.empty(D * D * 8, dtype=torch.uint8, device="cuda"))
+    dead = len(range(1, D, 9))
+    assert (lam[-dead:] == 0).all() and (lam[:-dead] > 0).all()
+
+
 def test_rotation_of_numbers_that_are_none_ends():
     signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0).cuda()
     ws = torch.empty(D * D * 8, dtype=torch.uint8, device="cuda")
