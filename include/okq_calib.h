@@ -64,7 +64,8 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
  * R = H U^T with the ordering and sign convention stated above.
  *   C  float [128][128] (symmetric; only read), signs  float [128] (+-1)
  *   R_out  float [128][128] (row = rotated coordinate), lambda_out  float [128] (descending)
- *   workspace: at least 128 KB (checked).
+ *   workspace: at least 128 KB (checked; the solvers keep everything in shared memory and, until the call has completed on
+ *   `stream`, in R_out and lambda_out: calls that overlap may share a workspace).
  * The device status convention of okq.h does not apply: the iterations have fixed limits (8 steps, 30 sweeps), which
  * a symmetric matrix does not reach; `sweeps_out` (device int32, may be null) receives the steps or sweeps used.
  */

@@ -597,7 +597,7 @@ __device__ __forceinline__ void eig_apply(cg::cluster_group& cluster, EigV& sv) 
 
 __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __restrict__ C, const float* __restrict__ signs,
                                                            float* __restrict__ R, float* __restrict__ lambda,
-                                                           int* __restrict__ sweeps_out, const int* __restrict__ left) {
+                                                           int* __restrict__ sweeps_out) {
   extern __shared__ __align__(16) unsigned char eig_raw[];
   __shared__ double red[32];
   cg::cluster_group cluster = cg::this_cluster();
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_calib_eigen(const float* __rest
   EigA<double>& sd = *reinterpret_cast<EigA<double>*>(eig_raw);
   EigA<float>& sf = *reinterpret_cast<EigA<float>*>(eig_raw);
   depend_wait();
-  if (*left == 0) return;   // the direct solver has done it
+  if (__float_as_uint(__ldcg(lambda)) != EIGEN_LEFT) return;   // the direct solver has done it
   cluster.sync();   // every block runs before its shared memory is written from outside
   // largest magnitude (the matrix is scaled by a power of two to at most 1) and trace
   double mx = 0.0, tr = 0.0;
@@ -770,6 +770,7 @@ size_t attn_bytes(int group, int n) {
   const size_t n_it = (size_t)(n + TQ_WS - 1) / TQ_WS;
   return ((size_t)group * n * 2 + n_it * group * n) * sizeof(float);
 }
+constexpr size_t EIGEN_BYTES = (size_t)D * D * sizeof(double);   // what the rotation documents; it touches none of it
 size_t moments_bytes() { return (size_t)MAX_CHUNKS * 3 * D * D * sizeof(float) + 16; }
 
 }  // namespace
@@ -854,11 +855,9 @@ okq_status okq_calib_rotation(const float* C, const float* signs, void* workspac
     attr_done(attr_mask, attr_dev);
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  double* ws = static_cast<double*>(workspace);
-  cudaError_t e = launch_calib_spectrum(C, signs, ws, R_out, lambda_out, sweeps_out, st);
+  cudaError_t e = launch_calib_spectrum(C, signs, R_out, lambda_out, sweeps_out, st);
   if (e == cudaSuccess)
-    e = launch_dependent(k_calib_eigen, dim3(1 + V_CTAS), EIG_THREADS, EIG_SMEM, st, 1 + V_CTAS, C, signs, R_out, lambda_out, sweeps_out,
-                         reinterpret_cast<const int*>(ws + EIGEN_LEFT));
+    e = launch_dependent(k_calib_eigen, dim3(1 + V_CTAS), EIG_THREADS, EIG_SMEM, st, 1 + V_CTAS, C, signs, R_out, lambda_out, sweeps_out);
   if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
   return launch_status();
 }

@@ -1,6 +1,6 @@
 // Direct eigensolver of the calibration: one symmetric 128 x 128 matrix by one cluster of eight blocks, all in fp64.
 //
-//   1. Householder reduction to a tridiagonal matrix (block 0, the matrix in registers); the reflectors go to the workspace
+//   1. Householder reduction to a tridiagonal matrix (block 0, the matrix in registers); the reflectors go to R's place
 //   2. eigenvalues by 33-section on Sturm counts, two eigenvalues per warp, 16 per block
 //   3. eigenvectors of the tridiagonal matrix from its two factorisations, twisted where the residual is least
 //   4. the reflectors applied to them, half a warp per two vectors
@@ -17,6 +17,9 @@
 // differ in scale has small eigenvalues that only the latter keeps.  Scales from 1 to 1e-6 over the channels: the smallest to
 // 3e-6 here, to fp32 there.  So matrices with diagonal elements below 2^-20 of the largest (and channels that are zero, whose
 // eigenvalues stay exactly 0) go there at once; at that ratio the error, 1e-16 times 2^20, is still hidden behind fp32's 6e-8.
+//
+// What the blocks exchange - the reflectors, then the vectors - passes through R's own 64 KB and shared memory: the workspace stays
+// untouched, so that calls which overlap may share it.
 //
 // Why: cyclic Jacobi is 11 to 13 sweeps of 127 dependent rounds of about a microsecond, whatever the number of SMs; the
 // reduction is 126 dependent steps of 0.9 us, and everything behind it is parallel over the vectors.  One matrix 1506 -> 203 us
@@ -45,7 +48,7 @@ constexpr int MAX_STEPS = 8;                // Newton-Schulz steps: 0.5 -> 0.19 
 
 struct Smem {
   union {
-    double refl[D][D];                      // reflectors (copies)
+    __align__(16) double refl[D][D];        // reflectors (copies)
     double all[D][PITCH];                   // all eigenvectors (rows), gathered from the blocks
   };
   __align__(16) double own[VEC][PITCH];     // this block's eigenvectors
@@ -121,7 +124,9 @@ __device__ __forceinline__ double fast_rcp(double x) {
 // What bounds it: the chain of a step (product 200 cycles, sums over 16 lanes 46 per level, barriers 40), and shared memory, which
 // delivers 128 bytes a cycle however many lanes read the same number: a tile of 8 x 8 elements per thread uses each number it
 // loads eight times.  Steps of product, w and update behind three barriers took 2500 cycles (3100 with one row per thread).
-__device__ void reduce_to_tridiagonal(Smem& sm, const float* __restrict__ C, double (*__restrict__ refl)[D]) {
+// Reflector k has components k + 1 .. 127: two of them share a row of 128 numbers of `rows`, and all fit into 64.  Row r: reflector r
+// from the left, 126 - r reversed.
+__device__ void reduce_to_tridiagonal(Smem& sm, const float* __restrict__ C, double* __restrict__ rows) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, u = lane & 15, r0 = 8 * (tid >> 4);
   auto& rd = sm.red;
   double a[8][8];
@@ -160,6 +165,8 @@ __device__ void reduce_to_tridiagonal(Smem& sm, const float* __restrict__ C, dou
   }
   if (tid < D) { rd.v[tid] = 0.0; rd.w[tid] = 0.0; }
   __syncthreads();
+  double* to = rows + tid;
+  int step = D;
 #pragma unroll 1
   for (int k = 0; k < D - 2; k++) {
     if (warp == 0) {
@@ -255,14 +262,16 @@ __device__ void reduce_to_tridiagonal(Smem& sm, const float* __restrict__ C, dou
       rd.x[tid] = tid > k + 2 ? next : 0.0;
       if (tid == k + 2) rd.alpha = next;
       if (tid == k + 1) sm.d[k + 1] = next;
-      refl[k][tid] = v;
+      if (tid > k) *to = v;
+      to += step;
+      if (k == D / 2 - 1) { to = rows + (D / 2 - 2) * D + D - 1 - tid; step = -D; }
     }
     __syncthreads();
   }
   // what is left: the last diagonal element and the one beside it
   if (tid == THREADS - 1) sm.d[D - 1] = fma(-2.0 * rd.v[D - 1], rd.w[D - 1], a[7][7]);
   if (tid == 0) { sm.e[D - 2] = rd.alpha; sm.e[D - 1] = 0.0; sm.tau[D - 2] = 0.0; sm.tau[D - 1] = 0.0; }
-  if (tid < D) refl[D - 2][tid] = 0.0;
+  if (tid == 0) rows[0] = 0.0;   // the last one, which reflects nothing
 }
 
 // Eigenvalues below x[n] of the rows lo .. hi of the tridiagonal matrix: sign changes of the sequence of leading minors,
@@ -296,13 +305,13 @@ __device__ __forceinline__ void sturm_count(const double2* de, int lo, int hi, c
   for (; i <= hi; i++) term(de[i]);
 }
 
-__global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __restrict__ C, const float* __restrict__ signs, double* __restrict__ ws,
-                                                              float* __restrict__ R, float* __restrict__ lambda, int* __restrict__ sweeps_out) {
+__global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __restrict__ C, const float* __restrict__ signs, float* __restrict__ R,
+                                                              float* __restrict__ lambda, int* __restrict__ sweeps_out) {
   extern __shared__ __align__(16) unsigned char raw[];
   Smem& sm = *reinterpret_cast<Smem*>(raw);
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x;
-  double (*refl)[D] = reinterpret_cast<double (*)[D]>(ws);
+  double* const rows = reinterpret_cast<double*>(R);   // exchanged between the blocks until R is written
   depend_wait();
   {
     float least = INFINITY, most = 0.f;
@@ -318,12 +327,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
       most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, s));
     }
     if (least < GRADED * most) {   // (the same in every warp of every block)
-      if (rank == 0 && tid == 0) reinterpret_cast<int*>(refl[D - 1])[0] = 1;
+      if (rank == 0 && tid == 0) lambda[0] = __uint_as_float(EIGEN_LEFT);
       return;
     }
   }
   if (rank == 0) {
-    reduce_to_tridiagonal(sm, C, refl);
+    reduce_to_tridiagonal(sm, C, rows);
     __threadfence();
   }
   cluster.sync();   // the tridiagonal matrix and the reflectors are there
@@ -332,9 +341,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
     if (tid < D) { sm.d[tid] = s0->d[tid]; sm.e[tid] = s0->e[tid]; sm.tau[tid] = s0->tau[tid]; }
     if (tid == 0) sm.expo = s0->expo;
   }
-  for (int i = tid; i < (D - 1) * D / 2; i += THREADS) copy_async16(&sm.refl[0][2 * i], &refl[0][2 * i]);
+  auto pairs = [&](auto f) {   // of the reflectors' 64 rows, the same ones of a thread each time
+    for (int i = tid; i < D / 2 * D / 2; i += THREADS) f(i / (D / 2), 2 * (i % (D / 2)));
+  };
+  pairs([&](int r, int c) {
+    copy_async16(&sm.refl[r][c], rows + r * D + c);
+    *reinterpret_cast<double2*>(&sm.refl[D / 2 + r][c]) = make_double2(0.0, 0.0);
+  });
   asm volatile("cp.async.commit_group;\n" ::);
-  if (tid < D) sm.refl[D - 1][tid] = 0.0;
   __syncthreads();
 
   // ---- sizes, blocks: an off-diagonal element at rounding level of the matrix is none
@@ -513,7 +527,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
     }
     resid_ok = resid_ok && isfinite(lam[n]);
   }
-  asm volatile("cp.async.wait_group 0;\n" ::);
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  pairs([&](int r, int c) {   // the reversed ones go to rows of their own
+    if (c > r) return;
+    const double2 x = *reinterpret_cast<const double2*>(&sm.refl[r][c]);
+    *reinterpret_cast<double2*>(&sm.refl[r][c]) = make_double2(0.0, c == r ? x.y : 0.0);
+    if (r < D / 2 - 1) *reinterpret_cast<double2*>(&sm.refl[126 - r][126 - c]) = make_double2(c == r ? 0.0 : x.y, x.x);
+  });
   const int bad = __syncthreads_or(!resid_ok);   // (the vectors and the reflectors are in place)
 
   // ---- V = H_0 H_1 ... H_125 Z: reflectors in groups of four, last ones first, their products with the vector taken together
@@ -599,18 +619,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
   bool good = false;
 #pragma unroll 1
   for (; steps < MAX_STEPS;) {
-    // through the workspace, whose reflectors every block has copied: L2 delivers them faster than the other blocks' shared memory
-    if (steps == 0) cluster.sync();
-    else __syncthreads();
-    for (int i = tid; i < VEC * D / 2; i += THREADS) {
-      const int row = i / (D / 2), c = 2 * (i % (D / 2));
-      __stcg(reinterpret_cast<double2*>(&refl[rank * VEC + row][c]), *reinterpret_cast<const double2*>(&sm.own[row][c]));
+    // half of the columns through R, whose reflectors every block has copied, half straight into the other blocks' shared memory
+    cluster.sync();   // (nobody reads the reflectors, or the vectors of the step before, any more)
+    for (int i = tid; i < VEC * D / 4; i += THREADS) {
+      const int row = i / (D / 4), c = 2 * (i % (D / 4));
+      const double2 x = *reinterpret_cast<const double2*>(&sm.own[row][D / 2 + c]);
+#pragma unroll
+      for (int r = 0; r < CTAS; r++) *reinterpret_cast<double2*>(cluster.map_shared_rank(&sm.all[rank * VEC + row][D / 2 + c], r)) = x;
+      __stcg(reinterpret_cast<double2*>(rows + (rank * VEC + row) * (D / 2) + c), *reinterpret_cast<const double2*>(&sm.own[row][c]));
     }
     __threadfence();
     cluster.sync();   // every block's vectors are there
-    for (int i = tid; i < D * D / 2; i += THREADS) {
-      const int row = i / (D / 2), c = 2 * (i % (D / 2));
-      copy_async16(&sm.all[row][c], &refl[row][c]);
+    for (int i = tid; i < D * D / 4; i += THREADS) {
+      const int row = i / (D / 4), c = 2 * (i % (D / 4));
+      copy_async16(&sm.all[row][c], rows + row * (D / 2) + c);
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
@@ -667,8 +689,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
     if (err < 1e-16) { good = true; break; }   // the step just made leaves 3/4 of that, the squared distance
   }
   if (rank == 0 && tid == 0) {
-    reinterpret_cast<int*>(refl[D - 1])[0] = good ? 0 : 1;   // (0: nothing left for the Jacobi solver)
-    if (good && sweeps_out) *sweeps_out = steps;
+    if (!good) lambda[0] = __uint_as_float(EIGEN_LEFT);
+    else if (sweeps_out) *sweeps_out = steps;
   }
   if (!good) return;   // (the same for every block, none of which reads another's memory any more)
 
@@ -740,7 +762,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_calib_spectrum(const float* __re
 
 }  // namespace
 
-cudaError_t launch_calib_spectrum(const float* C, const float* signs, double* ws, float* R, float* lambda, int* sweeps, cudaStream_t s) {
+cudaError_t launch_calib_spectrum(const float* C, const float* signs, float* R, float* lambda, int* sweeps, cudaStream_t s) {
   static thread_local unsigned long long attr_mask = 0;
   int dev = 0;
   if (attr_needed(attr_mask, dev)) {
@@ -748,7 +770,7 @@ cudaError_t launch_calib_spectrum(const float* C, const float* signs, double* ws
     if (e != cudaSuccess) return e;
     attr_done(attr_mask, dev);
   }
-  return launch_dependent(k_calib_spectrum, dim3(CTAS), THREADS, sizeof(Smem), s, CTAS, C, signs, ws, R, lambda, sweeps);
+  return launch_dependent(k_calib_spectrum, dim3(CTAS), THREADS, sizeof(Smem), s, CTAS, C, signs, R, lambda, sweeps);
 }
 
 }  // namespace okq

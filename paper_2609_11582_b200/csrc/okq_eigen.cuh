@@ -6,10 +6,11 @@
 
 namespace okq {
 
-constexpr size_t EIGEN_BYTES = (size_t)D * D * sizeof(double);   // workspace: 126 reflectors and the word below
-constexpr size_t EIGEN_LEFT = (size_t)(D - 1) * D;               // double whose first int says that the matrix is left to the Jacobi solver
+// In the place of lambda[0], until the Jacobi solver behind has run: the matrix is left to it.  (A NaN that no result has: eigenvalues
+// of the direct solver are numbers.)
+constexpr unsigned EIGEN_LEFT = 0x7fe11e57u;
 
-// eigenvalues and R = H U^T of one symmetric matrix, or the word at EIGEN_LEFT set
-cudaError_t launch_calib_spectrum(const float* C, const float* signs, double* ws, float* R, float* lambda, int* sweeps, cudaStream_t s);
+// eigenvalues and R = H U^T of one symmetric matrix, or lambda[0] = EIGEN_LEFT
+cudaError_t launch_calib_spectrum(const float* C, const float* signs, float* R, float* lambda, int* sweeps, cudaStream_t s);
 
 }  // namespace okq

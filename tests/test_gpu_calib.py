@@ -246,6 +246,24 @@ def test_rotation_of_channels_without_values():
     assert (lam[-dead:] == 0).all() and (lam[:-dead] > 0).all()
 
 
+def test_rotations_that_overlap_may_share_a_workspace():
+    """Different matrices on streams of their own with one workspace give what each gives by itself, and the workspace stays as it was."""
+    signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0).cuda()
+    mats = [torch.from_numpy(_matrices()[k]).float().cuda() for k in ("definite", "indefinite", "low rank", "two eigenvalues", "cluster")]
+    ws = torch.full((D * D * 8,), 0x5a, dtype=torch.uint8, device="cuda")
+    alone = [B.calib_rotation(C, signs, ws) for C in mats]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in mats]
+    for _ in range(5):
+        got = []
+        for C, st in zip(mats, streams):
+            with torch.cuda.stream(st):
+                got.append(B.calib_rotation(C, signs, ws))
+        torch.cuda.synchronize()
+        assert all((x == y).all() for a, b in zip(alone, got) for x, y in zip(a, b))
+    assert (ws == 0x5a).all()
+
+
 def test_rotation_of_numbers_that_are_none_ends():
     signs = WL.gen_signs(WL.WORKLOADS["layer7b"], 0).cuda()
     ws = torch.empty(D * D * 8, dtype=torch.uint8, device="cuda")
