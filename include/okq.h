@@ -282,6 +282,15 @@ void okq_profile_events(void* before, void* after);
 int32_t okq_decode_select(int32_t impl);
 
 /*
+ * How okq_decode_attention would take a call (of its launches the first) given `workspace_bytes`, 0 meaning the least it accepts;
+ * for tests of the rules (the paper has no counterpart).  Positive: the one-launch kernel, with this many blocks per (sequence, KV
+ * head).  Negative: the split-K pair, whose combine kernel gives a (sequence, KV head) four blocks or one, or four sequences a
+ * block.  0: arguments that the call would refuse.  Only the sizes of `cache` are looked at.
+ */
+enum { OKQ_PLAN_PAIR_QUARTER = -1, OKQ_PLAN_PAIR_ONE = -2, OKQ_PLAN_PAIR_FOUR = -3 };
+int32_t okq_debug_decode_plan(const okq_cache* cache, int32_t layer_count, int32_t num_splits, size_t workspace_bytes);
+
+/*
  * Canonical view of one layer (checkpointing and parity checks; the paper has no
  * counterpart, the arrays are simply Eq. 2-4 and Eq. 6 outputs in natural order).
  * All windows up to capacity are converted, whatever seq_len says.

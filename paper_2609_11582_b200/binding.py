@@ -18,6 +18,8 @@ RECORD_BYTES_MX, MX_META_BYTES = 2312, 136
 META_FP16, META_MXFP4 = 0, 1
 SCHEDULE_WINDOW, SCHEDULE_CAPTION = 0, 1
 
+PLAN_PAIR_QUARTER, PLAN_PAIR_ONE, PLAN_PAIR_FOUR = -1, -2, -3
+
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_CAPACITY, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(8)
 
 
@@ -85,6 +87,8 @@ def lib():
         L.okq_decode_attention_noalloc.restype = C.c_int
         L.okq_decode_attention_noalloc.argtypes = [C.POINTER(okq_cache), C.c_int32, C.c_int32, C.c_void_p, C.c_float,
                                                    C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p]
+        L.okq_debug_decode_plan.restype = C.c_int32
+        L.okq_debug_decode_plan.argtypes = [C.POINTER(okq_cache), C.c_int32, C.c_int32, C.c_size_t]
         L.okq_decode_select.restype = C.c_int32
         L.okq_decode_select.argtypes = [C.c_int32]
         L.okq_profile_events.restype = None
@@ -133,7 +137,7 @@ def lib():
 def exported_symbols():
     return ["okq_status_string", "okq_last_cuda_error", "okq_cache_sizes", "okq_decode_workspace_bytes",
             "okq_quantize_keys", "okq_quantize_values", "okq_append", "okq_decode_attention", "okq_cache_export",
-            "okq_cache_import", "okq_profile_events", "okq_decode_select", "okq_decode_attention_simt",
+            "okq_cache_import", "okq_profile_events", "okq_decode_select", "okq_debug_decode_plan", "okq_decode_attention_simt",
             "okq_decode_attention_noalloc", "okq_quantize_values_bulk", "okq_debug_bulk_timeout", "okq_cache_export_mx",
             "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_debug_calib_timeout", "okq_calib_moments", "okq_calib_rotation",
             "okq_ladder_codebook", "okq_ladder_quantize_keys", "okq_ladder_quantize_values",
@@ -268,6 +272,11 @@ def decode_attention_noalloc(cache: Cache, layer: int, layer_count: int, q, sign
     _check(lib().okq_decode_attention_noalloc(C.byref(cache.c), layer, layer_count, _ptr(q), scale, _ptr(signs),
                                               _ptr(R), n_R, num_splits, _ptr(out), _stream(stream)),
            "okq_decode_attention_noalloc")
+
+
+def decode_plan(c: okq_cache, layer_count: int, num_splits=0, workspace_bytes=0) -> int:
+    """okq_debug_decode_plan: which kernels a decode call on a cache of these sizes would take."""
+    return lib().okq_debug_decode_plan(C.byref(c), layer_count, num_splits, workspace_bytes)
 
 
 def decode_select(impl: int) -> int:

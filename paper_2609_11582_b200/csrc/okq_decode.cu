@@ -485,6 +485,15 @@ int32_t okq_decode_select(int32_t impl) {
   return prev;
 }
 
+int32_t okq_debug_decode_plan(const okq_cache* cache, int32_t layer_count, int32_t num_splits, size_t workspace_bytes) {
+  if (check_cache(cache, false) != OKQ_OK || layer_count <= 0 || num_splits < 0 || cache->batch > MAX_ENTRIES) return 0;
+  const int per_launch = MAX_ENTRIES / cache->batch, lc = layer_count < per_launch ? layer_count : per_launch;
+  const size_t partials = mma_partials_bytes(cache, lc, num_splits);
+  DecodeParams P = make_params(cache, 0, lc, nullptr, 0.f, nullptr, nullptr, 1, nullptr, num_splits);
+  P.piece_slots = workspace_bytes > partials ? (long long)((workspace_bytes - partials) / sizeof(WarpPiece)) : 0;
+  return decode_plan(P, mma_ctas(cache, lc, num_splits));
+}
+
 size_t okq_decode_workspace_bytes(const okq_cache* cache, int32_t layer_count, int32_t num_splits) {
   if (check_cache(cache, false) != OKQ_OK || layer_count <= 0 || num_splits < 0) return 0;
   const size_t a = simt_workspace(cache, layer_count, num_splits), b = mma_workspace(cache, layer_count, num_splits);

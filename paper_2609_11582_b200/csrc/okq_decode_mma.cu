@@ -820,30 +820,44 @@ static void combine_launch(const DecodeParams& P, int n_cta, cudaStream_t s) {
   launch_dependent(k_combine_mma<CAPTION, NS, SEQ>, grid, SEQ * 128, sizeof(CombineSmem<CAPTION, SEQ>), s, 1, P, n_cta);
 }
 
+static int combine_form(const CacheView& cv, int layer_count, int n_cta) {
+  // A block per sequence and head while they all run at once, four sequences per block, whose product is on the tensor cores, from there
+  // on (30000 tokens: 132 units of 3 sequences 166 us against 175 with blocks of four, 152 units of 2, 3 and 4 sequences 196, 198 and 198
+  // against 188, 194 and 197; 28 layers x 4 sequences x 4 heads at 2000 / 8192 tokens 123 / 192 against 90 / 163).  The captioning
+  // schedule's long raw tails make four full sequences as slow as two waves of single ones (8192 tokens: 152 units of 4 sequences 122
+  // against 125 us, 304 units 184 against 165; of 3 sequences 180 units 132 against 126).  A single sequence would leave three quarters
+  // of such a block idle.  A handful of units (e.g. a single-layer call) shares four blocks each, a quarter of the output columns per
+  // block.
+  const int units = cv.n_kv_heads * cv.batch * layer_count, waves = cv.sched == SCHED_CAPTION && cv.batch >= CB_SEQ_MAX ? 2 : 1;
+  const int n_blocks = cv.n_kv_heads * ((cv.batch + CB_SEQ_MAX - 1) / CB_SEQ_MAX) * layer_count;
+  if (4 * n_blocks <= n_cta) return OKQ_PLAN_PAIR_QUARTER;
+  return cv.batch < 2 || units <= waves * sm_count() ? OKQ_PLAN_PAIR_ONE : OKQ_PLAN_PAIR_FOUR;
+}
+
 template <bool CAPTION>
-static void combine_dispatch(const DecodeParams& P, int n_cta, cudaStream_t s) {
-  // Four sequences per block, whose product runs on the tensor cores, wherever there are so many: 28 layers x 4 sequences x 4 heads at
-  // 2000 / 8192 tokens 89 / 163 us against 125 / 193 with one per block, 14 x 4 x 4 at 16384 163 against 167.  Two sequences fill half
-  // of such a block: worth it once there are blocks for half of the SMs (28 x 2 x 4 at 16384 tokens 160 against 167, 12 x 2 x 4 at
-  // 30000 138 against 134).  A single sequence per block otherwise, and a handful of blocks (e.g. a single-layer call) share it, a
-  // quarter of the output columns each.
-  const int n_blocks = P.cv.n_kv_heads * ((P.cv.batch + CB_SEQ_MAX - 1) / CB_SEQ_MAX) * P.layer_count;
-  if (4 * n_blocks <= n_cta) combine_launch<CAPTION, 4, 1>(P, n_cta, s);
-  else if (P.cv.batch < 2 || (P.cv.batch == 2 && 2 * n_blocks < n_cta)) combine_launch<CAPTION, 1, 1>(P, n_cta, s);
-  else combine_launch<CAPTION, 1, CB_SEQ_MAX>(P, n_cta, s);
+static void combine_dispatch(const DecodeParams& P, int form, int n_cta, cudaStream_t s) {
+  switch (form) {
+    case OKQ_PLAN_PAIR_QUARTER: combine_launch<CAPTION, 4, 1>(P, n_cta, s); break;
+    case OKQ_PLAN_PAIR_ONE: combine_launch<CAPTION, 1, 1>(P, n_cta, s); break;
+    default: combine_launch<CAPTION, 1, CB_SEQ_MAX>(P, n_cta, s);
+  }
 }
 
 int g_decode_impl = 1;
 
+int decode_plan(const DecodeParams& P, int n_cta) {
+  // (the one-launch kernel: where the library chooses the grid itself)
+  const int cs = P.n_splits == 0 && g_decode_impl == 1 ? decode_small_cluster(P.cv, P.layer_count, P.piece_slots) : 0;
+  return cs > 0 ? cs : combine_form(P.cv, P.layer_count, n_cta);
+}
+
 okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, cudaEvent_t before, cudaEvent_t after) {
-  if (P.n_splits == 0 && g_decode_impl == 1) {   // the library's own choice of the grid
-    const int cs = decode_small_cluster(P.cv, P.layer_count, P.piece_slots);
-    if (cs > 0) {
-      if (before) cudaEventRecord(before, s);
-      const okq_status st = launch_decode_small(P, cs, s);
-      if (after) cudaEventRecord(after, s);
-      return st;
-    }
+  const int plan = decode_plan(P, n_cta);
+  if (plan > 0) {
+    if (before) cudaEventRecord(before, s);
+    const okq_status st = launch_decode_small(P, plan, s);
+    if (after) cudaEventRecord(after, s);
+    return st;
   }
   static thread_local unsigned long long attr_mask = 0;
   int attr_dev = 0;
@@ -869,8 +883,8 @@ okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, c
   } else if (P.cv.fmt == FMT_MXFP4) launch_dependent(k_decode_mma<FMT_MXFP4>, dim3(n_cta), NTHREADS, sizeof(MmaSmem<FMT_MXFP4>), s, 1, P);
   else launch_dependent(k_decode_mma<FMT_FP16>, dim3(n_cta), NTHREADS, sizeof(MmaSmem<FMT_FP16>), s, 1, P);
   if (after) cudaEventRecord(after, s);
-  if (P.cv.sched == SCHED_CAPTION) combine_dispatch<true>(P, n_cta, s);
-  else combine_dispatch<false>(P, n_cta, s);
+  if (P.cv.sched == SCHED_CAPTION) combine_dispatch<true>(P, plan, n_cta, s);
+  else combine_dispatch<false>(P, plan, n_cta, s);
   return OKQ_OK;
 }
 

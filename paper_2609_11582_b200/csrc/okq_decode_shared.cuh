@@ -87,6 +87,8 @@ extern int g_decode_impl;
 int decode_small_cluster(const CacheView& cv, int layer_count, long long piece_slots);
 okq_status launch_decode_small(const DecodeParams& P, int cs, cudaStream_t s);
 
+// how launch_decode_mma takes a call: blocks of a cluster of the one-launch kernel, or the pair's OKQ_PLAN_PAIR_*
+int decode_plan(const DecodeParams& P, int n_cta);
 // launches the tensor-core split kernel (bracketed by the optional events) and its combine kernel
 okq_status launch_decode_mma(const DecodeParams& P, int n_cta, cudaStream_t s, cudaEvent_t before, cudaEvent_t after);
 

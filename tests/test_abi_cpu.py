@@ -83,6 +83,22 @@ def test_pointer_validation_before_any_launch(L):
     assert L.okq_append(C.byref(c8), 0, 1, fake, fake, fake, fake, fake, 1, None) == B.ERR_ALIGNMENT
 
 
+@pytest.mark.parametrize("schedule,batch,heads,layers,plan", [
+    (B.SCHEDULE_WINDOW, 4, 1, 37, B.PLAN_PAIR_QUARTER), (B.SCHEDULE_WINDOW, 4, 1, 38, B.PLAN_PAIR_FOUR),
+    (B.SCHEDULE_WINDOW, 3, 4, 12, B.PLAN_PAIR_ONE), (B.SCHEDULE_WINDOW, 3, 1, 50, B.PLAN_PAIR_FOUR),
+    (B.SCHEDULE_WINDOW, 2, 2, 37, B.PLAN_PAIR_ONE), (B.SCHEDULE_WINDOW, 2, 1, 75, B.PLAN_PAIR_FOUR),
+    (B.SCHEDULE_WINDOW, 5, 2, 14, B.PLAN_PAIR_ONE), (B.SCHEDULE_WINDOW, 5, 1, 30, B.PLAN_PAIR_FOUR),
+    (B.SCHEDULE_WINDOW, 1, 4, 48, B.PLAN_PAIR_ONE), (B.SCHEDULE_WINDOW, 1, 4, 9, B.PLAN_PAIR_QUARTER),
+    (B.SCHEDULE_CAPTION, 4, 2, 37, B.PLAN_PAIR_ONE), (B.SCHEDULE_CAPTION, 4, 1, 75, B.PLAN_PAIR_FOUR),
+    (B.SCHEDULE_CAPTION, 3, 4, 12, B.PLAN_PAIR_ONE), (B.SCHEDULE_CAPTION, 3, 1, 50, B.PLAN_PAIR_FOUR)])
+def test_combine_kernel_of_the_split_k_pair(L, schedule, batch, heads, layers, plan):
+    """Either side of the steps of the rule, at 148 SMs: blocks of four sequences from the 149th (sequence, head) on, under the
+    captioning schedule with four sequences or more from the 297th."""
+    c = B.okq_cache(layers, batch, heads, 7 * heads, 128, 32, 32768, B.META_FP16, schedule, 0)
+    assert B.decode_plan(c, layers) == plan
+    assert B.decode_plan(c, 0) == 0
+
+
 def test_calibration_argument_checks(L):
     assert L.okq_calib_workspace_bytes(0, 16) == 0 and L.okq_calib_workspace_bytes(7, 0) == 0
     # the largest of: row statistics + per-(query tile, head) column sums; 64 partial moment sets; 128 x 128 fp64
