@@ -45,7 +45,9 @@ def test_one_launch_decode_in_clusters_of_six(schedule, batch, heads, n):
     outs = []
     for splits in (0, 2):   # against the split-K pair
         out = torch.full((1, batch, 7 * heads, D), float("nan"), device=dev)
-        B.decode_attention(cache, 0, 1, q, signs, R, Hn.decode_workspace(cache, 1, splits), out, num_splits=splits)
+        ws = Hn.decode_workspace(cache, 1, splits)
+        assert (B.decode_plan(cache.c, 1, splits, ws.numel()) == 6) == (splits == 0)
+        B.decode_attention(cache, 0, 1, q, signs, R, ws, out, num_splits=splits)
         outs.append(out.cpu().numpy().astype(np.float64))
     Hn.assert_attention_close(outs[0], outs[1])
 
@@ -74,7 +76,7 @@ def test_one_launch_decode_captioning_schedule(meta, n, batch):
     Hn.assert_attention_close(outs[0], outs[1])
 
 
-# blocks of four sequences (more than 148 of them), the last one partly filled; no packed window, one, several; a full raw tail.
+# blocks of four sequences (152 of them), the last one partly filled; no packed window, one, several; a full raw tail.
 # The matrices may be of any size: the combine kernel's product takes them as they are.
 @pytest.mark.parametrize("schedule", [B.SCHEDULE_WINDOW, B.SCHEDULE_CAPTION])
 @pytest.mark.parametrize("batch,group,n,size", [(5, 5, 31, 1.0), (6, 8, 32 * 9 + 31, 1.0), (7, 1, 32 * 12, 1e20), (8, 7, 32 * 9 + 1, 1e-20)])
@@ -90,8 +92,17 @@ def test_combine_blocks_of_several_sequences(schedule, batch, group, n, size):
         B.quantize_keys(cache, l, k.to(dev).roll(l, dims=2), signs[l])
         B.quantize_values(cache, l, v.to(dev).roll(l, dims=2), mod, R[l])
     q = torch.stack([WL.gen_queries(w, l) for l in range(layers)]).to(dev)
-    out, ref = (torch.full((layers, batch, heads * group, D), float("nan"), device=dev) for _ in range(2))
-    B.decode_attention(cache, 0, layers, q, signs, size * R, Hn.decode_workspace(cache, layers, 2), out, num_splits=2)
+    ref = torch.full((layers, batch, heads * group, D), float("nan"), device=dev)
+
+    def call(ws):
+        out = torch.full_like(ref, float("nan"))
+        B.decode_attention(cache, 0, layers, q, signs, size * R, ws, out)
+        torch.cuda.synchronize()
+        return out
+
+    ws = Hn.decode_workspace(cache, layers, 0, call)   # no room for the one-launch kernel's pieces
+    assert B.decode_plan(cache.c, layers, 0, ws.numel()) == B.PLAN_PAIR_FOUR
+    out = call(ws)
     one = Hn.decode_workspace(cache, 1)
     for l in range(layers):   # the one-launch kernel, whose product is on CUDA cores
         B.decode_attention(cache, l, 1, q[l], signs[l], size * R[l], one, ref[l])
@@ -127,7 +138,7 @@ def test_combine_product_in_blocks_of_several_sequences(schedule, batch, group, 
     ws = Hn.decode_workspace(cache, layers, 0, call)   # no room for the one-launch kernel's pieces
     raw = call(ws, torch.zeros_like(R))
     sums = call(ws, torch.eye(D, device=dev).expand_as(R).contiguous()) - raw
-    assert Hn.ran_split_k(ws)
+    assert B.decode_plan(cache.c, layers, 0, ws.numel()) == B.PLAN_PAIR_FOUR and Hn.ran_split_k(ws)
     ref = torch.einsum("lbhr,lrc->lbhc", sums, R[:, 0, mod_id].double())
     assert (call(ws) - raw - ref).norm() <= 2.0 ** -22 * ref.norm()
 
