@@ -3,9 +3,9 @@
 // The split-K kernel and its combine kernel are a chain of launch, prefix, partials through memory, launch, prefix,
 // merge; with a handful of windows per warp that chain is the whole time (35 + 20 us for one layer of 4 sequences at
 // 4096 tokens).  Here a thread-block cluster (or one block) owns one unit: its CS x 12 warps walk the unit's windows (the same code as
-// the split-K kernel), leave their sums as pieces in global memory (L2), and after one cluster barrier every CTA merges
-// 1 / CS of the rotated channels over all pieces.  The merged sums are pushed into every CTA's shared memory, and after
-// the second barrier each CTA applies R_m^T for 1 / CS of the output columns.  The raw tail is scored by every CTA (its
+// the split-K kernel), leave their sums as pieces in global memory (L2), and after one cluster barrier MS of them (all; four of six)
+// merge 1 / MS of the rotated channels each over all pieces.  The merged sums are pushed into those CTAs' shared memory, and after
+// the second barrier each of them applies R_m^T for 1 / MS of the output columns.  The raw tail is scored by each of them (its
 // rows are staged at the start) while the first barrier is on its way.
 // What bounds it: latency (launch, query rotation, the first window of a warp, two cluster barriers, L2 round trips of the
 // merge).  One sequence, one head group of seven, 2048 tokens: 59 -> 11.3 us per call; one layer of 4 sequences x 4 heads at
@@ -32,8 +32,9 @@ struct __align__(16) Place {
   int v_pk, k_pk, nwin, n_tail, npc, n_rawk;
   // The windows make `used` pieces of at most cnt windows, dealt out evenly over the CTAs (this one has [piece0, piece1)): one CTA
   // filled after the other, 64 windows over 192 warps were one for every warp of five CTAs, three to a sub-partition's dispatch, and
-  // nothing for the rest (13.6 -> 11.6 us).  Fewer windows per piece, spread over all warps, is no better: what a warp does once,
-  // whatever its windows, is dispatch of the same SM.
+  // nothing for the rest (13.5 -> 11.3 us).  Up to four pieces stay with the first CTA, a sub-partition each, except in a cluster of 16
+  // (32 units, 64 tokens: 9.6 -> 9.3 us).  Fewer windows per piece, spread over all warps, is no better: what a warp does once, whatever
+  // its windows, is dispatch of the same SM.
   int cnt, used, piece0, piece1;
 };
 
@@ -116,24 +117,36 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = P.group;
-  depend_wait();
-  WalkEnd we{-INFINITY, 0.f, 0u};
-  auto pieces_of = [](const Place& a) { return a.cnt > 1 ? (a.nwin + a.cnt - 1) / a.cnt : a.nwin; };
   Place at;
+  at.unit = blockIdx.x / CS; at.rank = blockIdx.x % CS;
   {
-    at.unit = blockIdx.x / CS; at.rank = blockIdx.x % CS;
     const int e = at.unit / cv.n_kv_heads;
     at.h = at.unit % cv.n_kv_heads; at.b = e % cv.batch; at.li = e / cv.batch; at.layer = P.layer0 + at.li;
+  }
+  depend_wait();
+  const __half *kt_kept, *vt_kept;
+  WarpPiece* pieces_kept;
+  // Headers of as many pieces as there are, in a cluster of 16; of all places in smaller ones, warps without windows filling those behind
+  // the pieces': loops of a fixed length are 0.3 us shorter there, 0.3 us longer here.
+  constexpr bool COUNTED = CS > 8;
+  WalkEnd we{-INFINITY, 0.f, 0u};
+  // (a single block with fp16 metadata has the registers to keep addresses and all across the walk)
+  constexpr bool KEEP = CS == 1 && FMT == FMT_FP16;
+  auto pieces_of = [](const Place& a) { return KEEP ? (a.cnt > 0 ? (a.nwin + a.cnt - 1) / a.cnt : 0) : a.cnt > 1 ? (a.nwin + a.cnt - 1) / a.cnt : a.nwin; };
+  {
     const int seq = cv.seq_len[at.layer * cv.batch + at.b];
     at.v_pk = cv.v_packed(seq); at.k_pk = cv.k_packed(seq); at.nwin = at.v_pk / W; at.n_tail = seq - at.v_pk;
     at.npc = (at.k_pk - at.v_pk) / W; at.n_rawk = seq - at.k_pk;
     at.cnt = (at.nwin + CS * NWARP - 1) / (CS * NWARP);
     at.used = CS > 1 ? pieces_of(at) : 0;   // (a single block's division can wait)
     at.piece0 = at.used * at.rank / CS; at.piece1 = CS > 1 ? at.used * (at.rank + 1) / CS : NWARP;
+    if (CS > 1 && !COUNTED && at.used <= 4) { at.piece0 = at.rank ? at.used : 0; at.piece1 = at.used; }   // (a warp per sub-partition)
     if (CS > 1 && tid == 0) sm.at = at;
     const __half* qbase = P.q + (((size_t)at.li * cv.batch + at.b) * cv.n_q_heads + (size_t)at.h * G) * D;
     const float* signs = P.signs + (size_t)at.li * D;
     const __half* kt = cv.k_tail + cv.k_tail_off(at.layer, at.b, at.h);
+    kt_kept = kt; vt_kept = cv.v_tail + cv.v_tail_off(at.layer, at.b, at.h);
+    pieces_kept = P.pieces + (size_t)at.unit * (CS * NWARP);
 
     // ---- on their way from the start: queries and the first raw keys
     for (int i = tid; i < G * (D / 8); i += NTHREADS) cp_async16(&sm.q[i / (D / 8)][8 * (i % (D / 8))], qbase + 8 * i);
@@ -174,12 +187,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   }
   cluster.barrier_wait();
   // ---- the piece's header goes to every merging CTA of the cluster
-  if (CS == 1 || at.piece0 + warp < at.piece1)   // (a single block: all of its warps, those without windows too)
+  const bool held = CS == 1 || warp < at.piece1 - at.piece0;
+  if (!COUNTED || held) {
+    const int slot = held ? at.piece0 + warp : at.used + at.rank * NWARP + warp - at.piece1;
     for (int r = 0; r < MS; r++) {
-      PieceMeta* pm = cluster.map_shared_rank(&sm.meta[at.piece0 + warp], r);
+      PieceMeta* pm = cluster.map_shared_rank(&sm.meta[slot], r);
       if ((lane & 3) == 0) { pm->m[lane >> 2] = we.m; pm->l[lane >> 2] = we.l; }
       if (lane == 0) pm->held = (int)we.held;
     }
+  }
   cluster.barrier_arrive();   // (release: the pieces and their headers)
   if (MS < CS && at.rank >= MS) {   // the rest is the merging CTAs'
     cp_async_wait<0>();
@@ -191,10 +207,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_decode_small(DecodeParams P) {
   __syncthreads();            // the record rings are idle: their space holds the rest from here on
 
   const int rank = at.rank, h = at.h, b = at.b, li = at.li, layer = at.layer;
-  const int v_pk = at.v_pk, k_pk = at.k_pk, nwin = at.nwin, n_tail = at.n_tail, npc = at.npc, n_rawk = at.n_rawk, n_meta = CS == 1 ? SM::NP : at.used;
-  const __half* kt = cv.k_tail + cv.k_tail_off(layer, b, h);
-  const __half* vt = cv.v_tail + cv.v_tail_off(layer, b, h);
-  WarpPiece* const pieces = P.pieces + (size_t)at.unit * (CS * NWARP);
+  const int v_pk = at.v_pk, k_pk = at.k_pk, nwin = at.nwin, n_tail = at.n_tail, npc = at.npc, n_rawk = at.n_rawk, n_meta = COUNTED ? at.used : SM::NP;
+  const __half* kt = KEEP ? kt_kept : cv.k_tail + cv.k_tail_off(layer, b, h);
+  const __half* vt = KEEP ? vt_kept : cv.v_tail + cv.v_tail_off(layer, b, h);
+  WarpPiece* const pieces = KEEP ? pieces_kept : P.pieces + (size_t)at.unit * (CS * NWARP);
   // ---- rest of the tail, value rows and matrices
   for (int i = tid; i < (n_rawk - W) * (D / 8); i += NTHREADS)
     cp_async16(&af.k[i / (D / 8)][8 * (i % (D / 8))], kt + cv.k_slot(k_pk + W + i / (D / 8)) * D + 8 * (i % (D / 8)));
@@ -453,7 +469,7 @@ static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s
 // measured; four units: 50 and 75).  The host knows the capacity, not the lengths, and takes sequences to be full: a cache mostly
 // empty goes the way it would go full.
 // Clusters of six are for the 16 units of a layer of 4 sequences x 4 heads and a few more, one too many for clusters of eight: all six
-// blocks walk, four of them merge.
+// blocks walk, four of them merge.  Of up to four windows, which one block walks, four blocks make 0.4 us less.
 template <int FMT>
 static int small_cluster(long long units, long long windows, long long piece_slots) {
   constexpr int SIZES = 6;
@@ -463,6 +479,7 @@ static int small_cluster(long long units, long long windows, long long piece_slo
   double best_cost = 31.0 + 2.0 * (double)units * (double)windows / ((double)sm_count() * NWARP) + 0.04 * (double)units;
   for (int i = SIZES - 1; i >= 0; i--) {   // (of equals the largest cluster)
     if (fit[i] <= 0 || units * size[i] * NWARP > piece_slots) continue;   // the warps' pieces have to fit the scratch
+    if (size[i] == 6 && windows <= 4) continue;
     const double waves = (double)((units + fit[i] - 1) / fit[i]), walk = (double)((windows + NWARP * size[i] - 1) / (NWARP * size[i]));
     const double cost = waves * (11.5 + 2.1 * walk);
     if (cost < best_cost) { best_cost = cost; best = size[i]; }

@@ -28,13 +28,23 @@ def test_one_launch_decode_at_its_edges(batch, heads, n):
     Hn.assert_attention_close(got, c.gpu_decode(0, simt=True)[0])
 
 
+# four windows stay with the first block of a cluster, five are dealt out (a cluster of 16 deals from the first on)
+@pytest.mark.parametrize("batch,heads,cluster", [(7, 1, 16), (15, 1, 8), (4, 4, 6), (33, 1, 4), (74, 1, 2), (148, 1, 1)])
+@pytest.mark.parametrize("n", [32 * 4 + 3, 32 * 5])
+def test_one_launch_decode_of_a_few_windows(batch, heads, cluster, n):
+    w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=7 * heads, prefix_text=40, video_chunk=70, audio_chunk=21)
+    c = Hn.Case(w, n_tokens=n, meta_format=B.META_MXFP4 if batch % 2 else B.META_FP16)
+    assert B.decode_plan(c.cache.c, 1, 0, B.decode_workspace_bytes(c.cache, 1)) == cluster
+    Hn.assert_attention_close(c.gpu_decode(0)[0], c.gpu_decode(0, simt=True)[0])
+
+
 # 16 to 22 units: clusters of six, of which four blocks merge.  No window, one, fewer than the 72 warps, one more, several per warp
 @pytest.mark.parametrize("schedule", [B.SCHEDULE_WINDOW, B.SCHEDULE_CAPTION])
 @pytest.mark.parametrize("batch,heads,n", [(16, 1, 31), (5, 4, 32), (11, 2, 32 * 13 + 31), (4, 4, 32 * 73), (9, 2, 32 * 200 + 5)])
 def test_one_launch_decode_in_clusters_of_six(schedule, batch, heads, n):
     w = WL.scaled(WL.WORKLOADS["layer7b"], batch=batch, n_kv_heads=heads, n_q_heads=7 * heads, prefix_text=40, video_chunk=70, audio_chunk=21)
     dev = torch.device("cuda")
-    cache = B.Cache(1, batch, heads, 7 * heads, (n + W - 1) // W * W, device=dev, schedule=schedule,
+    cache = B.Cache(1, batch, heads, 7 * heads, max(8, (n + W - 1) // W) * W, device=dev, schedule=schedule,
                     meta_format=B.META_MXFP4 if batch % 2 else B.META_FP16)
     k, v = WL.gen_kv(w, 0, n_tokens=n)
     signs, R = WL.gen_signs(w, 0).to(dev), WL.gen_rotations(w, 0)[None].contiguous().to(dev)
