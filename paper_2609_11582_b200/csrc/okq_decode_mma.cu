@@ -231,15 +231,14 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
 
 // CAPTION: the captioning schedule keeps up to 159 raw values (and up to 127 raw keys) per sequence, and
 // the keys of the raw values' tokens may already be packed
-// SEQ: sequences per CTA (4 for full grids: the matrices are streamed once per four sequences; 1 when the
-// grid would otherwise leave most SMs idle, e.g. a single-layer call)
+// SEQ: sequences per CTA, one or four (combine_form below)
 template <bool CAPTION, int SEQ>
 struct CombineSmem {
   static constexpr int CB_SEQ = SEQ, CB_ROWS = SEQ * GP;
   static constexpr int TAIL = CAPTION ? CAPTION_V_SLOTS : W;   // most raw-value tokens of a sequence
-  // ring of 16-row slices of the rotation matrices; with one sequence per block it is large enough for a quarter
-  // of the columns of all three matrices, which the four-slice configuration fetches whole at the start
   static constexpr bool SPLIT = SEQ == CB_SEQ_MAX;   // the product with R_m^T on the tensor cores, from three bf16 terms
+  // one sequence per block: ring of 16-row slices of the rotation matrices, large enough for a quarter of the columns of all
+  // three matrices, which the four-slice configuration fetches whole at the start
   __align__(16) float Rbuf[SPLIT ? 4 : 3 * D * (D / 4)];
   // per partial and head: rescale factor, weight sums of the modalities (one-sequence blocks have room for the
   // partials of a long single sequence, which is spread over many CTAs of the split-K kernel)
@@ -293,7 +292,7 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
   const __half* qbase = P.q + (((size_t)li * cv.batch + bb) * cv.n_q_heads + h * G) * D;
   const __half* kt = cv.k_tail + cv.k_tail_off(layer, bb, h);
   const __half* vt = cv.v_tail + cv.v_tail_off(layer, bb, h);
-  // Scratch inside the rotated-sum array (written much later), per sequence: the raw key rows of a chunk of the
+  // Scratch inside the array of the rotated sums or of their terms (written much later), per sequence: the raw key rows of a chunk of the
   // tail (272-byte rows: 16-byte reads of 32 different rows hit different banks) or, under the captioning
   // schedule, the key parts of the up to four packed windows among the raw-value tokens; then the group's query
   // rows.  Everything is fetched with cp.async so that all the loads are in flight together.
@@ -541,7 +540,7 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
       araw[6] = fmaf(w1.z, x, araw[6]); araw[7] = fmaf(w1.w, x, araw[7]);
     }
   }
-  // (the value rows passed through scratch inside the rotated-sum array, which the merge below fills: a sequence
+  // (the value rows passed through scratch inside the array of the terms, which the merge below fills: a sequence
   // group must not start writing it while another still reads its rows)
   if (SEQ != 1) __syncthreads();
   // merge of the split-K partials, four heads at a time: per partial the twelve accumulator fragments of this
@@ -694,115 +693,114 @@ __global__ void __launch_bounds__(SEQ * 128, SEQ == CB_SEQ_MAX ? 2 : 1) k_combin
       *reinterpret_cast<float4*>(&P.out[(((size_t)li * cv.batch + ob) * cv.n_q_heads + h * G + j) * D + cl]) =
           make_float4((x.x + y.x + rv.x) * inv, (x.y + y.y + rv.y) * inv, (x.z + y.z + rv.z) * inv, (x.w + y.w + rv.w) * inv);
     }
-    return;
-  }
-
-  // out[row][c] = raw[row][c] + sum_m sum_r R_m[r][c] * vec[m][row][r].  The first half of the threads compute
-  // a 4-row x 4-column tile each; the second half stream the matrices through shared memory in 16-row
-  // slices, three slices ahead.
-  // (with the matrices preloaded there is nothing to stream: both halves compute, each every other 16-row slice)
-  constexpr bool PRE = NS == 4;
-  const int khalf = PRE ? threadIdx.x / (CB_SEQ * 64) : 0;
-  const bool comp = PRE || threadIdx.x < CB_SEQ * 64;
-  constexpr int CW = 4 / NS;          // output columns per compute thread
-  constexpr int SW = D / NS;          // output columns of this CTA = floats per staged matrix row
-  static_assert(NS == 1 || NS == 4, "column slices");
-  const int rw = ((threadIdx.x % (CB_SEQ * 64)) >> 5) * 4, cl = (threadIdx.x & 31) * CW;   // first row / column (inside the slice) of the tile
-  const float* Rset = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D + sl * SW;
-  constexpr int N_CHUNK = 3 * D / CB_CHUNK;
-  float* rbuf = &sm.Rbuf[0];          // ring of CB_NBUF slices of CB_CHUNK x SW floats (or, preloaded, all rows)
-  auto stage = [&](int chunk) {   // rows [16*chunk, 16*chunk+16) of the three stacked matrices, this CTA's columns
-    const float* src = Rset + (size_t)chunk * CB_CHUNK * D;
-    float* dst = rbuf + (chunk % CB_NBUF) * CB_CHUNK * SW;
-    if (chunk < N_CHUNK)
-      for (int i = threadIdx.x - CB_SEQ * 64; i < CB_CHUNK * SW / 4; i += CB_SEQ * 64) {
-        const int row = i / (SW / 4), c4 = i % (SW / 4);
-        cp_async16(dst + row * SW + 4 * c4, src + (size_t)row * D + 4 * c4);
-      }
-    cp_async_commit();
-  };
-  float o[4][CW];
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int k = 0; k < CW; k++) o[i][k] = 0.f;
-  if (PRELOAD) {
-    cp_async_wait<0>();
-    __syncthreads();   // the matrices have landed and vec is complete
   } else {
-    if (!comp)
-      for (int pre = 0; pre < CB_NBUF - 1; pre++) stage(pre);
-  }
-  for (int chunk = 0; chunk < N_CHUNK; chunk++) {
-    if (!PRELOAD) {
-      if (!comp) cp_async_wait<CB_NBUF - 2>();
-      __syncthreads();   // slice `chunk` has landed; everyone is done with slice chunk-1 (and, first time, vec is complete)
+    // out[row][c] = raw[row][c] + sum_m sum_r R_m[r][c] * vec[m][row][r].  The first half of the threads compute
+    // a 4-row x 4-column tile each; the second half stream the matrices through shared memory in 16-row
+    // slices, three slices ahead.
+    // (with the matrices preloaded there is nothing to stream: both halves compute, each every other 16-row slice)
+    constexpr bool PRE = NS == 4;
+    const int khalf = PRE ? threadIdx.x / 64 : 0;
+    const bool comp = PRE || threadIdx.x < 64;
+    constexpr int CW = 4 / NS;          // output columns per compute thread
+    constexpr int SW = D / NS;          // output columns of this CTA = floats per staged matrix row
+    static_assert(NS == 1 || NS == 4, "column slices");
+    const int rw = ((threadIdx.x & 63) >> 5) * 4, cl = (threadIdx.x & 31) * CW;   // first row / column (inside the slice) of the tile
+    const float* Rset = P.R + ((size_t)li * P.n_R + (P.n_R == 1 ? 0 : h)) * 3 * D * D + sl * SW;
+    constexpr int N_CHUNK = 3 * D / CB_CHUNK;
+    float* rbuf = &sm.Rbuf[0];          // ring of CB_NBUF slices of CB_CHUNK x SW floats (or, preloaded, all rows)
+    auto stage = [&](int chunk) {   // rows [16*chunk, 16*chunk+16) of the three stacked matrices, this CTA's columns
+      const float* src = Rset + (size_t)chunk * CB_CHUNK * D;
+      float* dst = rbuf + (chunk % CB_NBUF) * CB_CHUNK * SW;
+      if (chunk < N_CHUNK)
+        for (int i = threadIdx.x - 64; i < CB_CHUNK * SW / 4; i += 64) {
+          const int row = i / (SW / 4), c4 = i % (SW / 4);
+          cp_async16(dst + row * SW + 4 * c4, src + (size_t)row * D + 4 * c4);
+        }
+      cp_async_commit();
+    };
+    float o[4][CW];
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+      for (int k = 0; k < CW; k++) o[i][k] = 0.f;
+    if (PRELOAD) {
+      cp_async_wait<0>();
+      __syncthreads();   // the matrices have landed and vec is complete
+    } else {
+      if (!comp)
+        for (int pre = 0; pre < CB_NBUF - 1; pre++) stage(pre);
     }
-    if (!comp) {
-      if (!PRELOAD) stage(chunk + CB_NBUF - 1);   // into the buffer of slice chunk-1
-    } else if (!PRE || (chunk & 1) == khalf) {
-      const int m = chunk / (D / CB_CHUNK), r0 = (chunk % (D / CB_CHUNK)) * CB_CHUNK;
-      const float* rb = rbuf + (PRELOAD ? chunk : chunk % CB_NBUF) * CB_CHUNK * SW;
+    for (int chunk = 0; chunk < N_CHUNK; chunk++) {
+      if (!PRELOAD) {
+        if (!comp) cp_async_wait<CB_NBUF - 2>();
+        __syncthreads();   // slice `chunk` has landed; everyone is done with slice chunk-1 (and, first time, vec is complete)
+      }
+      if (!comp) {
+        if (!PRELOAD) stage(chunk + CB_NBUF - 1);   // into the buffer of slice chunk-1
+      } else if (!PRE || (chunk & 1) == khalf) {
+        const int m = chunk / (D / CB_CHUNK), r0 = (chunk % (D / CB_CHUNK)) * CB_CHUNK;
+        const float* rb = rbuf + (PRELOAD ? chunk : chunk % CB_NBUF) * CB_CHUNK * SW;
 #pragma unroll 2
-      for (int r = 0; r < CB_CHUNK; r += 4) {
-        float4 x[4];
+        for (int r = 0; r < CB_CHUNK; r += 4) {
+          float4 x[4];
 #pragma unroll
-        for (int i = 0; i < 4; i++) x[i] = *reinterpret_cast<const float4*>(&sm.vec[m][rw + i][r0 + r]);
-        if (NS == 1) {
-          float4 rr[4];
+          for (int i = 0; i < 4; i++) x[i] = *reinterpret_cast<const float4*>(&sm.vec[m][rw + i][r0 + r]);
+          if (NS == 1) {
+            float4 rr[4];
 #pragma unroll
-          for (int k = 0; k < 4; k++) rr[k] = *reinterpret_cast<const float4*>(&rb[(r + k) * SW + cl]);
+            for (int k = 0; k < 4; k++) rr[k] = *reinterpret_cast<const float4*>(&rb[(r + k) * SW + cl]);
 #pragma unroll
-          for (int i = 0; i < 4; i++) {
-            o[i][0] = fmaf(rr[0].x, x[i].x, o[i][0]); o[i][1 % CW] = fmaf(rr[0].y, x[i].x, o[i][1 % CW]);
-            o[i][2 % CW] = fmaf(rr[0].z, x[i].x, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[0].w, x[i].x, o[i][3 % CW]);
-            o[i][0] = fmaf(rr[1].x, x[i].y, o[i][0]); o[i][1 % CW] = fmaf(rr[1].y, x[i].y, o[i][1 % CW]);
-            o[i][2 % CW] = fmaf(rr[1].z, x[i].y, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[1].w, x[i].y, o[i][3 % CW]);
-            o[i][0] = fmaf(rr[2].x, x[i].z, o[i][0]); o[i][1 % CW] = fmaf(rr[2].y, x[i].z, o[i][1 % CW]);
-            o[i][2 % CW] = fmaf(rr[2].z, x[i].z, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[2].w, x[i].z, o[i][3 % CW]);
-            o[i][0] = fmaf(rr[3].x, x[i].w, o[i][0]); o[i][1 % CW] = fmaf(rr[3].y, x[i].w, o[i][1 % CW]);
-            o[i][2 % CW] = fmaf(rr[3].z, x[i].w, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[3].w, x[i].w, o[i][3 % CW]);
+            for (int i = 0; i < 4; i++) {
+              o[i][0] = fmaf(rr[0].x, x[i].x, o[i][0]); o[i][1 % CW] = fmaf(rr[0].y, x[i].x, o[i][1 % CW]);
+              o[i][2 % CW] = fmaf(rr[0].z, x[i].x, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[0].w, x[i].x, o[i][3 % CW]);
+              o[i][0] = fmaf(rr[1].x, x[i].y, o[i][0]); o[i][1 % CW] = fmaf(rr[1].y, x[i].y, o[i][1 % CW]);
+              o[i][2 % CW] = fmaf(rr[1].z, x[i].y, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[1].w, x[i].y, o[i][3 % CW]);
+              o[i][0] = fmaf(rr[2].x, x[i].z, o[i][0]); o[i][1 % CW] = fmaf(rr[2].y, x[i].z, o[i][1 % CW]);
+              o[i][2 % CW] = fmaf(rr[2].z, x[i].z, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[2].w, x[i].z, o[i][3 % CW]);
+              o[i][0] = fmaf(rr[3].x, x[i].w, o[i][0]); o[i][1 % CW] = fmaf(rr[3].y, x[i].w, o[i][1 % CW]);
+              o[i][2 % CW] = fmaf(rr[3].z, x[i].w, o[i][2 % CW]); o[i][3 % CW] = fmaf(rr[3].w, x[i].w, o[i][3 % CW]);
+            }
+          } else {   // one column per thread
+            const float r0v = rb[(r + 0) * SW + cl], r1v = rb[(r + 1) * SW + cl], r2v = rb[(r + 2) * SW + cl], r3v = rb[(r + 3) * SW + cl];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+              o[i][0] = fmaf(r3v, x[i].w, fmaf(r2v, x[i].z, fmaf(r1v, x[i].y, fmaf(r0v, x[i].x, o[i][0]))));
           }
-        } else {   // one column per thread
-          const float r0v = rb[(r + 0) * SW + cl], r1v = rb[(r + 1) * SW + cl], r2v = rb[(r + 2) * SW + cl], r3v = rb[(r + 3) * SW + cl];
-#pragma unroll
-          for (int i = 0; i < 4; i++)
-            o[i][0] = fmaf(r3v, x[i].w, fmaf(r2v, x[i].z, fmaf(r1v, x[i].y, fmaf(r0v, x[i].x, o[i][0]))));
         }
       }
     }
-  }
-  if (PRE) {   // the second half's sums reach the first through the tail-score array, idle by now
-    float* red = &sm.tsc_own[0] + (threadIdx.x % (CB_SEQ * 64)) * 4 * CW;
-    static_assert(!PRE || CB_SEQ * 64 * 4 * CW <= CB_SEQ * W * GP, "reduction scratch");
-    if (khalf) {
+    if (PRE) {   // the second half's sums reach the first through the tail-score array, idle by now
+      float* red = &sm.tsc_own[0] + (threadIdx.x & 63) * 4 * CW;
+      static_assert(!PRE || 64 * 4 * CW <= W * GP, "reduction scratch");
+      if (khalf) {
 #pragma unroll
-      for (int i = 0; i < 4; i++)
+        for (int i = 0; i < 4; i++)
 #pragma unroll
-        for (int k = 0; k < CW; k++) red[i * CW + k] = o[i][k];
+          for (int k = 0; k < CW; k++) red[i * CW + k] = o[i][k];
+      }
+      __syncthreads();
+      if (!khalf) {
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+          for (int k = 0; k < CW; k++) o[i][k] += red[i * CW + k];
+      }
     }
-    __syncthreads();
-    if (!khalf) {
+    if (comp && !khalf) {
 #pragma unroll
-      for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int k = 0; k < CW; k++) o[i][k] += red[i * CW + k];
-    }
-  }
-  if (comp && !khalf) {
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-      const int row = rw + i, ob = blockIdx.y * CB_SEQ + row / GP, j = row % GP;
-      if (ob >= cv.batch || j >= G) continue;
-      const float L = sm.Ls[row / GP][j];
-      const float inv = L > 0.f ? 1.0f / L : 0.f;
-      float* dst = &P.out[(((size_t)li * cv.batch + ob) * cv.n_q_heads + h * G + j) * D + sl * SW + cl];
-      if (NS == 1) {
-        const float4 rv = *reinterpret_cast<const float4*>(&sm.rawv[row][cl]);
-        *reinterpret_cast<float4*>(dst) = make_float4((o[i][0] + rv.x) * inv, (o[i][1 % CW] + rv.y) * inv,
-                                                      (o[i][2 % CW] + rv.z) * inv, (o[i][3 % CW] + rv.w) * inv);
-      } else {
-        dst[0] = (o[i][0] + sm.rawv[row][sl * SW + cl]) * inv;
+      for (int i = 0; i < 4; i++) {
+        const int row = rw + i;   // head of the group
+        if (row >= G) continue;
+        const float L = sm.Ls[0][row];
+        const float inv = L > 0.f ? 1.0f / L : 0.f;
+        float* dst = &P.out[(((size_t)li * cv.batch + b) * cv.n_q_heads + h * G + row) * D + sl * SW + cl];
+        if (NS == 1) {
+          const float4 rv = *reinterpret_cast<const float4*>(&sm.rawv[row][cl]);
+          *reinterpret_cast<float4*>(dst) = make_float4((o[i][0] + rv.x) * inv, (o[i][1 % CW] + rv.y) * inv,
+                                                        (o[i][2 % CW] + rv.z) * inv, (o[i][3 % CW] + rv.w) * inv);
+        } else {
+          dst[0] = (o[i][0] + sm.rawv[row][sl * SW + cl]) * inv;
+        }
       }
     }
   }
