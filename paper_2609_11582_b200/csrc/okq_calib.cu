@@ -14,6 +14,7 @@
 #include "../../include/okq_calib.h"
 #include "okq_calib_scores.cuh"
 #include "okq_common.cuh"
+#include "okq_device.cuh"
 #include "okq_eigen.cuh"
 
 namespace cg = cooperative_groups;
@@ -33,15 +34,6 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // One pass over the key tiles of a 128-query block of one head; scores in the log2 domain, s = (q . k) * scale2.
 //   PASS 0: rowstat[g * n + i] = (-2 m_i, 1 / l_i^2), m_i = max_j s_ij, l_i = sum_j 2^(s_ij - m_i)
@@ -157,10 +149,10 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
             for (int nt = 0; nt < 4; nt++) mx = fmaxf(mx, fmaxf(d[mt][nt][2 * hf], d[mt][nt][2 * hf + 1]));
             const float mn = fmaxf(m[mt][hf], mx * scale2);
             if (mn != -INFINITY) {
-              float a = l[mt][hf] * ex2f(m[mt][hf] - mn);   // 0 for the first finite maximum
+              float a = l[mt][hf] * ex2(m[mt][hf] - mn);   // 0 for the first finite maximum
 #pragma unroll
               for (int nt = 0; nt < 4; nt++)
-                a += ex2f(fmaf(d[mt][nt][2 * hf], scale2, -mn)) + ex2f(fmaf(d[mt][nt][2 * hf + 1], scale2, -mn));
+                a += ex2(fmaf(d[mt][nt][2 * hf], scale2, -mn)) + ex2(fmaf(d[mt][nt][2 * hf + 1], scale2, -mn));
               l[mt][hf] = a;
               m[mt][hf] = mn;
             }
@@ -172,8 +164,8 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
         for (int nt = 0; nt < 4; nt++)
 #pragma unroll
           for (int e = 0; e < 2; e++)
-            c[2 * nt + e] = fmaf(ex2f(fmaf(d[0][nt][e], two, m[0][0])), l[0][0], ex2f(fmaf(d[0][nt][2 + e], two, m[0][1])) * l[0][1]) +
-                            fmaf(ex2f(fmaf(d[1][nt][e], two, m[1][0])), l[1][0], ex2f(fmaf(d[1][nt][2 + e], two, m[1][1])) * l[1][1]);
+            c[2 * nt + e] = fmaf(ex2(fmaf(d[0][nt][e], two, m[0][0])), l[0][0], ex2(fmaf(d[0][nt][2 + e], two, m[0][1])) * l[0][1]) +
+                            fmaf(ex2(fmaf(d[1][nt][e], two, m[1][0])), l[1][0], ex2(fmaf(d[1][nt][2 + e], two, m[1][1])) * l[1][1]);
         // over the eight row groups, each lane ending with one column: n-tile bits 1, 0 and e by lane bits 4, 3, 2
 #pragma unroll
         for (int w = 4, bit = 16; w >= 1; w >>= 1, bit >>= 1) {
@@ -208,7 +200,7 @@ __global__ void __launch_bounds__(128, 3) k_calib_pass(const __half* __restrict_
         for (int dl = 1; dl < 4; dl <<= 1) {
           const float mo = __shfl_xor_sync(0xffffffffu, mm, dl), lo = __shfl_xor_sync(0xffffffffu, ll, dl);
           const float mn = fmaxf(mm, mo);
-          ll = (mm == -INFINITY ? 0.f : ll * ex2f(mm - mn)) + (mo == -INFINITY ? 0.f : lo * ex2f(mo - mn));
+          ll = (mm == -INFINITY ? 0.f : ll * ex2(mm - mn)) + (mo == -INFINITY ? 0.f : lo * ex2(mo - mn));
           mm = mn;
         }
         if (t == 0 && row[mt][hf] < n) rowstat[(size_t)head * n + row[mt][hf]] = make_float2(-2.0f * mm, 1.0f / (ll * ll));

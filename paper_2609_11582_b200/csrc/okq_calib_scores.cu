@@ -17,6 +17,7 @@
 // for which are busy 73 % of the time; the tensor pipe is a third busy.  8192 tokens x 7 heads 578 -> 195 us against the mma.sync
 // kernels of okq_calib.cu, 512 x 7 39 -> 21 (most of it the four launches).
 #include "okq_calib_scores.cuh"
+#include "okq_device.cuh"
 #include "okq_tc.cuh"
 
 namespace okq {
@@ -83,22 +84,6 @@ template <int PASS> struct Cursor {
   __device__ int qtile() const { return PASS == 0 ? t : q; }
   __device__ int ktile() const { return PASS == 0 ? pos : t; }
 };
-
-__device__ __forceinline__ float ex2a(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-  return y;
-}
-// two fp32 numbers in a register pair: one issue slot for two operations
-struct P2 { unsigned long long v; };
-__device__ __forceinline__ P2 pk(float x, float y) { P2 r; asm("mov.b64 %0, {%1, %2};\n" : "=l"(r.v) : "f"(x), "f"(y)); return r; }
-__device__ __forceinline__ float2 up(P2 a) { float2 r; asm("mov.b64 {%0, %1}, %2;\n" : "=f"(r.x), "=f"(r.y) : "l"(a.v)); return r; }
-__device__ __forceinline__ P2 padd(P2 a, P2 b) { P2 r; asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
-__device__ __forceinline__ P2 pfma(P2 a, P2 b, P2 c) {
-  P2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
 
 __device__ __forceinline__ void tma_tile(const CUtensorMap* map, void* dst, int row, int slab, uint32_t bar) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"((uint32_t)OP_BYTES) : "memory");
@@ -209,11 +194,11 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
     // ------------------------------------------------------------------ worker warps (after a timeout they run on, waits failing at once)
     const int eq = warp & 3, wq = warp >> 2;   // quarter of the lanes, quarter of the columns
     const uint32_t taddr = tmem + ((uint32_t)(eq * 32) << 16) + 32u * (uint32_t)wq;
-    const P2 two2 = pk(2.0f * scale2, 2.0f * scale2), one2 = pk(scale2, scale2);
+    const F2 two2 = f2(2.0f * scale2, 2.0f * scale2), one2 = f2(scale2, scale2);
     float m = -INFINITY, l = 0.f;              // pass 0: this thread's query over its columns
-    P2 acc[16];                                // pass 1: sums of this thread's columns over the lane's queries
+    F2 acc[16];                                // pass 1: sums of this thread's columns over the lane's queries
 #pragma unroll
-    for (int i = 0; i < 16; i++) acc[i] = pk(0.f, 0.f);
+    for (int i = 0; i < 16; i++) acc[i] = f2(0.f, 0.f);
     float tot = 0.f;                           // ... of earlier steps, one column per lane
     int items = 0;
     const int ragged = n % TS ? n / TS : -1;   // the tile that is not full
@@ -258,15 +243,15 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
         const float mn = fmaxf(m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2);
         if (!edge || mn != -INFINITY) {
           const float at = mn == -INFINITY ? 0.f : mn;   // (whole tiles of infinite keys: every term is 0)
-          const P2 neg = pk(-at, -at);
-          P2 s[2] = {pk(0.f, 0.f), pk(0.f, 0.f)};   // (on their own: a long sum takes one rounding per tile)
+          const F2 neg = f2(-at, -at);
+          F2 s[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};   // (on their own: a long sum takes one rounding per tile)
 #pragma unroll
           for (int c = 0; c < 16; c++) {
-            const float2 x = up(pfma(pk(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), one2, neg));
-            s[c & 1] = padd(s[c & 1], pk(ex2a(x.x), ex2a(x.y)));
+            const float2 x = un2(fma2(f2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), one2, neg));
+            s[c & 1] = add2(s[c & 1], f2(ex2(x.x), ex2(x.y)));
           }
-          const float2 u = up(padd(s[0], s[1]));
-          l = fmaf(l, ex2a(m - at), u.x + u.y);     // (a factor 0 for the first finite maximum)
+          const float2 u = un2(add2(s[0], s[1]));
+          l = fmaf(l, ex2(m - at), u.x + u.y);     // (a factor 0 for the first finite maximum)
           m = mn;
         }
         if (last) {
@@ -279,7 +264,7 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
 #pragma unroll
             for (int q = 0; q < 4; q++) { p[q] = sm.row[items & 1][q][32 * eq + lane]; M = fmaxf(M, p[q].x); }
 #pragma unroll
-            for (int q = 0; q < 4; q++) L += p[q].x == -INFINITY ? 0.f : p[q].y * ex2a(p[q].x - M);
+            for (int q = 0; q < 4; q++) L += p[q].x == -INFINITY ? 0.f : p[q].y * ex2(p[q].x - M);
             stat[((size_t)piece * G + head) * n + row] = sm.abort ? make_float2(NAN, NAN) : make_float2(M, L);
           }
           items++;
@@ -287,18 +272,18 @@ __global__ void __launch_bounds__(NT_ALL, 1) k_calib_scores(const __grid_constan
           l = 0.f;
         }
       } else {
-        const P2 m2 = pk(rs.x, rs.x), c2 = pk(rs.y, rs.y);
+        const F2 m2 = f2(rs.x, rs.x), c2 = f2(rs.y, rs.y);
 #pragma unroll
         for (int c = 0; c < 16; c++) {
-          const float2 x = up(pfma(pk(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), two2, m2));
-          acc[c] = pfma(pk(ex2a(x.x), ex2a(x.y)), c2, acc[c]);
+          const float2 x = un2(fma2(f2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), two2, m2));
+          acc[c] = fma2(f2(ex2(x.x), ex2(x.y)), c2, acc[c]);
         }
         // over the lanes, each ending with one column: bits 4..0 of the column by lane bits 4..0.  Every 16 steps: the exchange is
         // hidden behind the exponentials, and sums of 98 terms in one register cost a factor two in the error.
         if (last || (i & 15) == 15) {
           float v[32];
 #pragma unroll
-          for (int c = 0; c < 16; c++) { const float2 x = up(acc[c]); v[2 * c] = x.x; v[2 * c + 1] = x.y; acc[c] = pk(0.f, 0.f); }
+          for (int c = 0; c < 16; c++) { const float2 x = un2(acc[c]); v[2 * c] = x.x; v[2 * c + 1] = x.y; acc[c] = f2(0.f, 0.f); }
 #pragma unroll
           for (int w = 16; w >= 1; w >>= 1) {
             const bool upper = (lane & w) != 0;
@@ -344,7 +329,7 @@ __global__ void __launch_bounds__(256) k_calib_rows(int G, int n, int causal, lo
   for (int q = 0; q < pieces; q++) {
     const float2 x = p[(size_t)q * G * n];
     const float mn = fmaxf(M, x.x);
-    L = (M == -INFINITY ? 0.f : L * ex2a(M - mn)) + (x.x == -INFINITY ? 0.f : x.y * ex2a(x.x - mn));
+    L = (M == -INFINITY ? 0.f : L * ex2(M - mn)) + (x.x == -INFINITY ? 0.f : x.y * ex2(x.x - mn));
     M = mn;
   }
   *p = make_float2(-2.0f * M, 1.0f / (L * L));
