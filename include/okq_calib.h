@@ -34,8 +34,12 @@ size_t okq_calib_workspace_bytes(int32_t group, int32_t n);
  * over j <= i (causal != 0) or over all j.
  *   q_fp16  fp16 [group][n][128], k_fp16  fp16 [n][128], w_out  float [n]
  * Scores on the tensor cores (fp16 products, fp32 accumulation), two passes over the keys (row maximum and
- * normaliser, then the squared weights); the sums over queries are taken in a fixed order.
- * Errors: OKQ_ERR_INVALID_ARG (null, n <= 0, group <= 0), OKQ_ERR_ALIGNMENT, OKQ_ERR_WORKSPACE.
+ * normaliser, then the squared weights); the sums over queries are taken in a fixed order.  A key whose scores are -inf has the
+ * weight 0; a query without a finite score, like any NaN, makes weights of keys that it sees NaN.
+ * From 257 tokens on (positive scales) the kernels' waits are bounded: should one run out, after about two seconds of SM clocks, the call
+ * still ends by itself, and the weights of the blocks that gave up are NaN, which okq_calib_moments hands on to the moments of
+ * the tokens' modalities and okq_calib_rotation to the eigenvalues.
+ * Errors: OKQ_ERR_INVALID_ARG (null, n <= 0, group <= 0), OKQ_ERR_ALIGNMENT, OKQ_ERR_WORKSPACE, OKQ_ERR_CUDA.
  */
 okq_status okq_calib_attention_weights(const void* q_fp16, const void* k_fp16, int32_t group, int32_t n,
                                        float sm_scale, int32_t causal, void* workspace, size_t workspace_bytes,
@@ -49,7 +53,8 @@ okq_status okq_debug_calib_timeout(const void* q_fp16, const void* k_fp16, int32
 
 /*
  * C_m = sum_{j: modality_j = m} w_j v_j^T v_j for m = 0 (text), 1 (audio), 2 (video); ids > 2 count as text.
- *   v_fp16  fp16 [n][128], w  float [n] (>= 0), modality  uint8 [n], C_out  float [3][128][128]
+ *   v_fp16  fp16 [n][128], w  float [n] (>= 0; a NaN makes its modality's moments NaN), modality  uint8 [n],
+ *   C_out  float [3][128][128]
  * A weighted 128 x 128 x n contraction per modality on the tensor cores: the values are one operand as they
  * are, w_j v_j split into two fp16 terms the other (weights first scaled by a power of two so that the
  * largest is at most 1), fp32 accumulation, partial sums over token ranges added in a fixed order.
@@ -62,7 +67,7 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
  * Newton-Schulz steps towards orthogonality; cyclic Jacobi where equal eigenvalues leave the vectors undetermined, and for
  * matrices with diagonal elements below 2^-20 of the largest, whose small eigenvalues it keeps to fp32) and
  * R = H U^T with the ordering and sign convention stated above.
- *   C  float [128][128] (symmetric; only read), signs  float [128] (+-1)
+ *   C  float [128][128] (symmetric; only read; with a NaN or an infinity in it every eigenvalue is NaN), signs  float [128] (+-1)
  *   R_out  float [128][128] (row = rotated coordinate), lambda_out  float [128] (descending)
  *   workspace: at least 128 KB (checked; the solvers keep everything in shared memory and, until the call has completed on
  *   `stream`, in R_out and lambda_out: calls that overlap may share a workspace).
@@ -71,6 +76,11 @@ okq_status okq_calib_moments(const void* v_fp16, const float* w, const uint8_t* 
  */
 okq_status okq_calib_rotation(const float* C, const float* signs, void* workspace, size_t workspace_bytes,
                               float* R_out, float* lambda_out, int32_t* sweeps_out, void* stream);
+
+/* Testing aid (the paper has no counterpart): the first of okq_calib_rotation's solvers alone.  A matrix that it leaves to the Jacobi
+ * solver has NaN in lambda_out[0] and anything in R_out. */
+okq_status okq_debug_calib_direct(const float* C, const float* signs, float* R_out, float* lambda_out, int32_t* sweeps_out,
+                                  void* stream);
 
 #ifdef __cplusplus
 }

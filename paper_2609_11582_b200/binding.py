@@ -105,6 +105,8 @@ def lib():
         L.okq_debug_calib_timeout.restype = C.c_int
         L.okq_debug_calib_timeout.argtypes = [C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_size_t, C.c_void_p,
                                               C.c_int64, C.c_void_p]
+        L.okq_debug_calib_direct.restype = C.c_int
+        L.okq_debug_calib_direct.argtypes = [C.c_void_p] * 6
         L.okq_calib_moments.restype = C.c_int
         L.okq_calib_moments.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t,
                                         C.c_void_p, C.c_void_p]
@@ -139,7 +141,8 @@ def exported_symbols():
             "okq_quantize_keys", "okq_quantize_values", "okq_append", "okq_decode_attention", "okq_cache_export",
             "okq_cache_import", "okq_profile_events", "okq_decode_select", "okq_debug_decode_plan", "okq_decode_attention_simt",
             "okq_decode_attention_noalloc", "okq_quantize_values_bulk", "okq_debug_bulk_timeout", "okq_cache_export_mx",
-            "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_debug_calib_timeout", "okq_calib_moments", "okq_calib_rotation",
+            "okq_calib_workspace_bytes", "okq_calib_attention_weights", "okq_debug_calib_timeout", "okq_debug_calib_direct",
+            "okq_calib_moments", "okq_calib_rotation",
             "okq_ladder_codebook", "okq_ladder_quantize_keys", "okq_ladder_quantize_values",
             "okq_debug_ladder_timeout", "okq_ladder_decode_attention", "okq_turboquant_encode", "okq_turboquant_decode"]
 
@@ -359,6 +362,14 @@ def calib_rotation(Cm, signs, workspace, stream=None):
     sweeps = torch.zeros(1, dtype=torch.int32, device=Cm.device)
     _check(lib().okq_calib_rotation(_ptr(Cm), _ptr(signs), _ptr(workspace), workspace.numel(), _ptr(R), _ptr(lam),
                                     _ptr(sweeps), _stream(stream)), "okq_calib_rotation")
+    return R, lam, sweeps
+
+
+def debug_calib_direct(Cm, signs, stream=None):
+    """okq_debug_calib_direct: as calib_rotation, by the direct solver alone; eigenvalue 0 is NaN for a matrix that it leaves."""
+    R, lam = torch.empty_like(Cm), torch.empty(HEAD_DIM, dtype=torch.float32, device=Cm.device)
+    sweeps = torch.zeros(1, dtype=torch.int32, device=Cm.device)
+    _check(lib().okq_debug_calib_direct(_ptr(Cm), _ptr(signs), _ptr(R), _ptr(lam), _ptr(sweeps), _stream(stream)), "okq_debug_calib_direct")
     return R, lam, sweeps
 
 

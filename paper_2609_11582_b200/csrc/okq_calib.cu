@@ -854,4 +854,12 @@ okq_status okq_calib_rotation(const float* C, const float* signs, void* workspac
   return launch_status();
 }
 
+okq_status okq_debug_calib_direct(const float* C, const float* signs, float* R_out, float* lambda_out, int32_t* sweeps_out, void* stream) {
+  if (!C || !signs || !R_out || !lambda_out) return OKQ_ERR_INVALID_ARG;
+  if (!aligned16(C) || !aligned16(R_out)) return OKQ_ERR_ALIGNMENT;
+  const cudaError_t e = launch_calib_spectrum(C, signs, R_out, lambda_out, sweeps_out, static_cast<cudaStream_t>(stream));
+  if (e != cudaSuccess) { set_last_cuda_error((int)e); return OKQ_ERR_CUDA; }
+  return launch_status();
+}
+
 }  // extern "C"

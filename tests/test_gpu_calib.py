@@ -213,6 +213,37 @@ def test_rotation_of_matrices_that_are_hard_for_a_solver(kind):
     assert np.abs(U @ Cm - lam[:, None] * U).max() <= 1e-6 * size
 
 
+LEFT = {"two eigenvalues", "pairs",                            # equal eigenvalues of one tridiagonal block
+        "diagonal, repeated", "one element"}                   # diagonal elements below 2^-20 of the largest
+
+
+@pytest.mark.parametrize("kind", list(_matrices()))
+def test_direct_solver_takes_all_matrices_but_those_meant_for_the_jacobi_one(kind):
+    """So that the tests of hard matrices run the solver that they are about; calibration data is all of the direct one's."""
+    signs = torch.ones(D, device="cuda")
+    lam = B.debug_calib_direct(torch.from_numpy(_matrices()[kind]).float().contiguous().cuda(), signs)[1]
+    assert bool(lam[0].isnan()) == (kind in LEFT)
+    assert kind in LEFT or lam.isfinite().all()
+
+
+@pytest.mark.parametrize("n", [256, 1000, 4096])
+def test_direct_solver_takes_calibration_data(n):
+    q, k, v, mod, signs = _case(n)
+    ws = B.calib_workspace(7, n)
+    C = B.calib_moments(v.cuda(), B.calib_attention_weights(q.cuda(), k.cuda(), ws), mod.cuda(), ws)
+    for m in range(3):
+        assert B.debug_calib_direct(C[m].contiguous(), signs.cuda())[1].isfinite().all()
+
+
+def test_weights_that_are_none_mark_the_moments_of_their_modality():
+    _, _, v, mod, _ = _case(600)
+    w = torch.ones(600)
+    w[mod == 1] = float("nan")
+    C = B.calib_moments(v.cuda(), w.cuda(), mod.cuda(), B.calib_workspace(1, 600))
+    assert C[1].isnan().all() and C[0].isfinite().all() and C[2].isfinite().all()
+    assert B.calib_rotation(C[1].contiguous(), torch.ones(D, device="cuda"), B.calib_workspace(1, 600))[1].isnan().all()
+
+
 @pytest.mark.parametrize("decades", [0, 2, 3, 4, 5, 6])
 def test_rotation_keeps_small_eigenvalues_of_graded_matrices(decades):
     """Channels whose scales differ by up to 10^6: every eigenvalue to a few roundings of fp32, relative to itself.  Reference: singular
@@ -270,7 +301,7 @@ def test_rotation_of_numbers_that_are_none_ends():
     for bad in (float("nan"), float("inf")):
         C = torch.eye(D, device="cuda")
         C[3, 4] = C[4, 3] = bad
-        B.calib_rotation(C, signs, ws)
+        assert B.calib_rotation(C, signs, ws)[1].isnan().all()
     R, lam, _ = B.calib_rotation(torch.eye(D, device="cuda"), signs, ws)
     assert (lam == 1).all() and R.isfinite().all()
 
