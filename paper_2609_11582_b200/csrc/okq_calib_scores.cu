@@ -15,7 +15,7 @@
 //
 // What bounds it: one exponential per score and pass (16 per cycle and SM; 8192 tokens x 7 heads, causal: 51 us a pass), the units
 // for which are busy 73 % of the time; the tensor pipe is a third busy.  8192 tokens x 7 heads 578 -> 195 us against the mma.sync
-// kernels of okq_calib.cu, 512 x 7 39 -> 21 (most of it the four launches).
+// kernels of okq_calib.cu, 512 x 7 34 -> 20 (most of it the four launches).
 #include "okq_calib_scores.cuh"
 #include "okq_device.cuh"
 #include "okq_tc.cuh"

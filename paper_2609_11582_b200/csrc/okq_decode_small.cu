@@ -464,7 +464,9 @@ static cudaError_t small_launch(const DecodeParams& P, int units, cudaStream_t s
 // unit, in waves of as many as run at once (on this GPU 7 clusters of 16, 15 of 8, 22 of 6, 33 of 4, 74 of 2, 148 blocks: a cluster
 // stays inside one of eight groups of SMs): 11.5 us a wave and 2.1 us per window of a warp.  The pair: 31 us, 2 us per window
 // of a warp with the windows balanced over all warps, 0.04 us per unit in the combine kernel.  Fitted to calls of 1 to 28
-// layers, 1 to 16 sequences, 1 to 8 heads and 200 to 32768 tokens.  Where a unit's windows spread over many blocks the pair costs
+// layers, 1 to 16 sequences, 1 to 8 heads and 200 to 32768 tokens with the pieces not yet dealt out and the combine kernel's product
+// on CUDA cores; both ways have become faster since (the smallest call takes 11.3 us of the 13.6 that this says) and the
+// constants have not been fitted again.  Where a unit's windows spread over many blocks the pair costs
 // more than this says, its combine kernel merging that many partials per unit (one unit of 131072 tokens: 36 us estimated, 214
 // measured; four units: 50 and 75).  The host knows the capacity, not the lengths, and takes sequences to be full: a cache mostly
 // empty goes the way it would go full.
